@@ -2,6 +2,7 @@
 // masks, materialisation of a stage output), global average pooling, gradient accumulation,
 // the SGD-momentum update and the two loss heads.  All are bandwidth-bound passes over
 // [pixels][channels] tensors; reductions are two-stage and deterministic (no float atomics).
+#include "fin.cuh"
 #include "kernels.h"
 
 namespace ast {
@@ -163,9 +164,11 @@ struct MaskBwdOp {
     }
 };
 
+// Block sums go to the channels' accumulators (`sums`, coefficients then formed by the next reader, fin.cuh) or, where there is no
+// BatchNorm (a bias gradient), to partial[block_y][acc][c] for the finishing kernel.
 template <typename T, int V, typename OP>
 __global__ void __launch_bounds__(512) chan_reduce_kernel(OP op, size_t pixels, int c, int cw, int rows, size_t pix_per_block,
-                                                          float* __restrict__ partial) {
+                                                          float* __restrict__ partial, double* sums, float* pivot_copy) {
     pdl_wait();
     pdl_launch();
     extern __shared__ float red[];
@@ -182,6 +185,10 @@ __global__ void __launch_bounds__(512) chan_reduce_kernel(OP op, size_t pixels, 
     if (active) {
         float ctx[OP::NCTX][V];
         op.template init<T, V>(c0, ctx);
+        if (pivot_copy && blockIdx.y == 0 && row == 0) {
+#pragma unroll
+            for (int q = 0; q < V; ++q) pivot_copy[c0 + q] = ctx[0][q];
+        }
         size_t pbeg = (size_t)blockIdx.y * pix_per_block, pend = min(pixels, pbeg + pix_per_block);
         size_t p = pbeg + row;
         if (V == Vec<T>::N) {
@@ -210,7 +217,8 @@ __global__ void __launch_bounds__(512) chan_reduce_kernel(OP op, size_t pixels, 
             if (ch < c) {
                 float s = 0.f;
                 for (int r2 = 0; r2 < rows; ++r2) s += red[r2 * width + e];
-                partial[((size_t)blockIdx.y * OP::NACC + t) * c + ch] = s;
+                if (sums) add_sum(sums + (size_t)t * c + ch, s);
+                else partial[((size_t)blockIdx.y * OP::NACC + t) * c + ch] = s;
             }
         }
         __syncthreads();
@@ -245,15 +253,16 @@ ReducePlan plan_reduce(int dtype, size_t pixels, int c, int nacc, size_t scratch
 double esz(int dtype) { return dtype == 0 ? 4.0 : 2.0; }
 
 template <typename OP>
-void launch_reduce(int dtype, const ReducePlan& p, const OP& op, size_t pixels, int c, float* partial, int kind, double bytes, cudaStream_t st) {
+void launch_reduce(int dtype, const ReducePlan& p, const OP& op, size_t pixels, int c, float* partial, double* sums, float* pivot_copy, int kind, double bytes,
+                   cudaStream_t st) {
     LaunchScope ls(kind, bytes + 8.0 * c * p.by, 4.0 * pixels * c, st);
     dim3 grid(p.gx, (unsigned)p.by);
     if (dtype == 0) {
-        if (p.V == 1) launch_pdl(chan_reduce_kernel<float, 1, OP>, grid, 512, p.smem, st, op, pixels, c, p.cw, p.rows, p.ppb, partial);
-        else launch_pdl(chan_reduce_kernel<float, 4, OP>, grid, 512, p.smem, st, op, pixels, c, p.cw, p.rows, p.ppb, partial);
+        if (p.V == 1) launch_pdl(chan_reduce_kernel<float, 1, OP>, grid, 512, p.smem, st, op, pixels, c, p.cw, p.rows, p.ppb, partial, sums, pivot_copy);
+        else launch_pdl(chan_reduce_kernel<float, 4, OP>, grid, 512, p.smem, st, op, pixels, c, p.cw, p.rows, p.ppb, partial, sums, pivot_copy);
     } else {
-        if (p.V == 1) launch_pdl(chan_reduce_kernel<__nv_bfloat16, 1, OP>, grid, 512, p.smem, st, op, pixels, c, p.cw, p.rows, p.ppb, partial);
-        else launch_pdl(chan_reduce_kernel<__nv_bfloat16, 8, OP>, grid, 512, p.smem, st, op, pixels, c, p.cw, p.rows, p.ppb, partial);
+        if (p.V == 1) launch_pdl(chan_reduce_kernel<__nv_bfloat16, 1, OP>, grid, 512, p.smem, st, op, pixels, c, p.cw, p.rows, p.ppb, partial, sums, pivot_copy);
+        else launch_pdl(chan_reduce_kernel<__nv_bfloat16, 8, OP>, grid, 512, p.smem, st, op, pixels, c, p.cw, p.rows, p.ppb, partial, sums, pivot_copy);
     }
 }
 
@@ -298,8 +307,7 @@ __device__ __forceinline__ bool sum_partials(const float* __restrict__ partial, 
     return true;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(1024) bn_stats_finish(const float* __restrict__ partial, int blocks, int c, const T* __restrict__ z, double count,
+__global__ void __launch_bounds__(1024) bn_stats_finish(const float* __restrict__ partial, int blocks, int c, double count,
                                                        const float* __restrict__ gamma, const float* __restrict__ beta, float eps, float momentum,
                                                        BnFwdOut o) {
     pdl_wait();
@@ -308,10 +316,9 @@ __global__ void __launch_bounds__(1024) bn_stats_finish(const float* __restrict_
     // kernel's global loads overlap
     const int chp = blockIdx.x * 32 + (threadIdx.x & 31);
     const bool owner = (threadIdx.x >> 5) == 0 && chp < c;
-    // pivot: the first pixel's value, or (z == nullptr: partials written by the producing kernel) the running mean
-    // as it stands before this update
+    // pivot: the running mean as it stands before this update (what the producing kernel subtracted)
     const float rm = owner ? o.run_mean[chp] : 0.f, rv = owner ? o.run_var[chp] : 0.f;
-    const float pv = owner ? (z ? to_f<T>(z[chp]) : rm) : 0.f, gm = owner ? gamma[chp] : 0.f, bt = owner ? beta[chp] : 0.f;
+    const float pv = rm, gm = owner ? gamma[chp] : 0.f, bt = owner ? beta[chp] : 0.f;
     int ch;
     double s1, s2;
     if (!sum_partials(partial, blocks, c, ch, s1, s2)) return;
@@ -454,10 +461,12 @@ template <typename T> __global__ void gap_bwd_kernel(const T* __restrict__ da, i
 }
 
 // ------------------------------------------------------------------ parameters
-__global__ void accumulate_kernel(float* __restrict__ G, const float* __restrict__ g, size_t n4, size_t n) {
+// Also sets the accumulators of the next backward pass's channel sums to zero: every pass is followed by its accumulate.
+__global__ void accumulate_kernel(float* __restrict__ G, const float* __restrict__ g, size_t n4, size_t n, double* __restrict__ zero, size_t n_zero) {
     pdl_wait();
     pdl_launch();
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (size_t k = i; k < n_zero; k += (size_t)gridDim.x * blockDim.x) zero[k] = 0.0;
     if (i < n4) {
         float4 a = reinterpret_cast<float4*>(G)[i];
         float4 b = reinterpret_cast<const float4*>(g)[i];
@@ -665,46 +674,64 @@ __global__ void __launch_bounds__(256) xent_kernel(const T* __restrict__ logits,
 }  // namespace
 
 // =================================================================== launchers
-void bn_stats(int dtype, const void* z, size_t pixels, int c, const float* gamma, const float* beta, float eps, float momentum, float* scratch,
-              size_t scratch_floats, const BnFwdOut& o, cudaStream_t st) {
+void bn_stats(int dtype, const void* z, size_t pixels, int c, const BnSumsOut& so, size_t scratch_floats, cudaStream_t st) {
     ReducePlan p = plan_reduce(dtype, pixels, c, 2, scratch_floats);
     StatsOp op{z};
-    launch_reduce(dtype, p, op, pixels, c, scratch, K_BN_STATS, (double)pixels * c * esz(dtype), st);
-    LaunchScope ls(K_BN_STATS_FINISH, 8.0 * c * (p.by + 4), 10.0 * c, st);
-    if (dtype == 0)
-        launch_pdl(bn_stats_finish<float>, (c + 31) / 32, 1024, 0, st, scratch, (int)p.by, c, (const float*)z, (double)pixels, gamma, beta, eps, momentum, o);
-    else
-        launch_pdl(bn_stats_finish<__nv_bfloat16>, (c + 31) / 32, 1024, 0, st, scratch, (int)p.by, c, (const __nv_bfloat16*)z, (double)pixels, gamma, beta, eps,
-                                                                       momentum, o);
+    launch_reduce(dtype, p, op, pixels, c, nullptr, so.sums, so.pivot_copy, K_BN_STATS, (double)pixels * c * esz(dtype), st);
 }
 
 void bn_stats_finish_partials(const float* partial, int blocks, size_t pixels, int c, const float* gamma, const float* beta, float eps,
                               float momentum, const BnFwdOut& o, cudaStream_t st) {
     LaunchScope ls(K_BN_STATS_FINISH, 8.0 * c * (blocks + 4), 10.0 * c, st);
-    launch_pdl(bn_stats_finish<float>, (c + 31) / 32, 1024, 0, st, partial, blocks, c, (const float*)nullptr, (double)pixels, gamma, beta, eps, momentum,
-               o);
+    launch_pdl(bn_stats_finish, (c + 31) / 32, 1024, 0, st, partial, blocks, c, (double)pixels, gamma, beta, eps, momentum, o);
 }
 
 void bn_bwd_reduce(int dtype, const void* dy, const void* z, size_t pixels, int c, const float* scale, const float* shift, int act,
-                   const float* mean, const float* rstd, const float* gamma, float* scratch, size_t scratch_floats, const BnBwdOut& o,
-                   cudaStream_t st) {
+                   const float* mean, const float* rstd, double* sums, size_t scratch_floats, cudaStream_t st) {
     ReducePlan p = plan_reduce(dtype, pixels, c, 2, scratch_floats);
     BwdOp op{GradSrc{dy, z, scale, shift, nullptr, nullptr, nullptr, act}, mean, rstd, act == ACT_NONE ? -INFINITY : 0.f,
              act == ACT_RELU6 ? 6.f : INFINITY};
-    launch_reduce(dtype, p, op, pixels, c, scratch, K_BN_BWD_REDUCE, (double)pixels * c * esz(dtype) * ((act != ACT_NONE || mean) ? 2.0 : 1.0), st);
+    launch_reduce(dtype, p, op, pixels, c, nullptr, sums, nullptr, K_BN_BWD_REDUCE, (double)pixels * c * esz(dtype) * ((act != ACT_NONE || mean) ? 2.0 : 1.0), st);
+}
+
+void bias_grad(int dtype, const void* dy, const void* z, size_t pixels, int c, int act, float* scratch, size_t scratch_floats, float* db, cudaStream_t st) {
+    ReducePlan p = plan_reduce(dtype, pixels, c, 2, scratch_floats);
+    BwdOp op{GradSrc{dy, z, nullptr, nullptr, nullptr, nullptr, nullptr, act}, nullptr, nullptr, act == ACT_NONE ? -INFINITY : 0.f, act == ACT_RELU6 ? 6.f : INFINITY};
+    launch_reduce(dtype, p, op, pixels, c, scratch, nullptr, nullptr, K_BN_BWD_REDUCE, (double)pixels * c * esz(dtype) * (act != ACT_NONE ? 2.0 : 1.0), st);
     LaunchScope ls(K_BN_BWD_FINISH, 8.0 * c * (p.by + 4), 10.0 * c, st);
-    launch_pdl(bn_bwd_finish, (c + 31) / 32, 1024, 0, st, scratch, (int)p.by, c, (double)pixels, mean, rstd, gamma, o);
+    launch_pdl(bn_bwd_finish, (c + 31) / 32, 1024, 0, st, scratch, (int)p.by, c, (double)pixels, (const float*)nullptr, (const float*)nullptr,
+               (const float*)nullptr, BnBwdOut{nullptr, db, nullptr, nullptr, nullptr});
 }
 
 bool ew_relu_mask_bn_sums(int dtype, const void* d, const void* out_val, const void* z, size_t pixels, int c, const float* mean, const float* rstd,
-                          const float* gamma, void* dst, float* scratch, size_t scratch_floats, const BnBwdOut& o, cudaStream_t st) {
+                          void* dst, double* sums, size_t scratch_floats, cudaStream_t st) {
     if (c % (dtype == 0 ? 4 : 8)) return false;          // whole vectors per thread (the op stores what it loads)
     ReducePlan p = plan_reduce(dtype, pixels, c, 2, scratch_floats);
     MaskBwdOp op{d, out_val, z, dst, mean, rstd};
-    launch_reduce(dtype, p, op, pixels, c, scratch, K_EW_MASK, (double)pixels * c * esz(dtype) * 4.0, st);
-    LaunchScope ls(K_BN_BWD_FINISH, 8.0 * c * (p.by + 4), 10.0 * c, st);
-    launch_pdl(bn_bwd_finish, (c + 31) / 32, 1024, 0, st, scratch, (int)p.by, c, (double)pixels, mean, rstd, gamma, o);
+    launch_reduce(dtype, p, op, pixels, c, nullptr, sums, nullptr, K_EW_MASK, (double)pixels * c * esz(dtype) * 4.0, st);
     return true;
+}
+
+// ---- pending coefficients settled by a kernel of their own: in front of a kernel that cannot form them itself
+__global__ void __launch_bounds__(128) bn_settle_fwd_kernel(BnPendFwd b) {
+    pdl_wait();
+    pdl_launch();
+    const int ch = blockIdx.x * 128 + threadIdx.x;
+    if (ch < b.c) bn_fwd_coef(b, ch, true);
+}
+__global__ void __launch_bounds__(128) bn_settle_bwd_kernel(BnPendBwd b) {
+    pdl_wait();
+    pdl_launch();
+    const int ch = blockIdx.x * 128 + threadIdx.x;
+    if (ch < b.c) bn_bwd_coef(b, ch, true);
+}
+void bn_settle_fwd(const BnPendFwd& b, cudaStream_t st) {
+    LaunchScope ls(K_BN_STATS_FINISH, 52.0 * b.c, 10.0 * b.c, st);
+    launch_pdl(bn_settle_fwd_kernel, (b.c + 127) / 128, 128, 0, st, b);
+}
+void bn_settle_bwd(const BnPendBwd& b, cudaStream_t st) {
+    LaunchScope ls(K_BN_BWD_FINISH, 48.0 * b.c, 10.0 * b.c, st);
+    launch_pdl(bn_settle_bwd_kernel, (b.c + 127) / 128, 128, 0, st, b);
 }
 
 void bn_bwd_finish_partials(const float* partial, int blocks, size_t pixels, int c, const float* mean, const float* rstd, const float* gamma,
@@ -716,21 +743,46 @@ void bn_bwd_finish_partials(const float* partial, int blocks, size_t pixels, int
 // Vector form with the per-channel coefficients in registers: the grid's threads are cut to a multiple of the vectors per
 // pixel, so that a thread striding by that count always lands on the same channels; four vectors of each operand are
 // loaded before any is used.
-template <typename T, int V>
-__global__ void __launch_bounds__(256) ew_add_vec_kernel(ValSrc a, ValSrc b, int act, size_t groups, int vpr, size_t stride, T* __restrict__ out,
-                                                          T* __restrict__ out2) {
+// PEND: coefficients of an operand may still be sums (fin.cuh); each block forms those of all channels in shared memory.
+template <typename T, int V, bool PEND>
+__global__ void __launch_bounds__(256) ew_add_vec_kernel(ValSrc a, ValSrc b, BnPendFwd pa, BnPendFwd pb, int act, size_t groups, int vpr, size_t stride,
+                                                          T* __restrict__ out, T* __restrict__ out2) {
     pdl_wait();
     pdl_launch();
+    extern __shared__ float coef[];           // [2][2][c]: scale and shift of a and b
+    if (PEND) {
+        const int c = vpr * V;
+        for (int i = threadIdx.x; i < 2 * c; i += 256) {
+            const bool second = i >= c;
+            const int ch = second ? i - c : i;
+            const BnPendFwd& p = second ? pb : pa;
+            const ValSrc& v = second ? b : a;
+            float2 k = make_float2(1.f, 0.f);
+            if (p.sums) k = bn_fwd_coef(p, ch, blockIdx.x == 0);
+            else if (v.scale) k = make_float2(v.scale[ch], v.shift[ch]);
+            coef[(second ? 2 * c : 0) + ch] = k.x;
+            coef[(second ? 3 * c : c) + ch] = k.y;
+        }
+        __syncthreads();
+    }
     const size_t id = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= stride) return;
     const int c0 = (int)(id % (size_t)vpr) * V;
     float as[V], ah[V], bs[V], bh[V];
 #pragma unroll
     for (int q = 0; q < V; ++q) {
-        as[q] = a.scale ? __ldg(a.scale + c0 + q) : 1.f;
-        ah[q] = a.scale ? __ldg(a.shift + c0 + q) : 0.f;
-        bs[q] = (b.p && b.scale) ? __ldg(b.scale + c0 + q) : 1.f;
-        bh[q] = (b.p && b.scale) ? __ldg(b.shift + c0 + q) : 0.f;
+        if (PEND) {
+            const int c = vpr * V;
+            as[q] = coef[c0 + q];
+            ah[q] = coef[c + c0 + q];
+            bs[q] = coef[2 * c + c0 + q];
+            bh[q] = coef[3 * c + c0 + q];
+        } else {
+            as[q] = a.scale ? __ldg(a.scale + c0 + q) : 1.f;
+            ah[q] = a.scale ? __ldg(a.shift + c0 + q) : 0.f;
+            bs[q] = (b.p && b.scale) ? __ldg(b.scale + c0 + q) : 1.f;
+            bh[q] = (b.p && b.scale) ? __ldg(b.shift + c0 + q) : 0.f;
+        }
     }
     const float alo = a.act == ACT_NONE ? -INFINITY : 0.f, ahi = a.act == ACT_RELU6 ? 6.f : INFINITY;
     const float blo = b.act == ACT_NONE ? -INFINITY : 0.f, bhi = b.act == ACT_RELU6 ? 6.f : INFINITY;
@@ -770,13 +822,15 @@ __global__ void __launch_bounds__(256) ew_add_vec_kernel(ValSrc a, ValSrc b, int
     }
 }
 
-template <typename T, int V> static void ew_add_launch(const ValSrc& a, const ValSrc& b, int act, size_t n, int c, void* out, void* out2, cudaStream_t st) {
+template <typename T, int V> static void ew_add_launch(const ValSrc& a, const ValSrc& b, const BnPendFwd& pa, const BnPendFwd& pb, int act, size_t n, int c, void* out, void* out2, cudaStream_t st) {
     size_t groups = n / V;
     LaunchScope ls(K_EW_ADD, (double)n * sizeof(T) * (1 + (b.p ? 1 : 0) + 1 + (out2 ? 1 : 0)), (double)n, st);
     if (V > 1) {
         const int vpr = c / V;
         size_t blocks = (groups + 4 * 256 - 1) / (4 * 256);
-        const size_t cap = (size_t)sm_count() * 8;
+        const bool pend = pa.sums || pb.sums;
+        // with pending coefficients every block first forms those of all channels: fewer, longer blocks
+        const size_t cap = (size_t)sm_count() * (pend ? 4 : 8);
         if (blocks > cap) blocks = cap;
         size_t threads = blocks * 256;
         if (threads < (size_t)vpr) {
@@ -784,26 +838,56 @@ template <typename T, int V> static void ew_add_launch(const ValSrc& a, const Va
             threads = blocks * 256;
         }
         const size_t stride = threads / vpr * vpr;
-        launch_pdl(ew_add_vec_kernel<T, V>, (unsigned)blocks, 256, 0, st, a, b, act, groups, vpr, stride, (T*)out, (T*)out2);
+        if (pend) launch_pdl(ew_add_vec_kernel<T, V, true>, (unsigned)blocks, 256, (size_t)16 * c, st, a, b, pa, pb, act, groups, vpr, stride, (T*)out, (T*)out2);
+        else launch_pdl(ew_add_vec_kernel<T, V, false>, (unsigned)blocks, 256, 0, st, a, b, pa, pb, act, groups, vpr, stride, (T*)out, (T*)out2);
         return;
     }
     launch_pdl(ew_add_kernel<T, V>, (unsigned)((groups + 255) / 256), 256, 0, st, a, b, act, groups, c, (T*)out, (T*)out2);
 }
 
-void ew_add(int dtype, const ValSrc& a, const ValSrc& b, int act, size_t pixels, int c, void* out, void* out2, cudaStream_t st) {
+// channel counts whose pending coefficients ew_add forms itself: whole vectors, and the shared memory a kernel has without asking
+bool ew_takes_pending(int dtype, int c) { return c % (dtype == 0 ? 4 : 8) == 0 && c <= 3072; }
+
+void ew_add(int dtype, const ValSrc& a, const ValSrc& b, const BnPendFwd& pa, const BnPendFwd& pb, int act, size_t pixels, int c, void* out, void* out2,
+            cudaStream_t st) {
     size_t n = pixels * c;
     if (dtype == 0) {
-        if (c % 4 == 0) ew_add_launch<float, 4>(a, b, act, n, c, out, out2, st);
-        else ew_add_launch<float, 1>(a, b, act, n, c, out, out2, st);
+        if (c % 4 == 0) ew_add_launch<float, 4>(a, b, pa, pb, act, n, c, out, out2, st);
+        else ew_add_launch<float, 1>(a, b, pa, pb, act, n, c, out, out2, st);
     } else {
-        if (c % 8 == 0) ew_add_launch<__nv_bfloat16, 8>(a, b, act, n, c, out, out2, st);
-        else ew_add_launch<__nv_bfloat16, 1>(a, b, act, n, c, out, out2, st);
+        if (c % 8 == 0) ew_add_launch<__nv_bfloat16, 8>(a, b, pa, pb, act, n, c, out, out2, st);
+        else ew_add_launch<__nv_bfloat16, 1>(a, b, pa, pb, act, n, c, out, out2, st);
     }
 }
 
-void ew_apply(int dtype, const ValSrc& a, size_t pixels, int c, void* out, cudaStream_t st) {
+void ew_apply(int dtype, const ValSrc& a, const BnPendFwd& pa, size_t pixels, int c, void* out, cudaStream_t st) {
     ValSrc none{nullptr, nullptr, nullptr, 0};
-    ew_add(dtype, a, none, ACT_NONE, pixels, c, out, nullptr, st);
+    ew_add(dtype, a, none, pa, BnPendFwd{}, ACT_NONE, pixels, c, out, nullptr, st);
+}
+
+// dst = src (16-byte units), and n_zero doubles set to zero by the same launch
+__global__ void __launch_bounds__(256) slot_copy_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t n, double* __restrict__ zero, size_t n_zero) {
+    pdl_wait();
+    pdl_launch();
+    const size_t stride = (size_t)gridDim.x * 256, id = (size_t)blockIdx.x * 256 + threadIdx.x;
+    for (size_t i = id; i < n_zero; i += stride) zero[i] = 0.0;
+    for (size_t i = id; i < n; i += 4 * stride) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u * stride < n) v[u] = src[i + u * stride];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u * stride < n) dst[i + u * stride] = v[u];
+    }
+}
+bool slot_copy(const void* src, void* dst, size_t bytes, double* zero, size_t n_zero, cudaStream_t st) {
+    if (bytes % 16 || (reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) % 16) return false;
+    LaunchScope ls(K_EW_ADD, 2.0 * bytes, 0.0, st);
+    size_t blocks = (bytes / 16 + 1023) / 1024;
+    const size_t cap = (size_t)sm_count() * 8;
+    launch_pdl(slot_copy_kernel, (unsigned)(blocks < 1 ? 1 : blocks > cap ? cap : blocks), 256, 0, st, (const uint4*)src, (uint4*)dst, bytes / 16, zero, n_zero);
+    return true;
 }
 
 template <typename T, int V> static void ew_flat_launch(int mode, const void* a, const void* b, size_t n, void* dst, cudaStream_t st) {
@@ -853,11 +937,11 @@ void gap_bwd(int dtype, const void* da, int n, int hw, int c, const void* addend
     else launch_pdl(gap_bwd_kernel<__nv_bfloat16>, blocks, 256, 0, st, (const __nv_bfloat16*)da, n, hw, c, (const __nv_bfloat16*)addend, (__nv_bfloat16*)dx);
 }
 
-void accumulate(float* G, const float* g, size_t n, cudaStream_t st) {
+void accumulate(float* G, const float* g, size_t n, double* zero, size_t n_zero, cudaStream_t st) {
     if (!n) return;
     size_t n4 = n / 4, threads = n4 + (n - n4 * 4);
     LaunchScope ls(K_ACCUMULATE, 12.0 * n, (double)n, st);
-    launch_pdl(accumulate_kernel, (unsigned)((threads + 255) / 256), 256, 0, st, G, g, n4, n);
+    launch_pdl(accumulate_kernel, (unsigned)((threads + 255) / 256), 256, 0, st, G, g, n4, n, zero, n_zero);
 }
 
 void sgd_step(float* w, float* v, float* G, size_t n, float inv_m, float lr, float mu, cudaStream_t st) {

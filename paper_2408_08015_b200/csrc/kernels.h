@@ -69,6 +69,38 @@ bool tracing();
 // records `msg` as the calling thread's last error and returns `code`
 int report_error(int code, const char* msg);
 
+struct BnFwdOut {
+    float *mean, *rstd, *scale, *shift, *run_mean, *run_var;
+};
+struct BnBwdOut {
+    float *dgamma, *dbeta, *k1, *k2, *k3;   // dgamma/k* null: only dbeta = sum of dpre (bias gradient)
+};
+// A BatchNorm whose sums have been taken and whose coefficients the next kernel that reads its tensor forms (fin.cuh).
+// sums: [2][c] doubles; sums == nullptr: nothing is pending, the coefficients are in memory.
+struct BnPendFwd {
+    const double* sums;
+    const float* pivot;      // what the producer subtracted (its copy: the running mean is updated by the reader)
+    const float *gamma, *beta;
+    double inv_count, unbias;
+    float eps, momentum;
+    int c;
+    BnFwdOut o;
+};
+struct BnPendBwd {
+    const double* sums;
+    const float *gamma, *mean, *rstd;
+    double inv_count;
+    int c;
+    BnBwdOut o;
+};
+// Where a kernel leaves the sums of the tensor it writes: accumulators [2][c] (zero at its start), forward the pivot it
+// subtracts (the running mean) and the place of its copy.
+struct BnSumsOut {
+    double* sums;
+    const float* pivot;
+    float* pivot_copy;
+};
+
 // BatchNorm-backward reduction fused into the kernel that writes the gradient dy of a conv->BN->activation unit's
 // output: z is that unit's raw conv output, scale/shift/mean/rstd its forward statistics, act its activation.
 struct BnRed {
@@ -112,6 +144,7 @@ int pw_bwd_data_tc(const ConvGeom& g, const GradSrc& dz, const __nv_bfloat16* wt
 // (bwd == false: x [P][K], w = [N][K]) or backward-data (bwd == true: dz [P][K], w = transposed weights [N][K]); false = does not fit
 bool pw_stream(bool bwd, int P, int K, int N, const ValSrc& x, const GradSrc& dz, const __nv_bfloat16* w, const void* addend, void* out, int* err,
                int kind, double bytes, cudaStream_t st);
+bool pw_wgrad_pipeline_fits(const ConvGeom& g, bool need_z, size_t scratch_floats);
 // gw[co][ci]; per-CTA partial sums in scratch, summed in fixed order by a second kernel
 void pw_bwd_weight_tc(const ConvGeom& g, const GradSrc& dz, const ValSrc& x, float* scratch, size_t scratch_floats, float* gw, int* err,
                       cudaStream_t st);
@@ -151,34 +184,37 @@ void dw_bwd_weight(int dtype, const ConvGeom& g, const GradSrc& dz, const ValSrc
                    float* gw, cudaStream_t st);
 
 // ---- BatchNorm statistics and backward reductions over a [pixels][c] tensor ----
-struct BnFwdOut {
-    float *mean, *rstd, *scale, *shift, *run_mean, *run_var;
-};
-void bn_stats(int dtype, const void* z, size_t pixels, int c, const float* gamma, const float* beta, float eps, float momentum,
-              float* scratch, size_t scratch_floats, const BnFwdOut& o, cudaStream_t st);
+// sums of a [pixels][c] tensor of its own pass; the coefficients are then pending (fin.cuh)
+void bn_stats(int dtype, const void* z, size_t pixels, int c, const BnSumsOut& so, size_t scratch_floats, cudaStream_t st);
 // finishing step alone, for statistics partials written by the producing kernel; the pivot is the running mean
 // as it stood before this call (the value the producer read)
 void bn_stats_finish_partials(const float* partial, int blocks, size_t pixels, int c, const float* gamma, const float* beta, float eps,
                               float momentum, const BnFwdOut& o, cudaStream_t st);
-struct BnBwdOut {
-    float *dgamma, *dbeta, *k1, *k2, *k3;   // dgamma/k* null: only dbeta = sum of dpre (bias gradient)
-};
 void bn_bwd_reduce(int dtype, const void* dy, const void* z, size_t pixels, int c, const float* scale, const float* shift, int act,
-                   const float* mean, const float* rstd, const float* gamma, float* scratch, size_t scratch_floats,
-                   const BnBwdOut& o, cudaStream_t st);
+                   const float* mean, const float* rstd, double* sums, size_t scratch_floats, cudaStream_t st);
+// db[c] = sum over the pixels of dy inside the activation's linear region
+void bias_grad(int dtype, const void* dy, const void* z, size_t pixels, int c, int act, float* scratch, size_t scratch_floats, float* db, cudaStream_t st);
+// pending coefficients formed by a kernel of their own
+void bn_settle_fwd(const BnPendFwd& b, cudaStream_t st);
+void bn_settle_bwd(const BnPendBwd& b, cudaStream_t st);
 
 // finishing step alone, for partial sums written by the kernel that produced dy
 void bn_bwd_finish_partials(const float* partial, int blocks, size_t pixels, int c, const float* mean, const float* rstd, const float* gamma,
                             const BnBwdOut& o, cudaStream_t st);
 
 // ---- elementwise over [pixels][c] ----
-void ew_add(int dtype, const ValSrc& a, const ValSrc& b, int act, size_t pixels, int c, void* out, void* out2, cudaStream_t st);
-void ew_apply(int dtype, const ValSrc& a, size_t pixels, int c, void* out, cudaStream_t st);
+// pa, pb: pending coefficients of the operands (sums null: none); ew_takes_pending says for which channel counts they may be given
+bool ew_takes_pending(int dtype, int c);
+void ew_add(int dtype, const ValSrc& a, const ValSrc& b, const BnPendFwd& pa, const BnPendFwd& pb, int act, size_t pixels, int c, void* out, void* out2,
+            cudaStream_t st);
+void ew_apply(int dtype, const ValSrc& a, const BnPendFwd& pa, size_t pixels, int c, void* out, cudaStream_t st);
+// dst = src, and n_zero doubles set to zero; false: not 16-byte aligned, nothing launched
+bool slot_copy(const void* src, void* dst, size_t bytes, double* zero, size_t n_zero, cudaStream_t st);
 void ew_relu_mask(int dtype, const void* d, const void* out_val, size_t n, void* dst, cudaStream_t st);
-// the same, fused with the BatchNorm-backward sums (and finishing step) of the operand branch whose raw conv output is z and whose
-// BatchNorm has no activation: dst's sums are that BatchNorm's; false = channel count not a whole number of vectors, nothing launched
+// the same, fused with the BatchNorm-backward sums of the operand branch whose raw conv output is z and whose BatchNorm has no
+// activation: dst's sums are that BatchNorm's; false = channel count not a whole number of vectors, nothing launched
 bool ew_relu_mask_bn_sums(int dtype, const void* d, const void* out_val, const void* z, size_t pixels, int c, const float* mean, const float* rstd,
-                          const float* gamma, void* dst, float* scratch, size_t scratch_floats, const BnBwdOut& o, cudaStream_t st);
+                          void* dst, double* sums, size_t scratch_floats, cudaStream_t st);
 void ew_sum(int dtype, const void* a, const void* b, size_t n, void* dst, cudaStream_t st);
 // bfloat16, channel counts multiples of 8: zero-inserted gradient / subsampled output of a stride-2 3x3 conv (see conv3_s2_tc_supported)
 void ew_upsample2_grad(const GradSrc& d, int n, int hi, int wi, int ho, int wo, int c, void* up, cudaStream_t st);
@@ -203,7 +239,8 @@ void dwk_bwd_data(int dtype, const ConvGeom& g, const GradSrc& dz, const float* 
 void dwk_bwd_weight(int dtype, const ConvGeom& g, const GradSrc& dz, const ValSrc& x, float* scratch, size_t scratch_floats, float* gw, cudaStream_t st);
 
 // ---- parameters ----
-void accumulate(float* G, const float* g, size_t n, cudaStream_t st);
+// G += g; n_zero doubles set to zero
+void accumulate(float* G, const float* g, size_t n, double* zero, size_t n_zero, cudaStream_t st);
 void sgd_step(float* w, float* v, float* G, size_t n, float inv_m, float lr, float mu, cudaStream_t st);
 // derived[i] = w[perm[i]]; wb[i] = bf16(w[i]); wtb[i] = bf16(w[perm[i]])  (wb/wtb may be null)
 void refresh_derived(const float* w, const int32_t* perm, float* derived, __nv_bfloat16* wb, __nv_bfloat16* wtb, size_t n, cudaStream_t st);

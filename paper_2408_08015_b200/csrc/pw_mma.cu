@@ -1,0 +1,165 @@
+// Launch side of the register-operand pointwise kernels (pw_mma.cuh): instantiations, shared-memory layout and the choice of a
+// tiling for a layer.
+#include <string.h>
+
+#include "pw_mma.cuh"
+#include "pw_mma.h"
+
+namespace ast {
+namespace {
+
+using namespace mma;
+
+typedef void (*KernelFn)(const Args);
+
+template <bool BWD, int NJ, int G, int XF> KernelFn pick(int mi, int wk) {
+    if (wk == 1) return mi == 1 ? pw_mma_kernel<BWD, 1, NJ, G, XF> : pw_mma_kernel<BWD, 2, NJ, G, XF>;
+    return wk == 2 ? pw_mma_split_kernel<BWD, NJ, G, 2, XF> : wk == 4 ? pw_mma_split_kernel<BWD, NJ, G, 4, XF> : pw_mma_split_kernel<BWD, NJ, G, 8, XF>;
+}
+template <bool BWD, int XF> KernelFn by_columns(const MmaTiling& c) {
+    switch (c.nj) {
+        case 2: return pick<BWD, 2, 2, XF>(c.mi, c.wk);
+        case 3: return pick<BWD, 3, 1, XF>(c.mi, c.wk);
+        case 4: return pick<BWD, 4, 4, XF>(c.mi, c.wk);
+        case 6: return pick<BWD, 6, 2, XF>(c.mi, c.wk);
+        default: return pick<BWD, 8, 4, XF>(c.mi, c.wk);
+    }
+}
+template <bool BWD> KernelFn kernel_for(const MmaTiling& c, int xf) {
+    return xf == XF_NONE ? by_columns<BWD, XF_NONE>(c) : xf == XF_AFFINE ? by_columns<BWD, XF_AFFINE>(c) : by_columns<BWD, XF_ACT>(c);
+}
+// the shared-memory limit of every instantiation, raised once per device
+template <bool BWD> void raise_limits() {
+    static std::atomic<unsigned long long> done{0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (done.load(std::memory_order_acquire) & bit) return;
+    for (int nj : {2, 3, 4, 6, 8})
+        for (int v = 0; v < 5; ++v)
+            for (int xf = XF_NONE; xf <= XF_ACT; ++xf) {
+                MmaTiling c{};
+                c.nj = nj;
+                c.mi = v == 1 ? 2 : 1;
+                c.wk = v < 2 ? 1 : 1 << (v - 1);
+                cudaFuncSetAttribute(kernel_for<BWD>(c, xf), cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+            }
+    done.fetch_or(bit, std::memory_order_release);
+}
+
+uint32_t w_pitch(int K) {
+    uint32_t b = (uint32_t)((K + 31) / 32) * 64u;      // whole 32-channel chunks
+    return b % 128 == 0 ? b + 64 : b;                  // an odd multiple of 64 bytes: a fragment read meets every bank once
+}
+
+}  // namespace
+
+// Which layers run here and how they are tiled.  Times below: one layer with its BatchNorm sums in a captured chain of launches, inputs
+// of large layers from HBM; "before" is the tensor-memory pipeline (or, above 256 channels, the one-tile / streaming kernels of
+// pw_tc.cu and pw_stream.cu) with its finishing kernel.
+//   - More than 256 x 64 products per pixel on more than 50 000 pixels: the arithmetic of mma.sync (and the shared-memory reads of its
+//     weights) is what bounds such a layer and the tensor-memory pipeline is as fast or faster (64 -> 256 at 100 352 pixels: 26.4 us
+//     against 27.4; 256 -> 128: 33.4 against 39.8).  It takes at most 256 channels a side, so wider layers run here (128 -> 512 at
+//     25 088 pixels: 33.5 -> 22.7 us; 512 -> 128: 27.4 -> 22.8).
+//   - A reduction of at most 192 channels, or at least 6 000 pixels, or twice as many output as reduction channels: the persistent
+//     form (24 -> 144 at 100 352 pixels 18.7 -> 13.8 us, backward 26.1 -> 24.2; 144 -> 24: 20.2 -> 12.7 and 30.4 -> 22.9; 160 -> 960 at 784
+//     pixels 18.4 -> 5.3 and 21.5 -> 6.8).
+//   - Else the split form: as many warps on the reduction as it takes to give the chip about one (backward) or one and a
+//     half (forward) CTAs per multiprocessor (960 -> 160 at 784 pixels 40.9 -> 6.9 us, backward 53.0 -> 9.8; 384 -> 64 at 784: 13.0 ->
+//     3.9 and 21.7 -> 4.6).
+bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {
+    if (K % 8 || N % 8 || (double)P * (K > N ? K : N) * 2.0 >= 4.0e9) return false;
+    if (P >= 50000 && K <= 256 && N <= 256 && K * N >= 256 * 64) return false;
+    const int KCH = (K + 31) / 32, sms = sm_count();
+    MmaTiling c{};
+    c.mi = 1; c.wm = 8; c.wn = 1; c.wk = 1; c.ctas = 1;
+    auto cols = [&](int nj) { return (N + 8 * nj - 1) / (8 * nj); };
+    if (KCH <= 6 || P >= 6000 || N >= 2 * K) {
+        // column tile: least padding, then fewest blocks; the backward epilogue holds too much per column for eight tiles unless N is 64
+        int best = 0, best_cost = 0;
+        for (int nj : {8, 6, 4, 3, 2}) {
+            if (bwd && nj == 8 && N > 64) continue;
+            const int cost = cols(nj) * nj * 8 * 4 + cols(nj) * 24;
+            if (!best || cost < best_cost) {
+                best = nj;
+                best_cost = cost;
+            }
+        }
+        c.nj = best;
+        c.mi = 2;
+        auto ctas = [&] { return (P + 16 * c.mi * c.wm - 1) / (16 * c.mi * c.wm) * cols(c.nj); };
+        if (ctas() < sms) c.mi = 1;
+        if (ctas() < sms && c.nj == 8) c.nj = 4;
+        if (ctas() < sms && c.nj == 6 && N % 32 == 0) c.nj = 4;
+        if (ctas() < sms) c.wm = 4;
+        if (!bwd && (c.mi == 1 || c.nj <= 3)) c.ctas = 2;
+        if (c.wm == 4) c.ctas = 4;
+    } else {
+        c.nj = N <= 16 ? 2 : N <= 24 ? 3 : 4;
+        c.wk = 2;
+        const int want = bwd ? sms * 4 / 5 : sms * 5 / 4;
+        while (c.wk < 8 && (P + 128 / c.wk - 1) / (128 / c.wk) * cols(c.nj) < want) c.wk *= 2;
+        c.wm = 8 / c.wk;
+    }
+    while (mma_smem(bwd, K, c) > 200 * 1024) {
+        if (c.nj <= 2) return false;
+        c.nj = c.nj == 8 ? 6 : c.nj == 6 ? 4 : c.nj - 1;
+    }
+    *out = c;
+    return true;
+}
+
+size_t mma_smem(bool bwd, int K, const MmaTiling& c) {
+    const int Kp = (K + 31) / 32 * 32, BN = c.wk == 1 ? c.wn * c.nj * 8 : c.nj * 8;
+    size_t b = (size_t)BN * w_pitch(K) + (size_t)(bwd ? 5 : 2) * Kp * 4 + (size_t)(bwd ? 4 : 1) * BN * 4;
+    if (c.wk == 1) b += (size_t)c.wm * 2 * BN * 4;
+    else {
+        const size_t acc = (size_t)128 * (BN + 4) * 4;
+        b += acc > 16384 ? acc : 16384;
+    }
+    return b < 8192 ? 8192 : b;
+}
+
+void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, double bytes, cudaStream_t st) {
+    Args a;
+    memset(&a, 0, sizeof a);
+    a.P = p.P; a.K = p.K; a.N = p.N;
+    a.KCH = (p.K + 31) / 32;
+    int xf;
+    if (bwd) {
+        a.a = p.dz.dy; a.az = p.dz.z; a.act = p.dz.act;
+        a.c0 = p.dz.k1; a.c1 = p.dz.k2; a.c2 = p.dz.k3; a.c3 = p.dz.scale; a.c4 = p.dz.shift;
+        a.pb = p.pb;
+        xf = p.dz.act != ACT_NONE ? XF_ACT : (p.dz.k1 || p.pb.sums) ? XF_AFFINE : XF_NONE;
+    } else {
+        a.a = p.x.p; a.act = p.x.act;
+        a.c0 = p.x.scale; a.c1 = p.x.shift;
+        a.pf = p.pf;
+        xf = p.x.act != ACT_NONE ? XF_ACT : (p.x.scale || p.pf.sums) ? XF_AFFINE : XF_NONE;
+    }
+    a.w = p.w; a.bias = p.bias; a.addend = p.addend; a.out = p.out;
+    a.WM = c.wm; a.WN = c.wn;
+    a.wpitch = w_pitch(p.K);
+    const int BN = c.wk == 1 ? c.wn * c.nj * 8 : c.nj * 8, BM = c.wk == 1 ? 16 * c.mi * c.wm : 16 * (8 / c.wk);
+    a.m_tiles = (p.P + BM - 1) / BM;
+    const int ny = (p.N + BN - 1) / BN;
+    int gx = a.m_tiles;
+    if (c.wk == 1) {
+        int cap = sm_count() * c.ctas / ny;
+        if (cap < 1) cap = 1;
+        if (gx > cap) gx = cap;
+    }
+    a.so = p.so;
+    if (p.red) {
+        a.rz = (const __nv_bfloat16*)p.red->z;
+        a.r_scale = p.red->scale; a.r_shift = p.red->shift; a.r_mean = p.red->mean; a.r_rstd = p.red->rstd;
+        a.r_act = p.red->act;
+    }
+    if (bwd) raise_limits<true>();
+    else raise_limits<false>();
+    const size_t smem = mma_smem(bwd, p.K, c);
+    LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 2.0 * p.P * p.N : 0.0), 2.0 * p.P * p.N * p.K, st);
+    launch_pdl(bwd ? kernel_for<true>(c, xf) : kernel_for<false>(c, xf), dim3(gx, ny), c.wk == 1 ? 32 * c.wm * c.wn : 256, smem, st, a);
+}
+
+}  // namespace ast

@@ -1,0 +1,50 @@
+// Host interface of the register-operand pointwise kernels (pw_mma.cu).
+#pragma once
+#include "kernels.h"
+
+namespace ast {
+
+// A tiling of the layer.  wk == 1: persistent CTAs of wm x wn warps, a warp owns 16*mi pixels x 8*nj columns and the whole reduction;
+// wk > 1: one tile of 16*(8/wk) pixels x 8*nj columns per CTA, the reduction split over wk warps.
+struct MmaTiling {
+    int mi, nj, wm, wn, wk;
+    int ctas;                  // wk == 1: CTAs per multiprocessor the grid is sized for
+};
+
+struct MmaProblem {
+    int P, K, N;
+    ValSrc x;                  // forward operand
+    GradSrc dz;                // backward operand
+    BnPendFwd pf;              // pending coefficients of x
+    BnPendBwd pb;              // pending coefficients of dz
+    const __nv_bfloat16* w;    // [N][K]
+    const float* bias;
+    const void* addend;
+    __nv_bfloat16* out;
+    BnSumsOut so;              // column sums of the output (sums null: none)
+    const BnRed* red;          // backward: the unit the sums belong to
+};
+
+// Chooses a tiling; false: the layer does not run here (pw_tc.cu has the kernels for it).
+bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out);
+size_t mma_smem(bool bwd, int K, const MmaTiling& c);
+void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, double bytes, cudaStream_t st);
+
+// ---- weight gradient (pw_wgrad_mma.cu)
+struct WgradProblem {
+    int P, CO, CI;
+    ValSrc x;
+    GradSrc dz;
+    BnPendBwd pb;              // pending coefficients of dz; pend_write: this kernel also writes them out
+    int pend_write;
+};
+// a CTA: 8*vm channels of the wider side x 8*vn of the narrower; `splits` pixel ranges, `cluster` of them summed in the kernel
+struct WgradTiling {
+    int vm, vn, splits, cluster;
+};
+// pipeline_fits: the pipelined kernel of pw_tc.cu takes the layer
+bool wgrad_mma_choose(int P, int CO, int CI, bool pipeline_fits, size_t scratch_floats, WgradTiling* out);
+size_t wgrad_mma_smem(const WgradTiling& c);
+void wgrad_mma_launch(const WgradProblem& p, const WgradTiling& c, float* scratch, float* gw, cudaStream_t st);
+
+}  // namespace ast

@@ -1492,25 +1492,35 @@ int pw_bwd_data_tc(const ConvGeom& g, const GradSrc& dz, const __nv_bfloat16* wt
     return 0;
 }
 
+// the weight-gradient pipeline's plan for a layer: the whole gradient in one CTA's tensor memory where its stages fit; else the wider side in
+// 2 or 4 channel sub-ranges (the other side's rows are then read once per sub-range, by CTAs that run side by side: a re-read from L2)
+static bool plan_wgrad_layer(WgArgs& wa, size_t* smem, size_t scratch_floats) {
+    static const int kSplits[3][2] = {{1, 1}, {4, 1}, {2, 1}};
+    for (int i = 0; i < 3; ++i) {
+        wa.nsa = wa.COf >= wa.CIf ? kSplits[i][0] : kSplits[i][1];
+        wa.nsb = wa.COf >= wa.CIf ? kSplits[i][1] : kSplits[i][0];
+        if (plan_wgrad(wa, smem, scratch_floats, sm_count())) return true;
+    }
+    return false;
+}
+bool pw_wgrad_pipeline_fits(const ConvGeom& g, bool need_z, size_t scratch_floats) {
+    WgArgs wa{};
+    wa.P = g.n * g.ho * g.wo; wa.COf = g.co; wa.CIf = g.ci;
+    wa.need_z = need_z ? 1 : 0;
+    size_t smem = 0;
+    return g.stride == 1 && plan_wgrad_layer(wa, &smem, scratch_floats);
+}
+
 void pw_bwd_weight_tc(const ConvGeom& g, const GradSrc& dz, const ValSrc& x, float* scratch, size_t scratch_floats, float* gw, int* err,
                       cudaStream_t st) {
     if (g.stride == 1) {
         smem_limit_once<104>(pw_wgrad_pipe_kernel, 226 * 1024);
-        const int n_sm = sm_count();
         WgArgs wa{};
         wa.dz = dz; wa.x = x; wa.partial = scratch; wa.gw = gw; wa.err = err;
         wa.P = g.n * g.ho * g.wo; wa.COf = g.co; wa.CIf = g.ci;
         wa.need_z = (dz.act != ACT_NONE || dz.k1) ? 1 : 0;
         size_t smem = 0;
-        // the whole gradient in one CTA's tensor memory where its stages fit; else the wider side in 2 or 4 channel sub-ranges
-        // (the other side's rows are then read once per sub-range, by CTAs that run side by side: a re-read from L2)
-        static const int kSplits[3][2] = {{1, 1}, {4, 1}, {2, 1}};
-        bool planned = false;
-        for (int i = 0; i < 3 && !planned; ++i) {
-            wa.nsa = g.co >= g.ci ? kSplits[i][0] : kSplits[i][1];
-            wa.nsb = g.co >= g.ci ? kSplits[i][1] : kSplits[i][0];
-            planned = plan_wgrad(wa, &smem, scratch_floats, n_sm);
-        }
+        bool planned = plan_wgrad_layer(wa, &smem, scratch_floats);
         alignas(64) CUtensorMap tm_dy, tm_z, tm_x;
         memset(&tm_dy, 0, sizeof(tm_dy)); memset(&tm_z, 0, sizeof(tm_z)); memset(&tm_x, 0, sizeof(tm_x));
         if (planned && wa.nsa * wa.nsb > 1) {

@@ -10,6 +10,7 @@
 
 #include "../../include/asteroid.h"
 #include "kernels.h"
+#include "pw_mma.h"
 
 namespace ast {
 
@@ -61,6 +62,7 @@ struct Unit {
     long w_off = -1, b_off = -1, gamma_off = -1, beta_off = -1;   // floats into the parameter arena
     size_t k_off = 0;       // floats into the backward-coefficient arena (k1,k2,k3)
     size_t run_off = 0;     // floats into the running-statistics arena
+    size_t sum_off = 0;     // BatchNorm units: channels before this unit's (its sums: 2c doubles at 2*sum_off, its pivots at sum_off)
     // dense conv with a short reduction, bfloat16 mode: forward and weight gradient run as pointwise tensor-core GEMMs
     // over an explicit im2col tensor kept in the slot (col_kp = padded reduction length, 0 = not such a unit)
     int col_kp = 0;
@@ -106,7 +108,7 @@ struct asteroid_stage {
     std::vector<int> val_of_layer;  // layer index - (first-1) -> value id or -1
     // n_params: values of the caller's flat state (layers back to back); n_pad: floats of the internal parameter arenas, where
     // every layer starts on a multiple of 8 floats (16-byte aligned in the bfloat16 copies, whatever precedes it)
-    size_t n_params = 0, n_pad = 0, n_run = 0, n_coef = 0;
+    size_t n_params = 0, n_pad = 0, n_run = 0, n_coef = 0, n_bn_ch = 0;
     struct Seg { size_t pub, in, n; };
     std::vector<Seg> segs;
     // device arenas
@@ -116,6 +118,11 @@ struct asteroid_stage {
     __nv_bfloat16* wpad = nullptr;                 // [co][Kp] bf16 weights of the im2col units
     float* gpad = nullptr;                         // [co][Kp] padded weight gradient of the im2col unit at hand
     size_t n_wpad = 0, n_gpad = 0;
+    // per-channel sums of the BatchNorms (fin.cuh), forward and backward, and the pivots the forward sums were taken with.  The forward sums
+    // are zeroed by a forward's first kernel, the backward sums by accumulate.
+    double *fsum = nullptr, *bsum = nullptr;
+    float* pivots = nullptr;
+    bool bsum_dirty = false;                       // a backward ran since its sums were zeroed (profile runs skip accumulate)
     int* err = nullptr;                            // device error word (bounded waits)
     // Weight-gradient kernels depend only on the BatchNorm-backward coefficients of their unit and nothing in the rest of
     // the backward pass depends on them: they run on a second stream (forked from and joined back into the caller's
@@ -364,6 +371,8 @@ static int build_plan(asteroid_stage* s) {
             ncoef += 3 * (size_t)o.c;
             u.run_off = nrun;
             nrun += 2 * (size_t)o.c;
+            u.sum_off = s->n_bn_ch;
+            s->n_bn_ch += (size_t)o.c;
         }
     }
     for (auto& u : s->units)
@@ -529,36 +538,114 @@ static void tick(asteroid_stage* s, size_t unit, int which, cudaStream_t st) {
     if (s->tm.on) cudaEventRecord(s->tm.ev[unit * 6 + which], st);
 }
 
+// ---- BatchNorm coefficients that are still sums (fin.cuh)
+static BnFwdOut fwd_out(asteroid_stage* s, const SlotView& sv, const Unit& u) {
+    const Val& o = s->vals[u.out];
+    float* stt = sv.stats + o.stat_off;
+    return BnFwdOut{stt, stt + o.c, stt + 2 * (size_t)o.c, stt + 3 * (size_t)o.c, s->run + u.run_off, s->run + u.run_off + o.c};
+}
+static BnBwdOut bwd_out(asteroid_stage* s, const Unit& u) {
+    float* kc = s->coef + u.k_off;
+    const size_t c = (size_t)s->vals[u.out].c;
+    return BnBwdOut{s->g + u.gamma_off, s->g + u.beta_off, kc, kc + c, kc + 2 * c};
+}
+static BnPendFwd pend_fwd(asteroid_stage* s, const SlotView& sv, const Unit& u) {
+    const Val& o = s->vals[u.out];
+    const double n = (double)(o.elems / o.c);
+    return BnPendFwd{s->fsum + 2 * u.sum_off, s->pivots + u.sum_off, s->w + u.gamma_off, s->w + u.beta_off, 1.0 / n, n > 1.0 ? n / (n - 1.0) : 1.0,
+                     s->eps, s->bn_mom, o.c, fwd_out(s, sv, u)};
+}
+static BnPendBwd pend_bwd(asteroid_stage* s, const SlotView& sv, const Unit& u) {
+    const Val& o = s->vals[u.out];
+    const float* stt = sv.stats + o.stat_off;
+    return BnPendBwd{s->bsum + 2 * u.sum_off, s->w + u.gamma_off, stt, stt + o.c, 1.0 / (double)(o.elems / o.c), o.c, bwd_out(s, u)};
+}
+static BnSumsOut sums_fwd(asteroid_stage* s, const Unit& u) { return BnSumsOut{s->fsum + 2 * u.sum_off, s->run + u.run_off, s->pivots + u.sum_off}; }
+
+// which BatchNorm units' coefficients are pending in the pass at hand
+struct Pending {
+    asteroid_stage* s;
+    SlotView sv;
+    cudaStream_t st;
+    std::vector<char> unit;
+    Pending(asteroid_stage* s_, const SlotView& v, cudaStream_t st_) : s(s_), sv(v), st(st_), unit(s_->units.size(), 0) {}
+    bool has(int u) const { return u >= 0 && unit[u] != 0; }
+    // the unit's pending coefficients for a kernel that forms them itself (nothing is pending afterwards); empty if none are
+    BnPendFwd take_fwd(int u) {
+        if (!has(u)) return BnPendFwd{};
+        unit[u] = 0;
+        return pend_fwd(s, sv, s->units[u]);
+    }
+    void settle_fwd(int u) {
+        if (has(u)) bn_settle_fwd(take_fwd(u), st);
+    }
+    void settle_bwd(int u) {
+        if (has(u)) bn_settle_bwd(pend_bwd(s, sv, s->units[u]), st);
+        if (u >= 0) unit[u] = 0;
+    }
+};
+
+// Pointwise problem of a unit on the register-operand kernels; false: it does not run there.
+static bool mma_unit(const asteroid_stage* s, const Unit& u, const ConvGeom& g, bool bwd, MmaTiling* t) {
+    if (s->dtype != AST_BF16 || g.k != 1 || g.stride != 1 || g.pad != 0) return false;
+    (void)u;
+    return bwd ? mma_choose(true, g.n * g.ho * g.wo, g.co, g.ci, t) : mma_choose(false, g.n * g.ho * g.wo, g.ci, g.co, t);
+}
+
 static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cudaStream_t st) {
     SlotView sv = slot_view(s, slot);
     const int dt = s->dtype;
     {
-        // the slot's copy of x (backward reads it); a kernel rather than a memcpy node where the channel count allows
-        // vector accesses, so that the chain of programmatic dependent launches is not interrupted
+        // the slot's copy of x (backward reads it); a kernel rather than a memcpy node where the alignment allows vector
+        // accesses, so that the chain of programmatic dependent launches is not interrupted.  It also zeroes the channel sums.
         const Val& v0 = s->vals[0];
-        if (v0.c % (dt == AST_F32 ? 4 : 8) == 0) ew_apply(dt, ValSrc{x, nullptr, nullptr, ACT_NONE}, v0.elems / v0.c, v0.c, sv.base + v0.buf_off, st);
-        else CU(cudaMemcpyAsync(sv.base + v0.buf_off, x, v0.elems * s->esz, cudaMemcpyDeviceToDevice, st));
+        if (!slot_copy(x, sv.base + v0.buf_off, v0.elems * s->esz, s->fsum, 2 * s->n_bn_ch, st)) {
+            CU(cudaMemcpyAsync(sv.base + v0.buf_off, x, v0.elems * s->esz, cudaMemcpyDeviceToDevice, st));
+            if (s->n_bn_ch) CU(cudaMemsetAsync(s->fsum, 0, 2 * s->n_bn_ch * sizeof(double), st));
+        }
     }
+    Pending pend(s, sv, st);
+    const auto producer = [&](int v) { return s->vals[v].affine ? s->vals[v].unit : -1; };
     for (size_t ui = 0; ui < s->units.size(); ++ui) {
         const Unit& u = s->units[ui];
         const Val& o = s->vals[u.out];
         const bool is_last = ui + 1 == s->units.size();
         void* obuf = sv.base + o.buf_off;
         tick(s, ui, 0, st);
-        int fused_stats = 0;       // > 0: the producing kernel wrote that many statistics partials into the scratch arena
-        if (u.kind == U_CONV) {
+        int fused_stats = 0;       // > 0: the producing kernel wrote that many statistics partials into the scratch arena; -1: it took the sums
+        const bool bn = u.l_bn >= 0;
+        MmaTiling til;
+        // the pointwise layer on the register-operand kernels: forms its input's pending coefficients, takes its output's sums
+        auto on_mma = [&](const ConvGeom& g, const ValSrc& xs, int in_unit, const __nv_bfloat16* w) {
+            MmaProblem p{};
+            p.P = g.n * g.ho * g.wo; p.K = g.ci; p.N = g.co;
+            p.x = xs; p.w = w; p.out = (__nv_bfloat16*)obuf;
+            p.bias = u.b_off >= 0 ? s->w + u.b_off : nullptr;
+            p.pf = pend.take_fwd(in_unit);
+            if (bn) p.so = sums_fwd(s, u);
+            mma_launch(false, p, til, K_PW_FWD_TC, 2.0 * ((double)p.P * p.K + (double)p.P * p.N) + 2.0 * p.N * p.K, st);
+            fused_stats = bn ? -1 : 0;
+        };
+        if (u.kind == U_CONV && !u.col_kp && u.sub_off < 0 && mma_unit(s, u, u.g, false, &til)) {
+            on_mma(u.g, val_src(s, sv, u.in), producer(u.in), s->wb + u.w_off);
+        } else if (u.kind == U_CONV) {
+            pend.settle_fwd(producer(u.in));
             const float* bias = u.b_off >= 0 ? s->w + u.b_off : nullptr;
-            const bool bn = u.l_bn >= 0;
             if (u.col_kp) {
                 void* col = sv.base + u.col_off;
                 conv_im2col(u.g, val_src(s, sv, u.in), u.col_kp, col, st);
-                fused_stats = pw_fwd_tc(col_geom(u), ValSrc{col, nullptr, nullptr, ACT_NONE}, s->wpad + u.wpad_off, nullptr, obuf,
+                const ValSrc cs{col, nullptr, nullptr, ACT_NONE};
+                if (mma_unit(s, u, col_geom(u), false, &til)) on_mma(col_geom(u), cs, -1, s->wpad + u.wpad_off);
+                else
+                fused_stats = pw_fwd_tc(col_geom(u), cs, s->wpad + u.wpad_off, nullptr, obuf,
                                         bn ? s->run + u.run_off : nullptr, bn ? s->scratch : nullptr, s->scratch_floats, s->err, st);
             } else if (u.sub_off >= 0) {
                 ValSrc xs = val_src(s, sv, u.in);
                 void* sub = sv.base + u.sub_off;
                 ew_subsample2(xs.p, u.g.n, u.g.hi, u.g.wi, u.g.ho, u.g.wo, u.g.ci, sub, st);
                 xs.p = sub;                                  // the producer's BatchNorm / activation is per channel: applied on load as before
+                if (mma_unit(s, u, sub_geom(u), false, &til)) on_mma(sub_geom(u), xs, -1, s->wb + u.w_off);
+                else
                 fused_stats = pw_fwd_tc(sub_geom(u), xs, s->wb + u.w_off, bias, obuf, bn ? s->run + u.run_off : nullptr,
                                         bn ? s->scratch : nullptr, s->scratch_floats, s->err, st);
             } else if (pw_tc_supported(dt, u.g, false))
@@ -571,38 +658,48 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
             }
             else conv_fwd(dt, u.g, val_src(s, sv, u.in), s->w + u.w_off, bias, obuf, st);
         } else if (u.kind == U_DW) {
-            const bool bn = u.l_bn >= 0;
+            pend.settle_fwd(producer(u.in));
             if (u.g.k != 3) dwk_fwd(dt, u.g, val_src(s, sv, u.in), s->derived + u.w_off, obuf, st);
             else
                 fused_stats = dw_fwd(dt, u.g, val_src(s, sv, u.in), s->derived + u.w_off, obuf, bn ? s->run + u.run_off : nullptr, bn ? s->scratch : nullptr,
                                      s->scratch_floats, st);
         } else if (u.kind == U_SILU) {
+            pend.settle_fwd(producer(u.in));
             silu_fwd(dt, val_src(s, sv, u.in), o.elems / o.c, o.c, obuf, is_last ? y : nullptr, st);
         } else if (u.kind == U_SE) {
+            pend.settle_fwd(producer(u.in));
             const int c = o.c, k = u.se_k;
             const float* wp = s->w + u.w_off;        // w1 [k][c], b1 [k], w2 [c][k], b2 [c]
             float* sev = sv.stats + u.se_off;        // s [B][c], p1 [B][k], gate [B][c]
             se_forward(dt, val_src(s, sv, u.in), s->B, o.h * o.w, c, k, wp, wp + (size_t)k * c, wp + (size_t)k * c + k, wp + 2 * (size_t)k * c + k, sev,
                        sev + (size_t)s->B * c, sev + (size_t)s->B * (c + k), s->scratch, s->scratch_floats, obuf, is_last ? y : nullptr, st);
         } else if (u.kind == U_ADD) {
-            ew_add(dt, val_src(s, sv, u.in), val_src(s, sv, u.in2), u.act, o.elems / o.c, o.c, obuf, is_last ? y : nullptr, st);
+            if (!ew_takes_pending(dt, o.c)) {
+                pend.settle_fwd(producer(u.in));
+                pend.settle_fwd(producer(u.in2));
+            }
+            const BnPendFwd pa = pend.take_fwd(producer(u.in)), pb = pend.take_fwd(producer(u.in2));
+            ew_add(dt, val_src(s, sv, u.in), val_src(s, sv, u.in2), pa, pb, u.act, o.elems / o.c, o.c, obuf, is_last ? y : nullptr, st);
         } else {
             const Val& a = s->vals[u.in];
+            pend.settle_fwd(producer(u.in));
             gap_fwd(dt, val_src(s, sv, u.in), s->B, a.h * a.w, a.c, obuf, st);
         }
         tick(s, ui, 1, st);
-        s->fwd_stats_blocks[ui] = fused_stats;
-        if (u.l_bn >= 0) {
-            float* stt = sv.stats + o.stat_off;
-            BnFwdOut bo{stt, stt + o.c, stt + 2 * (size_t)o.c, stt + 3 * (size_t)o.c, s->run + u.run_off, s->run + u.run_off + o.c};
+        s->fwd_stats_blocks[ui] = fused_stats < 0 ? 1 : fused_stats;
+        if (bn) {
             if (fused_stats > 0)
-                bn_stats_finish_partials(s->scratch, fused_stats, o.elems / o.c, o.c, s->w + u.gamma_off, s->w + u.beta_off, s->eps, s->bn_mom, bo, st);
-            else
-                bn_stats(dt, obuf, o.elems / o.c, o.c, s->w + u.gamma_off, s->w + u.beta_off, s->eps, s->bn_mom, s->scratch, s->scratch_floats, bo, st);
+                bn_stats_finish_partials(s->scratch, fused_stats, o.elems / o.c, o.c, s->w + u.gamma_off, s->w + u.beta_off, s->eps, s->bn_mom,
+                                         fwd_out(s, sv, u), st);
+            else {
+                if (fused_stats == 0) bn_stats(dt, obuf, o.elems / o.c, o.c, sums_fwd(s, u), s->scratch_floats, st);
+                pend.unit[ui] = 1;
+            }
         }
         tick(s, ui, 2, st);
         if (is_last) {
-            if (u.kind == U_CONV || u.kind == U_DW) ew_apply(dt, val_src(s, sv, u.out), o.elems / o.c, o.c, y, st);
+            if (!ew_takes_pending(dt, o.c)) pend.settle_fwd(producer(u.out));
+            if (u.kind == U_CONV || u.kind == U_DW) ew_apply(dt, val_src(s, sv, u.out), pend.take_fwd(producer(u.out)), o.elems / o.c, o.c, y, st);
             else if (u.kind == U_GAP) CU(cudaMemcpyAsync(y, obuf, o.elems * s->esz, cudaMemcpyDeviceToDevice, st));
         }
     }
@@ -656,6 +753,9 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
     gs.back().state = G_ALIAS;
     gs.back().ptr = dy;
     std::vector<char> reduced(s->units.size(), 0);   // BatchNorm-backward sums already taken by the kernel that wrote dy
+    Pending pend(s, sv, st);                         // ... and not yet turned into coefficients
+    if (s->bsum_dirty && s->n_bn_ch) CU(cudaMemsetAsync(s->bsum, 0, 2 * s->n_bn_ch * sizeof(double), st));
+    s->bsum_dirty = true;
     std::fill(s->bwd_sums_by.begin(), s->bwd_sums_by.end(), -1);
     // weight gradients go to the second stream (not while a profile run times the units one by one, nor while a
     // per-launch trace brackets every kernel with events: a kernel's duration is then that of the kernel running alone)
@@ -688,17 +788,28 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             if (u.l_bn >= 0) {
                 d.scale = stt + 2 * (size_t)o.c;
                 d.shift = stt + 3 * (size_t)o.c;
-                BnBwdOut bo{s->g + u.gamma_off, s->g + u.beta_off, kc, kc + o.c, kc + 2 * (size_t)o.c};
-                if (!reduced[ui])
-                    bn_bwd_reduce(dt, d.dy, d.z, o.elems / o.c, o.c, d.scale, d.shift, u.act, stt, stt + o.c, s->w + u.gamma_off, s->scratch,
-                                  s->scratch_floats, bo, st);
+                if (!reduced[ui]) {
+                    bn_bwd_reduce(dt, d.dy, d.z, o.elems / o.c, o.c, d.scale, d.shift, u.act, stt, stt + o.c, s->bsum + 2 * u.sum_off, s->scratch_floats, st);
+                    pend.unit[ui] = 1;
+                }
                 d.k1 = kc; d.k2 = kc + o.c; d.k3 = kc + 2 * (size_t)o.c;
             }
             if (u.b_off >= 0) {
-                BnBwdOut bo{nullptr, s->g + u.b_off, nullptr, nullptr, nullptr};
-                bn_bwd_reduce(dt, d.dy, d.z, o.elems / o.c, o.c, nullptr, nullptr, u.act, nullptr, nullptr, nullptr, s->scratch, s->scratch_floats,
-                              bo, st);
+                bias_grad(dt, d.dy, d.z, o.elems / o.c, o.c, u.act, s->scratch, s->scratch_floats, s->g + u.b_off, st);
             }
+            // pending coefficients stay pending where both kernels of the unit can form them
+            MmaTiling til_d{};
+            WgradTiling til_w{};
+            ConvGeom wg = u.g;
+            if (u.col_kp) wg = col_geom(u);
+            else if (u.sub_off >= 0) wg = sub_geom(u);
+            const bool pw = u.kind == U_CONV && dt == AST_BF16 && wg.k == 1 && wg.stride == 1 && wg.pad == 0;
+            const bool mma_w = pw && wgrad_mma_choose(wg.n * wg.ho * wg.wo, wg.co, wg.ci, pw_wgrad_pipeline_fits(wg, grad_needs_z(d), s->scratch_floats),
+                                                      s->scratch_floats, &til_w);
+            const bool mma_d = want_in && u.kind == U_CONV && !u.col_kp && mma_unit(s, u, u.g, true, &til_d);
+            if (!mma_w || (want_in && !mma_d)) pend.settle_bwd(ui);
+            const BnPendBwd pb = pend.has(ui) ? pend_bwd(s, sv, u) : BnPendBwd{};
+            pend.unit[ui] = 0;
             tick(s, ui, 4, st);
             ValSrc xin = val_src(s, sv, u.in);
             if (u.kind == U_DW && want_in && u.g.k == 3) {
@@ -723,7 +834,15 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             }
             if (s2_tc && conv3_wgrad_tc_supported(dt, s1_geom(u)))
                 conv3_bwd_weight_tc(s1_geom(u), dup, xin, wscratch, s->scratch_floats, s->g + u.w_off, s->err, wst, conv_flops(u.g));
-            else if (u.kind == U_CONV && u.col_kp) {
+            else if (mma_w) {
+                WgradProblem p{};
+                p.P = wg.n * wg.ho * wg.wo; p.CO = wg.co; p.CI = wg.ci;
+                p.dz = d; p.x = xin; p.pb = pb; p.pend_write = want_in ? 0 : 1;
+                if (u.col_kp) p.x = ValSrc{sv.base + u.col_off, nullptr, nullptr, ACT_NONE};
+                else if (u.sub_off >= 0) p.x.p = sv.base + u.sub_off;                  // written by the forward of this micro-batch
+                wgrad_mma_launch(p, til_w, wscratch, u.col_kp ? s->gpad : s->g + u.w_off, wst);
+                if (u.col_kp) conv_unpad_grad(s->gpad, u.g.co, u.g.k * u.g.k * u.g.ci, u.col_kp, s->g + u.w_off, wst);
+            } else if (u.kind == U_CONV && u.col_kp) {
                 pw_bwd_weight_tc(col_geom(u), d, ValSrc{sv.base + u.col_off, nullptr, nullptr, ACT_NONE}, wscratch, s->scratch_floats, s->gpad, s->err, wst);
                 conv_unpad_grad(s->gpad, u.g.co, u.g.k * u.g.k * u.g.ci, u.col_kp, s->g + u.w_off, wst);
             } else if (u.kind == U_CONV && u.sub_off >= 0) {
@@ -743,7 +862,25 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 // this kernel writes the complete gradient of its input value: let it also take the BatchNorm-backward
                 // sums of the unit that gradient belongs to
                 const int tgt = s->vals[u.in].first_cons == ui ? bn_reduce_target(s, u.in) : -1;
-                if (u.kind == U_CONV && pw_tc_supported(dt, u.g, true)) {
+                if (mma_d) {
+                    MmaProblem p{};
+                    BnRed red{};
+                    p.P = u.g.n * u.g.ho * u.g.wo; p.K = u.g.co; p.N = u.g.ci;
+                    p.dz = d; p.pb = pb; p.w = s->wtb + u.w_off; p.addend = addend; p.out = (__nv_bfloat16*)own(u.in);
+                    if (tgt >= 0) {
+                        const Unit& tu = s->units[tgt];
+                        const Val& tv = s->vals[tu.out];
+                        float* ts = sv.stats + tv.stat_off;
+                        red = BnRed{sv.base + tv.buf_off, ts + 2 * (size_t)tv.c, ts + 3 * (size_t)tv.c, ts, ts + tv.c, tu.act, nullptr, 0};
+                        p.red = &red;
+                        p.so = BnSumsOut{s->bsum + 2 * tu.sum_off, nullptr, nullptr};
+                        pend.unit[tgt] = 1;
+                        reduced[tgt] = 1;
+                        s->bwd_sums_by[tgt] = ui;
+                    }
+                    mma_launch(true, p, til_d, K_PW_BWD_DATA_TC, 2.0 * (double)p.P * p.K * (grad_needs_z(d) ? 2.0 : 1.0) +
+                               2.0 * (double)p.P * p.N * (addend ? 2.0 : 1.0) + 2.0 * p.N * p.K, st);
+                } else if (u.kind == U_CONV && pw_tc_supported(dt, u.g, true)) {
                     BnRed red{};
                     if (tgt >= 0) {
                         const Unit& tu = s->units[tgt];
@@ -788,11 +925,10 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                     const Unit& tu = s->units[tgt];
                     const Val& tv = s->vals[tu.out];
                     float* ts = sv.stats + tv.stat_off;
-                    float* tk = s->coef + tu.k_off;
-                    BnBwdOut tbo{s->g + tu.gamma_off, s->g + tu.beta_off, tk, tk + tv.c, tk + 2 * (size_t)tv.c};
-                    fused = ew_relu_mask_bn_sums(dt, go.ptr, sv.base + o.buf_off, sv.base + tv.buf_off, o.elems / o.c, o.c, ts, ts + tv.c, s->w + tu.gamma_off,
-                                                 own(u.out), s->scratch, s->scratch_floats, tbo, st);
+                    fused = ew_relu_mask_bn_sums(dt, go.ptr, sv.base + o.buf_off, sv.base + tv.buf_off, o.elems / o.c, o.c, ts, ts + tv.c, own(u.out),
+                                                 s->bsum + 2 * tu.sum_off, s->scratch_floats, st);
                     if (fused) {
+                        pend.unit[tgt] = 1;
                         reduced[tgt] = 1;
                         s->bwd_sums_by[tgt] = ui;
                     }
@@ -881,6 +1017,9 @@ static int create_impl(const ast_layer* net, int n_layers, int first, int last, 
         if ((rc = arena_alloc(s, "padded weights", &s->wpad, s->n_wpad * 2, &mod))) return rc;
         if ((rc = arena_alloc(s, "padded weight gradient", &s->gpad, s->n_gpad * 4, &work))) return rc;
     }
+    if ((rc = arena_alloc(s, "forward channel sums", &s->fsum, s->n_bn_ch * 2 * sizeof(double), &work))) return rc;
+    if ((rc = arena_alloc(s, "backward channel sums", &s->bsum, s->n_bn_ch * 2 * sizeof(double), &work))) return rc;
+    if ((rc = arena_alloc(s, "statistics pivots", &s->pivots, s->n_bn_ch * 4, &work))) return rc;
     if ((rc = arena_alloc(s, "error word", &s->err, 256, &work))) return rc;
     if ((rc = arena_alloc(s, "momentum", &s->v, np * 4, &opt))) return rc;
     if ((rc = arena_alloc(s, "activation slots", &s->slot_mem, s->slot_bytes * s->slots, &act))) return rc;
@@ -1064,7 +1203,8 @@ int asteroid_stage_accumulate(asteroid_stage* s, int mb, void* stream) {
     if (!s) return fail(AST_ERR_ARG, "null argument");
     if (s->pending_g != mb) return fail(AST_ERR_ORDER, "accumulate(%d): the last backward was of micro-batch %d", mb, s->pending_g);
     if (s->n_acc >= s->M) return fail(AST_ERR_ORDER, "already accumulated %d micro-batches this round", s->M);
-    accumulate(s->G, s->g, s->n_pad, (cudaStream_t)stream);
+    accumulate(s->G, s->g, s->n_pad, s->bsum, 2 * s->n_bn_ch, (cudaStream_t)stream);
+    s->bsum_dirty = s->bsum_dirty && s->n_pad == 0;
     CU(cudaGetLastError());
     s->pending_g = -1;
     s->n_acc++;

@@ -170,18 +170,23 @@ bool conv3_wgrad_tc_supported(int dtype, const ConvGeom& g);
 void conv3_bwd_weight_tc(const ConvGeom& g, const GradSrc& dz, const ValSrc& x, float* scratch, size_t scratch_floats, float* gw, int* err,
                          cudaStream_t st, double useful_flops = 0);
 
-// ---- depthwise 3x3 (weights tap-major: w9c[r*3+s][c]) ----
-// With `pivot` and `partial` given, the stride-1 kernel also writes the BatchNorm statistics partials of its output
-// (layout and meaning as for pw_fwd_tc) and returns the number of blocks that wrote them; 0 = none.
-int dw_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const float* w9c, void* z, const float* pivot, float* partial, size_t partial_floats,
-           cudaStream_t st);
-void dw_bwd_data(int dtype, const ConvGeom& g, const GradSrc& dz, const float* w9c, const void* addend, void* dx, cudaStream_t st);
-// stride-1 bf16 layers with enough image columns: input gradient and weight gradient in one pass; false = not applicable
-bool dw_bwd_fused(int dtype, const ConvGeom& g, const GradSrc& dz, const ValSrc& x, const float* w9c, const void* addend, void* dx,
-                  float* scratch, size_t scratch_floats, float* gw, cudaStream_t st);
-// gw[c][r][s]
-void dw_bwd_weight(int dtype, const ConvGeom& g, const GradSrc& dz, const ValSrc& x, float* scratch, size_t scratch_floats,
-                   float* gw, cudaStream_t st);
+// ---- depthwise 3x3 (weights tap-major: w9c[r*3+s][c]), pending coefficients in and channel sums out (dw3.cu) ----
+// tw: strip width in pixels (backward, stride 2: in columns of dz); th: rows per strip; ctas: blocks per multiprocessor the grid is sized for
+struct DwTiling {
+    int tw, th, ctas;
+};
+// one depthwise layer of dw3_settle: offsets of its accumulators [9][c] and of its weight gradient [c][9]
+struct DwSettle {
+    size_t acc_off, g_off;
+    int c;
+};
+DwTiling dw3_choose(int dtype, bool bwd, const ConvGeom& g);
+void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf, const float* w9c, void* z, const BnSumsOut& so, const DwTiling& t, cudaStream_t st);
+// dx may be null (weight gradient only); gw: [9][c] accumulators; sums [2][c] (may be null), mean, rstd: of the unit that produced x
+void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* w9c, const void* addend, void* dx, double* gw,
+             double* sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st);
+// accumulators -> weight gradients, all layers of the table (device memory); total: sum of 9*c
+void dw3_settle(const double* acc, const DwSettle* tab, int layers, size_t total, float* g, cudaStream_t st);
 
 // ---- BatchNorm statistics and backward reductions over a [pixels][c] tensor ----
 // sums of a [pixels][c] tensor of its own pass; the coefficients are then pending (fin.cuh)

@@ -62,6 +62,7 @@ struct Unit {
     long w_off = -1, b_off = -1, gamma_off = -1, beta_off = -1;   // floats into the parameter arena
     size_t k_off = 0;       // floats into the backward-coefficient arena (k1,k2,k3)
     size_t run_off = 0;     // floats into the running-statistics arena
+    size_t acc_off = 0;     // 3x3 depthwise units: the weight gradient's accumulators, [9][c] doubles, in the backward sums
     size_t sum_off = 0;     // BatchNorm units: channels before this unit's (its sums: 2c doubles at 2*sum_off, its pivots at sum_off)
     // dense conv with a short reduction, bfloat16 mode: forward and weight gradient run as pointwise tensor-core GEMMs
     // over an explicit im2col tensor kept in the slot (col_kp = padded reduction length, 0 = not such a unit)
@@ -108,7 +109,7 @@ struct asteroid_stage {
     std::vector<int> val_of_layer;  // layer index - (first-1) -> value id or -1
     // n_params: values of the caller's flat state (layers back to back); n_pad: floats of the internal parameter arenas, where
     // every layer starts on a multiple of 8 floats (16-byte aligned in the bfloat16 copies, whatever precedes it)
-    size_t n_params = 0, n_pad = 0, n_run = 0, n_coef = 0, n_bn_ch = 0;
+    size_t n_params = 0, n_pad = 0, n_run = 0, n_coef = 0, n_bn_ch = 0, n_bsum = 0, n_dw_weights = 0;
     struct Seg { size_t pub, in, n; };
     std::vector<Seg> segs;
     // device arenas
@@ -119,9 +120,12 @@ struct asteroid_stage {
     float* gpad = nullptr;                         // [co][Kp] padded weight gradient of the im2col unit at hand
     size_t n_wpad = 0, n_gpad = 0;
     // per-channel sums of the BatchNorms (fin.cuh), forward and backward, and the pivots the forward sums were taken with.  The forward sums
-    // are zeroed by a forward's first kernel, the backward sums by accumulate.
+    // are zeroed by a forward's first kernel, the backward sums by accumulate.  The backward sums also hold the accumulators of the 3x3
+    // depthwise weight gradients.
     double *fsum = nullptr, *bsum = nullptr;
     float* pivots = nullptr;
+    DwSettle* dw_tab = nullptr;                    // the 3x3 depthwise units' accumulators and weight gradients
+    int n_dw = 0;
     bool bsum_dirty = false;                       // a backward ran since its sums were zeroed (profile runs skip accumulate)
     int* err = nullptr;                            // device error word (bounded waits)
     // Weight-gradient kernels depend only on the BatchNorm-backward coefficients of their unit and nothing in the rest of
@@ -372,9 +376,17 @@ static int build_plan(asteroid_stage* s) {
             u.run_off = nrun;
             nrun += 2 * (size_t)o.c;
             u.sum_off = s->n_bn_ch;
-            s->n_bn_ch += (size_t)o.c;
+            s->n_bn_ch += align_up((size_t)o.c, 4);   // kernels read and write pivots in vectors
         }
     }
+    s->n_bsum = 2 * s->n_bn_ch;
+    for (auto& u : s->units)
+        if (u.kind == U_DW && u.g.k == 3) {
+            u.acc_off = s->n_bsum;
+            s->n_bsum += 9 * (size_t)u.g.ci;
+            s->n_dw_weights += 9 * (size_t)u.g.ci;
+            ++s->n_dw;
+        }
     for (auto& u : s->units)
         if (u.kind == U_SE) {
             u.se_off = nstat;
@@ -658,11 +670,14 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
             }
             else conv_fwd(dt, u.g, val_src(s, sv, u.in), s->w + u.w_off, bias, obuf, st);
         } else if (u.kind == U_DW) {
-            pend.settle_fwd(producer(u.in));
-            if (u.g.k != 3) dwk_fwd(dt, u.g, val_src(s, sv, u.in), s->derived + u.w_off, obuf, st);
-            else
-                fused_stats = dw_fwd(dt, u.g, val_src(s, sv, u.in), s->derived + u.w_off, obuf, bn ? s->run + u.run_off : nullptr, bn ? s->scratch : nullptr,
-                                     s->scratch_floats, st);
+            if (u.g.k != 3) {
+                pend.settle_fwd(producer(u.in));
+                dwk_fwd(dt, u.g, val_src(s, sv, u.in), s->derived + u.w_off, obuf, st);
+            } else {
+                const BnPendFwd pf = pend.take_fwd(producer(u.in));
+                dw3_fwd(dt, u.g, val_src(s, sv, u.in), pf, s->derived + u.w_off, obuf, bn ? sums_fwd(s, u) : BnSumsOut{}, dw3_choose(dt, false, u.g), st);
+                fused_stats = bn ? -1 : 0;
+            }
         } else if (u.kind == U_SILU) {
             pend.settle_fwd(producer(u.in));
             silu_fwd(dt, val_src(s, sv, u.in), o.elems / o.c, o.c, obuf, is_last ? y : nullptr, st);
@@ -754,7 +769,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
     gs.back().ptr = dy;
     std::vector<char> reduced(s->units.size(), 0);   // BatchNorm-backward sums already taken by the kernel that wrote dy
     Pending pend(s, sv, st);                         // ... and not yet turned into coefficients
-    if (s->bsum_dirty && s->n_bn_ch) CU(cudaMemsetAsync(s->bsum, 0, 2 * s->n_bn_ch * sizeof(double), st));
+    if (s->bsum_dirty && s->n_bsum) CU(cudaMemsetAsync(s->bsum, 0, s->n_bsum * sizeof(double), st));
     s->bsum_dirty = true;
     std::fill(s->bwd_sums_by.begin(), s->bwd_sums_by.end(), -1);
     // weight gradients go to the second stream (not while a profile run times the units one by one, nor while a
@@ -807,20 +822,36 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             const bool mma_w = pw && wgrad_mma_choose(wg.n * wg.ho * wg.wo, wg.co, wg.ci, pw_wgrad_pipeline_fits(wg, grad_needs_z(d), s->scratch_floats),
                                                       s->scratch_floats, &til_w);
             const bool mma_d = want_in && u.kind == U_CONV && !u.col_kp && mma_unit(s, u, u.g, true, &til_d);
-            if (!mma_w || (want_in && !mma_d)) pend.settle_bwd(ui);
+            const bool dw3 = u.kind == U_DW && u.g.k == 3;
+            if (!dw3 && (!mma_w || (want_in && !mma_d))) pend.settle_bwd(ui);
             const BnPendBwd pb = pend.has(ui) ? pend_bwd(s, sv, u) : BnPendBwd{};
             pend.unit[ui] = 0;
             tick(s, ui, 4, st);
             ValSrc xin = val_src(s, sv, u.in);
-            if (u.kind == U_DW && want_in && u.g.k == 3) {
+            if (dw3) {
+                // input gradient, weight gradient and, where x is the raw output of a conv -> BatchNorm unit read by nobody after this one, that
+                // BatchNorm's sums
                 GradState& gi = gs[u.in];
                 const void* addend = gi.state == G_NONE ? nullptr : gi.ptr;
-                if (dw_bwd_fused(dt, u.g, d, xin, s->derived + u.w_off, addend, own(u.in), s->scratch, s->scratch_floats, s->g + u.w_off, st)) {
+                const int tgt = want_in && s->vals[u.in].first_cons == ui && bn_reduce_target(s, u.in) == s->vals[u.in].unit ? s->vals[u.in].unit : -1;
+                double* sums = nullptr;
+                const float* ts = nullptr;
+                if (tgt >= 0) {
+                    const Unit& tu = s->units[tgt];
+                    sums = s->bsum + 2 * tu.sum_off;
+                    ts = sv.stats + s->vals[tu.out].stat_off;
+                    pend.unit[tgt] = 1;
+                    reduced[tgt] = 1;
+                    s->bwd_sums_by[tgt] = ui;
+                }
+                dw3_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, want_in ? own(u.in) : nullptr, s->bsum + u.acc_off, sums, ts, ts ? ts + u.g.ci : nullptr,
+                        dw3_choose(dt, true, u.g), st);
+                if (want_in) {
                     gi.state = G_OWNED;
                     gi.ptr = own(u.in);
-                    tick(s, ui, 5, st);
-                    continue;
                 }
+                tick(s, ui, 5, st);
+                continue;
             }
             const bool s2_tc = u.kind == U_CONV && u.up_off >= 0;
             void* up = s2_tc ? s->up_mem + u.up_off : nullptr;
@@ -854,8 +885,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             else if (u.kind == U_CONV && conv3_wgrad_tc_supported(dt, u.g))
                 conv3_bwd_weight_tc(u.g, d, xin, wscratch, s->scratch_floats, s->g + u.w_off, s->err, wst);
             else if (u.kind == U_CONV) conv_bwd_weight(dt, u.g, d, xin, wscratch, s->scratch_floats, s->g + u.w_off, wst);
-            else if (u.g.k != 3) dwk_bwd_weight(dt, u.g, d, xin, wscratch, s->scratch_floats, s->g + u.w_off, wst);
-            else dw_bwd_weight(dt, u.g, d, xin, wscratch, s->scratch_floats, s->g + u.w_off, wst);
+            else dwk_bwd_weight(dt, u.g, d, xin, wscratch, s->scratch_floats, s->g + u.w_off, wst);
             if (want_in) {
                 GradState& gi = gs[u.in];
                 const void* addend = gi.state == G_NONE ? nullptr : gi.ptr;
@@ -902,8 +932,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 } else if (u.kind == U_CONV && conv3_tc_supported(dt, u.g)) conv3_bwd_data_tc(u.g, d, s->wtb + u.w_off, addend, own(u.in), s->err, st);
                 else if (s2_tc) conv3_bwd_data_tc(s1_geom(u), dup, s->wtb + u.w_off, addend, own(u.in), s->err, st, conv_flops(u.g));
                 else if (u.kind == U_CONV) conv_bwd_data(dt, u.g, d, s->derived + u.w_off, addend, own(u.in), st);
-                else if (u.g.k != 3) dwk_bwd_data(dt, u.g, d, s->derived + u.w_off, addend, own(u.in), st);
-                else dw_bwd_data(dt, u.g, d, s->derived + u.w_off, addend, own(u.in), st);
+                else dwk_bwd_data(dt, u.g, d, s->derived + u.w_off, addend, own(u.in), st);
                 gi.state = G_OWNED;
                 gi.ptr = own(u.in);
             }
@@ -974,6 +1003,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
     }
     if (s->need_dx && gs[0].state == G_ALIAS)
         CU(cudaMemcpyAsync(dx, gs[0].ptr, s->vals[0].elems * s->esz, cudaMemcpyDeviceToDevice, st));
+    if (s->n_dw_weights) dw3_settle(s->bsum, s->dw_tab, s->n_dw, s->n_dw_weights, s->g, st);
     if (side_used) {            // join: the call's work is complete, in the caller's stream order, when the second stream's is
         CU(cudaEventRecord(s->ev_join, s->side));
         CU(cudaStreamWaitEvent(st, s->ev_join, 0));
@@ -1018,7 +1048,14 @@ static int create_impl(const ast_layer* net, int n_layers, int first, int last, 
         if ((rc = arena_alloc(s, "padded weight gradient", &s->gpad, s->n_gpad * 4, &work))) return rc;
     }
     if ((rc = arena_alloc(s, "forward channel sums", &s->fsum, s->n_bn_ch * 2 * sizeof(double), &work))) return rc;
-    if ((rc = arena_alloc(s, "backward channel sums", &s->bsum, s->n_bn_ch * 2 * sizeof(double), &work))) return rc;
+    if ((rc = arena_alloc(s, "backward channel sums", &s->bsum, s->n_bsum * sizeof(double), &work))) return rc;
+    if (s->n_dw) {
+        std::vector<DwSettle> tab;
+        for (const auto& u : s->units)
+            if (u.kind == U_DW && u.g.k == 3) tab.push_back(DwSettle{u.acc_off, (size_t)u.w_off, u.g.ci});
+        if ((rc = arena_alloc(s, "depthwise layer table", &s->dw_tab, tab.size() * sizeof(DwSettle), &work))) return rc;
+        CU(cudaMemcpy(s->dw_tab, tab.data(), tab.size() * sizeof(DwSettle), cudaMemcpyHostToDevice));
+    }
     if ((rc = arena_alloc(s, "statistics pivots", &s->pivots, s->n_bn_ch * 4, &work))) return rc;
     if ((rc = arena_alloc(s, "error word", &s->err, 256, &work))) return rc;
     if ((rc = arena_alloc(s, "momentum", &s->v, np * 4, &opt))) return rc;
@@ -1203,7 +1240,7 @@ int asteroid_stage_accumulate(asteroid_stage* s, int mb, void* stream) {
     if (!s) return fail(AST_ERR_ARG, "null argument");
     if (s->pending_g != mb) return fail(AST_ERR_ORDER, "accumulate(%d): the last backward was of micro-batch %d", mb, s->pending_g);
     if (s->n_acc >= s->M) return fail(AST_ERR_ORDER, "already accumulated %d micro-batches this round", s->M);
-    accumulate(s->G, s->g, s->n_pad, s->bsum, 2 * s->n_bn_ch, (cudaStream_t)stream);
+    accumulate(s->G, s->g, s->n_pad, s->bsum, s->n_bsum, (cudaStream_t)stream);
     s->bsum_dirty = s->bsum_dirty && s->n_pad == 0;
     CU(cudaGetLastError());
     s->pending_g = -1;

@@ -54,31 +54,78 @@ uint32_t w_pitch(int K) {
 
 }  // namespace
 
-// Which layers run here and how they are tiled.  Times below: one layer with its BatchNorm sums in a captured chain of launches, inputs
-// of large layers from HBM; "before" is the tensor-memory pipeline (or, above 256 channels, the one-tile / streaming kernels of
+// Backward tilings by a cost model (us), fitted to 1 500 timings over 49 layers (512 to 200 704 pixels, 16 to 1280 channels, with and without an
+// addend): within 2.2 % of the best tiling on average, at worst 27 %.  Persistent form: a CTA's tile takes the longer of its own latency
+// and the issue time of all warps on the multiprocessor, per 32-channel chunk and column tile, plus the epilogue, which an addend makes longer;
+// weights are staged once per CTA.  Split form: one tile per CTA, waves over the chip.  Offered are the tilings that won somewhere: with two
+// pixel tiles per warp one CTA of eight warps or two of four; eight column tiles per warp only with one pixel tile (the epilogue holds four
+// vectors per column tile).  Before the model (one rule as in the forward): 128 -> 512 at 25 088 pixels 57.6 -> 52.2 us, 64 -> 64 at 100 352
+// 27.5 -> 21.4, 160 -> 960 at 784 8.1 -> 6.0, 384 -> 64 at 3136 10.5 -> 6.7.
+bool bwd_choose(int P, int K, int N, MmaTiling* out) {
+    const int KCH = (K + 31) / 32, sms = sm_count();
+    double best = 0;
+    auto offer = [&](int mi, int nj, int wm, int wk, int ctas) {
+        const MmaTiling c{mi, nj, wm, 1, wk, ctas};
+        if (mma_smem(true, K, c) * (wk == 1 ? ctas : 1) > 200 * 1024) return;
+        const int cols = (N + 8 * nj - 1) / (8 * nj);
+        double t;
+        if (wk == 1) {
+            const int tiles = (P + 16 * mi * wm - 1) / (16 * mi * wm), cap = sms * ctas / cols > 0 ? sms * ctas / cols : 1, gx = tiles < cap ? tiles : cap;
+            const int turns = (tiles + gx - 1) / gx;
+            int r = (gx * cols + sms - 1) / sms;
+            if (r > ctas) r = ctas;
+            const double issue = (double)r * wm * mi * (KCH * (0.0502 + 0.00418 * nj) + nj * 0.0315);
+            const double lat = 1.01 + 0.476 * KCH * (1.0 + 0.269 * (mi - 1)) + 0.0202 * mi * nj;
+            t = 1.53 + 0.0154 * r * nj * KCH + turns * (lat > issue ? lat : issue);
+        } else {
+            const int bm = 128 / wk, waves = ((P + bm - 1) / bm * cols + sms - 1) / sms, kc = (KCH + wk - 1) / wk;
+            t = 0.714 + waves * (1.85 + kc * (0.651 + 0.00019 * nj) + nj * 0.0301 * (1.0 + 0.0529 * wk) + 0.0224 * nj * KCH);
+        }
+        if (best == 0 || t < best) {
+            best = t;
+            *out = c;
+        }
+    };
+    for (int nj : {8, 6, 4, 3, 2}) {
+        const bool narrow = (nj == 2 && N > 16) || (nj == 3 && N > 24);       // only where the weights of more columns do not fit
+        if (narrow ? best != 0 : (N + 8 * nj - 1) / (8 * nj) * nj * 8 > N * 1.35 + 8) continue;
+        if (nj == 8) {
+            offer(1, 8, 4, 1, 2);
+            offer(1, 8, 8, 1, 1);
+        } else {
+            offer(2, nj, 8, 1, 1);
+            offer(2, nj, 4, 1, 2);
+            offer(1, nj, 8, 1, 2);
+        }
+        if (P <= 30000)
+            for (int wk : {2, 4, 8}) offer(1, nj, 8 / wk, wk, 1);
+    }
+    return best != 0;
+}
+
+// Which layers run here and how the forward is tiled.  Times below: one layer with its BatchNorm sums in a captured chain of launches,
+// inputs of large layers from HBM; "before" is the tensor-memory pipeline (or, above 256 channels, the one-tile / streaming kernels of
 // pw_tc.cu and pw_stream.cu) with its finishing kernel.
 //   - More than 256 x 64 products per pixel on more than 50 000 pixels: the arithmetic of mma.sync (and the shared-memory reads of its
 //     weights) is what bounds such a layer and the tensor-memory pipeline is as fast or faster (64 -> 256 at 100 352 pixels: 26.4 us
-//     against 27.4; 256 -> 128: 33.4 against 39.8).  It takes at most 256 channels a side, so wider layers run here (128 -> 512 at
-//     25 088 pixels: 33.5 -> 22.7 us; 512 -> 128: 27.4 -> 22.8).
+//     against 27.4; 256 -> 128: 33.4 against 39.8; backward to 256 channels 71 against 77, but to 64 channels 45 against 42.5).  It takes at
+//     most 256 channels a side, so wider layers run here (128 -> 512 at 25 088 pixels: 33.5 -> 22.7 us; 512 -> 128: 27.4 -> 22.8).
 //   - A reduction of at most 192 channels, or at least 6 000 pixels, or twice as many output as reduction channels: the persistent
-//     form (24 -> 144 at 100 352 pixels 18.7 -> 13.8 us, backward 26.1 -> 24.2; 144 -> 24: 20.2 -> 12.7 and 30.4 -> 22.9; 160 -> 960 at 784
-//     pixels 18.4 -> 5.3 and 21.5 -> 6.8).
-//   - Else the split form: as many warps on the reduction as it takes to give the chip about one (backward) or one and a
-//     half (forward) CTAs per multiprocessor (960 -> 160 at 784 pixels 40.9 -> 6.9 us, backward 53.0 -> 9.8; 384 -> 64 at 784: 13.0 ->
-//     3.9 and 21.7 -> 4.6).
+//     form (24 -> 144 at 100 352 pixels 18.7 -> 13.8 us; 144 -> 24: 20.2 -> 12.7; 160 -> 960 at 784 pixels 18.4 -> 5.3).
+//   - Else the split form: as many warps on the reduction as it takes to give the chip about one and a half CTAs per multiprocessor
+//     (960 -> 160 at 784 pixels 40.9 -> 6.9 us; 384 -> 64 at 784: 13.0 -> 3.9).
 bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {
     if (K % 8 || N % 8 || (double)P * (K > N ? K : N) * 2.0 >= 4.0e9) return false;
-    if (P >= 50000 && K <= 256 && N <= 256 && K * N >= 256 * 64) return false;
+    if (P >= 50000 && K <= 256 && N <= 256 && K * N >= 256 * 64 && !(bwd && N <= 64)) return false;
+    if (bwd) return bwd_choose(P, K, N, out);
     const int KCH = (K + 31) / 32, sms = sm_count();
     MmaTiling c{};
     c.mi = 1; c.wm = 8; c.wn = 1; c.wk = 1; c.ctas = 1;
     auto cols = [&](int nj) { return (N + 8 * nj - 1) / (8 * nj); };
     if (KCH <= 6 || P >= 6000 || N >= 2 * K) {
-        // column tile: least padding, then fewest blocks; the backward epilogue holds too much per column for eight tiles unless N is 64
+        // column tile: least padding, then fewest blocks
         int best = 0, best_cost = 0;
         for (int nj : {8, 6, 4, 3, 2}) {
-            if (bwd && nj == 8 && N > 64) continue;
             const int cost = cols(nj) * nj * 8 * 4 + cols(nj) * 24;
             if (!best || cost < best_cost) {
                 best = nj;
@@ -92,16 +139,16 @@ bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {
         if (ctas() < sms && c.nj == 8) c.nj = 4;
         if (ctas() < sms && c.nj == 6 && N % 32 == 0) c.nj = 4;
         if (ctas() < sms) c.wm = 4;
-        if (!bwd && (c.mi == 1 || c.nj <= 3)) c.ctas = 2;
+        if (c.mi == 1 || c.nj <= 3) c.ctas = 2;
         if (c.wm == 4) c.ctas = 4;
     } else {
         c.nj = N <= 16 ? 2 : N <= 24 ? 3 : 4;
         c.wk = 2;
-        const int want = bwd ? sms * 4 / 5 : sms * 5 / 4;
+        const int want = sms * 5 / 4;
         while (c.wk < 8 && (P + 128 / c.wk - 1) / (128 / c.wk) * cols(c.nj) < want) c.wk *= 2;
         c.wm = 8 / c.wk;
     }
-    while (mma_smem(bwd, K, c) > 200 * 1024) {
+    while (mma_smem(false, K, c) > 200 * 1024) {
         if (c.nj <= 2) return false;
         c.nj = c.nj == 8 ? 6 : c.nj == 6 ? 4 : c.nj - 1;
     }
@@ -137,7 +184,7 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
         a.pf = p.pf;
         xf = p.x.act != ACT_NONE ? XF_ACT : (p.x.scale || p.pf.sums) ? XF_AFFINE : XF_NONE;
     }
-    a.w = p.w; a.bias = p.bias; a.addend = p.addend; a.out = p.out;
+    a.w = (const __nv_bfloat16*)p.w; a.bias = p.bias; a.addend = p.addend; a.out = (__nv_bfloat16*)p.out;
     a.WM = c.wm; a.WN = c.wn;
     a.wpitch = w_pitch(p.K);
     const int BN = c.wk == 1 ? c.wn * c.nj * 8 : c.nj * 8, BM = c.wk == 1 ? 16 * c.mi * c.wm : 16 * (8 / c.wk);

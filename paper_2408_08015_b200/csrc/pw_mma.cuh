@@ -298,8 +298,19 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
         }
     };
     if (BWD && sums) fetch_z(tile);
+    // the addend one column group ahead (the first one before the products), where registers allow
+    constexpr bool AHEAD = MI * NJ < 16;
+    CVec<C> av[2][MI][2];
+    auto fetch_add = [&](int gr, int row0, CVec<C> (*v)[2]) {
+        const uint32_t n = (uint32_t)min(n0 + wn * NJ * 8 + gr * 8 * G + C * t, a.N - C);
+#pragma unroll
+        for (int mi = 0; mi < MI; ++mi)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) v[mi][h].load(a.addend, ((uint32_t)min(row0 + mi * 16 + h * 8, a.P - 1) * (uint32_t)a.N + n) * 2u);
+    };
     for (; tile < a.m_tiles; tile += gridDim.x) {
         const int row0 = tile * BM + warp_row;
+        if (BWD && AHEAD && a.addend) fetch_add(0, row0, av[0]);
         float acc[MI][NJ][4];
 #pragma unroll
         for (int mi = 0; mi < MI; ++mi)
@@ -333,6 +344,8 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
 #pragma unroll
         for (int gr = 0; gr < NG; ++gr) {
             const int cl = wn * NJ * 8 + gr * 8 * G + C * t, n = n0 + cl;
+            if (BWD && AHEAD && a.addend && gr + 1 < NG) fetch_add(gr + 1, row0, av[(gr + 1) & 1]);
+            if (BWD && !AHEAD && a.addend) fetch_add(gr, row0, av[gr & 1]);
             if (n >= a.N) continue;
             SumCoef<BWD> sc[G];
             if (sums) {
@@ -346,12 +359,11 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
                     const int p = row0 + mi * 16 + h * 8;
                     if (p >= a.P) continue;
                     const uint32_t e = ((uint32_t)p * (uint32_t)a.N + (uint32_t)n) * 2u;
-                    CVec<C> av, ov;
-                    if (BWD && a.addend) av.load(a.addend, e);
+                    CVec<C> ov;
 #pragma unroll
                     for (int q = 0; q < G; ++q) {
                         float2 v = make_float2(acc[mi][gr * G + q][2 * h], acc[mi][gr * G + q][2 * h + 1]);
-                        if (BWD && a.addend) v = __fadd2_rn(v, unpack2(av.w[q]));
+                        if (BWD && a.addend) v = __fadd2_rn(v, unpack2(av[gr & 1][mi][h].w[q]));
                         if (!BWD && a.bias) v = __fadd2_rn(v, make_float2(__ldg(a.bias + n + 2 * q), __ldg(a.bias + n + 2 * q + 1)));
                         ov.w[q] = pack2(v);
                         if (sums) sc[q].add(ov.w[q], BWD ? zv[gr][mi][h].w[q] : 0u, rlo, rhi, s1[gr * G + q], s2[gr * G + q]);

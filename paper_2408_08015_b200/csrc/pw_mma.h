@@ -17,10 +17,10 @@ struct MmaProblem {
     GradSrc dz;                // backward operand
     BnPendFwd pf;              // pending coefficients of x
     BnPendBwd pb;              // pending coefficients of dz
-    const __nv_bfloat16* w;    // [N][K]
+    const void* w;             // [N][K]
     const float* bias;
     const void* addend;
-    __nv_bfloat16* out;
+    void* out;
     BnSumsOut so;              // column sums of the output (sums null: none)
     const BnRed* red;          // backward: the unit the sums belong to
 };
@@ -46,5 +46,19 @@ struct WgradTiling {
 bool wgrad_mma_choose(int P, int CO, int CI, bool pipeline_fits, size_t scratch_floats, WgradTiling* out);
 size_t wgrad_mma_smem(const WgradTiling& c);
 void wgrad_mma_launch(const WgradProblem& p, const WgradTiling& c, float* scratch, float* gw, cudaStream_t st);
+
+// ---- float32 (pw_f32.cu): columns per lane, warps on the reduction, CTAs per multiprocessor; false: not whole vectors of four channels
+struct F32Tiling {
+    int tn, wk, ctas;
+};
+bool f32_choose(bool bwd, int P, int K, int N, F32Tiling* out);
+size_t f32_smem(bool bwd, int K, const F32Tiling& c);
+void f32_launch(bool bwd, const MmaProblem& p, const F32Tiling& c, int kind, double bytes, cudaStream_t st);
+// narrow-side channels per lane; pixel ranges, `cluster` of them summed in the kernel
+struct F32WgradTiling {
+    int tn, splits, cluster;
+};
+bool f32_wgrad_choose(int P, int CO, int CI, size_t scratch_floats, F32WgradTiling* out);
+void f32_wgrad_launch(const WgradProblem& p, const F32WgradTiling& c, float* scratch, float* gw, cudaStream_t st);
 
 }  // namespace ast

@@ -604,6 +604,13 @@ static bool mma_unit(const asteroid_stage* s, const Unit& u, const ConvGeom& g, 
     return bwd ? mma_choose(true, g.n * g.ho * g.wo, g.co, g.ci, t) : mma_choose(false, g.n * g.ho * g.wo, g.ci, g.co, t);
 }
 
+// ... and on the float32 ones
+static bool f32_unit(const asteroid_stage* s, const Unit& u, bool bwd, F32Tiling* t) {
+    const ConvGeom& g = u.g;
+    if (s->dtype != AST_F32 || u.kind != U_CONV || g.k != 1 || g.stride != 1 || g.pad != 0) return false;
+    return bwd ? f32_choose(true, g.n * g.ho * g.wo, g.co, g.ci, t) : f32_choose(false, g.n * g.ho * g.wo, g.ci, g.co, t);
+}
+
 static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cudaStream_t st) {
     SlotView sv = slot_view(s, slot);
     const int dt = s->dtype;
@@ -627,19 +634,24 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
         int fused_stats = 0;       // > 0: the producing kernel wrote that many statistics partials into the scratch arena; -1: it took the sums
         const bool bn = u.l_bn >= 0;
         MmaTiling til;
+        F32Tiling til32;
         // the pointwise layer on the register-operand kernels: forms its input's pending coefficients, takes its output's sums
-        auto on_mma = [&](const ConvGeom& g, const ValSrc& xs, int in_unit, const __nv_bfloat16* w) {
+        auto on_mma = [&](const ConvGeom& g, const ValSrc& xs, int in_unit, const void* w) {
             MmaProblem p{};
             p.P = g.n * g.ho * g.wo; p.K = g.ci; p.N = g.co;
-            p.x = xs; p.w = w; p.out = (__nv_bfloat16*)obuf;
+            p.x = xs; p.w = w; p.out = obuf;
             p.bias = u.b_off >= 0 ? s->w + u.b_off : nullptr;
             p.pf = pend.take_fwd(in_unit);
             if (bn) p.so = sums_fwd(s, u);
-            mma_launch(false, p, til, K_PW_FWD_TC, 2.0 * ((double)p.P * p.K + (double)p.P * p.N) + 2.0 * p.N * p.K, st);
+            const double elems = (double)p.P * p.K + (double)p.P * p.N + (double)p.N * p.K;
+            if (dt == AST_F32) f32_launch(false, p, til32, K_CONV_FWD, 4.0 * elems, st);
+            else mma_launch(false, p, til, K_PW_FWD_TC, 2.0 * elems, st);
             fused_stats = bn ? -1 : 0;
         };
         if (u.kind == U_CONV && !u.col_kp && u.sub_off < 0 && mma_unit(s, u, u.g, false, &til)) {
             on_mma(u.g, val_src(s, sv, u.in), producer(u.in), s->wb + u.w_off);
+        } else if (f32_unit(s, u, false, &til32)) {
+            on_mma(u.g, val_src(s, sv, u.in), producer(u.in), s->w + u.w_off);
         } else if (u.kind == U_CONV) {
             pend.settle_fwd(producer(u.in));
             const float* bias = u.b_off >= 0 ? s->w + u.b_off : nullptr;
@@ -822,8 +834,13 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             const bool mma_w = pw && wgrad_mma_choose(wg.n * wg.ho * wg.wo, wg.co, wg.ci, pw_wgrad_pipeline_fits(wg, grad_needs_z(d), s->scratch_floats),
                                                       s->scratch_floats, &til_w);
             const bool mma_d = want_in && u.kind == U_CONV && !u.col_kp && mma_unit(s, u, u.g, true, &til_d);
+            F32Tiling til_d32{};
+            F32WgradTiling til_w32{};
+            const bool f32_d = want_in && f32_unit(s, u, true, &til_d32);
+            const bool f32_w = u.kind == U_CONV && dt == AST_F32 && wg.k == 1 && wg.stride == 1 && wg.pad == 0 &&
+                               f32_wgrad_choose(wg.n * wg.ho * wg.wo, wg.co, wg.ci, s->scratch_floats, &til_w32);
             const bool dw3 = u.kind == U_DW && u.g.k == 3;
-            if (!dw3 && (!mma_w || (want_in && !mma_d))) pend.settle_bwd(ui);
+            if (!dw3 && ((!mma_w && !f32_w) || (want_in && !mma_d && !f32_d))) pend.settle_bwd(ui);
             const BnPendBwd pb = pend.has(ui) ? pend_bwd(s, sv, u) : BnPendBwd{};
             pend.unit[ui] = 0;
             tick(s, ui, 4, st);
@@ -865,13 +882,14 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             }
             if (s2_tc && conv3_wgrad_tc_supported(dt, s1_geom(u)))
                 conv3_bwd_weight_tc(s1_geom(u), dup, xin, wscratch, s->scratch_floats, s->g + u.w_off, s->err, wst, conv_flops(u.g));
-            else if (mma_w) {
+            else if (mma_w || f32_w) {
                 WgradProblem p{};
                 p.P = wg.n * wg.ho * wg.wo; p.CO = wg.co; p.CI = wg.ci;
                 p.dz = d; p.x = xin; p.pb = pb; p.pend_write = want_in ? 0 : 1;
                 if (u.col_kp) p.x = ValSrc{sv.base + u.col_off, nullptr, nullptr, ACT_NONE};
                 else if (u.sub_off >= 0) p.x.p = sv.base + u.sub_off;                  // written by the forward of this micro-batch
-                wgrad_mma_launch(p, til_w, wscratch, u.col_kp ? s->gpad : s->g + u.w_off, wst);
+                if (f32_w) f32_wgrad_launch(p, til_w32, wscratch, s->g + u.w_off, wst);
+                else wgrad_mma_launch(p, til_w, wscratch, u.col_kp ? s->gpad : s->g + u.w_off, wst);
                 if (u.col_kp) conv_unpad_grad(s->gpad, u.g.co, u.g.k * u.g.k * u.g.ci, u.col_kp, s->g + u.w_off, wst);
             } else if (u.kind == U_CONV && u.col_kp) {
                 pw_bwd_weight_tc(col_geom(u), d, ValSrc{sv.base + u.col_off, nullptr, nullptr, ACT_NONE}, wscratch, s->scratch_floats, s->gpad, s->err, wst);
@@ -892,11 +910,11 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 // this kernel writes the complete gradient of its input value: let it also take the BatchNorm-backward
                 // sums of the unit that gradient belongs to
                 const int tgt = s->vals[u.in].first_cons == ui ? bn_reduce_target(s, u.in) : -1;
-                if (mma_d) {
+                if (mma_d || f32_d) {
                     MmaProblem p{};
                     BnRed red{};
                     p.P = u.g.n * u.g.ho * u.g.wo; p.K = u.g.co; p.N = u.g.ci;
-                    p.dz = d; p.pb = pb; p.w = s->wtb + u.w_off; p.addend = addend; p.out = (__nv_bfloat16*)own(u.in);
+                    p.dz = d; p.pb = pb; p.w = f32_d ? (const void*)(s->derived + u.w_off) : s->wtb + u.w_off; p.addend = addend; p.out = own(u.in);
                     if (tgt >= 0) {
                         const Unit& tu = s->units[tgt];
                         const Val& tv = s->vals[tu.out];
@@ -908,8 +926,9 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                         reduced[tgt] = 1;
                         s->bwd_sums_by[tgt] = ui;
                     }
-                    mma_launch(true, p, til_d, K_PW_BWD_DATA_TC, 2.0 * (double)p.P * p.K * (grad_needs_z(d) ? 2.0 : 1.0) +
-                               2.0 * (double)p.P * p.N * (addend ? 2.0 : 1.0) + 2.0 * p.N * p.K, st);
+                    const double elems = (double)p.P * p.K * (grad_needs_z(d) ? 2.0 : 1.0) + (double)p.P * p.N * (addend ? 2.0 : 1.0) + (double)p.N * p.K;
+                    if (f32_d) f32_launch(true, p, til_d32, K_CONV_BWD_DATA, 4.0 * elems, st);
+                    else mma_launch(true, p, til_d, K_PW_BWD_DATA_TC, 2.0 * elems, st);
                 } else if (u.kind == U_CONV && pw_tc_supported(dt, u.g, true)) {
                     BnRed red{};
                     if (tgt >= 0) {

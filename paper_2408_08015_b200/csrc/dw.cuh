@@ -1,4 +1,4 @@
-// Depthwise 3x3 convolution, NHWC: pieces shared by the forward and the fused backward kernels (dw3.cu).
+// Depthwise convolution, NHWC: pieces shared by the 3x3 (dw3.cu) and 5x5 (dw5.cu) kernels.
 //
 // A thread owns two channels and a strip of TW pixels and walks down its rows.  Two channels, not four or eight: the nine weights, the
 // coefficients of every transform and the nine weight-gradient sums of two channels fit in registers (72 of them), where four channels'
@@ -76,14 +76,15 @@ __device__ __forceinline__ void stage_grad(const GradSrc& g, const BnPendBwd& p,
     }
 }
 
-// Sum over the block's threads that own the same channels (tid % lanes), in thread order, of N pairs per thread; channel c's sum k goes to
-// acc[k * c_total + c0 + c].  red: N * blockDim.x pairs.
-template <int N> __device__ __forceinline__ void block_sums(const float2* v, int lanes, int rows, int c0, int c, double* acc, float* red) {
-    const int width = 2 * lanes, pitch = 2 * lanes * rows;
+// Sum over the block's threads that own the same channels (tid % lanes), in thread order, of N values of V (float: one channel a lane, float2:
+// two) per thread; channel c's sum k goes to acc[k * c_total + c0 + c].  red: N * blockDim.x V.
+template <int N, typename V> __device__ __forceinline__ void block_sums(const V* v, int lanes, int rows, int c0, int c, double* acc, float* red) {
+    constexpr int CH = sizeof(V) / 4;
+    const int width = CH * lanes, pitch = CH * lanes * rows;
     __syncthreads();
     if ((int)threadIdx.x < lanes * rows)
 #pragma unroll
-        for (int k = 0; k < N; ++k) *reinterpret_cast<float2*>(red + k * pitch + threadIdx.x * 2) = v[k];
+        for (int k = 0; k < N; ++k) *reinterpret_cast<V*>(red + k * pitch + threadIdx.x * CH) = v[k];
     __syncthreads();
     for (int i = threadIdx.x; i < N * width; i += blockDim.x) {
         const int k = i / width, j = i - k * width;
@@ -94,6 +95,63 @@ template <int N> __device__ __forceinline__ void block_sums(const float2* v, int
         }
     }
 }
+
+// the thread's N weights of its two channels
+template <int N> __device__ __forceinline__ void load_weights(const float* wkc, int c, int c0, bool live, float2* w) {
+#pragma unroll
+    for (int t = 0; t < N; ++t) w[t] = live ? __ldg(reinterpret_cast<const float2*>(wkc + (size_t)t * c + c0)) : zero2();
+}
+
+constexpr int BT = 128;
+
+struct DwGeom {
+    int n, hi, wi, ho, wo, c;
+    int lanes, rows;             // channel groups per block; strips a block works on side by side
+    int th, nrc, sw, items;      // rows per strip, row chunks, strips across, work items
+};
+
+struct DwFwdArgs {
+    DwGeom g;
+    ValSrc x;
+    BnPendFwd pf;
+    const float* wkc;           // tap-major weights
+    void* out;
+    BnSumsOut so;
+    bool first;                  // writes the pending coefficients out
+};
+
+struct DwBwdArgs {
+    DwGeom g;
+    GradSrc dz;
+    BnPendBwd pb;
+    ValSrc x;                    // raw input with its (final) coefficients
+    const float* wkc;           // tap-major weights
+    const void* addend;
+    void* dx;                    // may be null: weight gradient only
+    double* gw;                  // [taps][c] accumulators of the weight gradient
+    double* sums;                // [2][c] of the unit that produced x, or null
+    const float *mean, *rstd;    // of that unit
+    bool first;
+};
+
+inline double esz(int dtype) { return dtype == 0 ? 4.0 : 2.0; }
+
+// lanes of a block over the groups of `per` channels: an even split in at most 32
+inline void cut_channels(DwGeom& d, int per = 2) {
+    const int cv = d.c / per, parts = (cv + 31) / 32;
+    d.lanes = (cv + parts - 1) / parts;
+    d.rows = BT / d.lanes;
+}
+inline dim3 cut_grid(const DwGeom& d, int ctas, int per = 2) {
+    const int gy = (d.c / per + d.lanes - 1) / d.lanes, gx = (d.items + d.rows - 1) / d.rows, cap = (int)((long long)sm_count() * ctas / gy);
+    return dim3(gx < cap ? gx : cap > 0 ? cap : 1, gy);
+}
+// images per launch: byte offsets within a launch are 32-bit
+inline int image_chunk(int dtype, const ConvGeom& g) {
+    const size_t img = (size_t)g.hi * g.wi * g.ci * (dtype == 0 ? 4 : 2), m = 0x7fffffffu / img;
+    return m < 1 ? 1 : m < (size_t)g.n ? (int)m : g.n;
+}
+inline const void* at(const void* p, size_t e, int dtype) { return p ? (const char*)p + e * (dtype == 0 ? 4 : 2) : nullptr; }
 
 }  // namespace dw
 }  // namespace ast

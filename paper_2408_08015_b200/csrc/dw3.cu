@@ -16,50 +16,12 @@
 //   bf16 stride 2, same  forward 24.4 -> 19.0  backward  79 -> 26.6    112x112x32 x16 17.9 -> 12.2, 62.7 -> 23.0
 //   bf16 14x14x384 x4    forward 12.6 ->  3.8  backward  27 ->  5.7    7x7x960 x16    21.5 -> 4.8, 40.6 -> 8.3
 //   f32  28x28x144 x16   forward 10.7 ->  5.9  backward  35 -> 13.0    f32 56x56x96 x16  16.8 -> 13.5, 45.5 -> 28.9
-#include "dw3.cuh"
+#include "dw.cuh"
 
 namespace ast {
 namespace {
 
 using namespace dw;
-constexpr int BT = 128;
-
-struct DwGeom {
-    int n, hi, wi, ho, wo, c;
-    int lanes, rows;             // channel pairs per block; strips a block works on side by side
-    int th, nrc, sw, items;      // rows per strip, row chunks, strips across, work items
-};
-
-struct DwFwdArgs {
-    DwGeom g;
-    ValSrc x;
-    BnPendFwd pf;
-    const float* w9c;
-    void* out;
-    BnSumsOut so;
-    bool first;                  // writes the pending coefficients out
-};
-
-struct DwBwdArgs {
-    DwGeom g;
-    GradSrc dz;
-    BnPendBwd pb;
-    ValSrc x;                    // raw input with its (final) coefficients
-    const float* w9c;
-    const void* addend;
-    void* dx;                    // may be null: weight gradient only
-    double* gw;                  // [9][c] accumulators of the weight gradient
-    double* sums;                // [2][c] of the unit that produced x, or null
-    const float *mean, *rstd;    // of that unit
-    bool first;
-};
-
-// the thread's nine weights of its two channels
-__device__ __forceinline__ void load_weights(const float* w9c, int c, int c0, bool live, float2* w) {
-#pragma unroll
-    for (int t = 0; t < 9; ++t) w[t] = live ? __ldg(reinterpret_cast<const float2*>(w9c + (size_t)t * c + c0)) : zero2();
-}
-
 // In all three kernels EX says that the strips cover the columns exactly, so that only the first and the last column a strip reads can lie
 // outside the image; the row loop is unrolled by three so that the rotating rows (or accumulators) need no moves.
 
@@ -74,7 +36,7 @@ __global__ void __launch_bounds__(BT) dw3_fwd_kernel(const DwFwdArgs a) {
     const bool live = row < g.rows && c0 < g.c;
     const uint32_t cby = g.c * sizeof(T);
     float2 w[9];
-    load_weights(a.w9c, g.c, c0, live, w);
+    load_weights<9>(a.wkc, g.c, c0, live, w);
     pdl_wait();
     int item = blockIdx.x * g.rows + row, wo0 = 0, oh0 = 0, oh1 = 0, n = 0;
     uint32_t col[NIN];
@@ -265,7 +227,7 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s1_kernel(const DwBwdArgs a) {
     const bool live = row < g.rows && c0 < g.c;
     const uint32_t cby = g.c * sizeof(T), rby = g.wi * cby;
     float2 w[9], gw[9];
-    load_weights(a.w9c, g.c, c0, live, w);
+    load_weights<9>(a.wkc, g.c, c0, live, w);
     pdl_wait();
     P2<T> nd[NZ], nz[NZ], nx[TW];
     uint32_t col[NZ];
@@ -387,7 +349,7 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s2_kernel(const DwBwdArgs a) {
     const bool live = row < g.rows && c0 < g.c;
     const uint32_t cby = g.c * sizeof(T);
     float2 w[9], gw[9];
-    load_weights(a.w9c, g.c, c0, live, w);
+    load_weights<9>(a.wkc, g.c, c0, live, w);
     pdl_wait();
     P2<T> nd[TZ + 1], nz[TZ + 1], nx[2][2 * TZ];
     uint32_t zcol[TZ + 1], xcol[2 * TZ];
@@ -518,16 +480,16 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s2_kernel(const DwBwdArgs a) {
     if (a.sums) block_sums<2>(fs, g.lanes, g.rows, cb, g.c, a.sums, sm);
 }
 
-// gw[c][t] = acc[t][c] for the weight gradients of several layers at once
-__global__ void __launch_bounds__(256) dw3_settle_kernel(const double* __restrict__ acc, const DwSettle* __restrict__ tab, int layers, float* __restrict__ g) {
+// (also of dw5.cu) gw[c][t] = acc[t][c] for the weight gradients of several layers at once
+__global__ void __launch_bounds__(256) dw_settle_kernel(const double* __restrict__ acc, const DwSettle* __restrict__ tab, int layers, float* __restrict__ g) {
     pdl_wait();
     pdl_launch();
     int i = blockIdx.x * 256 + threadIdx.x;
     for (int l = 0; l < layers; ++l) {
         const DwSettle e = tab[l];
-        const int n = 9 * e.c;
+        const int n = e.taps * e.c;
         if (i < n) {
-            const int c = i / 9, t = i - 9 * c;
+            const int c = i / e.taps, t = i - e.taps * c;
             g[e.g_off + i] = (float)acc[e.acc_off + (size_t)t * e.c + c];
             return;
         }
@@ -535,28 +497,9 @@ __global__ void __launch_bounds__(256) dw3_settle_kernel(const double* __restric
     }
 }
 
-double esz(int dtype) { return dtype == 0 ? 4.0 : 2.0; }
-
-// lanes of a block over the channel pairs: an even split in at most 32
-void cut_channels(DwGeom& d) {
-    const int cv = d.c / 2, parts = (cv + 31) / 32;
-    d.lanes = (cv + parts - 1) / parts;
-    d.rows = BT / d.lanes;
-}
-dim3 cut_grid(const DwGeom& d, int ctas) {
-    const int gy = (d.c / 2 + d.lanes - 1) / d.lanes, gx = (d.items + d.rows - 1) / d.rows, cap = (int)((long long)sm_count() * ctas / gy);
-    return dim3(gx < cap ? gx : cap > 0 ? cap : 1, gy);
-}
-// images per launch: byte offsets within a launch are 32-bit
-int image_chunk(int dtype, const ConvGeom& g) {
-    const size_t per = (size_t)g.hi * g.wi * g.ci * (dtype == 0 ? 4 : 2), m = 0x7fffffffu / per;
-    return m < 1 ? 1 : m < (size_t)g.n ? (int)m : g.n;
-}
-const void* at(const void* p, size_t e, int dtype) { return p ? (const char*)p + e * (dtype == 0 ? 4 : 2) : nullptr; }
-
 }  // namespace
 
-void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf, const float* w9c, void* z, const BnSumsOut& so, const DwTiling& t, cudaStream_t st) {
+void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf, const float* wkc, void* z, const BnSumsOut& so, const DwTiling& t, cudaStream_t st) {
     typedef void (*Fn)(const DwFwdArgs);
     using B = __nv_bfloat16;
     Fn f;
@@ -570,7 +513,7 @@ void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf,
     for (int n0 = 0; n0 < g.n; n0 += chunk) {
         const int n = g.n - n0 < chunk ? g.n - n0 : chunk;
         DwFwdArgs a{};
-        a.x = x; a.pf = pf; a.w9c = w9c; a.so = so; a.first = n0 == 0;
+        a.x = x; a.pf = pf; a.wkc = wkc; a.so = so; a.first = n0 == 0;
         a.x.p = at(x.p, (size_t)n0 * g.hi * g.wi * g.ci, dtype);
         a.out = (void*)at(z, (size_t)n0 * g.ho * g.wo * g.ci, dtype);
         DwGeom& d = a.g;
@@ -582,7 +525,7 @@ void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf,
     }
 }
 
-void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* w9c, const void* addend, void* dx, double* gw,
+void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* wkc, const void* addend, void* dx, double* gw,
              double* sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st) {
     typedef void (*Fn)(const DwBwdArgs);
     using B = __nv_bfloat16;
@@ -600,7 +543,7 @@ void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& p
         const int n = g.n - n0 < chunk ? g.n - n0 : chunk;
         const size_t ie = (size_t)n0 * g.hi * g.wi * g.ci, oe = (size_t)n0 * g.ho * g.wo * g.ci;
         DwBwdArgs a{};
-        a.dz = dz; a.pb = pb; a.x = x; a.w9c = w9c; a.gw = gw; a.sums = dx ? sums : nullptr; a.mean = mean; a.rstd = rstd; a.first = n0 == 0;
+        a.dz = dz; a.pb = pb; a.x = x; a.wkc = wkc; a.gw = gw; a.sums = dx ? sums : nullptr; a.mean = mean; a.rstd = rstd; a.first = n0 == 0;
         a.dz.dy = at(dz.dy, oe, dtype);
         a.dz.z = at(dz.z, oe, dtype);
         a.x.p = at(x.p, ie, dtype);
@@ -615,9 +558,9 @@ void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& p
     }
 }
 
-void dw3_settle(const double* acc, const DwSettle* tab, int layers, size_t total, float* g, cudaStream_t st) {
+void dw_settle(const double* acc, const DwSettle* tab, int layers, size_t total, float* g, cudaStream_t st) {
     LaunchScope ls(K_DW_BWD_WEIGHT_FINISH, 12.0 * total, 0.0, st);
-    launch_pdl(dw3_settle_kernel, (unsigned)((total + 255) / 256), 256, 0, st, acc, tab, layers, g);
+    launch_pdl(dw_settle_kernel, (unsigned)((total + 255) / 256), 256, 0, st, acc, tab, layers, g);
 }
 
 // Strips of 4 pixels (2 where registers or the halo do not allow 4) and the height that makes the longest chain of row steps cheapest.

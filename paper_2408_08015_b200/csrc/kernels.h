@@ -175,18 +175,23 @@ void conv3_bwd_weight_tc(const ConvGeom& g, const GradSrc& dz, const ValSrc& x, 
 struct DwTiling {
     int tw, th, ctas;
 };
-// one depthwise layer of dw3_settle: offsets of its accumulators [9][c] and of its weight gradient [c][9]
+// one depthwise layer of dw_settle: offsets of its accumulators [taps][c] and of its weight gradient [c][taps]
 struct DwSettle {
     size_t acc_off, g_off;
-    int c;
+    int c, taps;
 };
 DwTiling dw3_choose(int dtype, bool bwd, const ConvGeom& g);
 void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf, const float* w9c, void* z, const BnSumsOut& so, const DwTiling& t, cudaStream_t st);
 // dx may be null (weight gradient only); gw: [9][c] accumulators; sums [2][c] (may be null), mean, rstd: of the unit that produced x
 void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* w9c, const void* addend, void* dx, double* gw,
              double* sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st);
-// accumulators -> weight gradients, all layers of the table (device memory); total: sum of 9*c
-void dw3_settle(const double* acc, const DwSettle* tab, int layers, size_t total, float* g, cudaStream_t st);
+// the same for 5x5 layers (dw5.cu)
+DwTiling dw5_choose(int dtype, bool bwd, const ConvGeom& g);
+void dw5_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf, const float* wkc, void* z, const BnSumsOut& so, const DwTiling& t, cudaStream_t st);
+void dw5_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* wkc, const void* addend, void* dx, double* gw,
+             double* sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st);
+// accumulators -> weight gradients, all layers of the table (device memory); total: sum of taps*c
+void dw_settle(const double* acc, const DwSettle* tab, int layers, size_t total, float* g, cudaStream_t st);
 
 // ---- BatchNorm statistics and backward reductions over a [pixels][c] tensor ----
 // sums of a [pixels][c] tensor of its own pass; the coefficients are then pending (fin.cuh)
@@ -228,17 +233,26 @@ void gap_fwd(int dtype, const ValSrc& x, int n, int hw, int c, void* out, cudaSt
 void gap_bwd(int dtype, const void* da, int n, int hw, int c, const void* addend, void* dx, cudaStream_t st);
 
 // ---- EfficientNet MBConv pieces (mbconv.cu) ----
-// SiLU as a materialising unit: out = silu(value(x)); dx = dy * silu'(value(x)) (+ addend)
-void silu_fwd(int dtype, const ValSrc& x, size_t pixels, int c, void* out, void* out2, cudaStream_t st);
-void silu_bwd(int dtype, const void* dy, const ValSrc& x, const void* addend, size_t pixels, int c, void* dx, cudaStream_t st);
+// SiLU as a materialising unit over [n][hw][c]: out = silu(value(x)); dx = dy * silu'(value(x)) (+ addend)
+// part: where the sums over runs of pixels of the output go, [returned count][n][c] (0: it does not fit, none written)
+int silu_fwd(int dtype, const ValSrc& x, const BnPendFwd& pf, int n, int hw, int c, void* out, void* out2, float* part, size_t part_floats, cudaStream_t st);
+// gate, ds (may be null): dy is the gradient behind a squeeze-excite layer whose own share is dy*gate + ds; sums (may be null), mean, rstd: of the
+// unit that produced x, which has no activation
+void silu_bwd(int dtype, const void* dy, const float* gate, const float* ds, const ValSrc& x, const void* addend, int n, int hw, int c, void* dx, double* sums,
+              const float* mean, const float* rstd, cudaStream_t st);
 // squeeze-excite over [n][hw][c] with k hidden units; s [n][c], p1 [n][k], gate [n][c] are float vectors kept for the backward pass;
-// work: >= n*(2c+k) floats; scratch: partials of the pixel-split reductions (any size >= n*c floats; more allows more splits)
+// scratch: partials of the pixel-split reductions (any size >= n*c floats; more allows more splits); splits > 0: that many are there already
 void se_forward(int dtype, const ValSrc& x, int n, int hw, int c, int k, const float* w1, const float* b1, const float* w2, const float* b2,
-                float* s, float* p1, float* gate, float* scratch, size_t scratch_floats, void* out, void* out2, cudaStream_t st);
-void se_backward(int dtype, const void* dout, const ValSrc& x, int n, int hw, int c, int k, const float* w1, const float* w2, const float* s,
-                 const float* p1, const float* gate, float* work, float* scratch, size_t scratch_floats, const void* addend, void* dx, float* gw1, float* gb1,
-                 float* gw2, float* gb2, cudaStream_t st);
-// depthwise conv of odd kernel size k <= 7, pad (k-1)/2, stride 1 or 2; weights tap-major wkc[r*k+s][c]; gw[c][k][k]
+                float* s, float* p1, float* gate, float* scratch, size_t scratch_floats, int splits, void* out, void* out2, cudaStream_t st);
+struct SeWork {
+    float *dp2, *ds, *dp1;     // [n][c], [n][c], [n][k]
+};
+// the gradient of the gate through the fully connected layers; then the parameter gradients; then dx = dout*gate + ds (+ addend)
+void se_backward_gate(int dtype, const void* dout, const ValSrc& x, int n, int hw, int c, int k, const float* w1, const float* w2, const float* p1,
+                      const float* gate, const SeWork& w, float* scratch, size_t scratch_floats, cudaStream_t st);
+void se_param_grads(const float* s, const float* p1, const SeWork& w, int n, int c, int k, float* gw1, float* gb1, float* gw2, float* gb2, cudaStream_t st);
+void se_backward_scale(int dtype, const void* dout, int n, int hw, int c, const float* gate, const float* ds, const void* addend, void* dx, cudaStream_t st);
+// 7x7 depthwise conv, pad 3, stride 1 or 2; weights tap-major wkc[r*k+s][c]; gw[c][k][k]
 void dwk_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const float* wkc, void* z, cudaStream_t st);
 void dwk_bwd_data(int dtype, const ConvGeom& g, const GradSrc& dz, const float* wkc, const void* addend, void* dx, cudaStream_t st);
 void dwk_bwd_weight(int dtype, const ConvGeom& g, const GradSrc& dz, const ValSrc& x, float* scratch, size_t scratch_floats, float* gw, cudaStream_t st);

@@ -1,9 +1,9 @@
 // Pieces of the EfficientNet MBConv block that the MobileNetV2 / ResNet kernels do not cover: the SiLU activation as a
 // materialising elementwise unit (forward and backward), the squeeze-excite layer (per-sample channel means, two tiny
-// fully connected layers, channel gate; forward and backward), and a depthwise convolution of any odd kernel size up to
-// 7 (the 5x5 layers of the network).  All are bandwidth-bound passes over [pixels][channels] tensors with the producer's
-// BatchNorm / activation applied while loading; reductions are two-stage and in fixed order (no float atomics).
-#include "kernels.h"
+// fully connected layers, channel gate; forward and backward), and the 7x7 depthwise convolution.  All are bandwidth-bound
+// passes over [pixels][channels] tensors with the producer's BatchNorm / activation applied while loading; reductions are two-stage
+// and in fixed order.
+#include "fin.cuh"
 
 namespace ast {
 namespace {
@@ -74,36 +74,192 @@ VecGrid vec_grid(size_t groups, int vpr, int per_thread) {
     return VecGrid{(unsigned)blocks, threads / vpr * vpr};
 }
 
-// ------------------------------------------------------------------------------------------ SiLU
-// forward: out = silu(value(x)); backward: dx = dy * silu'(value(x)) (+ addend), value(x) recomputed from the raw tensor
-template <typename T, int V, bool BWD>
-__global__ void __launch_bounds__(256) silu_kernel(ValSrc x, const T* __restrict__ dy, const T* addend, size_t groups, int vpr, size_t stride,
-                                                   T* __restrict__ out, T* __restrict__ out2) {
-    pdl_wait();
-    pdl_launch();
-    const size_t id = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= stride) return;
-    ChanVal<V> cv;
-    cv.init(x, (int)(id % (size_t)vpr) * V);
-    for (size_t i = id; i < groups; i += stride) {
-        float p[V], d[V], a[V];
-        ld_raw_w<T, V>(x.p, i * V, p);
-        cv.apply(p);
-        if (BWD) {
-            ld_raw_w<T, V>(dy, i * V, d);
-            if (addend) ld_raw_w<T, V>(addend, i * V, a);
-#pragma unroll
-            for (int q = 0; q < V; ++q) {
-                const float sg = sigmoidf_(p[q]);
-                p[q] = d[q] * sg * fmaf(p[q], 1.f - sg, 1.f) + (addend ? a[q] : 0.f);
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < V; ++q) p[q] = p[q] * sigmoidf_(p[q]);
-        }
-        st_raw_w<T, V>(out, i * V, p);
-        if (out2) st_raw_w<T, V>(out2, i * V, p);
+// ------------------------------------------------------------------------------------------ passes over [sample][pixel][channel]
+// A block owns one sample, a run of its pixels and up to 256 channel vectors: a thread keeps its channels' coefficients (and the sample's
+// gates) in registers and requests four pixels before it uses the first.  Before, threads strode over the flat tensor, one vector at a time,
+// with two 64-bit divisions per vector to find the sample: 28x28x240 at 32 images took 10.6 us forward (12 MB each way).
+struct PassCut {
+    int lanes, rows, parts, splits, ppb;   // channel vectors per block, pixels side by side, blocks along the channels and the pixels, pixels per block
+};
+PassCut pass_cut(int n, int hw, int vpr) {
+    PassCut c;
+    c.parts = (vpr + 255) / 256;
+    c.lanes = (vpr + c.parts - 1) / c.parts;
+    c.rows = 256 / c.lanes;
+    int want = (int)((long long)sm_count() * 4 / ((long long)n * c.parts));
+    const int most = (hw + 4 * c.rows - 1) / (4 * c.rows);
+    if (want > most) want = most;
+    if (want < 1) want = 1;
+    c.ppb = (hw + want - 1) / want;
+    c.splits = (hw + c.ppb - 1) / c.ppb;
+    return c;
+}
+struct PassIdx {
+    int jl, row, c0, pbeg, pend, sample, split;
+    size_t base;               // element of the thread's channels in the sample's first pixel
+    bool live;
+    template <int V> __device__ __forceinline__ void init(const PassCut& k, int hw, int c) {
+        jl = threadIdx.x % k.lanes;
+        row = threadIdx.x / k.lanes;
+        const int j = blockIdx.y * k.lanes + jl;
+        live = row < k.rows && j * V < c;
+        c0 = j * V;
+        sample = blockIdx.x / k.splits;
+        split = blockIdx.x - sample * k.splits;
+        pbeg = split * k.ppb;
+        pend = min(hw, pbeg + k.ppb);
+        base = (size_t)sample * hw * c + (live ? c0 : 0);
     }
+};
+// sum over the block's rows, in row order, of V values per thread -> sm[jl * V + q] of the first row's threads' channels, in out
+template <int V> __device__ __forceinline__ void rows_sum(const PassCut& k, const PassIdx& x, const float* v, float* sm, float* out) {
+    __syncthreads();
+    if (x.row < k.rows)
+#pragma unroll
+        for (int q = 0; q < V; ++q) sm[(x.row * k.lanes + x.jl) * V + q] = v[q];
+    __syncthreads();
+    if (x.row == 0)
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            float s = 0.f;
+            for (int r = 0; r < k.rows; ++r) s += sm[(r * k.lanes + x.jl) * V + q];
+            out[q] = s;
+        }
+}
+
+// ------------------------------------------------------------------------------------------ SiLU
+// out = silu(value(x)), with pending coefficients formed here; `part`, may be null: sums over the block's pixels of out as stored, [split][sample][c]
+// (the squeeze of a squeeze-excite layer behind)
+template <typename T, int V>
+__global__ void __launch_bounds__(256) silu_fwd_kernel(ValSrc x, BnPendFwd pf, PassCut k, int hw, int c, T* __restrict__ out, T* __restrict__ out2,
+                                                       float* __restrict__ part) {
+    pdl_launch();
+    pdl_wait();
+    extern __shared__ float sm[];              // scale and shift of the block's channels; then the sums
+    PassIdx ix;
+    ix.init<V>(k, hw, c);
+    const int width = k.lanes * V, cb = blockIdx.y * width;
+    for (int i = threadIdx.x; i < width; i += 256) {
+        float2 f = make_float2(1.f, 0.f);
+        if (cb + i < c) {
+            if (pf.sums) f = bn_fwd_coef(pf, cb + i, blockIdx.x == 0);
+            else if (x.scale) f = make_float2(x.scale[cb + i], x.shift[cb + i]);
+        }
+        sm[i] = f.x;
+        sm[width + i] = f.y;
+    }
+    __syncthreads();
+    ChanVal<V> cv;
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+        cv.sc[q] = sm[ix.jl * V + q];
+        cv.sh[q] = sm[width + ix.jl * V + q];
+    }
+    cv.lo = x.act == ACT_NONE ? -INFINITY : 0.f;
+    cv.hi = x.act == ACT_RELU6 ? 6.f : INFINITY;
+    float acc[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) acc[q] = 0.f;
+    if (ix.live)
+        for (int p0 = ix.pbeg + ix.row; p0 < ix.pend; p0 += 4 * k.rows) {
+            float v[4][V];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (p0 + u * k.rows < ix.pend) ld_raw_w<T, V>(x.p, ix.base + (size_t)(p0 + u * k.rows) * c, v[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (p0 + u * k.rows >= ix.pend) break;
+                const size_t e = ix.base + (size_t)(p0 + u * k.rows) * c;
+                cv.apply(v[u]);
+#pragma unroll
+                for (int q = 0; q < V; ++q) {
+                    v[u][q] *= sigmoidf_(v[u][q]);
+                    if (part) acc[q] += to_f<T>(from_f<T>(v[u][q]));
+                }
+                st_raw_w<T, V>(out, e, v[u]);
+                if (out2) st_raw_w<T, V>(out2, e, v[u]);
+            }
+        }
+    if (!part) return;
+    float s[V];
+    rows_sum<V>(k, ix, acc, sm, s);
+    if (ix.row == 0 && ix.live)
+#pragma unroll
+        for (int q = 0; q < V; ++q) part[((size_t)ix.split * (gridDim.x / k.splits) + ix.sample) * c + ix.c0 + q] = s[q];
+}
+
+// dx = dy' * silu'(value(x)) (+ addend), value(x) recomputed from the raw tensor; dy' = dy, or dy*gate + ds where a squeeze-excite layer behind left
+// its backward to this kernel; `sums`, may be null: the BatchNorm-backward sums of the unit in front, [2][c], taken from dx as stored
+struct SiluBwdArgs {
+    ValSrc x;
+    const void *dy, *addend;
+    const float *gate, *ds;    // [sample][c]
+    double* sums;
+    const float *mean, *rstd;
+    int hw, c;
+    void* dx;
+};
+template <typename T, int V> __global__ void __launch_bounds__(256) silu_bwd_kernel(SiluBwdArgs a, PassCut k) {
+    pdl_launch();
+    pdl_wait();
+    extern __shared__ float sm[];
+    PassIdx ix;
+    ix.init<V>(k, a.hw, a.c);
+    ChanVal<V> cv;
+    float gt[V], dsv[V], s1[V], s2[V];
+    if (ix.live) {
+        cv.init(a.x, ix.c0);
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            gt[q] = a.gate ? a.gate[(size_t)ix.sample * a.c + ix.c0 + q] : 1.f;
+            dsv[q] = a.gate ? a.ds[(size_t)ix.sample * a.c + ix.c0 + q] : 0.f;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < V; ++q) s1[q] = s2[q] = 0.f;
+    if (ix.live)
+        for (int p0 = ix.pbeg + ix.row; p0 < ix.pend; p0 += 2 * k.rows) {
+            float z[2][V], d[2][V], ad[2][V];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (p0 + u * k.rows >= ix.pend) break;
+                const size_t e = ix.base + (size_t)(p0 + u * k.rows) * a.c;
+                ld_raw_w<T, V>(a.x.p, e, z[u]);
+                ld_raw_w<T, V>(a.dy, e, d[u]);
+                if (a.addend) ld_raw_w<T, V>(a.addend, e, ad[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (p0 + u * k.rows >= ix.pend) break;
+                const size_t e = ix.base + (size_t)(p0 + u * k.rows) * a.c;
+                float o[V];
+#pragma unroll
+                for (int q = 0; q < V; ++q) {
+                    const float v = fminf(fmaxf(fmaf(z[u][q], cv.sc[q], cv.sh[q]), cv.lo), cv.hi), sg = sigmoidf_(v);
+                    o[q] = fmaf(d[u][q], gt[q], dsv[q]) * sg * fmaf(v, 1.f - sg, 1.f) + (a.addend ? ad[u][q] : 0.f);
+                }
+                st_raw_w<T, V>(a.dx, e, o);
+                if (a.sums) {
+                    // sum of dx * z here; mean and rstd enter at the end
+#pragma unroll
+                    for (int q = 0; q < V; ++q) {
+                        const float r = to_f<T>(from_f<T>(o[q]));
+                        s1[q] += r;
+                        s2[q] = fmaf(r, z[u][q] - __ldg(a.mean + ix.c0 + q), s2[q]);
+                    }
+                }
+            }
+        }
+    if (!a.sums) return;
+    float t1[V], t2[V];
+    rows_sum<V>(k, ix, s1, sm, t1);
+    rows_sum<V>(k, ix, s2, sm, t2);
+    if (ix.row == 0 && ix.live)
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            add_sum(a.sums + ix.c0 + q, t1[q]);
+            add_sum(a.sums + a.c + ix.c0 + q, t2[q] * a.rstd[ix.c0 + q]);
+        }
 }
 
 // ------------------------------------------------------------------------------------------ squeeze-excite
@@ -152,27 +308,51 @@ __global__ void __launch_bounds__(256) se_reduce_kernel(ValSrc x, const T* __res
     }
 }
 
+// w1 [k][c] and w2 [c][k] into shared memory, before the dependency wait (weights are not written by a kernel that releases its dependents early):
+// each of the fully connected products below then costs shared-memory reads instead of two more memory latencies
+__device__ __forceinline__ void stage_fc(const float* w1, const float* w2, int n, float* sw) {
+    for (int i = threadIdx.x; i < n; i += 256) {
+        sw[i] = __ldg(w1 + i);
+        sw[n + i] = __ldg(w2 + i);
+    }
+}
+// sum over the splits of part[z][n][i], in index order
+__device__ __forceinline__ float split_sum(const float* part, int splits, size_t stride) {
+    float a = 0.f;
+    for (int z0 = 0; z0 < splits; z0 += 8) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = z0 + u < splits ? part[(size_t)(z0 + u) * stride] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) a += v[u];
+    }
+    return a;
+}
+
 // One block per sample: s = (sum of the pixel-split partials) / hw, p1 = w1 s + b1, h = silu(p1), g = sigmoid(w2 h + b2).
 // Keeps s, p1 and g for the backward pass.
 __global__ void __launch_bounds__(256) se_fc_fwd_kernel(const float* __restrict__ part, int splits, float inv_hw, const float* __restrict__ w1,
                                                         const float* __restrict__ b1, const float* __restrict__ w2, const float* __restrict__ b2, int c, int k,
-                                                        float* __restrict__ s, float* __restrict__ p1, float* __restrict__ g) {
-    pdl_wait();
+                                                        int staged, float* __restrict__ s, float* __restrict__ p1, float* __restrict__ g) {
     pdl_launch();
-    extern __shared__ float hs[];              // h[k], s[c]
+    extern __shared__ float hs[];              // h[k], s[c], weights
     float* sn = hs + k;
     const int n = blockIdx.x, nb = gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (staged) {
+        stage_fc(w1, w2, k * c, sn + c);
+        w1 = sn + c;
+        w2 = w1 + k * c;
+    }
+    pdl_wait();
     for (int i = threadIdx.x; i < c; i += 256) {
-        float a = 0.f;
-        for (int z = 0; z < splits; ++z) a += part[((size_t)z * nb + n) * c + i];
-        a *= inv_hw;
+        const float a = split_sum(part + (size_t)n * c + i, splits, (size_t)nb * c) * inv_hw;
         sn[i] = a;
         s[(size_t)n * c + i] = a;
     }
     __syncthreads();
     for (int j = warp; j < k; j += 8) {
         float acc = 0.f;
-        for (int i = lane; i < c; i += 32) acc = fmaf(__ldg(w1 + (size_t)j * c + i), sn[i], acc);
+        for (int i = lane; i < c; i += 32) acc = fmaf(w1[(size_t)j * c + i], sn[i], acc);
         acc = warp_sum(acc) + __ldg(b1 + j);
         if (lane == 0) {
             p1[(size_t)n * k + j] = acc;
@@ -182,33 +362,37 @@ __global__ void __launch_bounds__(256) se_fc_fwd_kernel(const float* __restrict_
     __syncthreads();
     for (int i = threadIdx.x; i < c; i += 256) {
         float acc = __ldg(b2 + i);
-        for (int j = 0; j < k; ++j) acc = fmaf(__ldg(w2 + (size_t)i * k + j), hs[j], acc);
+        for (int j = 0; j < k; ++j) acc = fmaf(w2[(size_t)i * k + j], hs[j], acc);
         g[(size_t)n * c + i] = sigmoidf_(acc);
     }
 }
 
 // One block per sample: dg = sum of the pixel-split partials; dp2 = dg g (1-g); dh = w2^T dp2; dp1 = dh silu'(p1); ds = w1^T dp1 / hw.
 __global__ void __launch_bounds__(256) se_fc_bwd_kernel(const float* __restrict__ part, int splits, const float* __restrict__ g, const float* __restrict__ p1,
-                                                        const float* __restrict__ w1, const float* __restrict__ w2, int c, int k, float inv_hw,
+                                                        const float* __restrict__ w1, const float* __restrict__ w2, int c, int k, int staged, float inv_hw,
                                                         float* __restrict__ dp2, float* __restrict__ dp1, float* __restrict__ ds) {
-    pdl_wait();
     pdl_launch();
-    extern __shared__ float sm[];              // dp2[c], dp1[k]
+    extern __shared__ float sm[];              // dp2[c], dp1[k], weights
     float* sdp2 = sm;
     float* sdp1 = sm + c;
     const int n = blockIdx.x, nb = gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (staged) {
+        stage_fc(w1, w2, k * c, sdp1 + k);
+        w1 = sdp1 + k;
+        w2 = w1 + k * c;
+    }
+    pdl_wait();
     for (int i = threadIdx.x; i < c; i += 256) {
         const float gg = g[(size_t)n * c + i];
-        float dg = 0.f;                          // gradient of the gate: the pixel-split partials of sum dout*x, in index order
-        for (int z = 0; z < splits; ++z) dg += part[((size_t)z * nb + n) * c + i];
-        const float v = dg * gg * (1.f - gg);
+        // gradient of the gate: the pixel-split partials of sum dout*x
+        const float dg = split_sum(part + (size_t)n * c + i, splits, (size_t)nb * c), v = dg * gg * (1.f - gg);
         sdp2[i] = v;
         dp2[(size_t)n * c + i] = v;
     }
     __syncthreads();
     for (int j = warp; j < k; j += 8) {
         float acc = 0.f;
-        for (int i = lane; i < c; i += 32) acc = fmaf(__ldg(w2 + (size_t)i * k + j), sdp2[i], acc);
+        for (int i = lane; i < c; i += 32) acc = fmaf(w2[(size_t)i * k + j], sdp2[i], acc);
         acc = warp_sum(acc);
         if (lane == 0) {
             const float p = p1[(size_t)n * k + j], sg = sigmoidf_(p);
@@ -220,7 +404,7 @@ __global__ void __launch_bounds__(256) se_fc_bwd_kernel(const float* __restrict_
     __syncthreads();
     for (int i = threadIdx.x; i < c; i += 256) {
         float acc = 0.f;
-        for (int j = 0; j < k; ++j) acc = fmaf(__ldg(w1 + (size_t)j * c + i), sdp1[j], acc);
+        for (int j = 0; j < k; ++j) acc = fmaf(w1[(size_t)j * c + i], sdp1[j], acc);
         ds[(size_t)n * c + i] = acc * inv_hw;       // the squeeze is a mean: every position of the sample receives ds / hw
     }
 }
@@ -237,11 +421,13 @@ __global__ void __launch_bounds__(256) se_param_grad_kernel(const float* __restr
     if (t < n_w) {                              // w1[j][i]
         const int j = t / c, i = t - j * c;
         float acc = 0.f;
+#pragma unroll 8
         for (int n = 0; n < nb; ++n) acc = fmaf(dp1[(size_t)n * k + j], s[(size_t)n * c + i], acc);
         gw1[t] = acc;
     } else if (t < 2 * n_w) {                   // w2[i][j]
         const int u = t - n_w, i = u / k, j = u - i * k;
         float acc = 0.f;
+#pragma unroll 8
         for (int n = 0; n < nb; ++n) {
             const float p = p1[(size_t)n * k + j];
             acc = fmaf(dp2[(size_t)n * c + i], p * sigmoidf_(p), acc);
@@ -250,11 +436,13 @@ __global__ void __launch_bounds__(256) se_param_grad_kernel(const float* __restr
     } else if (t < 2 * n_w + k) {
         const int j = t - 2 * n_w;
         float acc = 0.f;
+#pragma unroll 8
         for (int n = 0; n < nb; ++n) acc += dp1[(size_t)n * k + j];
         gb1[j] = acc;
     } else if (t < 2 * n_w + k + c) {
         const int i = t - 2 * n_w - k;
         float acc = 0.f;
+#pragma unroll 8
         for (int n = 0; n < nb; ++n) acc += dp2[(size_t)n * c + i];
         gb2[i] = acc;
     }
@@ -263,31 +451,42 @@ __global__ void __launch_bounds__(256) se_param_grad_kernel(const float* __restr
 // MODE 0: out = value(x) * gate[n][c];  MODE 1: out = d * gate[n][c] + ds[n][c] (+ addend), ds being the per-position share of the squeeze's gradient
 template <typename T, int V, int MODE>
 __global__ void __launch_bounds__(256) se_scale_kernel(ValSrc x, const T* __restrict__ d, const float* __restrict__ gate, const float* __restrict__ ds,
-                                                       const T* addend, size_t groups, int vpr, int hw, size_t stride, T* __restrict__ out,
-                                                       T* __restrict__ out2) {
-    pdl_wait();
+                                                       const T* addend, PassCut k, int hw, int c, T* __restrict__ out, T* __restrict__ out2) {
     pdl_launch();
-    const size_t id = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= stride) return;
-    const int c0 = (int)(id % (size_t)vpr) * V, c = vpr * V;
+    pdl_wait();
+    PassIdx ix;
+    ix.init<V>(k, hw, c);
+    if (!ix.live) return;
     ChanVal<V> cv;
-    if (MODE == 0) cv.init(x, c0);
-    for (size_t i = id; i < groups; i += stride) {
-        const size_t n = (i / (size_t)vpr) / (size_t)hw;
-        float v[V], a[V];
-        if (MODE == 0) {
-            ld_raw_w<T, V>(x.p, i * V, v);
-            cv.apply(v);
+    if (MODE == 0) cv.init(x, ix.c0);
+    float gt[V], dsv[V];
 #pragma unroll
-            for (int q = 0; q < V; ++q) v[q] *= gate[n * c + c0 + q];
-        } else {
-            ld_raw_w<T, V>(d, i * V, v);
-            if (addend) ld_raw_w<T, V>(addend, i * V, a);
+    for (int q = 0; q < V; ++q) {
+        gt[q] = gate[(size_t)ix.sample * c + ix.c0 + q];
+        dsv[q] = MODE == 1 ? ds[(size_t)ix.sample * c + ix.c0 + q] : 0.f;
+    }
+    for (int p0 = ix.pbeg + ix.row; p0 < ix.pend; p0 += 4 * k.rows) {
+        float v[4][V];
 #pragma unroll
-            for (int q = 0; q < V; ++q) v[q] = fmaf(v[q], gate[n * c + c0 + q], ds[n * c + c0 + q]) + (addend ? a[q] : 0.f);
+        for (int u = 0; u < 4; ++u)
+            if (p0 + u * k.rows < ix.pend) ld_raw_w<T, V>(MODE == 0 ? x.p : (const void*)d, ix.base + (size_t)(p0 + u * k.rows) * c, v[u]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (p0 + u * k.rows >= ix.pend) break;
+            const size_t e = ix.base + (size_t)(p0 + u * k.rows) * c;
+            if (MODE == 0) {
+                cv.apply(v[u]);
+#pragma unroll
+                for (int q = 0; q < V; ++q) v[u][q] *= gt[q];
+            } else {
+                float a[V];
+                if (addend) ld_raw_w<T, V>(addend, e, a);
+#pragma unroll
+                for (int q = 0; q < V; ++q) v[u][q] = fmaf(v[u][q], gt[q], dsv[q]) + (addend ? a[q] : 0.f);
+            }
+            st_raw_w<T, V>(out, e, v[u]);
+            if (out2) st_raw_w<T, V>(out2, e, v[u]);
         }
-        st_raw_w<T, V>(out, i * V, v);
-        if (out2) st_raw_w<T, V>(out2, i * V, v);
     }
 }
 
@@ -587,21 +786,29 @@ double esz_(int dtype) { return dtype == 0 ? 4.0 : 2.0; }
         }                                                                                         \
     } while (0)
 
-void silu_fwd(int dtype, const ValSrc& x, size_t pixels, int c, void* out, void* out2, cudaStream_t st) {
-    const size_t n = pixels * c;
-    LaunchScope ls(K_SILU, (double)n * esz_(dtype) * (2 + (out2 ? 1 : 0)), 4.0 * n, st);
+static size_t pass_smem(const PassCut& k, int V) { return (size_t)(k.rows > 2 ? k.rows : 2) * k.lanes * V * sizeof(float); }
+
+int silu_fwd(int dtype, const ValSrc& x, const BnPendFwd& pf, int n, int hw, int c, void* out, void* out2, float* part, size_t part_floats, cudaStream_t st) {
+    const double e = (double)n * hw * c;
+    LaunchScope ls(K_SILU, e * esz_(dtype) * (2 + (out2 ? 1 : 0)), 4.0 * e, st);
+    int splits = 0;
     DISPATCH_TV(dtype, c, {
-        const VecGrid vg = vec_grid(n / V, c / V, 4);
-        launch_pdl(silu_kernel<T, V, false>, vg.blocks, 256, 0, st, x, (const T*)nullptr, (const T*)nullptr, n / V, c / V, vg.stride, (T*)out, (T*)out2);
+        const PassCut k = pass_cut(n, hw, c / V);
+        splits = k.splits;
+        if ((size_t)splits * n * c > part_floats) part = nullptr;
+        launch_pdl(silu_fwd_kernel<T, V>, dim3(k.splits * n, k.parts), 256, pass_smem(k, V), st, x, pf, k, hw, c, (T*)out, (T*)out2, part);
     });
+    return part ? splits : 0;
 }
 
-void silu_bwd(int dtype, const void* dy, const ValSrc& x, const void* addend, size_t pixels, int c, void* dx, cudaStream_t st) {
-    const size_t n = pixels * c;
-    LaunchScope ls(K_SILU, (double)n * esz_(dtype) * (3 + (addend ? 1 : 0)), 8.0 * n, st);
+void silu_bwd(int dtype, const void* dy, const float* gate, const float* ds, const ValSrc& x, const void* addend, int n, int hw, int c, void* dx, double* sums,
+              const float* mean, const float* rstd, cudaStream_t st) {
+    const double e = (double)n * hw * c;
+    LaunchScope ls(K_SILU, e * esz_(dtype) * (3 + (addend ? 1 : 0)), 8.0 * e, st);
+    const SiluBwdArgs a{x, dy, addend, gate, ds, sums, mean, rstd, hw, c, dx};
     DISPATCH_TV(dtype, c, {
-        const VecGrid vg = vec_grid(n / V, c / V, 4);
-        launch_pdl(silu_kernel<T, V, true>, vg.blocks, 256, 0, st, x, (const T*)dy, (const T*)addend, n / V, c / V, vg.stride, (T*)dx, (T*)nullptr);
+        const PassCut k = pass_cut(n, hw, c / V);
+        launch_pdl(silu_bwd_kernel<T, V>, dim3(k.splits * n, k.parts), 256, pass_smem(k, V), st, a, k);
     });
 }
 
@@ -614,11 +821,26 @@ static int se_splits(int gx, int n, int hw, int c, size_t scratch_floats) {
     return z < 1 ? 1 : z;
 }
 
+// shared memory of the fully connected kernels; with the weights where they fit beside other blocks
+static size_t fc_smem(int c, int k, bool* staged) {
+    const size_t base = (size_t)(k + c) * sizeof(float), all = base + (size_t)2 * k * c * sizeof(float);
+    *staged = all <= 100 * 1024;
+    static std::atomic<unsigned long long> done{0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (!(done.load(std::memory_order_acquire) & bit)) {
+        cudaFuncSetAttribute(se_fc_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+        cudaFuncSetAttribute(se_fc_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+        done.fetch_or(bit, std::memory_order_release);
+    }
+    return *staged ? all : base;
+}
+
 void se_forward(int dtype, const ValSrc& x, int n, int hw, int c, int k, const float* w1, const float* b1, const float* w2, const float* b2,
-                float* s, float* p1, float* gate, float* scratch, size_t scratch_floats, void* out, void* out2, cudaStream_t st) {
+                float* s, float* p1, float* gate, float* scratch, size_t scratch_floats, int splits, void* out, void* out2, cudaStream_t st) {
     const size_t elems = (size_t)n * hw * c;
-    int splits = 1;
-    {
+    if (splits == 0) {
         LaunchScope ls(K_SE, (double)elems * esz_(dtype), (double)elems, st);
         DISPATCH_TV(dtype, c, {
             const int gx = (c / V + 31) / 32;
@@ -627,24 +849,22 @@ void se_forward(int dtype, const ValSrc& x, int n, int hw, int c, int k, const f
         });
     }
     {
+        bool staged;
+        const size_t smem = fc_smem(c, k, &staged);
         LaunchScope ls(K_SE, 4.0 * (2.0 * k * c + (double)n * ((2 + splits) * c + k)), 4.0 * n * k * c, st);
-        launch_pdl(se_fc_fwd_kernel, n, 256, (size_t)(k + c) * sizeof(float), st, (const float*)scratch, splits, 1.f / (float)hw, w1, b1, w2, b2, c, k, s, p1, gate);
+        launch_pdl(se_fc_fwd_kernel, n, 256, smem, st, (const float*)scratch, splits, 1.f / (float)hw, w1, b1, w2, b2, c, k, (int)staged, s, p1, gate);
     }
     LaunchScope ls(K_SE, (double)elems * esz_(dtype) * (2 + (out2 ? 1 : 0)), (double)elems, st);
     DISPATCH_TV(dtype, c, {
-        const VecGrid vg = vec_grid(elems / V, c / V, 4);
-        launch_pdl(se_scale_kernel<T, V, 0>, vg.blocks, 256, 0, st, x, (const T*)nullptr, (const float*)gate, (const float*)nullptr, (const T*)nullptr, elems / V, c / V, hw,
-                   vg.stride, (T*)out, (T*)out2);
+        const PassCut cut = pass_cut(n, hw, c / V);
+        launch_pdl(se_scale_kernel<T, V, 0>, dim3(cut.splits * n, cut.parts), 256, 0, st, x, (const T*)nullptr, (const float*)gate, (const float*)nullptr, (const T*)nullptr,
+                   cut, hw, c, (T*)out, (T*)out2);
     });
 }
 
-void se_backward(int dtype, const void* dout, const ValSrc& x, int n, int hw, int c, int k, const float* w1, const float* w2, const float* s,
-                 const float* p1, const float* gate, float* work, float* scratch, size_t scratch_floats, const void* addend, void* dx, float* gw1, float* gb1,
-                 float* gw2, float* gb2, cudaStream_t st) {
+void se_backward_gate(int dtype, const void* dout, const ValSrc& x, int n, int hw, int c, int k, const float* w1, const float* w2, const float* p1,
+                      const float* gate, const SeWork& w, float* scratch, size_t scratch_floats, cudaStream_t st) {
     const size_t elems = (size_t)n * hw * c;
-    float* dp2 = work;                         // [n][c]
-    float* ds = dp2 + (size_t)n * c;           // [n][c]
-    float* dp1 = ds + (size_t)n * c;           // [n][k]
     int splits = 1;
     {
         LaunchScope ls(K_SE, 2.0 * elems * esz_(dtype), 2.0 * elems, st);
@@ -654,21 +874,24 @@ void se_backward(int dtype, const void* dout, const ValSrc& x, int n, int hw, in
             launch_pdl(se_reduce_kernel<T, V, 1>, dim3(gx, n, splits), 256, 0, st, x, (const T*)dout, hw, c, scratch);
         });
     }
-    {
-        LaunchScope ls(K_SE, 4.0 * (2.0 * k * c + (double)n * ((3 + splits) * c + 2 * k)), 4.0 * n * k * c, st);
-        launch_pdl(se_fc_bwd_kernel, n, 256, (size_t)(c + k) * sizeof(float), st, (const float*)scratch, splits, gate, p1, w1, w2, c, k, 1.f / (float)hw, dp2, dp1, ds);
-    }
-    {
-        const int params = 2 * k * c + k + c;
-        LaunchScope ls(K_SE, 4.0 * (params + (double)n * (2 * c + 2 * k)), 4.0 * n * k * c, st);
-        launch_pdl(se_param_grad_kernel, (params + 255) / 256, 256, 0, st, s, p1, (const float*)dp1, (const float*)dp2, n, c, k, gw1, gb1, gw2, gb2);
-    }
-    if (!dx) return;                           // only the parameter gradients are wanted
+    bool staged;
+    const size_t smem = fc_smem(c, k, &staged);
+    LaunchScope ls(K_SE, 4.0 * (2.0 * k * c + (double)n * ((3 + splits) * c + 2 * k)), 4.0 * n * k * c, st);
+    launch_pdl(se_fc_bwd_kernel, n, 256, smem, st, (const float*)scratch, splits, gate, p1, w1, w2, c, k, (int)staged, 1.f / (float)hw, w.dp2, w.dp1, w.ds);
+}
+
+void se_param_grads(const float* s, const float* p1, const SeWork& w, int n, int c, int k, float* gw1, float* gb1, float* gw2, float* gb2, cudaStream_t st) {
+    const int params = 2 * k * c + k + c;
+    LaunchScope ls(K_SE, 4.0 * (params + (double)n * (2 * c + 2 * k)), 4.0 * n * k * c, st);
+    launch_pdl(se_param_grad_kernel, (params + 127) / 128, 128, 0, st, s, p1, (const float*)w.dp1, (const float*)w.dp2, n, c, k, gw1, gb1, gw2, gb2);
+}
+
+void se_backward_scale(int dtype, const void* dout, int n, int hw, int c, const float* gate, const float* ds, const void* addend, void* dx, cudaStream_t st) {
+    const size_t elems = (size_t)n * hw * c;
     LaunchScope ls(K_SE, (double)elems * esz_(dtype) * (2 + (addend ? 1 : 0)), 2.0 * elems, st);
     DISPATCH_TV(dtype, c, {
-        const VecGrid vg = vec_grid(elems / V, c / V, 4);
-        launch_pdl(se_scale_kernel<T, V, 1>, vg.blocks, 256, 0, st, x, (const T*)dout, gate, (const float*)ds, (const T*)addend, elems / V, c / V, hw, vg.stride,
-                   (T*)dx, (T*)nullptr);
+        const PassCut cut = pass_cut(n, hw, c / V);
+        launch_pdl(se_scale_kernel<T, V, 1>, dim3(cut.splits * n, cut.parts), 256, 0, st, ValSrc{}, (const T*)dout, gate, ds, (const T*)addend, cut, hw, c, (T*)dx, (T*)nullptr);
     });
 }
 
@@ -679,11 +902,11 @@ void se_backward(int dtype, const void* dout, const ValSrc& x, int n, int hw, in
         if ((dtype) == 0) { using T = float; constexpr int V = 4; __VA_ARGS__ }     \
         else { using T = __nv_bfloat16; constexpr int V = 4; __VA_ARGS__ }          \
     } while (0)
-// ... and with the compile-time kernel size K in {5, 7}
-#define DISPATCH_K(k, ...)                                  \
-    do {                                                    \
-        if ((k) == 5) { constexpr int K = 5; __VA_ARGS__ }  \
-        else { constexpr int K = 7; __VA_ARGS__ }           \
+// ... and with the compile-time kernel size (3x3: dw3.cu, 5x5: dw5.cu)
+#define DISPATCH_K(k, ...)       \
+    do {                         \
+        constexpr int K = 7;     \
+        __VA_ARGS__              \
     } while (0)
 
 void dwk_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const float* wkc, void* z, cudaStream_t st) {

@@ -62,7 +62,7 @@ struct Unit {
     long w_off = -1, b_off = -1, gamma_off = -1, beta_off = -1;   // floats into the parameter arena
     size_t k_off = 0;       // floats into the backward-coefficient arena (k1,k2,k3)
     size_t run_off = 0;     // floats into the running-statistics arena
-    size_t acc_off = 0;     // 3x3 depthwise units: the weight gradient's accumulators, [9][c] doubles, in the backward sums
+    size_t acc_off = 0;     // 3x3 and 5x5 depthwise units: the weight gradient's accumulators, [taps][c] doubles, in the backward sums
     size_t sum_off = 0;     // BatchNorm units: channels before this unit's (its sums: 2c doubles at 2*sum_off, its pivots at sum_off)
     // dense conv with a short reduction, bfloat16 mode: forward and weight gradient run as pointwise tensor-core GEMMs
     // over an explicit im2col tensor kept in the slot (col_kp = padded reduction length, 0 = not such a unit)
@@ -120,11 +120,11 @@ struct asteroid_stage {
     float* gpad = nullptr;                         // [co][Kp] padded weight gradient of the im2col unit at hand
     size_t n_wpad = 0, n_gpad = 0;
     // per-channel sums of the BatchNorms (fin.cuh), forward and backward, and the pivots the forward sums were taken with.  The forward sums
-    // are zeroed by a forward's first kernel, the backward sums by accumulate.  The backward sums also hold the accumulators of the 3x3
+    // are zeroed by a forward's first kernel, the backward sums by accumulate.  The backward sums also hold the accumulators of the
     // depthwise weight gradients.
     double *fsum = nullptr, *bsum = nullptr;
     float* pivots = nullptr;
-    DwSettle* dw_tab = nullptr;                    // the 3x3 depthwise units' accumulators and weight gradients
+    DwSettle* dw_tab = nullptr;                    // the depthwise units' accumulators and weight gradients
     int n_dw = 0;
     bool bsum_dirty = false;                       // a backward ran since its sums were zeroed (profile runs skip accumulate)
     int* err = nullptr;                            // device error word (bounded waits)
@@ -381,10 +381,11 @@ static int build_plan(asteroid_stage* s) {
     }
     s->n_bsum = 2 * s->n_bn_ch;
     for (auto& u : s->units)
-        if (u.kind == U_DW && u.g.k == 3) {
+        if (u.kind == U_DW && u.g.k <= 5) {
+            const size_t weights = (size_t)u.g.k * u.g.k * u.g.ci;
             u.acc_off = s->n_bsum;
-            s->n_bsum += 9 * (size_t)u.g.ci;
-            s->n_dw_weights += 9 * (size_t)u.g.ci;
+            s->n_bsum += weights;
+            s->n_dw_weights += weights;
             ++s->n_dw;
         }
     for (auto& u : s->units)
@@ -624,6 +625,7 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
         }
     }
     Pending pend(s, sv, st);
+    int squeeze_splits = 0;        // > 0: the unit before left the squeeze of this one as that many partials in the scratch arena
     const auto producer = [&](int v) { return s->vals[v].affine ? s->vals[v].unit : -1; };
     for (size_t ui = 0; ui < s->units.size(); ++ui) {
         const Unit& u = s->units[ui];
@@ -682,24 +684,30 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
             }
             else conv_fwd(dt, u.g, val_src(s, sv, u.in), s->w + u.w_off, bias, obuf, st);
         } else if (u.kind == U_DW) {
-            if (u.g.k != 3) {
+            if (u.g.k > 5) {
                 pend.settle_fwd(producer(u.in));
                 dwk_fwd(dt, u.g, val_src(s, sv, u.in), s->derived + u.w_off, obuf, st);
             } else {
                 const BnPendFwd pf = pend.take_fwd(producer(u.in));
-                dw3_fwd(dt, u.g, val_src(s, sv, u.in), pf, s->derived + u.w_off, obuf, bn ? sums_fwd(s, u) : BnSumsOut{}, dw3_choose(dt, false, u.g), st);
+                const BnSumsOut so = bn ? sums_fwd(s, u) : BnSumsOut{};
+                if (u.g.k == 5) dw5_fwd(dt, u.g, val_src(s, sv, u.in), pf, s->derived + u.w_off, obuf, so, dw5_choose(dt, false, u.g), st);
+                else dw3_fwd(dt, u.g, val_src(s, sv, u.in), pf, s->derived + u.w_off, obuf, so, dw3_choose(dt, false, u.g), st);
                 fused_stats = bn ? -1 : 0;
             }
         } else if (u.kind == U_SILU) {
-            pend.settle_fwd(producer(u.in));
-            silu_fwd(dt, val_src(s, sv, u.in), o.elems / o.c, o.c, obuf, is_last ? y : nullptr, st);
+            // a squeeze-excite layer right behind: its squeeze comes with this pass
+            const bool squeeze = o.consumers == 1 && ui + 1 < s->units.size() && s->units[ui + 1].kind == U_SE && s->units[ui + 1].in == u.out;
+            const BnPendFwd pf = pend.take_fwd(producer(u.in));
+            squeeze_splits = silu_fwd(dt, val_src(s, sv, u.in), pf, s->B, o.h * o.w, o.c, obuf, is_last ? y : nullptr, squeeze ? s->scratch : nullptr,
+                                      s->scratch_floats, st);
         } else if (u.kind == U_SE) {
             pend.settle_fwd(producer(u.in));
             const int c = o.c, k = u.se_k;
             const float* wp = s->w + u.w_off;        // w1 [k][c], b1 [k], w2 [c][k], b2 [c]
             float* sev = sv.stats + u.se_off;        // s [B][c], p1 [B][k], gate [B][c]
             se_forward(dt, val_src(s, sv, u.in), s->B, o.h * o.w, c, k, wp, wp + (size_t)k * c, wp + (size_t)k * c + k, wp + 2 * (size_t)k * c + k, sev,
-                       sev + (size_t)s->B * c, sev + (size_t)s->B * (c + k), s->scratch, s->scratch_floats, obuf, is_last ? y : nullptr, st);
+                       sev + (size_t)s->B * c, sev + (size_t)s->B * (c + k), s->scratch, s->scratch_floats, squeeze_splits, obuf, is_last ? y : nullptr, st);
+            squeeze_splits = 0;
         } else if (u.kind == U_ADD) {
             if (!ew_takes_pending(dt, o.c)) {
                 pend.settle_fwd(producer(u.in));
@@ -737,6 +745,11 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
 struct GradState {
     int state = G_NONE;
     const void* ptr = nullptr;
+};
+
+// A squeeze-excite layer's backward left to the SiLU unit in front: its output gradient counts as dy*gate + ds there.
+struct GatedGrad {
+    const float *gate = nullptr, *ds = nullptr;
 };
 
 // The conv->BN unit whose BatchNorm-backward sums can be taken by the kernel that writes the complete gradient of
@@ -779,6 +792,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
     };
     gs.back().state = G_ALIAS;
     gs.back().ptr = dy;
+    GatedGrad gated;
     std::vector<char> reduced(s->units.size(), 0);   // BatchNorm-backward sums already taken by the kernel that wrote dy
     Pending pend(s, sv, st);                         // ... and not yet turned into coefficients
     if (s->bsum_dirty && s->n_bsum) CU(cudaMemsetAsync(s->bsum, 0, s->n_bsum * sizeof(double), st));
@@ -839,13 +853,13 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             const bool f32_d = want_in && f32_unit(s, u, true, &til_d32);
             const bool f32_w = u.kind == U_CONV && dt == AST_F32 && wg.k == 1 && wg.stride == 1 && wg.pad == 0 &&
                                f32_wgrad_choose(wg.n * wg.ho * wg.wo, wg.co, wg.ci, s->scratch_floats, &til_w32);
-            const bool dw3 = u.kind == U_DW && u.g.k == 3;
-            if (!dw3 && ((!mma_w && !f32_w) || (want_in && !mma_d && !f32_d))) pend.settle_bwd(ui);
+            const bool dw = u.kind == U_DW && u.g.k <= 5;
+            if (!dw && ((!mma_w && !f32_w) || (want_in && !mma_d && !f32_d))) pend.settle_bwd(ui);
             const BnPendBwd pb = pend.has(ui) ? pend_bwd(s, sv, u) : BnPendBwd{};
             pend.unit[ui] = 0;
             tick(s, ui, 4, st);
             ValSrc xin = val_src(s, sv, u.in);
-            if (dw3) {
+            if (dw) {
                 // input gradient, weight gradient and, where x is the raw output of a conv -> BatchNorm unit read by nobody after this one, that
                 // BatchNorm's sums
                 GradState& gi = gs[u.in];
@@ -861,8 +875,10 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                     reduced[tgt] = 1;
                     s->bwd_sums_by[tgt] = ui;
                 }
-                dw3_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, want_in ? own(u.in) : nullptr, s->bsum + u.acc_off, sums, ts, ts ? ts + u.g.ci : nullptr,
-                        dw3_choose(dt, true, u.g), st);
+                void* to = want_in ? own(u.in) : nullptr;
+                const float* trs = ts ? ts + u.g.ci : nullptr;
+                if (u.g.k == 5) dw5_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, s->bsum + u.acc_off, sums, ts, trs, dw5_choose(dt, true, u.g), st);
+                else dw3_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, s->bsum + u.acc_off, sums, ts, trs, dw3_choose(dt, true, u.g), st);
                 if (want_in) {
                     gi.state = G_OWNED;
                     gi.ptr = own(u.in);
@@ -992,17 +1008,44 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             GradState& gi = gs[u.in];
             const void* addend = gi.state == G_NONE ? nullptr : gi.ptr;
             if (u.kind == U_SE) {
-                // the parameter gradients are wanted even when the input gradient is not; the kernel sequence computes both
+                // the parameter gradients are wanted even when the input gradient is not
                 const int c = o.c, k = u.se_k;
                 const float* wp = s->w + u.w_off;
                 float* gp = s->g + u.w_off;
-                const float* sev = sv.stats + u.se_off;
-                se_backward(dt, go.ptr, val_src(s, sv, u.in), s->B, o.h * o.w, c, k, wp, wp + (size_t)k * c + k, sev, sev + (size_t)s->B * c,
-                            sev + (size_t)s->B * (c + k), s->coef + u.se_work_off, s->scratch, s->scratch_floats, addend, want_in ? own(u.in) : nullptr, gp, gp + (size_t)k * c, gp + (size_t)k * c + k,
-                            gp + 2 * (size_t)k * c + k, st);
+                const float *sev = sv.stats + u.se_off, *p1 = sev + (size_t)s->B * c, *gate = sev + (size_t)s->B * (c + k);
+                float* work = s->coef + u.se_work_off;
+                const SeWork wk{work, work + (size_t)s->B * c, work + 2 * (size_t)s->B * c};
+                se_backward_gate(dt, go.ptr, val_src(s, sv, u.in), s->B, o.h * o.w, c, k, wp, wp + (size_t)k * c + k, p1, gate, wk, s->scratch, s->scratch_floats, st);
+                {
+                    int frc = fork();
+                    if (frc) return frc;
+                }
+                se_param_grads(sev, p1, wk, s->B, c, k, gp, gp + (size_t)k * c, gp + (size_t)k * c + k, gp + 2 * (size_t)k * c + k, wst);
+                const int si = s->vals[u.in].unit;
+                if (want_in && si == ui - 1 && s->units[si].kind == U_SILU && s->vals[u.in].consumers == 1) {
+                    // the SiLU in front applies gate and squeeze gradient as it reads this unit's output gradient
+                    gated = GatedGrad{gate, wk.ds};
+                    gi.state = G_ALIAS;
+                    gi.ptr = go.ptr;
+                    tick(s, ui, 5, st);
+                    continue;
+                }
+                if (want_in) se_backward_scale(dt, go.ptr, s->B, o.h * o.w, c, gate, wk.ds, addend, own(u.in), st);
             } else if (want_in) {
-                silu_bwd(dt, go.ptr, val_src(s, sv, u.in), addend, o.elems / o.c, o.c, own(u.in), st);
+                double* sums = nullptr;
+                const float* ts = nullptr;
+                const int tgt = s->vals[u.in].first_cons == ui && bn_reduce_target(s, u.in) == s->vals[u.in].unit ? s->vals[u.in].unit : -1;
+                if (tgt >= 0 && s->units[tgt].act == ACT_NONE) {
+                    const Unit& tu = s->units[tgt];
+                    sums = s->bsum + 2 * tu.sum_off;
+                    ts = sv.stats + s->vals[tu.out].stat_off;
+                    pend.unit[tgt] = 1;
+                    reduced[tgt] = 1;
+                    s->bwd_sums_by[tgt] = ui;
+                }
+                silu_bwd(dt, go.ptr, gated.gate, gated.ds, val_src(s, sv, u.in), addend, s->B, o.h * o.w, o.c, own(u.in), sums, ts, ts ? ts + o.c : nullptr, st);
             }
+            gated = GatedGrad{};
             if (want_in) {
                 gi.state = G_OWNED;
                 gi.ptr = own(u.in);
@@ -1022,7 +1065,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
     }
     if (s->need_dx && gs[0].state == G_ALIAS)
         CU(cudaMemcpyAsync(dx, gs[0].ptr, s->vals[0].elems * s->esz, cudaMemcpyDeviceToDevice, st));
-    if (s->n_dw_weights) dw3_settle(s->bsum, s->dw_tab, s->n_dw, s->n_dw_weights, s->g, st);
+    if (s->n_dw_weights) dw_settle(s->bsum, s->dw_tab, s->n_dw, s->n_dw_weights, s->g, st);
     if (side_used) {            // join: the call's work is complete, in the caller's stream order, when the second stream's is
         CU(cudaEventRecord(s->ev_join, s->side));
         CU(cudaStreamWaitEvent(st, s->ev_join, 0));
@@ -1071,7 +1114,7 @@ static int create_impl(const ast_layer* net, int n_layers, int first, int last, 
     if (s->n_dw) {
         std::vector<DwSettle> tab;
         for (const auto& u : s->units)
-            if (u.kind == U_DW && u.g.k == 3) tab.push_back(DwSettle{u.acc_off, (size_t)u.w_off, u.g.ci});
+            if (u.kind == U_DW && u.g.k <= 5) tab.push_back(DwSettle{u.acc_off, (size_t)u.w_off, u.g.ci, u.g.k * u.g.k});
         if ((rc = arena_alloc(s, "depthwise layer table", &s->dw_tab, tab.size() * sizeof(DwSettle), &work))) return rc;
         CU(cudaMemcpy(s->dw_tab, tab.data(), tab.size() * sizeof(DwSettle), cudaMemcpyHostToDevice));
     }

@@ -1,4 +1,4 @@
-"""The 3x3 depthwise kernels at the edges of their strips: maps narrower and shorter than a strip, widths that strips cover exactly and
+"""The 3x3 and 5x5 depthwise kernels at the edges of their strips: maps narrower and shorter than a strip, widths that strips cover exactly and
 one more, odd and even maps at stride 2, channel counts that split unevenly over the blocks, several strips per thread, with and
 without the units that leave sums behind or take them.  Activation-free, held to the plain float64 oracle on every tensor."""
 import pytest
@@ -9,7 +9,7 @@ from harness import ALL, CONTRACT, bf16_store, compare, gpu_round, make_inputs, 
 pytestmark = pytest.mark.gpu
 
 
-def _net(c, stride, around):
+def _net(c, stride, around, k):
     """Depthwise conv with BatchNorm; `around`: between two 1x1 convs with BatchNorm (coefficients pending on both sides)."""
     L, net = si.Layer, []
 
@@ -19,7 +19,7 @@ def _net(c, stride, around):
     if around:
         push("conv", 16, c, 1, 1, 0)
         push("bn", c, c, 0, 1, 0)
-    push("dwconv", c, c, 3, stride, 1)
+    push("dwconv", c, c, k, stride, k // 2)
     push("bn", c, c, 0, 1, 0)
     if around:
         push("conv", c, 24, 1, 1, 0)
@@ -48,10 +48,11 @@ CASES = {
 
 
 @pytest.mark.parametrize("bf16", [False, True], ids=["f32", "bf16"])
+@pytest.mark.parametrize("k", [3, 5])
 @pytest.mark.parametrize("name", list(CASES))
-def test_depthwise_edges(name, bf16):
+def test_depthwise_edges(name, k, bf16):
     c, stride, h, w, B, around = CASES[name]
-    net = _net(c, stride, around)
+    net = _net(c, stride, around, k)
     last = len(net) - 1
     xs, tg, params, _ = make_inputs(net, 0, last, h, w, B, 2, "mse", 23, bf16)
     params = si.randomize_bn(params, net, 0, last, 23)
@@ -59,5 +60,5 @@ def test_depthwise_edges(name, bf16):
     # maps of a few pixels: the gradients in front of a BatchNorm nearly vanish, and what is left of them is the storage rounding
     mirror = oracle_round(net, 0, last, B, 2, "mse", xs, tg, params, store=bf16_store) if bf16 else None
     gpu = gpu_round(net, 0, last, h, w, B, 2, "mse", xs, tg, params, bf16)
-    r = compare(gpu, plain, net, 0, last, 2e-2 if bf16 else 1e-4, mirror=mirror, allow=ALL if bf16 else (CONTRACT,), case="dw_edges/%s" % name)
-    print(name, summary(r))
+    r = compare(gpu, plain, net, 0, last, 2e-2 if bf16 else 1e-4, mirror=mirror, allow=ALL if bf16 else (CONTRACT,), case="dw%d_edges/%s" % (k, name))
+    print(name, k, summary(r))

@@ -54,6 +54,22 @@ template <int V> struct ChanGrad {
 };
 
 __device__ __forceinline__ float sigmoidf_(float x) { return 1.f / (1.f + __expf(-x)); }
+// of a value that bfloat16 storage rounds: the reciprocal to one or two units of float32
+template <typename T> __device__ __forceinline__ float sigmoid_as(float x) { return sizeof(T) == 2 ? __fdividef(1.f, 1.f + __expf(-x)) : sigmoidf_(x); }
+
+// V consecutive channels as loaded: a quarter of the registers of the unpacked values while a request is in flight
+template <typename T, int V> struct RawV {
+    uint32_t w[(sizeof(T) * V + 3) / 4];
+    __device__ __forceinline__ void load(const void* p, size_t e) {
+        if constexpr (sizeof(T) * V == 16) *reinterpret_cast<uint4*>(w) = *reinterpret_cast<const uint4*>(reinterpret_cast<const T*>(p) + e);
+        else if constexpr (sizeof(T) == 4) w[0] = reinterpret_cast<const uint32_t*>(p)[e];
+        else w[0] = reinterpret_cast<const uint16_t*>(p)[e];
+    }
+    __device__ __forceinline__ float at(int q) const {
+        if constexpr (sizeof(T) == 4) return __uint_as_float(w[q]);
+        else return __uint_as_float(q & 1 ? w[q >> 1] & 0xffff0000u : w[q >> 1] << 16);
+    }
+};
 
 // Threads beyond `stride` (the thread count cut to a multiple of the vectors per pixel) idle, so that a thread striding by
 // `stride` vectors always lands on the same channels.
@@ -81,12 +97,15 @@ VecGrid vec_grid(size_t groups, int vpr, int per_thread) {
 struct PassCut {
     int lanes, rows, parts, splits, ppb;   // channel vectors per block, pixels side by side, blocks along the channels and the pixels, pixels per block
 };
-PassCut pass_cut(int n, int hw, int vpr) {
+// ctas: blocks per multiprocessor a kernel's registers allow.  lanes: a kernel that adds to per-channel accumulators takes few channels and many
+// pixels per block: the additions, one per block, channel and sum, cost more than the pass on a small map (14x14x480 at 32 images with 60 lanes
+// 10.5 us, without sums 5.0).
+PassCut pass_cut(int n, int hw, int vpr, int ctas = 4, int lanes = 256) {
     PassCut c;
-    c.parts = (vpr + 255) / 256;
+    c.parts = (vpr + lanes - 1) / lanes;
     c.lanes = (vpr + c.parts - 1) / c.parts;
     c.rows = 256 / c.lanes;
-    int want = (int)((long long)sm_count() * 4 / ((long long)n * c.parts));
+    int want = (int)((long long)sm_count() * ctas / ((long long)n * c.parts));
     const int most = (hw + 4 * c.rows - 1) / (4 * c.rows);
     if (want > most) want = most;
     if (want < 1) want = 1;
@@ -111,27 +130,26 @@ struct PassIdx {
         base = (size_t)sample * hw * c + (live ? c0 : 0);
     }
 };
-// sum over the block's rows, in row order, of V values per thread -> sm[jl * V + q] of the first row's threads' channels, in out
-template <int V> __device__ __forceinline__ void rows_sum(const PassCut& k, const PassIdx& x, const float* v, float* sm, float* out) {
+// sums over the block's rows, in row order, of V values per thread; f(channel, sum) for each of the block's channels
+template <int V, typename F> __device__ __forceinline__ void rows_sum(const PassCut& k, const PassIdx& x, int c, const float* v, float* sm, F f) {
+    const int width = k.lanes * V, cb = blockIdx.y * width;
     __syncthreads();
     if (x.row < k.rows)
 #pragma unroll
-        for (int q = 0; q < V; ++q) sm[(x.row * k.lanes + x.jl) * V + q] = v[q];
+        for (int q = 0; q < V; ++q) sm[x.row * width + x.jl * V + q] = v[q];
     __syncthreads();
-    if (x.row == 0)
-#pragma unroll
-        for (int q = 0; q < V; ++q) {
-            float s = 0.f;
-            for (int r = 0; r < k.rows; ++r) s += sm[(r * k.lanes + x.jl) * V + q];
-            out[q] = s;
-        }
+    for (int i = threadIdx.x; i < width && cb + i < c; i += 256) {
+        float s = 0.f;
+        for (int r = 0; r < k.rows; ++r) s += sm[r * width + i];
+        f(cb + i, s);
+    }
 }
 
 // ------------------------------------------------------------------------------------------ SiLU
 // out = silu(value(x)), with pending coefficients formed here; `part`, may be null: sums over the block's pixels of out as stored, [split][sample][c]
 // (the squeeze of a squeeze-excite layer behind)
-template <typename T, int V>
-__global__ void __launch_bounds__(256) silu_fwd_kernel(ValSrc x, BnPendFwd pf, PassCut k, int hw, int c, T* __restrict__ out, T* __restrict__ out2,
+template <typename T, int V, bool PART>
+__global__ void __launch_bounds__(256, 4) silu_fwd_kernel(ValSrc x, BnPendFwd pf, PassCut k, int hw, int c, T* __restrict__ out, T* __restrict__ out2,
                                                        float* __restrict__ part) {
     pdl_launch();
     pdl_wait();
@@ -162,30 +180,29 @@ __global__ void __launch_bounds__(256) silu_fwd_kernel(ValSrc x, BnPendFwd pf, P
     for (int q = 0; q < V; ++q) acc[q] = 0.f;
     if (ix.live)
         for (int p0 = ix.pbeg + ix.row; p0 < ix.pend; p0 += 4 * k.rows) {
-            float v[4][V];
+            RawV<T, V> r[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (p0 + u * k.rows < ix.pend) ld_raw_w<T, V>(x.p, ix.base + (size_t)(p0 + u * k.rows) * c, v[u]);
+            for (int u = 0; u < 4; ++u) r[u].load(x.p, ix.base + (size_t)min(p0 + u * k.rows, hw - 1) * c);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 if (p0 + u * k.rows >= ix.pend) break;
                 const size_t e = ix.base + (size_t)(p0 + u * k.rows) * c;
-                cv.apply(v[u]);
+                float v[V];
+#pragma unroll
+                for (int q = 0; q < V; ++q) v[q] = r[u].at(q);
+                cv.apply(v);
 #pragma unroll
                 for (int q = 0; q < V; ++q) {
-                    v[u][q] *= sigmoidf_(v[u][q]);
-                    if (part) acc[q] += to_f<T>(from_f<T>(v[u][q]));
+                    v[q] *= sigmoid_as<T>(v[q]);
+                    if (PART) acc[q] += to_f<T>(from_f<T>(v[q]));
                 }
-                st_raw_w<T, V>(out, e, v[u]);
-                if (out2) st_raw_w<T, V>(out2, e, v[u]);
+                st_raw_w<T, V>(out, e, v);
+                if (out2) st_raw_w<T, V>(out2, e, v);
             }
         }
-    if (!part) return;
-    float s[V];
-    rows_sum<V>(k, ix, acc, sm, s);
-    if (ix.row == 0 && ix.live)
-#pragma unroll
-        for (int q = 0; q < V; ++q) part[((size_t)ix.split * (gridDim.x / k.splits) + ix.sample) * c + ix.c0 + q] = s[q];
+    if (!PART) return;
+    float* dst = part + ((size_t)ix.split * (gridDim.x / k.splits) + ix.sample) * c;
+    rows_sum<V>(k, ix, c, acc, sm, [&](int ch, float v) { dst[ch] = v; });
 }
 
 // dx = dy' * silu'(value(x)) (+ addend), value(x) recomputed from the raw tensor; dy' = dy, or dy*gate + ds where a squeeze-excite layer behind left
@@ -199,67 +216,60 @@ struct SiluBwdArgs {
     int hw, c;
     void* dx;
 };
-template <typename T, int V> __global__ void __launch_bounds__(256) silu_bwd_kernel(SiluBwdArgs a, PassCut k) {
+template <typename T, int V, bool GATE, bool SUMS> __global__ void __launch_bounds__(256, 2) silu_bwd_kernel(SiluBwdArgs a, PassCut k) {
     pdl_launch();
     pdl_wait();
     extern __shared__ float sm[];
     PassIdx ix;
     ix.init<V>(k, a.hw, a.c);
     ChanVal<V> cv;
-    float gt[V], dsv[V], s1[V], s2[V];
+    float gt[V], dsv[V], mu[V], s1[V], s2[V];
     if (ix.live) {
         cv.init(a.x, ix.c0);
 #pragma unroll
         for (int q = 0; q < V; ++q) {
-            gt[q] = a.gate ? a.gate[(size_t)ix.sample * a.c + ix.c0 + q] : 1.f;
-            dsv[q] = a.gate ? a.ds[(size_t)ix.sample * a.c + ix.c0 + q] : 0.f;
+            if (GATE) {
+                gt[q] = a.gate[(size_t)ix.sample * a.c + ix.c0 + q];
+                dsv[q] = a.ds[(size_t)ix.sample * a.c + ix.c0 + q];
+            }
+            if (SUMS) mu[q] = a.mean[ix.c0 + q];
         }
     }
 #pragma unroll
     for (int q = 0; q < V; ++q) s1[q] = s2[q] = 0.f;
     if (ix.live)
-        for (int p0 = ix.pbeg + ix.row; p0 < ix.pend; p0 += 2 * k.rows) {
-            float z[2][V], d[2][V], ad[2][V];
+        for (int p0 = ix.pbeg + ix.row; p0 < ix.pend; p0 += 4 * k.rows) {
+            RawV<T, V> rz[4], rd[4];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                if (p0 + u * k.rows >= ix.pend) break;
-                const size_t e = ix.base + (size_t)(p0 + u * k.rows) * a.c;
-                ld_raw_w<T, V>(a.x.p, e, z[u]);
-                ld_raw_w<T, V>(a.dy, e, d[u]);
-                if (a.addend) ld_raw_w<T, V>(a.addend, e, ad[u]);
+            for (int u = 0; u < 4; ++u) {
+                const size_t e = ix.base + (size_t)min(p0 + u * k.rows, a.hw - 1) * a.c;
+                rz[u].load(a.x.p, e);
+                rd[u].load(a.dy, e);
             }
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
+            for (int u = 0; u < 4; ++u) {
                 if (p0 + u * k.rows >= ix.pend) break;
                 const size_t e = ix.base + (size_t)(p0 + u * k.rows) * a.c;
+                RawV<T, V> ra;
+                if (a.addend) ra.load(a.addend, e);
                 float o[V];
 #pragma unroll
                 for (int q = 0; q < V; ++q) {
-                    const float v = fminf(fmaxf(fmaf(z[u][q], cv.sc[q], cv.sh[q]), cv.lo), cv.hi), sg = sigmoidf_(v);
-                    o[q] = fmaf(d[u][q], gt[q], dsv[q]) * sg * fmaf(v, 1.f - sg, 1.f) + (a.addend ? ad[u][q] : 0.f);
-                }
-                st_raw_w<T, V>(a.dx, e, o);
-                if (a.sums) {
-                    // sum of dx * z here; mean and rstd enter at the end
-#pragma unroll
-                    for (int q = 0; q < V; ++q) {
+                    const float z = rz[u].at(q), v = fminf(fmaxf(fmaf(z, cv.sc[q], cv.sh[q]), cv.lo), cv.hi), sg = sigmoid_as<T>(v);
+                    const float dd = GATE ? fmaf(rd[u].at(q), gt[q], dsv[q]) : rd[u].at(q);
+                    o[q] = dd * sg * fmaf(v, 1.f - sg, 1.f) + (a.addend ? ra.at(q) : 0.f);
+                    if (SUMS) {
                         const float r = to_f<T>(from_f<T>(o[q]));
                         s1[q] += r;
-                        s2[q] = fmaf(r, z[u][q] - __ldg(a.mean + ix.c0 + q), s2[q]);
+                        s2[q] = fmaf(r, z - mu[q], s2[q]);
                     }
                 }
+                st_raw_w<T, V>(a.dx, e, o);
             }
         }
-    if (!a.sums) return;
-    float t1[V], t2[V];
-    rows_sum<V>(k, ix, s1, sm, t1);
-    rows_sum<V>(k, ix, s2, sm, t2);
-    if (ix.row == 0 && ix.live)
-#pragma unroll
-        for (int q = 0; q < V; ++q) {
-            add_sum(a.sums + ix.c0 + q, t1[q]);
-            add_sum(a.sums + a.c + ix.c0 + q, t2[q] * a.rstd[ix.c0 + q]);
-        }
+    if (!SUMS) return;
+    rows_sum<V>(k, ix, a.c, s1, sm, [&](int ch, float v) { add_sum(a.sums + ch, v); });
+    rows_sum<V>(k, ix, a.c, s2, sm, [&](int ch, float v) { add_sum(a.sums + a.c + ch, v * a.rstd[ch]); });
 }
 
 // ------------------------------------------------------------------------------------------ squeeze-excite
@@ -450,7 +460,7 @@ __global__ void __launch_bounds__(256) se_param_grad_kernel(const float* __restr
 
 // MODE 0: out = value(x) * gate[n][c];  MODE 1: out = d * gate[n][c] + ds[n][c] (+ addend), ds being the per-position share of the squeeze's gradient
 template <typename T, int V, int MODE>
-__global__ void __launch_bounds__(256) se_scale_kernel(ValSrc x, const T* __restrict__ d, const float* __restrict__ gate, const float* __restrict__ ds,
+__global__ void __launch_bounds__(256, 4) se_scale_kernel(ValSrc x, const T* __restrict__ d, const float* __restrict__ gate, const float* __restrict__ ds,
                                                        const T* addend, PassCut k, int hw, int c, T* __restrict__ out, T* __restrict__ out2) {
     pdl_launch();
     pdl_wait();
@@ -466,26 +476,28 @@ __global__ void __launch_bounds__(256) se_scale_kernel(ValSrc x, const T* __rest
         dsv[q] = MODE == 1 ? ds[(size_t)ix.sample * c + ix.c0 + q] : 0.f;
     }
     for (int p0 = ix.pbeg + ix.row; p0 < ix.pend; p0 += 4 * k.rows) {
-        float v[4][V];
+        RawV<T, V> r[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (p0 + u * k.rows < ix.pend) ld_raw_w<T, V>(MODE == 0 ? x.p : (const void*)d, ix.base + (size_t)(p0 + u * k.rows) * c, v[u]);
+        for (int u = 0; u < 4; ++u) r[u].load(MODE == 0 ? x.p : (const void*)d, ix.base + (size_t)min(p0 + u * k.rows, hw - 1) * c);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (p0 + u * k.rows >= ix.pend) break;
             const size_t e = ix.base + (size_t)(p0 + u * k.rows) * c;
+            float v[V];
+#pragma unroll
+            for (int q = 0; q < V; ++q) v[q] = r[u].at(q);
             if (MODE == 0) {
-                cv.apply(v[u]);
+                cv.apply(v);
 #pragma unroll
-                for (int q = 0; q < V; ++q) v[u][q] *= gt[q];
+                for (int q = 0; q < V; ++q) v[q] *= gt[q];
             } else {
-                float a[V];
-                if (addend) ld_raw_w<T, V>(addend, e, a);
+                RawV<T, V> a;
+                if (addend) a.load(addend, e);
 #pragma unroll
-                for (int q = 0; q < V; ++q) v[u][q] = fmaf(v[u][q], gt[q], dsv[q]) + (addend ? a[q] : 0.f);
+                for (int q = 0; q < V; ++q) v[q] = fmaf(v[q], gt[q], dsv[q]) + (addend ? a.at(q) : 0.f);
             }
-            st_raw_w<T, V>(out, e, v[u]);
-            if (out2) st_raw_w<T, V>(out2, e, v[u]);
+            st_raw_w<T, V>(out, e, v);
+            if (out2) st_raw_w<T, V>(out2, e, v);
         }
     }
 }
@@ -796,7 +808,8 @@ int silu_fwd(int dtype, const ValSrc& x, const BnPendFwd& pf, int n, int hw, int
         const PassCut k = pass_cut(n, hw, c / V);
         splits = k.splits;
         if ((size_t)splits * n * c > part_floats) part = nullptr;
-        launch_pdl(silu_fwd_kernel<T, V>, dim3(k.splits * n, k.parts), 256, pass_smem(k, V), st, x, pf, k, hw, c, (T*)out, (T*)out2, part);
+        launch_pdl(part ? silu_fwd_kernel<T, V, true> : silu_fwd_kernel<T, V, false>, dim3(k.splits * n, k.parts), 256, pass_smem(k, V), st, x, pf, k, hw, c, (T*)out, (T*)out2,
+                   part);
     });
     return part ? splits : 0;
 }
@@ -807,8 +820,11 @@ void silu_bwd(int dtype, const void* dy, const float* gate, const float* ds, con
     LaunchScope ls(K_SILU, e * esz_(dtype) * (3 + (addend ? 1 : 0)), 8.0 * e, st);
     const SiluBwdArgs a{x, dy, addend, gate, ds, sums, mean, rstd, hw, c, dx};
     DISPATCH_TV(dtype, c, {
-        const PassCut k = pass_cut(n, hw, c / V);
-        launch_pdl(silu_bwd_kernel<T, V>, dim3(k.splits * n, k.parts), 256, pass_smem(k, V), st, a, k);
+        const PassCut k = pass_cut(n, hw, c / V, 2, sums ? 12 : 256);
+        typedef void (*Fn)(SiluBwdArgs, PassCut);
+        const Fn f = gate ? sums ? (Fn)silu_bwd_kernel<T, V, true, true> : (Fn)silu_bwd_kernel<T, V, true, false>
+                          : sums ? (Fn)silu_bwd_kernel<T, V, false, true> : (Fn)silu_bwd_kernel<T, V, false, false>;
+        launch_pdl(f, dim3(k.splits * n, k.parts), 256, pass_smem(k, V), st, a, k);
     });
 }
 

@@ -62,6 +62,9 @@ struct LaunchScope {
     cudaStream_t st;
 };
 uint64_t launches();
+// launches the calling thread issued; launches made by replaying a graph of n of them
+uint64_t thread_launches();
+void count_launches(uint64_t n);
 // number of multiprocessors of the calling thread's current device (queried once per device)
 int sm_count();
 // true while a per-launch event trace is being recorded

@@ -18,6 +18,7 @@ struct Rec {
 };
 std::mutex g_mu;
 uint64_t g_launches = 0;
+thread_local uint64_t t_launches = 0;
 bool g_tracing = false;
 std::vector<Rec> g_recs;
 std::vector<cudaEvent_t> g_pool;
@@ -53,11 +54,17 @@ int sm_count() {
 
 const char* kernel_name(int kind) { return (kind >= 0 && kind < K_KINDS) ? kNames[kind] : "?"; }
 uint64_t launches() { return g_launches; }
+uint64_t thread_launches() { return t_launches; }
+void count_launches(uint64_t n) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    g_launches += n;
+}
 bool tracing() { return g_tracing; }
 
 LaunchScope::LaunchScope(int kind, double alg_bytes, double flops, cudaStream_t s) : slot(-1), st(s) {
     std::lock_guard<std::mutex> lk(g_mu);
     ++g_launches;
+    ++t_launches;
     if (g_tracing) {
         Rec r{kind, alg_bytes, flops, take_event(), take_event()};
         cudaEventRecord(r.e0, st);

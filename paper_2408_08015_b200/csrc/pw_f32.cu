@@ -34,6 +34,9 @@ struct F32Args {
     int bp;                    // floats between the rows of the staged weights
     int m_tiles;
     BnPendFwd pf;
+    BnPendFwd pf2;             // a deferred residual sum: the second operand's coefficients (the tensor is az), and where the sum goes
+    const float *d0, *d1;
+    float* sum_out;
     BnPendBwd pb;
     BnSumsOut so;
     const float* rz;           // backward sums: raw output of the unit whose gradient this is
@@ -52,7 +55,8 @@ __device__ __forceinline__ float grad1(float d, float z, float k1, float k2, flo
 // that the float4 fragments of both operands (four k of one row) feed packed FMAs as they are: 4 + TN shared-memory reads for 8*TN of them.
 // WK warps share a tile's reduction where the map is small.  The operand goes global -> registers (one chunk ahead) -> transform -> shared memory;
 // the weights of the CTA's columns stay in shared memory, row order permuted so that a lane's columns come in groups of G consecutive ones.
-template <bool BWD, int TN, int WK, bool XF>
+enum { XF_NONE = 0, XF_VALUE = 1, XF_ADD = 2 };
+template <bool BWD, int TN, int WK, int XF>
 __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
     pdl_launch();
     constexpr int WM = 4 / WK, BM = 32 * WM, BK = 16 * WK, AP = BK + 4, QC = BK / 4, BN = 4 * TN, G = TN % 4 == 0 ? 4 : 2, NG = TN / G;
@@ -60,8 +64,8 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r = lane >> 2, t = lane & 3, wm = warp % WM, wk = warp / WM;
     const int n0 = blockIdx.y * BN, Kp = (a.K + 15) & ~15;
     float* sB = sm;                                        // [BN][bp]
-    float* sK = sB + BN * a.bp;                            // operand coefficients [5 | 2][Kp]
-    float* sN = sK + (BWD ? 5 : 2) * Kp;                   // column coefficients [4][BN]
+    float* sK = sB + BN * a.bp;                            // operand coefficients [5 | 3][Kp]
+    float* sN = sK + (BWD ? 5 : 3) * Kp;                   // column coefficients [4][BN]
     float* sA = sN + 4 * BN;                               // [2][BM][AP]
     float* sR = sA + 2 * BM * AP;                          // partial tiles of the other WK - 1 warps; the column sums [WM][2][BN]
     {
@@ -86,7 +90,7 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
         for (int j = 0; j < 4; ++j) {
             const size_t e = (size_t)min(tile * BM + prow + j * (NT / QC), a.P - 1) * a.K + k;
             nx[j] = ld4(a.a + e);
-            if (BWD && XF) nz[j] = ld4(a.az + e);
+            if ((BWD && XF) || XF == XF_ADD) nz[j] = ld4(a.az + e);
         }
     };
     int tile = blockIdx.x;
@@ -108,6 +112,13 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
                 if (a.pf.sums) k = bn_fwd_coef(a.pf, c, first);
                 else if (a.c0) k = make_float2(a.c0[c], a.c1[c]);
                 sK[c] = k.x;
+                if (XF == XF_ADD) {
+                    float2 k2 = make_float2(1.f, 0.f);
+                    if (a.pf2.sums) k2 = bn_fwd_coef(a.pf2, c, first);
+                    else if (a.d0) k2 = make_float2(a.d0[c], a.d1[c]);
+                    sK[2 * Kp + c] = k2.x;
+                    k.y += k2.y;
+                }
                 sK[Kp + c] = k.y;
             }
         }
@@ -162,14 +173,22 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
                         *reinterpret_cast<float4*>(d + (prow + j * (NT / QC)) * AP + kq * 4) = v;
                     }
                 } else {
-                    float4 s, h;
+                    float4 s, h, s2;
                     if (XF) {
                         s = ld4(sK + k); h = ld4(sK + Kp + k);
+                        if (XF == XF_ADD) s2 = ld4(sK + 2 * Kp + k);
                     }
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         float4 v = nx[j];
-                        if (XF) {
+                        if (XF == XF_ADD) {
+                            v.x = clampf(fmaf(v.x, s.x, fmaf(nz[j].x, s2.x, h.x)), a.lo, a.hi);
+                            v.y = clampf(fmaf(v.y, s.y, fmaf(nz[j].y, s2.y, h.y)), a.lo, a.hi);
+                            v.z = clampf(fmaf(v.z, s.z, fmaf(nz[j].z, s2.z, h.z)), a.lo, a.hi);
+                            v.w = clampf(fmaf(v.w, s.w, fmaf(nz[j].w, s2.w, h.w)), a.lo, a.hi);
+                            const int p = tile * BM + prow + j * (NT / QC);
+                            if (blockIdx.y == 0 && p < a.P) *reinterpret_cast<float4*>(a.sum_out + (size_t)p * a.K + k) = v;
+                        } else if (XF) {
                             v.x = clampf(fmaf(v.x, s.x, h.x), a.lo, a.hi);
                             v.y = clampf(fmaf(v.y, s.y, h.y), a.lo, a.hi);
                             v.z = clampf(fmaf(v.z, s.z, h.z), a.lo, a.hi);
@@ -522,9 +541,12 @@ template <int TN, bool MDZ> __global__ void __launch_bounds__(NT) pw_f32_wgrad_k
 }
 
 typedef void (*Fn)(const F32Args);
-template <bool BWD, int TN, bool XF> Fn by_wk(int wk) { return wk == 1 ? pw_f32_kernel<BWD, TN, 1, XF> : wk == 2 ? pw_f32_kernel<BWD, TN, 2, XF> : pw_f32_kernel<BWD, TN, 4, XF>; }
-template <bool BWD, bool XF> Fn by_tn(const F32Tiling& c) { return c.tn == 4 ? by_wk<BWD, 4, XF>(c.wk) : c.tn == 6 ? by_wk<BWD, 6, XF>(c.wk) : by_wk<BWD, 8, XF>(c.wk); }
-Fn kernel_for(bool bwd, bool xf, const F32Tiling& c) { return bwd ? xf ? by_tn<true, true>(c) : by_tn<true, false>(c) : xf ? by_tn<false, true>(c) : by_tn<false, false>(c); }
+template <bool BWD, int TN, int XF> Fn by_wk(int wk) { return wk == 1 ? pw_f32_kernel<BWD, TN, 1, XF> : wk == 2 ? pw_f32_kernel<BWD, TN, 2, XF> : pw_f32_kernel<BWD, TN, 4, XF>; }
+template <bool BWD, int XF> Fn by_tn(const F32Tiling& c) { return c.tn == 4 ? by_wk<BWD, 4, XF>(c.wk) : c.tn == 6 ? by_wk<BWD, 6, XF>(c.wk) : by_wk<BWD, 8, XF>(c.wk); }
+Fn kernel_for(bool bwd, int xf, const F32Tiling& c) {
+    if (bwd) return xf ? by_tn<true, XF_VALUE>(c) : by_tn<true, XF_NONE>(c);
+    return xf == XF_ADD ? by_tn<false, XF_ADD>(c) : xf ? by_tn<false, XF_VALUE>(c) : by_tn<false, XF_NONE>(c);
+}
 
 int w_pitch(int K) { return ((K + 15) & ~15) + 4; }        // 4 or 20 modulo 32 banks: the rows of four lanes in distinct banks
 
@@ -533,7 +555,7 @@ int w_pitch(int K) { return ((K + 15) & ~15) + 4; }        // 4 or 20 modulo 32 
 size_t f32_smem(bool bwd, int K, const F32Tiling& c) {
     const int BN = 4 * c.tn, WM = 4 / c.wk, Kp = (K + 15) & ~15;
     const size_t part = (size_t)(c.wk - 1) * WM * 32 * 4 * c.tn, sums = (size_t)WM * 2 * BN;
-    return 4 * ((size_t)BN * w_pitch(K) + (size_t)(bwd ? 5 : 2) * Kp + 4 * BN + (size_t)2 * 32 * WM * (16 * c.wk + 4) + (part > sums ? part : sums));
+    return 4 * ((size_t)BN * w_pitch(K) + (size_t)(bwd ? 5 : 3) * Kp + 4 * BN + (size_t)2 * 32 * WM * (16 * c.wk + 4) + (part > sums ? part : sums));
 }
 
 // Column tile: 16, 24 or 32, the one with the least padding.  The reduction is split over two or four warps (32- and 64-deep chunks) where tiles of
@@ -570,25 +592,31 @@ void f32_launch(bool bwd, const MmaProblem& p, const F32Tiling& c, int kind, dou
     if (!(done.load(std::memory_order_acquire) & bit)) {
         for (int tn : {4, 6, 8})
             for (int wk : {1, 2, 4})
-                for (int v = 0; v < 4; ++v)
-                    cudaFuncSetAttribute(kernel_for(v & 1, v >> 1, F32Tiling{tn, wk, 0}), cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+                for (int v = 0; v < 5; ++v)
+                    cudaFuncSetAttribute(kernel_for(v < 2, v < 2 ? v : v - 2, F32Tiling{tn, wk, 0}), cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         done.fetch_or(bit, std::memory_order_release);
     }
     F32Args a;
     memset(&a, 0, sizeof a);
     a.P = p.P; a.K = p.K; a.N = p.N;
-    bool xf;
-    const int act = bwd ? p.dz.act : p.x.act;
+    int xf;
+    const int act = bwd ? p.dz.act : p.sum_out ? p.sum_act : p.x.act;
     if (bwd) {
         a.a = (const float*)p.dz.dy; a.az = (const float*)p.dz.z;
         a.c0 = p.dz.k1; a.c1 = p.dz.k2; a.c2 = p.dz.k3; a.c3 = p.dz.scale; a.c4 = p.dz.shift;
         a.pb = p.pb;
-        xf = act != ACT_NONE || p.dz.k1 || p.pb.sums;
+        xf = act != ACT_NONE || p.dz.k1 || p.pb.sums ? XF_VALUE : XF_NONE;
     } else {
         a.a = (const float*)p.x.p;
         a.c0 = p.x.scale; a.c1 = p.x.shift;
         a.pf = p.pf;
-        xf = act != ACT_NONE || p.x.scale || p.pf.sums;
+        xf = act != ACT_NONE || p.x.scale || p.pf.sums ? XF_VALUE : XF_NONE;
+        if (p.sum_out) {
+            xf = XF_ADD;
+            a.az = (const float*)p.x2.p; a.d0 = p.x2.scale; a.d1 = p.x2.shift;
+            a.pf2 = p.pf2;
+            a.sum_out = (float*)p.sum_out;
+        }
     }
     a.lo = act == ACT_NONE ? -INFINITY : 0.f;
     a.hi = act == ACT_RELU6 ? 6.f : INFINITY;
@@ -606,7 +634,7 @@ void f32_launch(bool bwd, const MmaProblem& p, const F32Tiling& c, int kind, dou
     int gx = sm_count() * c.ctas / ny;
     if (gx < 1) gx = 1;
     if (gx > a.m_tiles) gx = a.m_tiles;
-    LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 4.0 * p.P * p.N : 0.0), 2.0 * p.P * p.N * p.K, st);
+    LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 4.0 * p.P * p.N : 0.0) + (p.sum_out ? 8.0 * p.P * p.K : 0.0), 2.0 * p.P * p.N * p.K, st);
     launch_pdl(kernel_for(bwd, xf, c), dim3(gx, ny), NT, f32_smem(bwd, p.K, c), st, a);
 }
 

@@ -26,6 +26,7 @@ template <bool BWD, int XF> KernelFn by_columns(const MmaTiling& c) {
     }
 }
 template <bool BWD> KernelFn kernel_for(const MmaTiling& c, int xf) {
+    if (!BWD && xf == XF_ADD) return by_columns<false, XF_ADD>(c);
     return xf == XF_NONE ? by_columns<BWD, XF_NONE>(c) : xf == XF_AFFINE ? by_columns<BWD, XF_AFFINE>(c) : by_columns<BWD, XF_ACT>(c);
 }
 // the shared-memory limit of every instantiation, raised once per device
@@ -37,7 +38,7 @@ template <bool BWD> void raise_limits() {
     if (done.load(std::memory_order_acquire) & bit) return;
     for (int nj : {2, 3, 4, 6, 8})
         for (int v = 0; v < 5; ++v)
-            for (int xf = XF_NONE; xf <= XF_ACT; ++xf) {
+            for (int xf = XF_NONE; xf <= (BWD ? XF_ACT : XF_ADD); ++xf) {
                 MmaTiling c{};
                 c.nj = nj;
                 c.mi = v == 1 ? 2 : 1;
@@ -158,7 +159,7 @@ bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {
 
 size_t mma_smem(bool bwd, int K, const MmaTiling& c) {
     const int Kp = (K + 31) / 32 * 32, BN = c.wk == 1 ? c.wn * c.nj * 8 : c.nj * 8;
-    size_t b = (size_t)BN * w_pitch(K) + (size_t)(bwd ? 5 : 2) * Kp * 4 + (size_t)(bwd ? 4 : 1) * BN * 4;
+    size_t b = (size_t)BN * w_pitch(K) + (size_t)(bwd ? 5 : 3) * Kp * 4 + (size_t)(bwd ? 4 : 1) * BN * 4;
     if (c.wk == 1) b += (size_t)c.wm * 2 * BN * 4;
     else {
         const size_t acc = (size_t)128 * (BN + 4) * 4;
@@ -183,6 +184,13 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
         a.c0 = p.x.scale; a.c1 = p.x.shift;
         a.pf = p.pf;
         xf = p.x.act != ACT_NONE ? XF_ACT : (p.x.scale || p.pf.sums) ? XF_AFFINE : XF_NONE;
+        if (p.sum_out) {
+            xf = XF_ADD;
+            a.az = p.x2.p; a.d0 = p.x2.scale; a.d1 = p.x2.shift;
+            a.pf2 = p.pf2;
+            a.sum_out = (__nv_bfloat16*)p.sum_out;
+            a.act = p.sum_act;
+        }
     }
     a.w = (const __nv_bfloat16*)p.w; a.bias = p.bias; a.addend = p.addend; a.out = (__nv_bfloat16*)p.out;
     a.WM = c.wm; a.WN = c.wn;
@@ -205,7 +213,7 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
     if (bwd) raise_limits<true>();
     else raise_limits<false>();
     const size_t smem = mma_smem(bwd, p.K, c);
-    LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 2.0 * p.P * p.N : 0.0), 2.0 * p.P * p.N * p.K, st);
+    LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 2.0 * p.P * p.N : 0.0) + (p.sum_out ? 4.0 * p.P * p.K : 0.0), 2.0 * p.P * p.N * p.K, st);
     launch_pdl(bwd ? kernel_for<true>(c, xf) : kernel_for<false>(c, xf), dim3(gx, ny), c.wk == 1 ? 32 * c.wm * c.wn : 256, smem, st, a);
 }
 

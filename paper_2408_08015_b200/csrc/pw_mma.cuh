@@ -25,7 +25,7 @@ namespace mma {
 
 struct Args {
     const void* a;             // [P][K]: x, or dy
-    const void* az;            // backward: z [P][K]
+    const void* az;            // backward: z [P][K]; forward of a deferred sum: its second operand
     const float *c0, *c1, *c2, *c3, *c4;   // operand transform: forward scale, shift; backward k1, k2, k3, scale, shift (null: identity)
     int act;
     const __nv_bfloat16* w;    // [N][K]
@@ -38,6 +38,9 @@ struct Args {
     int m_tiles;
     uint32_t wpitch;           // bytes between rows of the staged weights
     BnPendFwd pf;              // pending coefficients of the operand (sums null: c0.. are final)
+    BnPendFwd pf2;             // deferred sum: pending coefficients of the second operand
+    const float *d0, *d1;      // ... its scale and shift (null: identity)
+    __nv_bfloat16* sum_out;    // ... where the sum goes, [P][K]
     BnPendBwd pb;
     BnSumsOut so;              // column sums of the output (sums null: none)
     const __nv_bfloat16* rz;   // backward sums: raw output [P][N] of the unit whose gradient this is, its coefficients and activation
@@ -70,21 +73,29 @@ __device__ __forceinline__ uint32_t pack2(float2 f) {
 // Operand transforms of 8 channels.  Forward: the activation is applied after rounding on packed pairs, as one integer
 // min-then-max-with-0 (the bit patterns of non-negative bfloat16 numbers order like integers and negative ones are negative
 // integers; rounding is monotonic and 0 and 6 are bfloat16 numbers, so clamping before or after it is the same).
-enum { XF_NONE = 0, XF_AFFINE = 1, XF_ACT = 2 };
+// XF_ADD (forward): the operand is a residual sum that has not been formed yet, act(x*s + z*s2 + h) of two tensors.
+enum { XF_NONE = 0, XF_AFFINE = 1, XF_ACT = 2, XF_ADD = 3 };
 template <int XF> struct XfFwd {
-    float s[8], h[8];
+    float s[8], h[8], s2[8];
     uint32_t top;
+    bool relu;
     __device__ __forceinline__ void load(const float* sm, int Kp, int c) {
         if (XF == XF_NONE) return;
         lds8(sm + c, s);
         lds8(sm + Kp + c, h);
+        if (XF == XF_ADD) lds8(sm + 2 * Kp + c, s2);
+    }
+    __device__ __forceinline__ uint32_t sum(uint32_t w, uint32_t z, int q) const {
+        const uint32_t r = pack2(__ffma2_rn(unpack2(w), make_float2(s[q], s[q + 1]), __ffma2_rn(unpack2(z), make_float2(s2[q], s2[q + 1]), make_float2(h[q], h[q + 1]))));
+        return relu ? __vimin_s16x2_relu(r, top) : r;
     }
     __device__ __forceinline__ uint32_t two(uint32_t w, int q) const {
         const uint32_t r = pack2(__ffma2_rn(unpack2(w), make_float2(s[q], s[q + 1]), make_float2(h[q], h[q + 1])));
         return XF == XF_ACT ? __vimin_s16x2_relu(r, top) : r;
     }
-    __device__ __forceinline__ uint4 apply(const uint4& v, const uint4&) const {
+    __device__ __forceinline__ uint4 apply(const uint4& v, const uint4& z) const {
         if (XF == XF_NONE) return v;
+        if (XF == XF_ADD) return make_uint4(sum(v.x, z.x, 0), sum(v.y, z.y, 2), sum(v.z, z.z, 4), sum(v.w, z.w, 6));
         return make_uint4(two(v.x, 0), two(v.y, 2), two(v.z, 4), two(v.w, 6));
     }
 };
@@ -120,7 +131,10 @@ template <int XF> struct XfBwd {
 };
 template <bool BWD, int XF> struct Xf;
 template <int XF> struct Xf<false, XF> : XfFwd<XF> {
-    __device__ __forceinline__ void set_act(int act) { this->top = act == ACT_RELU6 ? 0x40C040C0u : 0x7F807F80u; }
+    __device__ __forceinline__ void set_act(int act) {
+        this->top = act == ACT_RELU6 ? 0x40C040C0u : 0x7F807F80u;
+        this->relu = act != ACT_NONE;
+    }
 };
 template <int XF> struct Xf<true, XF> : XfBwd<XF> {
     __device__ __forceinline__ void set_act(int act) { this->hi = act == ACT_RELU6 ? 6.f : INFINITY; }
@@ -163,6 +177,13 @@ template <bool BWD, int XF> __device__ __forceinline__ void stage_coefs(const Ar
                 if (ok && a.pf.sums) k = bn_fwd_coef(a.pf, c, first);
                 else if (ok && a.c0) k = make_float2(a.c0[c], a.c1[c]);
                 sK[c] = k.x;
+                if (XF == XF_ADD) {
+                    float2 k2 = make_float2(1.f, 0.f);
+                    if (ok && a.pf2.sums) k2 = bn_fwd_coef(a.pf2, c, first);
+                    else if (ok && a.d0) k2 = make_float2(a.d0[c], a.d1[c]);
+                    sK[2 * Kp + c] = k2.x;
+                    k.y += k2.y;
+                }
                 sK[Kp + c] = k.y;
             }
         }
@@ -239,14 +260,14 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
     const int BN = a.WN * NJ * 8, n0 = blockIdx.y * BN, Kp = a.KCH * 32;
     uint8_t* sW = sm;
     float* sK = reinterpret_cast<float*>(sW + (size_t)BN * a.wpitch);
-    float* sN = sK + (BWD ? 5 : 2) * Kp;
+    float* sN = sK + (BWD ? 5 : 3) * Kp;
     float* red = sN + (BWD ? 4 : 1) * BN;                  // [WM][2][BN]
     stage_weights<G>(a, sW, n0, BN);
     pdl_wait();
 
     const uint8_t* pa = reinterpret_cast<const uint8_t*>(a.a);
     const uint8_t* pz = reinterpret_cast<const uint8_t*>(a.az);
-    constexpr bool USE_Z = BWD && XF != XF_NONE;
+    constexpr bool USE_Z = BWD ? XF != XF_NONE : XF == XF_ADD;
     const int warp_row = wm * (16 * MI) + g, BM = a.WM * 16 * MI;
     const uint32_t row_bytes = (uint32_t)a.K * 2u;
     const uint32_t last_off = (uint32_t)min((a.KCH - 1) * 64 + t * 16, a.K * 2 - 16);     // beyond K: any finite value, its weights are zero
@@ -326,6 +347,14 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
             for (int mi = 0; mi < MI; ++mi)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) cu[mi][h] = xf.apply(nx[mi][h], nz[mi][h]);
+            if (!BWD && XF == XF_ADD && blockIdx.y == 0 && wn == 0 && kc * 64 + t * 16 < a.K * 2)
+#pragma unroll
+                for (int mi = 0; mi < MI; ++mi)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int p = row0 + mi * 16 + h * 8;
+                        if (p < a.P) *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(a.sum_out) + (size_t)p * row_bytes + (uint32_t)(kc * 64 + t * 16)) = cu[mi][h];
+                    }
             if (kc + 1 < a.KCH) fetch(kc + 1);
             else if (tile + (int)gridDim.x < a.m_tiles) {
                 set_rows(tile + gridDim.x);
@@ -410,13 +439,13 @@ __global__ void __launch_bounds__(256) pw_mma_split_kernel(const Args a) {
     pdl_launch();
     extern __shared__ __align__(16) uint8_t sm[];
     constexpr int WM = 8 / WK, BM = 16 * WM, BN = 8 * NJ, RP = BN + 4, D = BWD ? 3 : 4;
-    constexpr bool USE_Z = BWD && XF != XF_NONE;
+    constexpr bool USE_Z = BWD ? XF != XF_NONE : XF == XF_ADD;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int wm = warp % WM, wk = warp / WM;
     const int n0 = blockIdx.y * BN, Kp = a.KCH * 32, p0 = blockIdx.x * BM;
     uint8_t* sW = sm;
     float* sK = reinterpret_cast<float*>(sW + (size_t)BN * a.wpitch);
-    float* sN = sK + (BWD ? 5 : 2) * Kp;
+    float* sN = sK + (BWD ? 5 : 3) * Kp;
     float* racc = sN + (BWD ? 4 : 1) * BN;                 // [WK][BM][RP]
     stage_weights<G>(a, sW, n0, BN);
     pdl_wait();
@@ -466,6 +495,12 @@ __global__ void __launch_bounds__(256) pw_mma_split_kernel(const Args a) {
             if (kc < a.KCH) {
                 xf.load(sK, Kp, kc * 32 + t * 8);
                 const uint4 c0 = xf.apply(rx[d][0], rzv[d][0]), c1 = xf.apply(rx[d][1], rzv[d][1]);
+                if (!BWD && XF == XF_ADD && blockIdx.y == 0 && kc * 64 + t * 16 < a.K * 2) {
+                    const int p = p0 + wm * 16 + g;
+                    uint8_t* so = reinterpret_cast<uint8_t*>(a.sum_out) + (size_t)p * a.K * 2 + (uint32_t)(kc * 64 + t * 16);
+                    if (p < a.P) *reinterpret_cast<uint4*>(so) = c0;
+                    if (p + 8 < a.P) *reinterpret_cast<uint4*>(so + (size_t)16 * a.K) = c1;
+                }
                 if (kc + D * WK < a.KCH) fetch(kc + D * WK, rx[d], rzv[d]);
 #pragma unroll
                 for (int j = 0; j < NJ; ++j) {

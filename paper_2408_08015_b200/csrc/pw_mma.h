@@ -16,6 +16,12 @@ struct MmaProblem {
     ValSrc x;                  // forward operand
     GradSrc dz;                // backward operand
     BnPendFwd pf;              // pending coefficients of x
+    // a deferred residual sum (sum_out not null): the forward operand is sum_act(x + x2), both without an activation of their own, and the
+    // kernel also writes it out
+    ValSrc x2;
+    BnPendFwd pf2;
+    void* sum_out;
+    int sum_act;
     BnPendBwd pb;              // pending coefficients of dz
     const void* w;             // [N][K]
     const float* bias;

@@ -630,6 +630,21 @@ static bool f32_unit(const asteroid_stage* s, const Unit& u, bool bwd, F32Tiling
     return bwd ? f32_choose(true, g.n * g.ho * g.wo, g.co, g.ci, t) : f32_choose(false, g.n * g.ho * g.wo, g.ci, g.co, t);
 }
 
+// A residual sum of two tensors without activations of their own, read next by a pointwise layer on the register-operand or float32
+// kernels: that layer forms it as it loads, and writes it out for the others.  Up to 4 M elements, where the sum is mostly a launch in the chain (a
+// round of a sixth of MobileNetV2 at batch 4 1681 -> 1647 us, of small images 1469 -> 1440); beyond, two operands to wait for cost the
+// pointwise layer more than the pass saves (ResNet stage at batch 32: 1 % slower).  Not while a profile times the units one by one.
+static bool defers_add(const asteroid_stage* s, size_t ui) {
+    const Unit& u = s->units[ui];
+    if (s->tm.on || ui + 1 >= s->units.size() || s->vals[u.out].elems > (size_t)4 << 20) return false;
+    const Unit& v = s->units[ui + 1];
+    MmaTiling t;
+    F32Tiling t32;
+    if (v.kind != U_CONV || v.in != u.out || v.col_kp || v.sub_off >= 0) return false;
+    if (u.in == u.in2 || s->vals[u.in].act != ACT_NONE || s->vals[u.in2].act != ACT_NONE) return false;
+    return mma_unit(s, v, v.g, false, &t) || f32_unit(s, v, false, &t32);
+}
+
 static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cudaStream_t st) {
     SlotView sv = slot_view(s, slot);
     const int dt = s->dtype;
@@ -643,6 +658,7 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
         }
     }
     Pending pend(s, sv, st);
+    int deferred = -1;             // a residual sum left to the pointwise layer behind it
     int squeeze_splits = 0;        // > 0: the unit before left the squeeze of this one as that many partials in the scratch arena
     const auto producer = [&](int v) { return s->vals[v].affine ? s->vals[v].unit : -1; };
     for (size_t ui = 0; ui < s->units.size(); ++ui) {
@@ -662,6 +678,14 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
             p.x = xs; p.w = w; p.out = obuf;
             p.bias = u.b_off >= 0 ? s->w + u.b_off : nullptr;
             p.pf = pend.take_fwd(in_unit);
+            if (deferred >= 0) {
+                const Unit& au = s->units[deferred];
+                p.x2 = val_src(s, sv, au.in2);
+                p.pf2 = pend.take_fwd(producer(au.in2));
+                p.sum_out = sv.base + s->vals[au.out].buf_off;
+                p.sum_act = au.act;
+                deferred = -1;
+            }
             if (bn) p.so = sums_fwd(s, u);
             const double elems = (double)p.P * p.K + (double)p.P * p.N + (double)p.N * p.K;
             if (dt == AST_F32) f32_launch(false, p, til32, K_CONV_FWD, 4.0 * elems, st);
@@ -669,9 +693,11 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
             fused_stats = bn ? -1 : 0;
         };
         if (u.kind == U_CONV && !u.col_kp && u.sub_off < 0 && mma_unit(s, u, u.g, false, &til)) {
-            on_mma(u.g, val_src(s, sv, u.in), producer(u.in), s->wb + u.w_off);
+            const int from = deferred >= 0 ? s->units[deferred].in : u.in;
+            on_mma(u.g, val_src(s, sv, from), producer(from), s->wb + u.w_off);
         } else if (f32_unit(s, u, false, &til32)) {
-            on_mma(u.g, val_src(s, sv, u.in), producer(u.in), s->w + u.w_off);
+            const int from = deferred >= 0 ? s->units[deferred].in : u.in;
+            on_mma(u.g, val_src(s, sv, from), producer(from), s->w + u.w_off);
         } else if (u.kind == U_CONV) {
             pend.settle_fwd(producer(u.in));
             const float* bias = u.b_off >= 0 ? s->w + u.b_off : nullptr;
@@ -726,6 +752,8 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
             se_forward(dt, val_src(s, sv, u.in), s->B, o.h * o.w, c, k, wp, wp + (size_t)k * c, wp + (size_t)k * c + k, wp + 2 * (size_t)k * c + k, sev,
                        sev + (size_t)s->B * c, sev + (size_t)s->B * (c + k), s->scratch, s->scratch_floats, squeeze_splits, obuf, is_last ? y : nullptr, st);
             squeeze_splits = 0;
+        } else if (u.kind == U_ADD && defers_add(s, ui)) {
+            deferred = (int)ui;
         } else if (u.kind == U_ADD) {
             if (!ew_takes_pending(dt, o.c)) {
                 pend.settle_fwd(producer(u.in));

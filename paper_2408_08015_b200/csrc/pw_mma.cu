@@ -53,7 +53,6 @@ uint32_t w_pitch(int K) {
     return b % 128 == 0 ? b + 64 : b;                  // an odd multiple of 64 bytes: a fragment read meets every bank once
 }
 
-}  // namespace
 
 // Backward tilings by a cost model (us), fitted to 1 500 timings over 49 layers (512 to 200 704 pixels, 16 to 1280 channels, with and without an
 // addend): within 2.2 % of the best tiling on average, at worst 27 %.  Persistent form: a CTA's tile takes the longer of its own latency
@@ -92,7 +91,7 @@ bool bwd_choose(int P, int K, int N, MmaTiling* out) {
         if (narrow ? best != 0 : (N + 8 * nj - 1) / (8 * nj) * nj * 8 > N * 1.35 + 8) continue;
         if (nj == 8) {
             offer(1, 8, 4, 1, 2);
-            offer(1, 8, 8, 1, 1);
+            if (P < 20000) offer(1, 8, 8, 1, 1);           // on larger maps 5 to 30 % slower than two CTAs of four warps, which the model does not see
         } else {
             offer(2, nj, 8, 1, 1);
             offer(2, nj, 4, 1, 2);
@@ -104,57 +103,60 @@ bool bwd_choose(int P, int K, int N, MmaTiling* out) {
     return best != 0;
 }
 
-// Which layers run here and how the forward is tiled.  Times below: one layer with its BatchNorm sums in a captured chain of launches,
-// inputs of large layers from HBM; "before" is the tensor-memory pipeline (or, above 256 channels, the one-tile / streaming kernels of
-// pw_tc.cu and pw_stream.cu) with its finishing kernel.
-//   - More than 256 x 64 products per pixel on more than 50 000 pixels: the arithmetic of mma.sync (and the shared-memory reads of its
-//     weights) is what bounds such a layer and the tensor-memory pipeline is as fast or faster (64 -> 256 at 100 352 pixels: 26.4 us
-//     against 27.4; 256 -> 128: 33.4 against 39.8; backward to 256 channels 71 against 77, but to 64 channels 45 against 42.5).  It takes at
-//     most 256 channels a side, so wider layers run here (128 -> 512 at 25 088 pixels: 33.5 -> 22.7 us; 512 -> 128: 27.4 -> 22.8).
-//   - A reduction of at most 192 channels, or at least 6 000 pixels, or twice as many output as reduction channels: the persistent
-//     form (24 -> 144 at 100 352 pixels 18.7 -> 13.8 us; 144 -> 24: 20.2 -> 12.7; 160 -> 960 at 784 pixels 18.4 -> 5.3).
-//   - Else the split form: as many warps on the reduction as it takes to give the chip about one and a half CTAs per multiprocessor
-//     (960 -> 160 at 784 pixels 40.9 -> 6.9 us; 384 -> 64 at 784: 13.0 -> 3.9).
+// Forward tilings by a model of the same form, fitted to 1 300 timings over the same layers: within 3.3 % of the best tiling on average, at worst 36 %.
+// The forward kernels need fewer registers, so two CTAs of eight warps or four of four share a multiprocessor where the warp's tile is small.
+// Before the model (a rule of thumb on the map and the channels, 11 % above the best on average): 24 -> 144 at 100 352 pixels 20.1 -> 15.7 us, 16 -> 96 at
+// 200 704 26.1 -> 18.6, 32 -> 192 at 12 544 7.4 -> 4.2, 64 -> 384 at 3 136 7.5 -> 4.1, 96 -> 576 8.8 -> 5.4, 512 -> 128 at 4 704 10.0 -> 7.5.
+bool fwd_choose(int P, int K, int N, MmaTiling* out) {
+    const int KCH = (K + 31) / 32, sms = sm_count();
+    double best = 0;
+    auto offer = [&](int mi, int nj, int wm, int wk, int ctas) {
+        const MmaTiling c{mi, nj, wm, 1, wk, ctas};
+        if (mma_smem(false, K, c) * (wk == 1 ? ctas : 1) > 200 * 1024) return;
+        const int cols = (N + 8 * nj - 1) / (8 * nj);
+        double t;
+        if (wk == 1) {
+            const int tiles = (P + 16 * mi * wm - 1) / (16 * mi * wm), cap = sms * ctas / cols > 0 ? sms * ctas / cols : 1, gx = tiles < cap ? tiles : cap;
+            const int turns = (tiles + gx - 1) / gx;
+            int r = (gx * cols + sms - 1) / sms;
+            if (r > ctas) r = ctas;
+            const double issue = (double)r * wm * mi * (KCH * (0.0108 + 0.00169 * nj) + nj * 0.01086);
+            const double lat = 0.0046 + 0.312 * KCH * (1.0 + 0.0966 * (mi - 1)) + 0.0912 * mi * nj;
+            t = 1.085 + 0.0253 * r * nj * KCH + turns * (lat > issue ? lat : issue);
+        } else {
+            const int bm = 128 / wk, per = ((P + bm - 1) / bm * cols + sms - 1) / sms, r = per < 2 ? per : 2, waves = (per + r - 1) / r, kc = (KCH + wk - 1) / wk;
+            t = 4.177 + waves * (kc * (0.447 + 0.00146 * nj * r) + r * (0.00019 * nj + 0.00831 * nj * KCH));
+        }
+        if (best == 0 || t < best) {
+            best = t;
+            *out = c;
+        }
+    };
+    for (int nj : {8, 6, 4, 3, 2}) {
+        const bool narrow = (nj == 2 && N > 32) || (nj == 3 && N > 24);       // only where the weights of more columns do not fit
+        if (narrow ? best != 0 : (N + 8 * nj - 1) / (8 * nj) * nj * 8 > N * 1.35 + 8) continue;
+        for (int mi = 2; mi >= 1; --mi) {
+            offer(mi, nj, 8, 1, 1);
+            if (mi == 1 || nj <= 3) offer(mi, nj, 8, 1, 2);
+            offer(mi, nj, 4, 1, 2);
+            if (nj == 4 || (mi == 1 && nj >= 3)) offer(mi, nj, 4, 1, 4);
+        }
+        if (P <= 30000)
+            for (int wk : {2, 4, 8}) offer(1, nj, 8 / wk, wk, 1);
+    }
+    return best != 0;
+}
+
+}  // namespace
+
+// Which layers run here: all whose channel counts are whole vectors, but for more than 256 x 64 products per pixel on more than 50 000 pixels with at most
+// 256 channels a side.  There the arithmetic of mma.sync (and the shared-memory reads of its weights) is the bound and the tensor-memory
+// pipeline of pw_tc.cu is as fast or faster: 64 -> 256 at 100 352 pixels 26.3 us against 29.3, backward to 256 channels 71 against 77.  To at
+// most 64 channels it is not: 256 -> 64 30.6 against 24.0, backward 45 against 42.  (One layer with its BatchNorm sums in a captured chain.)
 bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {
     if (K % 8 || N % 8 || (double)P * (K > N ? K : N) * 2.0 >= 4.0e9) return false;
-    if (P >= 50000 && K <= 256 && N <= 256 && K * N >= 256 * 64 && !(bwd && N <= 64)) return false;
-    if (bwd) return bwd_choose(P, K, N, out);
-    const int KCH = (K + 31) / 32, sms = sm_count();
-    MmaTiling c{};
-    c.mi = 1; c.wm = 8; c.wn = 1; c.wk = 1; c.ctas = 1;
-    auto cols = [&](int nj) { return (N + 8 * nj - 1) / (8 * nj); };
-    if (KCH <= 6 || P >= 6000 || N >= 2 * K) {
-        // column tile: least padding, then fewest blocks
-        int best = 0, best_cost = 0;
-        for (int nj : {8, 6, 4, 3, 2}) {
-            const int cost = cols(nj) * nj * 8 * 4 + cols(nj) * 24;
-            if (!best || cost < best_cost) {
-                best = nj;
-                best_cost = cost;
-            }
-        }
-        c.nj = best;
-        c.mi = 2;
-        auto ctas = [&] { return (P + 16 * c.mi * c.wm - 1) / (16 * c.mi * c.wm) * cols(c.nj); };
-        if (ctas() < sms) c.mi = 1;
-        if (ctas() < sms && c.nj == 8) c.nj = 4;
-        if (ctas() < sms && c.nj == 6 && N % 32 == 0) c.nj = 4;
-        if (ctas() < sms) c.wm = 4;
-        if (c.mi == 1 || c.nj <= 3) c.ctas = 2;
-        if (c.wm == 4) c.ctas = 4;
-    } else {
-        c.nj = N <= 16 ? 2 : N <= 24 ? 3 : 4;
-        c.wk = 2;
-        const int want = sms * 5 / 4;
-        while (c.wk < 8 && (P + 128 / c.wk - 1) / (128 / c.wk) * cols(c.nj) < want) c.wk *= 2;
-        c.wm = 8 / c.wk;
-    }
-    while (mma_smem(false, K, c) > 200 * 1024) {
-        if (c.nj <= 2) return false;
-        c.nj = c.nj == 8 ? 6 : c.nj == 6 ? 4 : c.nj - 1;
-    }
-    *out = c;
-    return true;
+    if (P >= 50000 && K <= 256 && N <= 256 && K * N >= 256 * 64 && N > 64) return false;
+    return bwd ? bwd_choose(P, K, N, out) : fwd_choose(P, K, N, out);
 }
 
 size_t mma_smem(bool bwd, int K, const MmaTiling& c) {

@@ -192,18 +192,21 @@ __global__ void __launch_bounds__(512) chan_reduce_kernel(OP op, size_t pixels, 
         size_t pbeg = (size_t)blockIdx.y * pix_per_block, pend = min(pixels, pbeg + pix_per_block);
         size_t p = pbeg + row;
         if (V == Vec<T>::N) {
-            // the loads of a batch of pixels (eight vectors per thread) are issued before any is used: with one block per SM
-            // the bytes in flight come from each thread's own batch
-            constexpr int U = 8 / OP::NLD;
-            for (; p + (size_t)(U - 1) * rows < pend; p += (size_t)U * rows) {
+            // the loads of a batch of pixels (eight to twelve vectors per thread) are issued before any is used: with one block per SM
+            // the bytes in flight come from each thread's own batch.  The last batch re-reads the last pixel where it is short: taken one by
+            // one, its pixels cost a memory latency each (masked sum of 100 352 x 256 43.1 us, with batches of two pixels).
+            constexpr int U = OP::NLD == 3 ? 4 : 8 / OP::NLD;
+            for (; p < pend; p += (size_t)U * rows) {
                 Vec<T> r[U][OP::NLD];
 #pragma unroll
-                for (int u = 0; u < U; ++u) op.template load<T>((p + (size_t)u * rows) * c + c0, r[u]);
+                for (int u = 0; u < U; ++u) op.template load<T>(min(p + (size_t)u * rows, pend - 1) * c + c0, r[u]);
 #pragma unroll
-                for (int u = 0; u < U; ++u) op.template acc_raw<T, V>((p + (size_t)u * rows) * c + c0, r[u], ctx, a);
+                for (int u = 0; u < U; ++u)
+                    if (p + (size_t)u * rows < pend) op.template acc_raw<T, V>((p + (size_t)u * rows) * c + c0, r[u], ctx, a);
             }
+        } else {
+            for (; p < pend; p += rows) op.template acc<T, V>(p * c + c0, ctx, a);
         }
-        for (; p < pend; p += rows) op.template acc<T, V>(p * c + c0, ctx, a);
     }
     const int width = cw * V;
     for (int t = 0; t < OP::NACC; ++t) {
@@ -827,11 +830,11 @@ template <typename T, int V> static void ew_add_launch(const ValSrc& a, const Va
     LaunchScope ls(K_EW_ADD, (double)n * sizeof(T) * (1 + (b.p ? 1 : 0) + 1 + (out2 ? 1 : 0)), (double)n, st);
     if (V > 1) {
         const int vpr = c / V;
-        size_t blocks = (groups + 4 * 256 - 1) / (4 * 256);
+        // one wave of two blocks per multiprocessor (the registers' limit), every thread with the same number of vectors but one: with eight blocks
+        // per multiprocessor and four vectors a round, 25 088 x 512 left a third of the second round empty (21.2 us for 77 MB)
         const bool pend = pa.sums || pb.sums;
-        // with pending coefficients every block first forms those of all channels: fewer, longer blocks
-        const size_t cap = (size_t)sm_count() * (pend ? 4 : 8);
-        if (blocks > cap) blocks = cap;
+        const size_t cap = (size_t)sm_count() * 2 * 256, each = (groups + cap - 1) / cap;
+        size_t blocks = (groups + each * 256 - 1) / (each * 256);
         size_t threads = blocks * 256;
         if (threads < (size_t)vpr) {
             blocks = ((size_t)vpr + 255) / 256;

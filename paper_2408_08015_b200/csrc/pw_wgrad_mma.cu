@@ -147,7 +147,8 @@ template <int VM, int VN, bool MDZ>
 __global__ void __launch_bounds__(WARPS * 32) pw_wgrad_mma_kernel(const WmArgs a) {
     pdl_launch();
     extern __shared__ __align__(16) float st[];
-    constexpr int BM = 8 * VM, BN = 8 * VN, SP = BN + 1, BLK = BM * SP, NM = MDZ ? 5 : 2, NN = MDZ ? 2 : 5;
+    // the block in shared memory with the input channels contiguous: what is summed over the cluster and written out is then read and written in rows
+    constexpr int BM = 8 * VM, BN = 8 * VN, BC = MDZ ? BN : BM, SP = BC + 1, BLK = (BM * BN / BC) * SP, NM = MDZ ? 5 : 2, NN = MDZ ? 2 : 5;
     __shared__ __align__(16) float coef[NM * BM + NN * BN];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int m0 = ((int)blockIdx.y % a.mb) * BM, n0 = ((int)blockIdx.y / a.mb) * BN;
@@ -214,15 +215,16 @@ __global__ void __launch_bounds__(WARPS * 32) pw_wgrad_mma_kernel(const WmArgs a
 #pragma unroll
             for (int j = 0; j < VN; ++j) {
                 const int m = VM * g + 2 * i, n = VN * 2 * t + j;
-                d[m * SP + n] = acc[i][j][0];
-                d[m * SP + n + VN] = acc[i][j][1];
-                d[(m + 1) * SP + n] = acc[i][j][2];
-                d[(m + 1) * SP + n + VN] = acc[i][j][3];
+                auto at = [&](int mm, int nn) -> float& { return d[MDZ ? mm * SP + nn : nn * SP + mm]; };
+                at(m, n) = acc[i][j][0];
+                at(m, n + VN) = acc[i][j][1];
+                at(m + 1, n) = acc[i][j][2];
+                at(m + 1, n + VN) = acc[i][j][3];
             }
     }
     __syncthreads();
     for (int e = tid; e < BM * BN; e += WARPS * 32) {
-        float* d = st + (e / BN) * SP + e % BN;
+        float* d = st + (e / BC) * SP + e % BC;
         float s = d[0];
 #pragma unroll
         for (int w = 1; w < WARPS; ++w) s += d[w * BLK];
@@ -237,19 +239,18 @@ __global__ void __launch_bounds__(WARPS * 32) pw_wgrad_mma_kernel(const WmArgs a
     const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(st);
     const int per = (BM * BN + (int)cs - 1) / (int)cs, e0 = (int)rank * per, e1 = min(BM * BN, e0 + per);
     for (int e = e0 + tid; e < e1; e += WARPS * 32) {
-        // consecutive threads write consecutive input channels
-        const int m = MDZ ? e / BN : e % BM, n = MDZ ? e % BN : e / BM;
+        const int kr = e / BC, cc = e - kr * BC;
         float s = 0.f;
-        if (cs == 1) s = st[m * SP + n];
+        if (cs == 1) s = st[kr * SP + cc];
         else {
-            const uint32_t ad = s0 + (uint32_t)(m * SP + n) * 4u;
+            const uint32_t ad = s0 + (uint32_t)(kr * SP + cc) * 4u;
             float q[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) q[k] = k < (int)cs ? ld_cluster(ad, k) : 0.f;
 #pragma unroll
             for (int k = 0; k < 8; ++k) s += q[k];
         }
-        const int k = MDZ ? m0 + m : n0 + n, c = MDZ ? n0 + n : m0 + m;
+        const int k = (MDZ ? m0 : n0) + kr, c = (MDZ ? n0 : m0) + cc;
         if (k < a.CO && c < a.CI) out[(size_t)k * a.CI + c] = s;
     }
     if (cs > 1) cluster_sync();               // no CTA leaves while another still reads its block
@@ -270,7 +271,8 @@ template <bool MDZ> WKernel wkernel(int vm, int vn) {
 //     15.9 us against 23.5), except over layers it does not fit (480 x 80 at 6 272 pixels: 34.5 -> 18.5) and gradients so small that one
 //     warp block holds them (16 x 32 at 200 704 pixels: 20.4 -> 14.0).
 //   - 32 x 32 blocks (64 x 64 from 960 x 320 up, where the re-reads of 32 x 32 blocks cost more than the idle multiprocessors); about one
-//     and a half CTAs per multiprocessor; up to eight pixel ranges are one cluster, which writes the gradient itself.
+//     and a half CTAs per multiprocessor, of which two fit one (one of the 64 x 64 blocks': a second wave for the last two of 150 CTAs made
+//     320 x 960 at 784 pixels 25.9 us instead of 14.9); up to eight pixel ranges are one cluster, which writes the gradient itself.
 bool wgrad_mma_choose(int P, int CO, int CI, bool pipeline_fits, size_t scratch_floats, WgradTiling* out) {
     if (CO % 8 || CI % 8) return false;
     if (P > 4096 && !(P <= 16384 && !pipeline_fits) && CO * CI > 512) return false;
@@ -278,7 +280,7 @@ bool wgrad_mma_choose(int P, int CO, int CI, bool pipeline_fits, size_t scratch_
     WgradTiling c{4, CN <= 16 ? 2 : 4, 1, 1};
     if ((size_t)CM * CN >= 300000) c = WgradTiling{8, 8, 1, 1};
     const int blocks = ((CM + 8 * c.vm - 1) / (8 * c.vm)) * ((CN + 8 * c.vn - 1) / (8 * c.vn));
-    int sp = sm_count() * 3 / 2 / blocks;
+    int sp = sm_count() * (c.vm == 8 ? 2 : 3) / 2 / blocks;
     const int most = P / 64 > 0 ? P / 64 : 1;
     if (sp > most) sp = most;
     if (P > 50000) sp = 2 * sm_count() / 8 * 8;
@@ -295,7 +297,10 @@ bool wgrad_mma_choose(int P, int CO, int CI, bool pipeline_fits, size_t scratch_
     return true;
 }
 
-size_t wgrad_mma_smem(const WgradTiling& c) { return (size_t)WARPS * 8 * c.vm * (8 * c.vn + 1) * 4; }
+size_t wgrad_mma_smem(const WgradTiling& c) {                // the larger of the two layouts
+    const size_t a = (size_t)8 * c.vm * (8 * c.vn + 1), b = (size_t)8 * c.vn * (8 * c.vm + 1);
+    return (size_t)WARPS * (a > b ? a : b) * 4;
+}
 
 void wgrad_mma_launch(const WgradProblem& p, const WgradTiling& c, float* scratch, float* gw, cudaStream_t st) {
     static std::atomic<unsigned long long> done{0};

@@ -232,7 +232,9 @@ void ew_sum(int dtype, const void* a, const void* b, size_t n, void* dst, cudaSt
 // bfloat16, channel counts multiples of 8: zero-inserted gradient / subsampled output of a stride-2 3x3 conv (see conv3_s2_tc_supported)
 void ew_upsample2_grad(const GradSrc& d, int n, int hi, int wi, int ho, int wo, int c, void* up, cudaStream_t st);
 void ew_subsample2(const void* full, int n, int hi, int wi, int ho, int wo, int c, void* z, cudaStream_t st);
-void gap_fwd(int dtype, const ValSrc& x, int n, int hw, int c, void* out, cudaStream_t st);
+// pf: pending coefficients of x, where the channel count is whole vectors
+bool gap_takes_pending(int dtype, int c);
+void gap_fwd(int dtype, const ValSrc& x, const BnPendFwd& pf, int n, int hw, int c, void* out, cudaStream_t st);
 void gap_bwd(int dtype, const void* da, int n, int hw, int c, const void* addend, void* dx, cudaStream_t st);
 
 // ---- EfficientNet MBConv pieces (mbconv.cu) ----
@@ -264,8 +266,15 @@ void dwk_bwd_weight(int dtype, const ConvGeom& g, const GradSrc& dz, const ValSr
 // G += g; n_zero doubles set to zero
 void accumulate(float* G, const float* g, size_t n, double* zero, size_t n_zero, cudaStream_t st);
 void sgd_step(float* w, float* v, float* G, size_t n, float inv_m, float lr, float mu, cudaStream_t st);
-// derived[i] = w[perm[i]]; wb[i] = bf16(w[i]); wtb[i] = bf16(w[perm[i]])  (wb/wtb may be null)
-void refresh_derived(const float* w, const int32_t* perm, float* derived, __nv_bfloat16* wb, __nv_bfloat16* wtb, size_t n, cudaStream_t st);
+// a dense layer's weights [co][taps][ci] at `off`, derived as [ci][taps][co] at the same place; tile0: its first tile
+struct RefreshSeg {
+    size_t off;
+    int co, ci, taps, tile0;
+};
+// derived = the weights rearranged; wb, wtb (may be null): bfloat16 copies of the weights and of derived.  Dense layers by the table (device memory),
+// the n_rest other elements by rest[i] (destination) and rest[n_rest + i] (source); n: all of them
+void refresh_derived(const float* w, const RefreshSeg* segs, int n_segs, int tiles, const int32_t* rest, int n_rest, float* derived, __nv_bfloat16* wb,
+                     __nv_bfloat16* wtb, size_t n, cudaStream_t st);
 
 // ---- losses (scratch: >= 1024 floats + 1 counter word) ----
 void loss_mse(int dtype, const void* y, const void* t, size_t n, void* dy, float* loss, float* scratch, cudaStream_t st);

@@ -820,7 +820,7 @@ void silu_bwd(int dtype, const void* dy, const float* gate, const float* ds, con
     LaunchScope ls(K_SILU, e * esz_(dtype) * (3 + (addend ? 1 : 0)), 8.0 * e, st);
     const SiluBwdArgs a{x, dy, addend, gate, ds, sums, mean, rstd, hw, c, dx};
     DISPATCH_TV(dtype, c, {
-        const PassCut k = pass_cut(n, hw, c / V, 2, sums ? 12 : 256);
+        const PassCut k = pass_cut(n, hw, c / V, 2, sums ? 16 : 256);
         typedef void (*Fn)(SiluBwdArgs, PassCut);
         const Fn f = gate ? sums ? (Fn)silu_bwd_kernel<T, V, true, true> : (Fn)silu_bwd_kernel<T, V, true, false>
                           : sums ? (Fn)silu_bwd_kernel<T, V, false, true> : (Fn)silu_bwd_kernel<T, V, false, false>;

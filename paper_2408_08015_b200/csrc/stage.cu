@@ -126,7 +126,9 @@ struct asteroid_stage {
     std::vector<Seg> segs;
     // device arenas
     float *w = nullptr, *v = nullptr, *G = nullptr, *g = nullptr, *derived = nullptr, *run = nullptr, *coef = nullptr, *scratch = nullptr;
-    int32_t* perm = nullptr;
+    RefreshSeg* dense = nullptr;                   // how the derived weights come about (plan_refresh)
+    int32_t* rest = nullptr;
+    int n_dense = 0, tiles = 0, n_rest = 0;
     __nv_bfloat16 *wb = nullptr, *wtb = nullptr;   // bf16 copies of the weights and of the derived (transposed) weights
     __nv_bfloat16* wpad = nullptr;                 // [co][Kp] bf16 weights of the im2col units
     float* gpad = nullptr;                         // [co][Kp] padded weight gradient of the im2col unit at hand
@@ -417,22 +419,27 @@ static int build_plan(asteroid_stage* s) {
     return AST_OK;
 }
 
-static void fill_perm(const asteroid_stage* s, std::vector<int32_t>& perm) {
-    perm.resize(s->n_pad);
-    for (size_t i = 0; i < perm.size(); ++i) perm[i] = (int32_t)i;
+// How the derived weights come from the weights: dense layers turned tile by tile, everything else by (destination, source) lists.
+static void plan_refresh(const asteroid_stage* s, std::vector<RefreshSeg>& segs, int* tiles, std::vector<int32_t>& rest) {
+    std::vector<int32_t> src(s->n_pad);
+    for (size_t i = 0; i < src.size(); ++i) src[i] = (int32_t)i;
+    *tiles = 0;
     for (const auto& u : s->units) {
+        const ConvGeom& g = u.g;
+        const int taps = g.k * g.k;
         if (u.kind == U_CONV) {          // derived: wt[c][r][s][ko] <- w[ko][r][s][c]
-            const ConvGeom& g = u.g;
-            for (int ko = 0; ko < g.co; ++ko)
-                for (int rs = 0; rs < g.k * g.k; ++rs)
-                    for (int c = 0; c < g.ci; ++c)
-                        perm[u.w_off + ((size_t)c * g.k * g.k + rs) * g.co + ko] = (int32_t)(u.w_off + ((size_t)ko * g.k * g.k + rs) * g.ci + c);
+            segs.push_back(RefreshSeg{(size_t)u.w_off, g.co, g.ci, taps, *tiles});
+            *tiles += ((g.ci + 31) / 32) * ((g.co + 31) / 32) * taps;
+            std::fill(src.begin() + u.w_off, src.begin() + u.w_off + (size_t)g.co * taps * g.ci, -1);
         } else if (u.kind == U_DW) {     // derived: tap-major wkc[t][c] <- w[c][t]
-            const int taps = u.g.k * u.g.k;
-            for (int c = 0; c < u.g.ci; ++c)
-                for (int t = 0; t < taps; ++t) perm[u.w_off + (size_t)t * u.g.ci + c] = (int32_t)(u.w_off + (size_t)c * taps + t);
+            for (int c = 0; c < g.ci; ++c)
+                for (int t = 0; t < taps; ++t) src[u.w_off + (size_t)t * g.ci + c] = (int32_t)(u.w_off + (size_t)c * taps + t);
         }
     }
+    for (size_t i = 0; i < src.size(); ++i)
+        if (src[i] >= 0) rest.push_back((int32_t)i);
+    const size_t n = rest.size();
+    for (size_t i = 0; i < n; ++i) rest.push_back(src[rest[i]]);
 }
 
 static void free_stage(asteroid_stage* s) {
@@ -508,7 +515,7 @@ static int reset_bn_running(asteroid_stage* s) {
 
 // derived weight copies of every kind, after the master weights changed
 static void refresh_weights(asteroid_stage* s, cudaStream_t st) {
-    refresh_derived(s->w, s->perm, s->derived, s->wb, s->wtb, s->n_pad, st);
+    refresh_derived(s->w, s->dense, s->n_dense, s->tiles, s->rest, s->n_rest, s->derived, s->wb, s->wtb, s->n_pad, st);
     for (const auto& u : s->units)
         if (u.col_kp) conv_pad_weights(s->w + u.w_off, u.g.co, u.g.k * u.g.k * u.g.ci, u.col_kp, s->wpad + u.wpad_off, st);
 }
@@ -763,8 +770,9 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
             ew_add(dt, val_src(s, sv, u.in), val_src(s, sv, u.in2), pa, pb, u.act, o.elems / o.c, o.c, obuf, is_last ? y : nullptr, st);
         } else {
             const Val& a = s->vals[u.in];
-            pend.settle_fwd(producer(u.in));
-            gap_fwd(dt, val_src(s, sv, u.in), s->B, a.h * a.w, a.c, obuf, st);
+            if (!gap_takes_pending(dt, a.c)) pend.settle_fwd(producer(u.in));
+            const BnPendFwd pf = pend.take_fwd(producer(u.in));
+            gap_fwd(dt, val_src(s, sv, u.in), pf, s->B, a.h * a.w, a.c, obuf, st);
         }
         tick(s, ui, 1, st);
         s->fwd_stats_blocks[ui] = fused_stats < 0 ? 1 : fused_stats;
@@ -1200,7 +1208,13 @@ static int create_impl(const ast_layer* net, int n_layers, int first, int last, 
     if ((rc = arena_alloc(s, "accumulated gradients", &s->G, np * 4, &mod))) return rc;
     if ((rc = arena_alloc(s, "micro-batch gradients", &s->g, np * 4, &mod))) return rc;
     if ((rc = arena_alloc(s, "derived weights", &s->derived, np * 4, &mod))) return rc;
-    if ((rc = arena_alloc(s, "permutation", &s->perm, np * 4, &mod))) return rc;
+    std::vector<RefreshSeg> segs;
+    std::vector<int32_t> rest;
+    plan_refresh(s, segs, &s->tiles, rest);
+    s->n_dense = (int)segs.size();
+    s->n_rest = (int)(rest.size() / 2);
+    if ((rc = arena_alloc(s, "weight layers", &s->dense, segs.size() * sizeof(RefreshSeg), &mod))) return rc;
+    if ((rc = arena_alloc(s, "other parameters", &s->rest, rest.size() * 4, &mod))) return rc;
     if ((rc = arena_alloc(s, "running statistics", &s->run, s->n_run * 4, &mod))) return rc;
     if (s->dtype == AST_BF16) {
         if ((rc = arena_alloc(s, "bf16 weights", &s->wb, np * 2, &mod))) return rc;
@@ -1240,9 +1254,8 @@ static int create_impl(const ast_layer* net, int n_layers, int first, int last, 
     CU(cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming));
     CU(cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming));
     s->bytes_mod = mod; s->bytes_opt = opt; s->bytes_work = work;
-    std::vector<int32_t> perm;
-    fill_perm(s, perm);
-    if (np) CU(cudaMemcpy(s->perm, perm.data(), np * 4, cudaMemcpyHostToDevice));
+    if (!segs.empty()) CU(cudaMemcpy(s->dense, segs.data(), segs.size() * sizeof(RefreshSeg), cudaMemcpyHostToDevice));
+    if (!rest.empty()) CU(cudaMemcpy(s->rest, rest.data(), rest.size() * 4, cudaMemcpyHostToDevice));
     if ((rc = reset_bn_running(s))) return rc;
     s->slot_of_mb.assign(M, -1);
     s->mb_of_slot.assign(s->slots, -1);

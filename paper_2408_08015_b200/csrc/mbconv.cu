@@ -99,14 +99,14 @@ struct PassCut {
 };
 // ctas: blocks per multiprocessor a kernel's registers allow.  lanes: a kernel that adds to per-channel accumulators takes few channels and many
 // pixels per block: the additions, one per block, channel and sum, cost more than the pass on a small map (14x14x480 at 32 images with 60 lanes
-// 10.5 us, without sums 5.0).
-PassCut pass_cut(int n, int hw, int vpr, int ctas = 4, int lanes = 256) {
+// 10.5 us, without sums 5.0).  each: pixels a thread gets at least; more where the blocks leave partials for the next kernel to add.
+PassCut pass_cut(int n, int hw, int vpr, int ctas = 4, int lanes = 256, int each = 4) {
     PassCut c;
     c.parts = (vpr + lanes - 1) / lanes;
     c.lanes = (vpr + c.parts - 1) / c.parts;
     c.rows = 256 / c.lanes;
     int want = (int)((long long)sm_count() * ctas / ((long long)n * c.parts));
-    const int most = (hw + 4 * c.rows - 1) / (4 * c.rows);
+    const int most = (hw + each * c.rows - 1) / (each * c.rows);
     if (want > most) want = most;
     if (want < 1) want = 1;
     c.ppb = (hw + want - 1) / want;
@@ -805,7 +805,7 @@ int silu_fwd(int dtype, const ValSrc& x, const BnPendFwd& pf, int n, int hw, int
     LaunchScope ls(K_SILU, e * esz_(dtype) * (2 + (out2 ? 1 : 0)), 4.0 * e, st);
     int splits = 0;
     DISPATCH_TV(dtype, c, {
-        const PassCut k = pass_cut(n, hw, c / V);
+        const PassCut k = pass_cut(n, hw, c / V, 4, 256, part ? 6 : 4);
         splits = k.splits;
         if ((size_t)splits * n * c > part_floats) part = nullptr;
         launch_pdl(part ? silu_fwd_kernel<T, V, true> : silu_fwd_kernel<T, V, false>, dim3(k.splits * n, k.parts), 256, pass_smem(k, V), st, x, pf, k, hw, c, (T*)out, (T*)out2,

@@ -558,8 +558,13 @@ size_t f32_smem(bool bwd, int K, const F32Tiling& c) {
     return 4 * ((size_t)BN * w_pitch(K) + (size_t)(bwd ? 5 : 3) * Kp + 4 * BN + (size_t)2 * 32 * WM * (16 * c.wk + 4) + (part > sums ? part : sums));
 }
 
-// Column tile: 16, 24 or 32, the one with the least padding.  The reduction is split over two or four warps (32- and 64-deep chunks) where tiles of
-// 128 pixels would leave multiprocessors without one and a half CTAs and every warp still gets a 16-deep share.
+// Column tile: 16, 24 or 32, the one with the least padding; 16 where even the widest split of the reduction leaves less than one and a half CTAs per
+// multiprocessor (192 -> 32 on 1 568 pixels 6.4 -> 5.5 us forward, 7.6 -> 6.5 backward; 16 -> 96 on 1 000 pixels 3.9 -> 3.0 and 5.2 -> 4.0), in the
+// backward only up to 256 channels, since every column tile transforms the gradient anew (384 -> 64 on 1 568 pixels 11.7 -> 12.4 with 16).  The
+// backward with several tiles of 24 columns takes 16 and three CTAs per multiprocessor (24 -> 144 on 25 088 pixels 20.4 -> 16.8, on 100 352 82.8 ->
+// 63.1), the forward with 24 columns three (13.9 -> 12.3, 40.8 -> 37.6).  The reduction is split over two or four warps (32- and 64-deep chunks)
+// where tiles of 128 pixels would leave multiprocessors without one and a half CTAs - three quarters of one in the backward with wide tiles, where
+// unsplit tiles read the gradient in longer rows (144 -> 24 on 25 088 pixels 21.5 -> 16.6) - and every warp still gets a 16-deep share.
 bool f32_choose(bool bwd, int P, int K, int N, F32Tiling* out) {
     if (K % 4 || N % 4) return false;
     const int sms = sm_count();
@@ -572,10 +577,14 @@ bool f32_choose(bool bwd, int P, int K, int N, F32Tiling* out) {
             best = cost;
         }
     }
+    const int most = K >= 64 ? 4 : K >= 32 ? 2 : 1;
+    if ((!bwd || K <= 256) && (P + 128 / most - 1) / (128 / most) * ((N + 4 * c.tn - 1) / (4 * c.tn)) < sms * 3 / 2) c.tn = 4;
+    const bool thin = bwd && c.tn == 6 && N > 24;
+    if (thin) c.tn = 4;
     const int cols = (N + 4 * c.tn - 1) / (4 * c.tn);
     c.wk = 1;
-    while (c.wk < 4 && K >= 32 * c.wk && (P + 128 / c.wk - 1) / (128 / c.wk) * cols < sms * 3 / 2) c.wk *= 2;
-    c.ctas = 4;
+    while (c.wk < 4 && K >= 32 * c.wk && (P + 128 / c.wk - 1) / (128 / c.wk) * cols < (bwd && c.tn > 4 ? sms * 3 / 4 : sms * 3 / 2)) c.wk *= 2;
+    c.ctas = thin || (!bwd && c.tn == 6 && c.wk == 1) ? 3 : 4;
     while (f32_smem(bwd, K, c) > 200 * 1024) {
         if (c.tn == 4) return false;
         c.tn -= 2;
@@ -638,7 +647,9 @@ void f32_launch(bool bwd, const MmaProblem& p, const F32Tiling& c, int kind, dou
     launch_pdl(kernel_for(bwd, xf, c), dim3(gx, ny), NT, f32_smem(bwd, p.K, c), st, a);
 }
 
-// About three CTAs per multiprocessor, no pixel range below 64; from 12 ranges up in clusters of eight, with a split sum behind.
+// Three CTAs per multiprocessor, four with 24 columns (24 x 144 on 100 352 pixels 41.8 -> 34.3 us), no pixel range below 64.  Up to 11 ranges one cluster adds its blocks and writes the result (160 x 960 on 784
+// pixels: 20.0 us, against 23.0 with a split sum).  From 12 ranges up the split sum runs in any case, and single CTAs that start and end on their own beat
+// clusters of eight: 24 x 144 on 25 088 pixels 22.3 -> 14.3 us, 32 x 192 on 6 272 19.1 -> 9.3, 16 x 96 on 8 192 9.9 -> 6.4.
 bool f32_wgrad_choose(int P, int CO, int CI, size_t scratch_floats, F32WgradTiling* out) {
     if (CO % 4 || CI % 4) return false;
     const int CM = CO > CI ? CO : CI, CN = CO > CI ? CI : CO;
@@ -652,11 +663,11 @@ bool f32_wgrad_choose(int P, int CO, int CI, size_t scratch_floats, F32WgradTili
         }
     }
     const int blocks = ((CM + WBM - 1) / WBM) * ((CN + 4 * c.tn - 1) / (4 * c.tn));
-    int sp = sm_count() * 3 / blocks;
+    int sp = sm_count() * (c.tn == 6 ? 4 : 3) / blocks;
     const int most = P / 64 > 0 ? P / 64 : 1;
     if (sp > most) sp = most;
-    c.cluster = sp >= 6 ? 8 : sp >= 3 ? 4 : sp >= 2 ? 2 : 1;
-    c.splits = sp <= 11 ? c.cluster : (sp + 4) / 8 * 8;
+    c.cluster = sp >= 12 ? 1 : sp >= 6 ? 8 : sp >= 3 ? 4 : sp >= 2 ? 2 : 1;
+    c.splits = sp >= 12 ? sp : c.cluster;
     while ((size_t)(c.splits / c.cluster) * CO * CI > scratch_floats && c.splits > c.cluster) c.splits -= c.cluster;
     *out = c;
     return true;

@@ -29,6 +29,8 @@ CASES = {
     "wide_on_both_sides": ((200, 260), 7, 7, 3),
     "long_reduction": ((1284, 20), 3, 3, 8),
     "several_clusters": ((48, 16), 75, 70, 4),
+    "ranges_left_empty": ((24, 144, 24), 28, 28, 1),
+    "thin_gradient_in_narrow_tiles": ((144, 24), 75, 70, 4),
 }
 
 

@@ -512,7 +512,7 @@ template <typename T> __global__ void gap_bwd_kernel(const T* __restrict__ da, i
 }
 
 // ------------------------------------------------------------------ parameters
-// Also sets the accumulators of the next backward pass's channel sums to zero: every pass is followed by its accumulate.
+// Also sets the accumulators of the backward pass it follows to zero.
 __global__ void accumulate_kernel(float* __restrict__ G, const float* __restrict__ g, size_t n4, size_t n, double* __restrict__ zero, size_t n_zero) {
     pdl_wait();
     pdl_launch();
@@ -959,12 +959,14 @@ void ew_apply(int dtype, const ValSrc& a, const BnPendFwd& pa, size_t pixels, in
     ew_add(dtype, a, none, pa, BnPendFwd{}, ACT_NONE, pixels, c, out, nullptr, st);
 }
 
-// dst = src (16-byte units), and n_zero doubles set to zero by the same launch
-__global__ void __launch_bounds__(256) slot_copy_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t n, double* __restrict__ zero, size_t n_zero) {
+// dst = src (16-byte units), and na doubles at a and nb at b set to zero by the same launch
+__global__ void __launch_bounds__(256) slot_copy_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t n, double* __restrict__ a, size_t na,
+                                                        double* __restrict__ b, size_t nb) {
     pdl_wait();
     pdl_launch();
     const size_t stride = (size_t)gridDim.x * 256, id = (size_t)blockIdx.x * 256 + threadIdx.x;
-    for (size_t i = id; i < n_zero; i += stride) zero[i] = 0.0;
+    for (size_t i = id; i < na; i += stride) a[i] = 0.0;
+    for (size_t i = id; i < nb; i += stride) b[i] = 0.0;
     for (size_t i = id; i < n; i += 4 * stride) {
         uint4 v[4];
 #pragma unroll
@@ -975,12 +977,12 @@ __global__ void __launch_bounds__(256) slot_copy_kernel(const uint4* __restrict_
             if (i + u * stride < n) dst[i + u * stride] = v[u];
     }
 }
-bool slot_copy(const void* src, void* dst, size_t bytes, double* zero, size_t n_zero, cudaStream_t st) {
+bool slot_copy(const void* src, void* dst, size_t bytes, double* a, size_t na, double* b, size_t nb, cudaStream_t st) {
     if (bytes % 16 || (reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) % 16) return false;
     LaunchScope ls(K_EW_ADD, 2.0 * bytes, 0.0, st);
-    size_t blocks = (bytes / 16 + 1023) / 1024;
+    size_t blocks = (std::max(bytes / 16, na + nb) + 1023) / 1024;
     const size_t cap = (size_t)sm_count() * 8;
-    launch_pdl(slot_copy_kernel, (unsigned)(blocks < 1 ? 1 : blocks > cap ? cap : blocks), 256, 0, st, (const uint4*)src, (uint4*)dst, bytes / 16, zero, n_zero);
+    launch_pdl(slot_copy_kernel, (unsigned)(blocks < 1 ? 1 : blocks > cap ? cap : blocks), 256, 0, st, (const uint4*)src, (uint4*)dst, bytes / 16, a, na, b, nb);
     return true;
 }
 

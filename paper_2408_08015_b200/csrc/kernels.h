@@ -221,8 +221,8 @@ bool ew_takes_pending(int dtype, int c);
 void ew_add(int dtype, const ValSrc& a, const ValSrc& b, const BnPendFwd& pa, const BnPendFwd& pb, int act, size_t pixels, int c, void* out, void* out2,
             cudaStream_t st);
 void ew_apply(int dtype, const ValSrc& a, const BnPendFwd& pa, size_t pixels, int c, void* out, cudaStream_t st);
-// dst = src, and n_zero doubles set to zero; false: not 16-byte aligned, nothing launched
-bool slot_copy(const void* src, void* dst, size_t bytes, double* zero, size_t n_zero, cudaStream_t st);
+// dst = src, and na doubles at a and nb at b set to zero; false: not 16-byte aligned, nothing launched
+bool slot_copy(const void* src, void* dst, size_t bytes, double* a, size_t na, double* b, size_t nb, cudaStream_t st);
 void ew_relu_mask(int dtype, const void* d, const void* out_val, size_t n, void* dst, cudaStream_t st);
 // the same, fused with the BatchNorm-backward sums of the operand branch whose raw conv output is z and whose BatchNorm has no
 // activation: dst's sums are that BatchNorm's; false = channel count not a whole number of vectors, nothing launched

@@ -133,14 +133,14 @@ struct asteroid_stage {
     __nv_bfloat16* wpad = nullptr;                 // [co][Kp] bf16 weights of the im2col units
     float* gpad = nullptr;                         // [co][Kp] padded weight gradient of the im2col unit at hand
     size_t n_wpad = 0, n_gpad = 0;
-    // per-channel sums of the BatchNorms (fin.cuh), forward and backward, and the pivots the forward sums were taken with.  The forward sums
-    // are zeroed by a forward's first kernel, the backward sums by accumulate.  The backward sums also hold the accumulators of the
-    // depthwise weight gradients.
-    double *fsum = nullptr, *bsum = nullptr;
+    // per-channel sums of the BatchNorms' forward (fin.cuh) and the pivots they were taken with.  The backward's lie in the slot, together with the
+    // accumulators of the depthwise weight gradients.  A forward's first kernel zeroes both, so that a backward starts from zero
+    // whatever ran on the stage before its forward: calls that an import dropped, a replay of a captured round.  Accumulate zeroes the
+    // backward's again, for graphs of a caller's own that hold a backward and its accumulate without the forward.
+    double* fsum = nullptr;
     float* pivots = nullptr;
     DwSettle* dw_tab = nullptr;                    // the depthwise units' accumulators and weight gradients
     int n_dw = 0;
-    bool bsum_dirty = false;                       // a backward ran since its sums were zeroed (profile runs skip accumulate)
     int* err = nullptr;                            // device error word (bounded waits)
     // Weight-gradient kernels depend only on the BatchNorm-backward coefficients of their unit and nothing in the rest of
     // the backward pass depends on them: they run on a second stream (forked from and joined back into the caller's
@@ -154,11 +154,13 @@ struct asteroid_stage {
     char* up_mem = nullptr;                        // zero-inserted gradients of the stride-2 3x3 units
     size_t up_bytes = 0;
     char *slot_mem = nullptr, *grad_mem = nullptr;
-    size_t slot_bytes = 0, slot_stat_off = 0, grad_bytes = 0, scratch_floats = 0;
+    size_t slot_bytes = 0, slot_stat_off = 0, slot_bsum_off = 0, grad_bytes = 0, scratch_floats = 0;
     size_t bytes_mod = 0, bytes_opt = 0, bytes_work = 0;
     // round state
     std::vector<int> slot_of_mb, mb_of_slot;
     int pending_g = -1, n_acc = 0;
+    int pending_slot = -1;                         // where that backward's sums lie
+    std::vector<char> sums_left;                   // per slot: its backward failed on the way and may have left sums behind
     Timing tm;
     std::vector<ast::Arena> arenas;                // every device allocation of the stage, with its guard bands
     bool check_guards = false;
@@ -412,7 +414,8 @@ static int build_plan(asteroid_stage* s) {
             u.se_work_off = ncoef;
             ncoef += (size_t)s->B * (3 * (size_t)u.g.ci + u.se_k);
         }
-    s->slot_bytes = align_up(sb + nstat * sizeof(float), 256);
+    s->slot_bsum_off = align_up(sb + nstat * sizeof(float), 256);
+    s->slot_bytes = align_up(s->slot_bsum_off + s->n_bsum * sizeof(double), 256);
     s->grad_bytes = gb;
     s->n_coef = ncoef;
     s->n_run = nrun;
@@ -555,11 +558,12 @@ static ConvGeom col_geom(const Unit& u) {
 struct SlotView {
     char* base;
     float* stats;
+    double* bsum;
 };
 
 static SlotView slot_view(asteroid_stage* s, int slot) {
     char* b = s->slot_mem + (size_t)slot * s->slot_bytes;
-    return SlotView{b, reinterpret_cast<float*>(b + s->slot_stat_off)};
+    return SlotView{b, reinterpret_cast<float*>(b + s->slot_stat_off), reinterpret_cast<double*>(b + s->slot_bsum_off)};
 }
 
 static ValSrc val_src(asteroid_stage* s, const SlotView& sv, int v) {
@@ -596,7 +600,7 @@ static BnPendFwd pend_fwd(asteroid_stage* s, const SlotView& sv, const Unit& u) 
 static BnPendBwd pend_bwd(asteroid_stage* s, const SlotView& sv, const Unit& u) {
     const Val& o = s->vals[u.out];
     const float* stt = sv.stats + o.stat_off;
-    return BnPendBwd{s->bsum + 2 * u.sum_off, s->w + u.gamma_off, stt, stt + o.c, 1.0 / (double)(o.elems / o.c), o.c, bwd_out(s, u)};
+    return BnPendBwd{sv.bsum + 2 * u.sum_off, s->w + u.gamma_off, stt, stt + o.c, 1.0 / (double)(o.elems / o.c), o.c, bwd_out(s, u)};
 }
 static BnSumsOut sums_fwd(asteroid_stage* s, const Unit& u) { return BnSumsOut{s->fsum + 2 * u.sum_off, s->run + u.run_off, s->pivots + u.sum_off}; }
 
@@ -657,11 +661,13 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
     const int dt = s->dtype;
     {
         // the slot's copy of x (backward reads it); a kernel rather than a memcpy node where the alignment allows vector
-        // accesses, so that the chain of programmatic dependent launches is not interrupted.  It also zeroes the channel sums.
+        // accesses, so that the chain of programmatic dependent launches is not interrupted.  It also zeroes the channel sums of
+        // this forward and of its backward.
         const Val& v0 = s->vals[0];
-        if (!slot_copy(x, sv.base + v0.buf_off, v0.elems * s->esz, s->fsum, 2 * s->n_bn_ch, st)) {
+        if (!slot_copy(x, sv.base + v0.buf_off, v0.elems * s->esz, s->fsum, 2 * s->n_bn_ch, sv.bsum, s->n_bsum, st)) {
             CU(cudaMemcpyAsync(sv.base + v0.buf_off, x, v0.elems * s->esz, cudaMemcpyDeviceToDevice, st));
             if (s->n_bn_ch) CU(cudaMemsetAsync(s->fsum, 0, 2 * s->n_bn_ch * sizeof(double), st));
+            if (s->n_bsum) CU(cudaMemsetAsync(sv.bsum, 0, s->n_bsum * sizeof(double), st));
         }
     }
     Pending pend(s, sv, st);
@@ -849,8 +855,6 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
     GatedGrad gated;
     std::vector<char> reduced(s->units.size(), 0);   // BatchNorm-backward sums already taken by the kernel that wrote dy
     Pending pend(s, sv, st);                         // ... and not yet turned into coefficients
-    if (s->bsum_dirty && s->n_bsum) CU(cudaMemsetAsync(s->bsum, 0, s->n_bsum * sizeof(double), st));
-    s->bsum_dirty = true;
     std::fill(s->bwd_sums_by.begin(), s->bwd_sums_by.end(), -1);
     // weight gradients go to the second stream (not while a profile run times the units one by one, nor while a
     // per-launch trace brackets every kernel with events: a kernel's duration is then that of the kernel running alone)
@@ -884,7 +888,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 d.scale = stt + 2 * (size_t)o.c;
                 d.shift = stt + 3 * (size_t)o.c;
                 if (!reduced[ui]) {
-                    bn_bwd_reduce(dt, d.dy, d.z, o.elems / o.c, o.c, d.scale, d.shift, u.act, stt, stt + o.c, s->bsum + 2 * u.sum_off, s->scratch_floats, st);
+                    bn_bwd_reduce(dt, d.dy, d.z, o.elems / o.c, o.c, d.scale, d.shift, u.act, stt, stt + o.c, sv.bsum + 2 * u.sum_off, s->scratch_floats, st);
                     pend.unit[ui] = 1;
                 }
                 d.k1 = kc; d.k2 = kc + o.c; d.k3 = kc + 2 * (size_t)o.c;
@@ -923,7 +927,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 const float* ts = nullptr;
                 if (tgt >= 0) {
                     const Unit& tu = s->units[tgt];
-                    sums = s->bsum + 2 * tu.sum_off;
+                    sums = sv.bsum + 2 * tu.sum_off;
                     ts = sv.stats + s->vals[tu.out].stat_off;
                     pend.unit[tgt] = 1;
                     reduced[tgt] = 1;
@@ -931,8 +935,8 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 }
                 void* to = want_in ? own(u.in) : nullptr;
                 const float* trs = ts ? ts + u.g.ci : nullptr;
-                if (u.g.k == 5) dw5_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, s->bsum + u.acc_off, sums, ts, trs, dw5_choose(dt, true, u.g), st);
-                else dw3_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, s->bsum + u.acc_off, sums, ts, trs, dw3_choose(dt, true, u.g), st);
+                if (u.g.k == 5) dw5_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, sv.bsum + u.acc_off, sums, ts, trs, dw5_choose(dt, true, u.g), st);
+                else dw3_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, sv.bsum + u.acc_off, sums, ts, trs, dw3_choose(dt, true, u.g), st);
                 if (want_in) {
                     gi.state = G_OWNED;
                     gi.ptr = own(u.in);
@@ -991,7 +995,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                         float* ts = sv.stats + tv.stat_off;
                         red = BnRed{sv.base + tv.buf_off, ts + 2 * (size_t)tv.c, ts + 3 * (size_t)tv.c, ts, ts + tv.c, tu.act, nullptr, 0};
                         p.red = &red;
-                        p.so = BnSumsOut{s->bsum + 2 * tu.sum_off, nullptr, nullptr};
+                        p.so = BnSumsOut{sv.bsum + 2 * tu.sum_off, nullptr, nullptr};
                         pend.unit[tgt] = 1;
                         reduced[tgt] = 1;
                         s->bwd_sums_by[tgt] = ui;
@@ -1044,7 +1048,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                     const Val& tv = s->vals[tu.out];
                     float* ts = sv.stats + tv.stat_off;
                     fused = ew_relu_mask_bn_sums(dt, go.ptr, sv.base + o.buf_off, sv.base + tv.buf_off, o.elems / o.c, o.c, ts, ts + tv.c, own(u.out),
-                                                 s->bsum + 2 * tu.sum_off, s->scratch_floats, st);
+                                                 sv.bsum + 2 * tu.sum_off, s->scratch_floats, st);
                     if (fused) {
                         pend.unit[tgt] = 1;
                         reduced[tgt] = 1;
@@ -1091,7 +1095,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 const int tgt = s->vals[u.in].first_cons == ui && bn_reduce_target(s, u.in) == s->vals[u.in].unit ? s->vals[u.in].unit : -1;
                 if (tgt >= 0 && s->units[tgt].act == ACT_NONE) {
                     const Unit& tu = s->units[tgt];
-                    sums = s->bsum + 2 * tu.sum_off;
+                    sums = sv.bsum + 2 * tu.sum_off;
                     ts = sv.stats + s->vals[tu.out].stat_off;
                     pend.unit[tgt] = 1;
                     reduced[tgt] = 1;
@@ -1119,7 +1123,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
     }
     if (s->need_dx && gs[0].state == G_ALIAS)
         CU(cudaMemcpyAsync(dx, gs[0].ptr, s->vals[0].elems * s->esz, cudaMemcpyDeviceToDevice, st));
-    if (s->n_dw_weights) dw_settle(s->bsum, s->dw_tab, s->n_dw, s->n_dw_weights, s->g, st);
+    if (s->n_dw_weights) dw_settle(sv.bsum, s->dw_tab, s->n_dw, s->n_dw_weights, s->g, st);
     if (side_used) {            // join: the call's work is complete, in the caller's stream order, when the second stream's is
         CU(cudaEventRecord(s->ev_join, s->side));
         CU(cudaStreamWaitEvent(st, s->ev_join, 0));
@@ -1131,11 +1135,10 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
 // Runs a forward or backward call; from the third call with the same slot and buffers on as a graph.  A call is 20 to 190 kernels of a few
 // microseconds, and launching them one by one costs the host 2.5 us each: on small maps or micro-batches more than the device needs (a sixth of
 // MobileNetV2 at batch 4: 52 launches, 240 us a micro-batch against 130 us from a graph).  Not while the caller captures (the
-// kernels then belong to the caller's graph), a trace or a profile brackets single launches, or sums of an unaccumulated backward
-// have to be cleared first.  The graphs of the MAX_REPLAYS most recent (slot, buffers) are kept, and go with the stage.
+// kernels then belong to the caller's graph), or a trace or a profile brackets single launches.  The graphs of the MAX_REPLAYS most recent (slot, buffers) are kept, and go with the stage.
 template <typename F> static int run_call(asteroid_stage* s, bool bwd, int slot, const void* a, const void* b, cudaStream_t st, F call) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (tracing() || s->tm.on || (bwd && s->bsum_dirty)) return call(st);
+    if (tracing() || s->tm.on) return call(st);
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
         cudaGetLastError();
         return call(st);
@@ -1174,12 +1177,10 @@ template <typename F> static int run_call(asteroid_stage* s, bool bwd, int slot,
             count_launches((uint64_t)0 - n);       // captured, not launched
         }
         cudaGetLastError();
-        if (bwd) s->bsum_dirty = false;            // as before the capture
     }
     if (!r->exec) return call(st);
     CU(cudaGraphLaunch(r->exec, st));
     count_launches(r->launches);
-    if (bwd) s->bsum_dirty = true;
     return AST_OK;
 }
 
@@ -1225,7 +1226,6 @@ static int create_impl(const ast_layer* net, int n_layers, int first, int last, 
         if ((rc = arena_alloc(s, "padded weight gradient", &s->gpad, s->n_gpad * 4, &work))) return rc;
     }
     if ((rc = arena_alloc(s, "forward channel sums", &s->fsum, s->n_bn_ch * 2 * sizeof(double), &work))) return rc;
-    if ((rc = arena_alloc(s, "backward channel sums", &s->bsum, s->n_bsum * sizeof(double), &work))) return rc;
     if (s->n_dw) {
         std::vector<DwSettle> tab;
         for (const auto& u : s->units)
@@ -1259,6 +1259,7 @@ static int create_impl(const ast_layer* net, int n_layers, int first, int last, 
     if ((rc = reset_bn_running(s))) return rc;
     s->slot_of_mb.assign(M, -1);
     s->mb_of_slot.assign(s->slots, -1);
+    s->sums_left.assign(s->slots, 0);
     s->fwd_stats_blocks.assign(s->units.size(), 0);
     s->bwd_sums_by.assign(s->units.size(), -1);
     return AST_OK;
@@ -1404,8 +1405,11 @@ int asteroid_stage_backward(asteroid_stage* s, int mb, const void* dy, void* dx,
     int slot = s->slot_of_mb[mb];
     if (slot < 0) return fail(AST_ERR_ORDER, "backward of micro-batch %d without a resident forward", mb);
     if (s->pending_g >= 0) return fail(AST_ERR_ORDER, "gradients of micro-batch %d have not been accumulated yet", s->pending_g);
+    if (s->sums_left[slot] && s->n_bsum) CU(cudaMemsetAsync(slot_view(s, slot).bsum, 0, s->n_bsum * sizeof(double), (cudaStream_t)stream));
     int rc = run_call(s, true, slot, dy, dx, (cudaStream_t)stream, [&](cudaStream_t st) { return backward_impl(s, slot, dy, dx, st); });
+    s->sums_left[slot] = rc != AST_OK;
     if (rc) return rc;
+    s->pending_slot = slot;
     s->slot_of_mb[mb] = -1;
     s->mb_of_slot[slot] = -1;
     s->pending_g = mb;
@@ -1416,8 +1420,7 @@ int asteroid_stage_accumulate(asteroid_stage* s, int mb, void* stream) {
     if (!s) return fail(AST_ERR_ARG, "null argument");
     if (s->pending_g != mb) return fail(AST_ERR_ORDER, "accumulate(%d): the last backward was of micro-batch %d", mb, s->pending_g);
     if (s->n_acc >= s->M) return fail(AST_ERR_ORDER, "already accumulated %d micro-batches this round", s->M);
-    accumulate(s->G, s->g, s->n_pad, s->bsum, s->n_bsum, (cudaStream_t)stream);
-    s->bsum_dirty = s->bsum_dirty && s->n_pad == 0;
+    accumulate(s->G, s->g, s->n_pad, slot_view(s, s->pending_slot).bsum, s->n_bsum, (cudaStream_t)stream);
     CU(cudaGetLastError());
     s->pending_g = -1;
     s->n_acc++;

@@ -1132,6 +1132,14 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
     return AST_OK;
 }
 
+// While it lives the calling thread may create streams and graphs although a capture is open elsewhere: one that the caller has begun in the
+// global mode, on another stream of this thread or in another thread, would be invalidated by such a call.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Runs a forward or backward call; from the third call with the same slot and buffers on as a graph.  A call is 20 to 190 kernels of a few
 // microseconds, and launching them one by one costs the host 2.5 us each: on small maps or micro-batches more than the device needs (a sixth of
 // MobileNetV2 at batch 4: 52 launches, 240 us a micro-batch against 130 us from a graph).  Not while the caller captures (the
@@ -1145,6 +1153,7 @@ template <typename F> static int run_call(asteroid_stage* s, bool bwd, int slot,
     }
     if (cs != cudaStreamCaptureStatusNone) return call(st);
     Replay* r = nullptr;
+    RelaxedCapture relaxed;
     for (Replay& q : s->replays)
         if (q.bwd == bwd && q.slot == slot && q.a == a && q.b == b) r = &q;
     if (!r) {

@@ -1,0 +1,63 @@
+"""The same backward gives the same gradients, bit for bit, on every run.  Each kernel that takes channel sums or depthwise weight gradients is
+given an output gradient with two entries of +-2^60 at far-away pixels among entries of about 1: the large ones cancel exactly, and
+a sum that rounded on the way (a double keeps 53 bits) would hold what the order of its additions left of the small ones."""
+import numpy as np
+import pytest
+import torch
+
+import stage_inputs as si
+
+pytestmark = pytest.mark.gpu
+
+B, H, W, RUNS = 16, 32, 32, 24
+L = si.Layer
+
+
+def _net(kind, c):
+    conv, bn = L("conv", c, c, 1, 1, 0, -1, -1), L("bn", c, c, 0, 1, 0, 0, -1)
+    if kind == "own_pass":                                       # the stage's last BatchNorm: a reduction of its own over dy
+        return [conv, bn]
+    if kind == "pointwise":                                      # ... by the pointwise layer behind it
+        return [conv, bn, L("conv", c, c, 1, 1, 0, 1, -1)]
+    if kind == "silu":
+        return [conv, bn, L("silu", c, c, 0, 1, 0, 1, -1)]
+    k = int(kind[-1])
+    return [conv, bn, L("dwconv", c, c, k, 1, (k - 1) // 2, 1, -1)]
+
+
+@pytest.mark.parametrize("bf16", [False, True], ids=["f32", "bf16"])
+@pytest.mark.parametrize("kind", ["own_pass", "pointwise", "depthwise3", "depthwise5", "silu"])
+def test_gradients_do_not_depend_on_the_order_of_additions(kind, bf16):
+    import paper_2408_08015_b200 as P
+    c = 32
+    net = _net(kind, c)
+    last = len(net) - 1
+    n = si.param_count(net, 0, last)
+    dt, tdt = (P.AST_BF16, torch.bfloat16) if bf16 else (P.AST_F32, torch.float32)
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    x = torch.ones(B, H, W, c, device="cuda", dtype=tdt)         # the same everywhere: what is large cancels behind every layer
+    x[:, 0] = torch.randn(B, W, c, generator=gen, device="cuda").to(tdt)
+    dy = torch.randn(B, H, W, c, generator=gen, device="cuda").to(tdt)
+    dy[1, 16, 16] = 2.0 ** 60
+    dy[B - 2, 16, 16] = -2.0 ** 60
+    y, dx = torch.empty_like(x), torch.empty_like(x)
+    hdl = P.asteroid_stage_create(net, 0, last, H, W, B, 1, dtype=dt)
+    try:
+        params = np.ascontiguousarray(si.init_params(net, 0, last, 4), np.float32)
+        first = None
+        for run in range(RUNS):
+            P.asteroid_stage_import_state(hdl, params)
+            sp = torch.cuda.current_stream().cuda_stream
+            P.asteroid_stage_forward(hdl, 0, x.data_ptr(), y.data_ptr(), sp)
+            P.asteroid_stage_backward(hdl, 0, dy.data_ptr(), dx.data_ptr(), sp)
+            g = np.empty(n, np.float32)
+            P.asteroid_stage_export_state(hdl, micro_grad=g)
+            P.asteroid_stage_accumulate(hdl, 0, sp)
+            P.asteroid_stage_step(hdl, 0.0, 0.0, sp)
+            got = (g, dx.float().cpu().numpy())
+            assert np.isfinite(got[0]).all()
+            first = first or got
+            for a, b in zip(first, got):
+                np.testing.assert_array_equal(a, b, err_msg="run %d" % run)
+    finally:
+        P.asteroid_stage_destroy(hdl)

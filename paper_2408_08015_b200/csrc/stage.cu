@@ -11,6 +11,7 @@
 #include "../../include/asteroid.h"
 #include "kernels.h"
 #include "pw_mma.h"
+#include "replay.h"
 
 namespace ast {
 
@@ -99,18 +100,6 @@ struct Timing {
 
 using namespace ast;
 
-// One forward or backward call as a graph: the kernels of a call depend on the slot and on the caller's two buffers only.
-struct Replay {
-    bool bwd;
-    int slot;
-    const void *a, *b;                             // x and y, or dy and dx
-    uint64_t used;                                 // when last asked for
-    int seen;                                      // direct calls so far; -1: cannot be captured
-    uint64_t launches;
-    cudaGraphExec_t exec;
-};
-constexpr size_t MAX_REPLAYS = 64;
-
 struct asteroid_stage {
     std::vector<ast_layer> net;
     int first = 0, last = 0, in_h = 0, in_w = 0, B = 0, M = 0, dtype = 0, slots = 0, need_dx = 1;
@@ -146,7 +135,7 @@ struct asteroid_stage {
     // the backward pass depends on them: they run on a second stream (forked from and joined back into the caller's
     // stream inside each backward call), with their own split-sum scratch, and fill the gaps of the dependent chain.
     std::vector<Replay> replays;
-    uint64_t replay_clock = 0;
+    uint64_t rounds = 0;                           // updates so far
     cudaStream_t cap = nullptr;                    // calls are captured on it
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -1143,7 +1132,8 @@ struct RelaxedCapture {
 // Runs a forward or backward call; from the third call with the same slot and buffers on as a graph.  A call is 20 to 190 kernels of a few
 // microseconds, and launching them one by one costs the host 2.5 us each: on small maps or micro-batches more than the device needs (a sixth of
 // MobileNetV2 at batch 4: 52 launches, 240 us a micro-batch against 130 us from a graph).  Not while the caller captures (the
-// kernels then belong to the caller's graph), or a trace or a profile brackets single launches.  The graphs of the MAX_REPLAYS most recent (slot, buffers) are kept, and go with the stage.
+// kernels then belong to the caller's graph), or a trace or a profile brackets single launches.  replay.h says which calls are kept; their graphs go with the
+// stage.
 template <typename F> static int run_call(asteroid_stage* s, bool bwd, int slot, const void* a, const void* b, cudaStream_t st, F call) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (tracing() || s->tm.on) return call(st);
@@ -1152,24 +1142,11 @@ template <typename F> static int run_call(asteroid_stage* s, bool bwd, int slot,
         return call(st);
     }
     if (cs != cudaStreamCaptureStatusNone) return call(st);
-    Replay* r = nullptr;
     RelaxedCapture relaxed;
-    for (Replay& q : s->replays)
-        if (q.bwd == bwd && q.slot == slot && q.a == a && q.b == b) r = &q;
-    if (!r) {
-        const Replay fresh{bwd, slot, a, b, 0, 0, 0, nullptr};
-        if (s->replays.size() < MAX_REPLAYS) {
-            s->replays.push_back(fresh);
-            r = &s->replays.back();
-        } else {
-            r = &s->replays[0];
-            for (Replay& q : s->replays)
-                if (q.used < r->used) r = &q;
-            if (r->exec) cudaGraphExecDestroy(r->exec);
-            *r = fresh;
-        }
-    }
-    r->used = ++s->replay_clock;
+    cudaGraphExec_t dropped;
+    Replay* r = replay_entry(s->replays, bwd, slot, a, b, s->rounds, &dropped);
+    if (dropped) cudaGraphExecDestroy(dropped);
+    if (!r) return call(st);
     if (!r->exec && r->seen >= 0 && r->seen < 2) ++r->seen;
     else if (!r->exec && r->seen == 2) {
         r->seen = -1;
@@ -1444,6 +1421,7 @@ int asteroid_stage_step(asteroid_stage* s, float lr, float momentum, void* strea
     refresh_weights(s, st);
     CU(cudaGetLastError());
     s->n_acc = 0;
+    ++s->rounds;
     return AST_OK;
 }
 

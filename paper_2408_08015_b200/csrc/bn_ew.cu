@@ -1,7 +1,7 @@
 // BatchNorm statistics / backward reductions, elementwise pieces (residual add, activation
 // masks, materialisation of a stage output), global average pooling, gradient accumulation,
 // the SGD-momentum update and the two loss heads.  All are bandwidth-bound passes over
-// [pixels][channels] tensors; reductions are two-stage and deterministic (no float atomics).
+// [pixels][channels] tensors; reductions give the same bits on every run: partials added in a fixed order, or as exact integers (fin.cuh).
 #include "fin.cuh"
 #include "kernels.h"
 
@@ -168,7 +168,7 @@ struct MaskBwdOp {
 // BatchNorm (a bias gradient), to partial[block_y][acc][c] for the finishing kernel.
 template <typename T, int V, typename OP>
 __global__ void __launch_bounds__(512) chan_reduce_kernel(OP op, size_t pixels, int c, int cw, int rows, size_t pix_per_block,
-                                                          float* __restrict__ partial, double* sums, float* pivot_copy) {
+                                                          float* __restrict__ partial, ChanSums sums, float* pivot_copy) {
     pdl_wait();
     pdl_launch();
     extern __shared__ float red[];
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(512) chan_reduce_kernel(OP op, size_t pixels, 
             if (ch < c) {
                 float s = 0.f;
                 for (int r2 = 0; r2 < rows; ++r2) s += red[r2 * width + e];
-                if (sums) add_sum(sums + (size_t)t * c + ch, s);
+                if (sums) add_sum(sums, (size_t)t * c + ch, s);
                 else partial[((size_t)blockIdx.y * OP::NACC + t) * c + ch] = s;
             }
         }
@@ -256,7 +256,7 @@ ReducePlan plan_reduce(int dtype, size_t pixels, int c, int nacc, size_t scratch
 double esz(int dtype) { return dtype == 0 ? 4.0 : 2.0; }
 
 template <typename OP>
-void launch_reduce(int dtype, const ReducePlan& p, const OP& op, size_t pixels, int c, float* partial, double* sums, float* pivot_copy, int kind, double bytes,
+void launch_reduce(int dtype, const ReducePlan& p, const OP& op, size_t pixels, int c, float* partial, const ChanSums& sums, float* pivot_copy, int kind, double bytes,
                    cudaStream_t st) {
     LaunchScope ls(kind, bytes + 8.0 * c * p.by, 4.0 * pixels * c, st);
     dim3 grid(p.gx, (unsigned)p.by);
@@ -513,11 +513,11 @@ template <typename T> __global__ void gap_bwd_kernel(const T* __restrict__ da, i
 
 // ------------------------------------------------------------------ parameters
 // Also sets the accumulators of the backward pass it follows to zero.
-__global__ void accumulate_kernel(float* __restrict__ G, const float* __restrict__ g, size_t n4, size_t n, double* __restrict__ zero, size_t n_zero) {
+__global__ void accumulate_kernel(float* __restrict__ G, const float* __restrict__ g, size_t n4, size_t n, ChanSums zero, size_t n_zero) {
     pdl_wait();
     pdl_launch();
     size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (size_t k = i; k < n_zero; k += (size_t)gridDim.x * blockDim.x) zero[k] = 0.0;
+    for (size_t k = i; k < n_zero; k += (size_t)gridDim.x * blockDim.x) zero_sum(zero, k);
     if (i < n4) {
         float4 a = reinterpret_cast<float4*>(G)[i];
         float4 b = reinterpret_cast<const float4*>(g)[i];
@@ -781,7 +781,7 @@ void bn_stats_finish_partials(const float* partial, int blocks, size_t pixels, i
 }
 
 void bn_bwd_reduce(int dtype, const void* dy, const void* z, size_t pixels, int c, const float* scale, const float* shift, int act,
-                   const float* mean, const float* rstd, double* sums, size_t scratch_floats, cudaStream_t st) {
+                   const float* mean, const float* rstd, const ChanSums& sums, size_t scratch_floats, cudaStream_t st) {
     ReducePlan p = plan_reduce(dtype, pixels, c, 2, scratch_floats);
     BwdOp op{GradSrc{dy, z, scale, shift, nullptr, nullptr, nullptr, act}, mean, rstd, act == ACT_NONE ? -INFINITY : 0.f,
              act == ACT_RELU6 ? 6.f : INFINITY};
@@ -791,14 +791,14 @@ void bn_bwd_reduce(int dtype, const void* dy, const void* z, size_t pixels, int 
 void bias_grad(int dtype, const void* dy, const void* z, size_t pixels, int c, int act, float* scratch, size_t scratch_floats, float* db, cudaStream_t st) {
     ReducePlan p = plan_reduce(dtype, pixels, c, 2, scratch_floats);
     BwdOp op{GradSrc{dy, z, nullptr, nullptr, nullptr, nullptr, nullptr, act}, nullptr, nullptr, act == ACT_NONE ? -INFINITY : 0.f, act == ACT_RELU6 ? 6.f : INFINITY};
-    launch_reduce(dtype, p, op, pixels, c, scratch, nullptr, nullptr, K_BN_BWD_REDUCE, (double)pixels * c * esz(dtype) * (act != ACT_NONE ? 2.0 : 1.0), st);
+    launch_reduce(dtype, p, op, pixels, c, scratch, ChanSums{}, nullptr, K_BN_BWD_REDUCE, (double)pixels * c * esz(dtype) * (act != ACT_NONE ? 2.0 : 1.0), st);
     LaunchScope ls(K_BN_BWD_FINISH, 8.0 * c * (p.by + 4), 10.0 * c, st);
     launch_pdl(bn_bwd_finish, (c + 31) / 32, 1024, 0, st, scratch, (int)p.by, c, (double)pixels, (const float*)nullptr, (const float*)nullptr,
                (const float*)nullptr, BnBwdOut{nullptr, db, nullptr, nullptr, nullptr});
 }
 
 bool ew_relu_mask_bn_sums(int dtype, const void* d, const void* out_val, const void* z, size_t pixels, int c, const float* mean, const float* rstd,
-                          void* dst, double* sums, size_t scratch_floats, cudaStream_t st) {
+                          void* dst, const ChanSums& sums, size_t scratch_floats, cudaStream_t st) {
     if (c % (dtype == 0 ? 4 : 8)) return false;          // whole vectors per thread (the op stores what it loads)
     ReducePlan p = plan_reduce(dtype, pixels, c, 2, scratch_floats);
     MaskBwdOp op{d, out_val, z, dst, mean, rstd};
@@ -959,14 +959,13 @@ void ew_apply(int dtype, const ValSrc& a, const BnPendFwd& pa, size_t pixels, in
     ew_add(dtype, a, none, pa, BnPendFwd{}, ACT_NONE, pixels, c, out, nullptr, st);
 }
 
-// dst = src (16-byte units), and na doubles at a and nb at b set to zero by the same launch
-__global__ void __launch_bounds__(256) slot_copy_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t n, double* __restrict__ a, size_t na,
-                                                        double* __restrict__ b, size_t nb) {
+// dst = src (16-byte units), and the na sums of a and nb of b set to zero by the same launch
+__global__ void __launch_bounds__(256) slot_copy_kernel(const uint4* __restrict__ src, uint4* __restrict__ dst, size_t n, ChanSums a, size_t na, ChanSums b, size_t nb) {
     pdl_wait();
     pdl_launch();
     const size_t stride = (size_t)gridDim.x * 256, id = (size_t)blockIdx.x * 256 + threadIdx.x;
-    for (size_t i = id; i < na; i += stride) a[i] = 0.0;
-    for (size_t i = id; i < nb; i += stride) b[i] = 0.0;
+    for (size_t i = id; i < na; i += stride) zero_sum(a, i);
+    for (size_t i = id; i < nb; i += stride) zero_sum(b, i);
     for (size_t i = id; i < n; i += 4 * stride) {
         uint4 v[4];
 #pragma unroll
@@ -977,7 +976,7 @@ __global__ void __launch_bounds__(256) slot_copy_kernel(const uint4* __restrict_
             if (i + u * stride < n) dst[i + u * stride] = v[u];
     }
 }
-bool slot_copy(const void* src, void* dst, size_t bytes, double* a, size_t na, double* b, size_t nb, cudaStream_t st) {
+bool slot_copy(const void* src, void* dst, size_t bytes, const ChanSums& a, size_t na, const ChanSums& b, size_t nb, cudaStream_t st) {
     if (bytes % 16 || (reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) % 16) return false;
     LaunchScope ls(K_EW_ADD, 2.0 * bytes, 0.0, st);
     size_t blocks = (std::max(bytes / 16, na + nb) + 1023) / 1024;
@@ -1041,7 +1040,7 @@ void gap_bwd(int dtype, const void* da, int n, int hw, int c, const void* addend
     else launch_pdl(gap_bwd_kernel<__nv_bfloat16>, blocks, 256, 0, st, (const __nv_bfloat16*)da, n, hw, c, (const __nv_bfloat16*)addend, (__nv_bfloat16*)dx);
 }
 
-void accumulate(float* G, const float* g, size_t n, double* zero, size_t n_zero, cudaStream_t st) {
+void accumulate(float* G, const float* g, size_t n, const ChanSums& zero, size_t n_zero, cudaStream_t st) {
     if (!n) return;
     size_t n4 = n / 4, threads = n4 + (n - n4 * 4);
     LaunchScope ls(K_ACCUMULATE, 12.0 * n, (double)n, st);

@@ -5,6 +5,8 @@
 // had to be re-read from shared memory for every row, 72 of the 116 shared-memory/L1 wavefronts a row of the backward took.  A warp's vector
 // is then 128 (bf16) or 256 (float) consecutive bytes, still whole sectors.
 #pragma once
+#include <algorithm>
+
 #include "fin.cuh"
 
 namespace ast {
@@ -78,7 +80,7 @@ __device__ __forceinline__ void stage_grad(const GradSrc& g, const BnPendBwd& p,
 
 // Sum over the block's threads that own the same channels (tid % lanes), in thread order, of N values of V (float: one channel a lane, float2:
 // two) per thread; channel c's sum k goes to acc[k * c_total + c0 + c].  red: N * blockDim.x V.
-template <int N, typename V> __device__ __forceinline__ void block_sums(const V* v, int lanes, int rows, int c0, int c, double* acc, float* red) {
+template <int N, typename V> __device__ __forceinline__ void block_sums(const V* v, int lanes, int rows, int c0, int c, const ChanSums& acc, float* red) {
     constexpr int CH = sizeof(V) / 4;
     const int width = CH * lanes, pitch = CH * lanes * rows;
     __syncthreads();
@@ -91,7 +93,7 @@ template <int N, typename V> __device__ __forceinline__ void block_sums(const V*
         if (c0 + j < c) {
             float s = 0.f;
             for (int r = 0; r < rows; ++r) s += red[k * pitch + r * width + j];
-            add_sum(acc + (size_t)k * c + c0 + j, s);
+            add_sum(acc, (size_t)k * c + c0 + j, s);
         }
     }
 }
@@ -128,8 +130,8 @@ struct DwBwdArgs {
     const float* wkc;           // tap-major weights
     const void* addend;
     void* dx;                    // may be null: weight gradient only
-    double* gw;                  // [taps][c] accumulators of the weight gradient
-    double* sums;                // [2][c] of the unit that produced x, or null
+    ChanSums gw;                 // [taps][c] accumulators of the weight gradient
+    ChanSums sums;               // [2][c] of the unit that produced x, or none
     const float *mean, *rstd;    // of that unit
     bool first;
 };
@@ -142,8 +144,10 @@ inline void cut_channels(DwGeom& d, int per = 2) {
     d.lanes = (cv + parts - 1) / parts;
     d.rows = BT / d.lanes;
 }
-inline dim3 cut_grid(const DwGeom& d, int ctas, int per = 2) {
-    const int gy = (d.c / per + d.lanes - 1) / d.lanes, gx = (d.items + d.rows - 1) / d.rows, cap = (int)((long long)sm_count() * ctas / gy);
+// launches: how many of them share the layer's images, and with them the room its sums have
+inline dim3 cut_grid(const DwGeom& d, int ctas, int launches, int per = 2) {
+    const int gy = (d.c / per + d.lanes - 1) / d.lanes, gx = (d.items + d.rows - 1) / d.rows;
+    const int cap = (int)std::min((long long)sm_count() * ctas / gy, (long long)MAX_SUM_BLOCKS / launches);
     return dim3(gx < cap ? gx : cap > 0 ? cap : 1, gy);
 }
 // images per launch: byte offsets within a launch are 32-bit

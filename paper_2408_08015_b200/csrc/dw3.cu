@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(BT) dw3_fwd_kernel(const DwFwdArgs a) {
     __syncthreads();
     const float2 sc = ld2(sm + 2 * jl), sh = ld2(sm + width + 2 * jl);
     float2 piv = zero2();
-    const bool stats = a.so.sums != nullptr;
+    const bool stats = (bool)a.so.sums;
     if (stats && live) {
         piv = ld2(a.so.pivot + c0);
         if (blockIdx.x == 0 && row == 0) *reinterpret_cast<float2*>(a.so.pivot_copy + c0) = piv;
@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s2_kernel(const DwBwdArgs a) {
 }
 
 // (also of dw5.cu) gw[c][t] = acc[t][c] for the weight gradients of several layers at once
-__global__ void __launch_bounds__(256) dw_settle_kernel(const double* __restrict__ acc, const DwSettle* __restrict__ tab, int layers, float* __restrict__ g) {
+__global__ void __launch_bounds__(256) dw_settle_kernel(const ChanSums acc, const DwSettle* __restrict__ tab, int layers, float* __restrict__ g) {
     pdl_wait();
     pdl_launch();
     int i = blockIdx.x * 256 + threadIdx.x;
@@ -490,7 +490,9 @@ __global__ void __launch_bounds__(256) dw_settle_kernel(const double* __restrict
         const int n = e.taps * e.c;
         if (i < n) {
             const int c = i / e.taps, t = i - e.taps * c;
-            g[e.g_off + i] = (float)acc[e.acc_off + (size_t)t * e.c + c];
+            const int at = (int)(e.acc_off + (size_t)t * e.c + c);
+            const longlong2 n = acc.near[at];
+            g[e.g_off + i] = (float)(n.x & 1 ? full_totals(acc.near, acc.far, acc.shift, at, at).x : near_total(n, acc.shift));
             return;
         }
         i -= n;
@@ -509,7 +511,7 @@ void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf,
     else f = g.stride == 2 ? DW3_FWD(B, 2, 2) : DW3_FWD(B, 1, 4);
 #undef DW3_FWD
     const double in_e = (double)g.hi * g.wi * g.ci, out_e = (double)g.ho * g.wo * g.ci;
-    const int chunk = image_chunk(dtype, g);
+    const int chunk = image_chunk(dtype, g), launches = (g.n + chunk - 1) / chunk;
     for (int n0 = 0; n0 < g.n; n0 += chunk) {
         const int n = g.n - n0 < chunk ? g.n - n0 : chunk;
         DwFwdArgs a{};
@@ -521,12 +523,12 @@ void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf,
         d.items = n * d.nrc * d.sw;
         cut_channels(d);
         LaunchScope ls(K_DW_FWD, n * (in_e + out_e) * esz(dtype) + 36.0 * g.ci, 18.0 * n * out_e, st);
-        launch_pdl(f, cut_grid(d, t.ctas), BT, (size_t)BT * 2 * 2 * 4, st, a);
+        launch_pdl(f, cut_grid(d, t.ctas, launches), BT, (size_t)BT * 2 * 2 * 4, st, a);
     }
 }
 
-void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* wkc, const void* addend, void* dx, double* gw,
-             double* sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st) {
+void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* wkc, const void* addend, void* dx, const ChanSums& gw,
+             const ChanSums& sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st) {
     typedef void (*Fn)(const DwBwdArgs);
     using B = __nv_bfloat16;
     const bool xf = grad_needs_z(dz) || pb.sums;
@@ -538,12 +540,12 @@ void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& p
 #undef DW3_BWD
     const int rows_out = g.stride == 1 ? g.hi : g.ho, cols_out = g.stride == 1 ? g.wi : g.wo;
     const double in_e = (double)g.hi * g.wi * g.ci, out_e = (double)g.ho * g.wo * g.ci;
-    const int chunk = image_chunk(dtype, g);
+    const int chunk = image_chunk(dtype, g), launches = (g.n + chunk - 1) / chunk;
     for (int n0 = 0; n0 < g.n; n0 += chunk) {
         const int n = g.n - n0 < chunk ? g.n - n0 : chunk;
         const size_t ie = (size_t)n0 * g.hi * g.wi * g.ci, oe = (size_t)n0 * g.ho * g.wo * g.ci;
         DwBwdArgs a{};
-        a.dz = dz; a.pb = pb; a.x = x; a.wkc = wkc; a.gw = gw; a.sums = dx ? sums : nullptr; a.mean = mean; a.rstd = rstd; a.first = n0 == 0;
+        a.dz = dz; a.pb = pb; a.x = x; a.wkc = wkc; a.gw = gw; a.sums = dx ? sums : ChanSums{}; a.mean = mean; a.rstd = rstd; a.first = n0 == 0;
         a.dz.dy = at(dz.dy, oe, dtype);
         a.dz.z = at(dz.z, oe, dtype);
         a.x.p = at(x.p, ie, dtype);
@@ -554,12 +556,12 @@ void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& p
         d.items = n * d.nrc * d.sw;
         cut_channels(d);
         LaunchScope ls(K_DW_BWD_FUSED, n * (out_e * (xf ? 2.0 : 1.0) + in_e * (dx ? (addend ? 3.0 : 2.0) : 1.0)) * esz(dtype) + 36.0 * g.ci, 36.0 * n * out_e, st);
-        launch_pdl(f, cut_grid(d, t.ctas), BT, (size_t)BT * 2 * 9 * 4, st, a);
+        launch_pdl(f, cut_grid(d, t.ctas, launches), BT, (size_t)BT * 2 * 9 * 4, st, a);
     }
 }
 
-void dw_settle(const double* acc, const DwSettle* tab, int layers, size_t total, float* g, cudaStream_t st) {
-    LaunchScope ls(K_DW_BWD_WEIGHT_FINISH, 12.0 * total, 0.0, st);
+void dw_settle(const ChanSums& acc, const DwSettle* tab, int layers, size_t total, float* g, cudaStream_t st) {
+    LaunchScope ls(K_DW_BWD_WEIGHT_FINISH, 20.0 * total, 0.0, st);
     launch_pdl(dw_settle_kernel, (unsigned)((total + 255) / 256), 256, 0, st, acc, tab, layers, g);
 }
 

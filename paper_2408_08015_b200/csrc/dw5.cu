@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(BT) dw5_fwd_kernel(const DwFwdArgs a) {
     __syncthreads();
     const float2 sc = ld2(sm + 2 * jl), sh = ld2(sm + width + 2 * jl);
     float2 piv = zero2();
-    const bool stats = a.so.sums != nullptr;
+    const bool stats = (bool)a.so.sums;
     if (stats && live) {
         piv = ld2(a.so.pivot + c0);
         if (blockIdx.x == 0 && row == 0) *reinterpret_cast<float2*>(a.so.pivot_copy + c0) = piv;
@@ -496,7 +496,7 @@ void dw5_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf,
     else f = g.stride == 2 ? DW5_FWD(B, 2, 2) : t.tw == 4 ? DW5_FWD(B, 1, 4) : DW5_FWD(B, 1, 2);
 #undef DW5_FWD
     const double in_e = (double)g.hi * g.wi * g.ci, out_e = (double)g.ho * g.wo * g.ci;
-    const int chunk = image_chunk(dtype, g);
+    const int chunk = image_chunk(dtype, g), launches = (g.n + chunk - 1) / chunk;
     for (int n0 = 0; n0 < g.n; n0 += chunk) {
         const int n = g.n - n0 < chunk ? g.n - n0 : chunk;
         DwFwdArgs a{};
@@ -508,12 +508,12 @@ void dw5_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf,
         d.items = n * d.nrc * d.sw;
         cut_channels(d);
         LaunchScope ls(K_DW_FWD, n * (in_e + out_e) * esz(dtype) + 100.0 * g.ci, 50.0 * n * out_e, st);
-        launch_pdl(f, cut_grid(d, t.ctas), BT, (size_t)BT * 2 * 2 * 4, st, a);
+        launch_pdl(f, cut_grid(d, t.ctas, launches), BT, (size_t)BT * 2 * 2 * 4, st, a);
     }
 }
 
-void dw5_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* wkc, const void* addend, void* dx, double* gw,
-             double* sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st) {
+void dw5_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* wkc, const void* addend, void* dx, const ChanSums& gw,
+             const ChanSums& sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st) {
     typedef void (*Fn)(const DwBwdArgs);
     using B = __nv_bfloat16;
     const int xf = dz.act != ACT_NONE ? Z_ACT : (grad_needs_z(dz) || pb.sums) ? Z_AFFINE : Z_PLAIN;
@@ -528,12 +528,12 @@ void dw5_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& p
 #undef DW5_X
     const int rows_out = g.stride == 1 ? g.hi : g.ho, cols_out = g.stride == 1 ? g.wi : g.wo;
     const double in_e = (double)g.hi * g.wi * g.ci, out_e = (double)g.ho * g.wo * g.ci;
-    const int chunk = image_chunk(dtype, g);
+    const int chunk = image_chunk(dtype, g), launches = (g.n + chunk - 1) / chunk;
     for (int n0 = 0; n0 < g.n; n0 += chunk) {
         const int n = g.n - n0 < chunk ? g.n - n0 : chunk;
         const size_t ie = (size_t)n0 * g.hi * g.wi * g.ci, oe = (size_t)n0 * g.ho * g.wo * g.ci;
         DwBwdArgs a{};
-        a.dz = dz; a.pb = pb; a.x = x; a.wkc = wkc; a.gw = gw; a.sums = dx ? sums : nullptr; a.mean = mean; a.rstd = rstd; a.first = n0 == 0;
+        a.dz = dz; a.pb = pb; a.x = x; a.wkc = wkc; a.gw = gw; a.sums = dx ? sums : ChanSums{}; a.mean = mean; a.rstd = rstd; a.first = n0 == 0;
         a.dz.dy = at(dz.dy, oe, dtype);
         a.dz.z = at(dz.z, oe, dtype);
         a.x.p = at(x.p, ie, dtype);
@@ -544,7 +544,7 @@ void dw5_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& p
         d.items = n * d.nrc * d.sw;
         cut_channels(d, 1);
         LaunchScope ls(K_DW_BWD_FUSED, n * (out_e * (xf ? 2.0 : 1.0) + in_e * (dx ? (addend ? 3.0 : 2.0) : 1.0)) * esz(dtype) + 100.0 * g.ci, 100.0 * n * out_e, st);
-        launch_pdl(f, cut_grid(d, t.ctas, 1), BT, (size_t)BT * 25 * 4, st, a);
+        launch_pdl(f, cut_grid(d, t.ctas, launches, 1), BT, (size_t)BT * 25 * 4, st, a);
     }
 }
 

@@ -72,6 +72,26 @@ bool tracing();
 // records `msg` as the calling thread's last error and returns `code`
 int report_error(int code, const char* msg);
 
+// Accumulators of per-channel sums: integers (fin.cuh).  A sum has two words that partial sums of ordinary size are added to, and, for the
+// others, words that cover every float; chan_sums_bytes(n) bytes hold n sums, zero before the first addition.
+struct FarSum {
+    long long word[10];
+};
+struct ChanSums {
+    longlong2* near;         // null: no sums
+    FarSum* far;
+    int shift;               // exponent field 1 lies this many places into the first word
+    __host__ __device__ explicit operator bool() const { return near != nullptr; }
+    __host__ __device__ ChanSums operator+(size_t i) const { return ChanSums{near + i, far + i, shift}; }
+};
+constexpr int MAX_SUM_BLOCKS = 4096;         // partial sums of a channel that the words have room for, whatever they are
+inline size_t chan_sums_bytes(size_t n) { return n * (sizeof(longlong2) + sizeof(FarSum)); }
+// ordinary: forward sums 2^-24 to 2^28, backward sums 2^-46 to 2^6
+inline ChanSums chan_sums(void* mem, size_t n, bool bwd) {
+    longlong2* p = static_cast<longlong2*>(mem);
+    return ChanSums{p, reinterpret_cast<FarSum*>(p + n), bwd ? 24 : 2};
+}
+
 struct BnFwdOut {
     float *mean, *rstd, *scale, *shift, *run_mean, *run_var;
 };
@@ -79,9 +99,9 @@ struct BnBwdOut {
     float *dgamma, *dbeta, *k1, *k2, *k3;   // dgamma/k* null: only dbeta = sum of dpre (bias gradient)
 };
 // A BatchNorm whose sums have been taken and whose coefficients the next kernel that reads its tensor forms (fin.cuh).
-// sums: [2][c] doubles; sums == nullptr: nothing is pending, the coefficients are in memory.
+// sums: [2][c] accumulators; none: nothing is pending, the coefficients are in memory.
 struct BnPendFwd {
-    const double* sums;
+    ChanSums sums;
     const float* pivot;      // what the producer subtracted (its copy: the running mean is updated by the reader)
     const float *gamma, *beta;
     double inv_count, unbias;
@@ -90,7 +110,7 @@ struct BnPendFwd {
     BnFwdOut o;
 };
 struct BnPendBwd {
-    const double* sums;
+    ChanSums sums;
     const float *gamma, *mean, *rstd;
     double inv_count;
     int c;
@@ -99,7 +119,7 @@ struct BnPendBwd {
 // Where a kernel leaves the sums of the tensor it writes: accumulators [2][c] (zero at its start), forward the pivot it
 // subtracts (the running mean) and the place of its copy.
 struct BnSumsOut {
-    double* sums;
+    ChanSums sums;
     const float* pivot;
     float* pivot_copy;
 };
@@ -186,15 +206,15 @@ struct DwSettle {
 DwTiling dw3_choose(int dtype, bool bwd, const ConvGeom& g);
 void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf, const float* w9c, void* z, const BnSumsOut& so, const DwTiling& t, cudaStream_t st);
 // dx may be null (weight gradient only); gw: [9][c] accumulators; sums [2][c] (may be null), mean, rstd: of the unit that produced x
-void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* w9c, const void* addend, void* dx, double* gw,
-             double* sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st);
+void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* w9c, const void* addend, void* dx, const ChanSums& gw,
+             const ChanSums& sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st);
 // the same for 5x5 layers (dw5.cu)
 DwTiling dw5_choose(int dtype, bool bwd, const ConvGeom& g);
 void dw5_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf, const float* wkc, void* z, const BnSumsOut& so, const DwTiling& t, cudaStream_t st);
-void dw5_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* wkc, const void* addend, void* dx, double* gw,
-             double* sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st);
+void dw5_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* wkc, const void* addend, void* dx, const ChanSums& gw,
+             const ChanSums& sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st);
 // accumulators -> weight gradients, all layers of the table (device memory); total: sum of taps*c
-void dw_settle(const double* acc, const DwSettle* tab, int layers, size_t total, float* g, cudaStream_t st);
+void dw_settle(const ChanSums& acc, const DwSettle* tab, int layers, size_t total, float* g, cudaStream_t st);
 
 // ---- BatchNorm statistics and backward reductions over a [pixels][c] tensor ----
 // sums of a [pixels][c] tensor of its own pass; the coefficients are then pending (fin.cuh)
@@ -204,7 +224,7 @@ void bn_stats(int dtype, const void* z, size_t pixels, int c, const BnSumsOut& s
 void bn_stats_finish_partials(const float* partial, int blocks, size_t pixels, int c, const float* gamma, const float* beta, float eps,
                               float momentum, const BnFwdOut& o, cudaStream_t st);
 void bn_bwd_reduce(int dtype, const void* dy, const void* z, size_t pixels, int c, const float* scale, const float* shift, int act,
-                   const float* mean, const float* rstd, double* sums, size_t scratch_floats, cudaStream_t st);
+                   const float* mean, const float* rstd, const ChanSums& sums, size_t scratch_floats, cudaStream_t st);
 // db[c] = sum over the pixels of dy inside the activation's linear region
 void bias_grad(int dtype, const void* dy, const void* z, size_t pixels, int c, int act, float* scratch, size_t scratch_floats, float* db, cudaStream_t st);
 // pending coefficients formed by a kernel of their own
@@ -221,13 +241,13 @@ bool ew_takes_pending(int dtype, int c);
 void ew_add(int dtype, const ValSrc& a, const ValSrc& b, const BnPendFwd& pa, const BnPendFwd& pb, int act, size_t pixels, int c, void* out, void* out2,
             cudaStream_t st);
 void ew_apply(int dtype, const ValSrc& a, const BnPendFwd& pa, size_t pixels, int c, void* out, cudaStream_t st);
-// dst = src, and na doubles at a and nb at b set to zero; false: not 16-byte aligned, nothing launched
-bool slot_copy(const void* src, void* dst, size_t bytes, double* a, size_t na, double* b, size_t nb, cudaStream_t st);
+// dst = src, and the na sums of a and nb of b set to zero; false: src or dst not 16-byte aligned, nothing launched
+bool slot_copy(const void* src, void* dst, size_t bytes, const ChanSums& a, size_t na, const ChanSums& b, size_t nb, cudaStream_t st);
 void ew_relu_mask(int dtype, const void* d, const void* out_val, size_t n, void* dst, cudaStream_t st);
 // the same, fused with the BatchNorm-backward sums of the operand branch whose raw conv output is z and whose BatchNorm has no
 // activation: dst's sums are that BatchNorm's; false = channel count not a whole number of vectors, nothing launched
 bool ew_relu_mask_bn_sums(int dtype, const void* d, const void* out_val, const void* z, size_t pixels, int c, const float* mean, const float* rstd,
-                          void* dst, double* sums, size_t scratch_floats, cudaStream_t st);
+                          void* dst, const ChanSums& sums, size_t scratch_floats, cudaStream_t st);
 void ew_sum(int dtype, const void* a, const void* b, size_t n, void* dst, cudaStream_t st);
 // bfloat16, channel counts multiples of 8: zero-inserted gradient / subsampled output of a stride-2 3x3 conv (see conv3_s2_tc_supported)
 void ew_upsample2_grad(const GradSrc& d, int n, int hi, int wi, int ho, int wo, int c, void* up, cudaStream_t st);
@@ -243,7 +263,7 @@ void gap_bwd(int dtype, const void* da, int n, int hw, int c, const void* addend
 int silu_fwd(int dtype, const ValSrc& x, const BnPendFwd& pf, int n, int hw, int c, void* out, void* out2, float* part, size_t part_floats, cudaStream_t st);
 // gate, ds (may be null): dy is the gradient behind a squeeze-excite layer whose own share is dy*gate + ds; sums (may be null), mean, rstd: of the
 // unit that produced x, which has no activation
-void silu_bwd(int dtype, const void* dy, const float* gate, const float* ds, const ValSrc& x, const void* addend, int n, int hw, int c, void* dx, double* sums,
+void silu_bwd(int dtype, const void* dy, const float* gate, const float* ds, const ValSrc& x, const void* addend, int n, int hw, int c, void* dx, const ChanSums& sums,
               const float* mean, const float* rstd, cudaStream_t st);
 // squeeze-excite over [n][hw][c] with k hidden units; s [n][c], p1 [n][k], gate [n][c] are float vectors kept for the backward pass;
 // scratch: partials of the pixel-split reductions (any size >= n*c floats; more allows more splits); splits > 0: that many are there already
@@ -263,8 +283,8 @@ void dwk_bwd_data(int dtype, const ConvGeom& g, const GradSrc& dz, const float* 
 void dwk_bwd_weight(int dtype, const ConvGeom& g, const GradSrc& dz, const ValSrc& x, float* scratch, size_t scratch_floats, float* gw, cudaStream_t st);
 
 // ---- parameters ----
-// G += g; n_zero doubles set to zero
-void accumulate(float* G, const float* g, size_t n, double* zero, size_t n_zero, cudaStream_t st);
+// G += g; n_zero sums set to zero
+void accumulate(float* G, const float* g, size_t n, const ChanSums& zero, size_t n_zero, cudaStream_t st);
 void sgd_step(float* w, float* v, float* G, size_t n, float inv_m, float lr, float mu, cudaStream_t st);
 // a dense layer's weights [co][taps][ci] at `off`, derived as [ci][taps][co] at the same place; tile0: its first tile
 struct RefreshSeg {

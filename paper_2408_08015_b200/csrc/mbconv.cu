@@ -211,7 +211,7 @@ struct SiluBwdArgs {
     ValSrc x;
     const void *dy, *addend;
     const float *gate, *ds;    // [sample][c]
-    double* sums;
+    ChanSums sums;
     const float *mean, *rstd;
     int hw, c;
     void* dx;
@@ -268,8 +268,8 @@ template <typename T, int V, bool GATE, bool SUMS> __global__ void __launch_boun
             }
         }
     if (!SUMS) return;
-    rows_sum<V>(k, ix, a.c, s1, sm, [&](int ch, float v) { add_sum(a.sums + ch, v); });
-    rows_sum<V>(k, ix, a.c, s2, sm, [&](int ch, float v) { add_sum(a.sums + a.c + ch, v * a.rstd[ch]); });
+    rows_sum<V>(k, ix, a.c, s1, sm, [&](int ch, float v) { add_sum(a.sums, ch, v); });
+    rows_sum<V>(k, ix, a.c, s2, sm, [&](int ch, float v) { add_sum(a.sums, (size_t)a.c + ch, v * a.rstd[ch]); });
 }
 
 // ------------------------------------------------------------------------------------------ squeeze-excite
@@ -814,7 +814,7 @@ int silu_fwd(int dtype, const ValSrc& x, const BnPendFwd& pf, int n, int hw, int
     return part ? splits : 0;
 }
 
-void silu_bwd(int dtype, const void* dy, const float* gate, const float* ds, const ValSrc& x, const void* addend, int n, int hw, int c, void* dx, double* sums,
+void silu_bwd(int dtype, const void* dy, const float* gate, const float* ds, const ValSrc& x, const void* addend, int n, int hw, int c, void* dx, const ChanSums& sums,
               const float* mean, const float* rstd, cudaStream_t st) {
     const double e = (double)n * hw * c;
     LaunchScope ls(K_SILU, e * esz_(dtype) * (3 + (addend ? 1 : 0)), 8.0 * e, st);

@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
                 sK[Kp + c] = k.y;
             }
         }
-    const bool sums = a.so.sums != nullptr;
+    const bool sums = (bool)a.so.sums;
     if (sums)
         for (int c = tid; c < BN; c += NT) {
             const bool ok = n0 + c < a.N;
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
         if (n0 + cl >= a.N) continue;
         float x = 0.f;
         for (int m = 0; m < WM; ++m) x += sR[(m * 2 + s) * BN + cl];
-        add_sum(a.so.sums + (size_t)s * a.N + n0 + cl, x);
+        add_sum(a.so.sums, (size_t)s * a.N + n0 + cl, x);
     }
 }
 

@@ -18,6 +18,8 @@
 // The column sums the BatchNorms need are taken from the registers the output is stored from; the coefficients of a
 // BatchNorm in front are formed in the prologue (fin.cuh).
 #pragma once
+#include <type_traits>
+
 #include "fin.cuh"
 
 namespace ast {
@@ -158,12 +160,25 @@ template <int G> __device__ __forceinline__ void stage_weights(const Args& a, ui
 template <bool BWD, int XF> __device__ __forceinline__ void stage_coefs(const Args& a, float* sK, float* sN, int n0, int BN) {
     const int Kp = a.KCH * 32;
     const bool first = blockIdx.x == 0 && blockIdx.y == 0;
-    if (XF != XF_NONE)
-        for (int c = threadIdx.x; c < Kp; c += blockDim.x) {
+    if (XF != XF_NONE) {
+        const int nt = blockDim.x;
+        typename std::conditional<BWD, BnBwdIn, BnFwdIn>::type in, next;         // the sums of the thread's next channel are under way
+        int c = threadIdx.x;
+        const auto request = [&](int ch, auto& to) {
+            if constexpr (BWD) {
+                if (ch < a.K && a.pb.sums) to.load(a.pb, ch);
+            } else {
+                if (ch < a.K && a.pf.sums) to.load(a.pf, ch);
+            }
+        };
+        request(c, in);
+#pragma unroll 1
+        for (; c < Kp; c += nt) {
             const bool ok = c < a.K;
-            if (BWD) {
+            request(c + nt, next);
+            if constexpr (BWD) {
                 float3 k = make_float3(1.f, 0.f, 0.f);
-                if (ok && a.pb.sums) k = bn_bwd_coef(a.pb, c, first);
+                if (ok && a.pb.sums) k = in.coef(a.pb, c, first);
                 else if (ok && a.c0) k = make_float3(a.c0[c], a.c1[c], a.c2[c]);
                 sK[c] = k.x;
                 sK[Kp + c] = k.y;
@@ -174,7 +189,7 @@ template <bool BWD, int XF> __device__ __forceinline__ void stage_coefs(const Ar
                 }
             } else {
                 float2 k = make_float2(1.f, 0.f);
-                if (ok && a.pf.sums) k = bn_fwd_coef(a.pf, c, first);
+                if (ok && a.pf.sums) k = in.coef(a.pf, c, first);
                 else if (ok && a.c0) k = make_float2(a.c0[c], a.c1[c]);
                 sK[c] = k.x;
                 if (XF == XF_ADD) {
@@ -186,7 +201,9 @@ template <bool BWD, int XF> __device__ __forceinline__ void stage_coefs(const Ar
                 }
                 sK[Kp + c] = k.y;
             }
+            in = next;
         }
+    }
     if (a.so.sums)
         for (int c = threadIdx.x; c < BN; c += blockDim.x) {
             const bool ok = n0 + c < a.N;
@@ -298,7 +315,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
 
     const float rlo = a.r_act == ACT_NONE ? -INFINITY : 0.f, rhi = a.r_act == ACT_RELU6 ? 6.f : INFINITY;
     const uint8_t* wb = sW + (uint32_t)(wn * NJ * 8 + g) * a.wpitch + t * 16;
-    const bool sums = a.so.sums != nullptr;
+    const bool sums = (bool)a.so.sums;
     float2 s1[NJ], s2[NJ];
 #pragma unroll
     for (int i = 0; i < NJ; ++i) s1[i] = s2[i] = make_float2(0.f, 0.f);
@@ -427,7 +444,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
         if (n0 + cl >= a.N) continue;
         float v = 0.f;
         for (int m = 0; m < a.WM; ++m) v += red[(m * 2 + s) * BN + cl];
-        add_sum(a.so.sums + (size_t)s * a.N + n0 + cl, v);
+        add_sum(a.so.sums, (size_t)s * a.N + n0 + cl, v);
     }
 }
 
@@ -469,7 +486,7 @@ __global__ void __launch_bounds__(256) pw_mma_split_kernel(const Args a) {
     // epilogue operands of this thread's first output vector (8 channels of one pixel): requested before the reduction
     constexpr int EPT = 256 / NJ;                          // pixel rows per epilogue pass
     const int er = tid / NJ, ej = tid - er * NJ, en = n0 + ej * 8;
-    const bool eact = er < EPT && en < a.N, sums = a.so.sums != nullptr;
+    const bool eact = er < EPT && en < a.N, sums = (bool)a.so.sums;
     uint4 ead = make_uint4(0, 0, 0, 0), erz = ead;
     if (BWD && eact && er < BM && p0 + er < a.P) {
         const size_t e = ((size_t)(p0 + er) * a.N + en) >> 3;
@@ -579,7 +596,7 @@ __global__ void __launch_bounds__(256) pw_mma_split_kernel(const Args a) {
         v += __shfl_xor_sync(0xffffffffu, v, 1);
         v += __shfl_xor_sync(0xffffffffu, v, 2);
         const int s = u >= BN ? 1 : 0, cl = u - s * BN;
-        if (part == 0 && u < 2 * BN && n0 + cl < a.N) add_sum(a.so.sums + (size_t)s * a.N + n0 + cl, v);
+        if (part == 0 && u < 2 * BN && n0 + cl < a.N) add_sum(a.so.sums, (size_t)s * a.N + n0 + cl, v);
     }
 }
 

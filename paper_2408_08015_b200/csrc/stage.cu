@@ -63,8 +63,8 @@ struct Unit {
     long w_off = -1, b_off = -1, gamma_off = -1, beta_off = -1;   // floats into the parameter arena
     size_t k_off = 0;       // floats into the backward-coefficient arena (k1,k2,k3)
     size_t run_off = 0;     // floats into the running-statistics arena
-    size_t acc_off = 0;     // 3x3 and 5x5 depthwise units: the weight gradient's accumulators, [taps][c] doubles, in the backward sums
-    size_t sum_off = 0;     // BatchNorm units: channels before this unit's (its sums: 2c doubles at 2*sum_off, its pivots at sum_off)
+    size_t acc_off = 0;     // 3x3 and 5x5 depthwise units: the weight gradient's accumulators, [taps][c], in the backward sums
+    size_t sum_off = 0;     // BatchNorm units: channels before this unit's (its sums: 2c at 2*sum_off, its pivots at sum_off)
     // dense conv with a short reduction, bfloat16 mode: forward and weight gradient run as pointwise tensor-core GEMMs
     // over an explicit im2col tensor kept in the slot (col_kp = padded reduction length, 0 = not such a unit)
     int col_kp = 0;
@@ -126,7 +126,7 @@ struct asteroid_stage {
     // accumulators of the depthwise weight gradients.  A forward's first kernel zeroes both, so that a backward starts from zero
     // whatever ran on the stage before its forward: calls that an import dropped, a replay of a captured round.  Accumulate zeroes the
     // backward's again, for graphs of a caller's own that hold a backward and its accumulate without the forward.
-    double* fsum = nullptr;
+    char* fsum = nullptr;
     float* pivots = nullptr;
     DwSettle* dw_tab = nullptr;                    // the depthwise units' accumulators and weight gradients
     int n_dw = 0;
@@ -404,7 +404,7 @@ static int build_plan(asteroid_stage* s) {
             ncoef += (size_t)s->B * (3 * (size_t)u.g.ci + u.se_k);
         }
     s->slot_bsum_off = align_up(sb + nstat * sizeof(float), 256);
-    s->slot_bytes = align_up(s->slot_bsum_off + s->n_bsum * sizeof(double), 256);
+    s->slot_bytes = align_up(s->slot_bsum_off + chan_sums_bytes(s->n_bsum), 256);
     s->grad_bytes = gb;
     s->n_coef = ncoef;
     s->n_run = nrun;
@@ -547,12 +547,12 @@ static ConvGeom col_geom(const Unit& u) {
 struct SlotView {
     char* base;
     float* stats;
-    double* bsum;
+    char* bsum;
 };
 
 static SlotView slot_view(asteroid_stage* s, int slot) {
     char* b = s->slot_mem + (size_t)slot * s->slot_bytes;
-    return SlotView{b, reinterpret_cast<float*>(b + s->slot_stat_off), reinterpret_cast<double*>(b + s->slot_bsum_off)};
+    return SlotView{b, reinterpret_cast<float*>(b + s->slot_stat_off), b + s->slot_bsum_off};
 }
 
 static ValSrc val_src(asteroid_stage* s, const SlotView& sv, int v) {
@@ -570,6 +570,8 @@ static void tick(asteroid_stage* s, size_t unit, int which, cudaStream_t st) {
 }
 
 // ---- BatchNorm coefficients that are still sums (fin.cuh)
+static ChanSums fsums(const asteroid_stage* s) { return chan_sums(s->fsum, 2 * s->n_bn_ch, false); }
+static ChanSums bsums(const asteroid_stage* s, const SlotView& sv) { return chan_sums(sv.bsum, s->n_bsum, true); }
 static BnFwdOut fwd_out(asteroid_stage* s, const SlotView& sv, const Unit& u) {
     const Val& o = s->vals[u.out];
     float* stt = sv.stats + o.stat_off;
@@ -583,15 +585,15 @@ static BnBwdOut bwd_out(asteroid_stage* s, const Unit& u) {
 static BnPendFwd pend_fwd(asteroid_stage* s, const SlotView& sv, const Unit& u) {
     const Val& o = s->vals[u.out];
     const double n = (double)(o.elems / o.c);
-    return BnPendFwd{s->fsum + 2 * u.sum_off, s->pivots + u.sum_off, s->w + u.gamma_off, s->w + u.beta_off, 1.0 / n, n > 1.0 ? n / (n - 1.0) : 1.0,
+    return BnPendFwd{fsums(s) + 2 * u.sum_off, s->pivots + u.sum_off, s->w + u.gamma_off, s->w + u.beta_off, 1.0 / n, n > 1.0 ? n / (n - 1.0) : 1.0,
                      s->eps, s->bn_mom, o.c, fwd_out(s, sv, u)};
 }
 static BnPendBwd pend_bwd(asteroid_stage* s, const SlotView& sv, const Unit& u) {
     const Val& o = s->vals[u.out];
     const float* stt = sv.stats + o.stat_off;
-    return BnPendBwd{sv.bsum + 2 * u.sum_off, s->w + u.gamma_off, stt, stt + o.c, 1.0 / (double)(o.elems / o.c), o.c, bwd_out(s, u)};
+    return BnPendBwd{bsums(s, sv) + 2 * u.sum_off, s->w + u.gamma_off, stt, stt + o.c, 1.0 / (double)(o.elems / o.c), o.c, bwd_out(s, u)};
 }
-static BnSumsOut sums_fwd(asteroid_stage* s, const Unit& u) { return BnSumsOut{s->fsum + 2 * u.sum_off, s->run + u.run_off, s->pivots + u.sum_off}; }
+static BnSumsOut sums_fwd(asteroid_stage* s, const Unit& u) { return BnSumsOut{fsums(s) + 2 * u.sum_off, s->run + u.run_off, s->pivots + u.sum_off}; }
 
 // which BatchNorm units' coefficients are pending in the pass at hand
 struct Pending {
@@ -653,10 +655,10 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
         // accesses, so that the chain of programmatic dependent launches is not interrupted.  It also zeroes the channel sums of
         // this forward and of its backward.
         const Val& v0 = s->vals[0];
-        if (!slot_copy(x, sv.base + v0.buf_off, v0.elems * s->esz, s->fsum, 2 * s->n_bn_ch, sv.bsum, s->n_bsum, st)) {
+        if (!slot_copy(x, sv.base + v0.buf_off, v0.elems * s->esz, fsums(s), 2 * s->n_bn_ch, bsums(s, sv), s->n_bsum, st)) {
             CU(cudaMemcpyAsync(sv.base + v0.buf_off, x, v0.elems * s->esz, cudaMemcpyDeviceToDevice, st));
-            if (s->n_bn_ch) CU(cudaMemsetAsync(s->fsum, 0, 2 * s->n_bn_ch * sizeof(double), st));
-            if (s->n_bsum) CU(cudaMemsetAsync(sv.bsum, 0, s->n_bsum * sizeof(double), st));
+            if (s->n_bn_ch) CU(cudaMemsetAsync(s->fsum, 0, chan_sums_bytes(2 * s->n_bn_ch), st));
+            if (s->n_bsum) CU(cudaMemsetAsync(sv.bsum, 0, chan_sums_bytes(s->n_bsum), st));
         }
     }
     Pending pend(s, sv, st);
@@ -877,7 +879,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 d.scale = stt + 2 * (size_t)o.c;
                 d.shift = stt + 3 * (size_t)o.c;
                 if (!reduced[ui]) {
-                    bn_bwd_reduce(dt, d.dy, d.z, o.elems / o.c, o.c, d.scale, d.shift, u.act, stt, stt + o.c, sv.bsum + 2 * u.sum_off, s->scratch_floats, st);
+                    bn_bwd_reduce(dt, d.dy, d.z, o.elems / o.c, o.c, d.scale, d.shift, u.act, stt, stt + o.c, bsums(s, sv) + 2 * u.sum_off, s->scratch_floats, st);
                     pend.unit[ui] = 1;
                 }
                 d.k1 = kc; d.k2 = kc + o.c; d.k3 = kc + 2 * (size_t)o.c;
@@ -912,11 +914,11 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 GradState& gi = gs[u.in];
                 const void* addend = gi.state == G_NONE ? nullptr : gi.ptr;
                 const int tgt = want_in && s->vals[u.in].first_cons == ui && bn_reduce_target(s, u.in) == s->vals[u.in].unit ? s->vals[u.in].unit : -1;
-                double* sums = nullptr;
+                ChanSums sums{};
                 const float* ts = nullptr;
                 if (tgt >= 0) {
                     const Unit& tu = s->units[tgt];
-                    sums = sv.bsum + 2 * tu.sum_off;
+                    sums = bsums(s, sv) + 2 * tu.sum_off;
                     ts = sv.stats + s->vals[tu.out].stat_off;
                     pend.unit[tgt] = 1;
                     reduced[tgt] = 1;
@@ -924,8 +926,8 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 }
                 void* to = want_in ? own(u.in) : nullptr;
                 const float* trs = ts ? ts + u.g.ci : nullptr;
-                if (u.g.k == 5) dw5_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, sv.bsum + u.acc_off, sums, ts, trs, dw5_choose(dt, true, u.g), st);
-                else dw3_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, sv.bsum + u.acc_off, sums, ts, trs, dw3_choose(dt, true, u.g), st);
+                if (u.g.k == 5) dw5_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, bsums(s, sv) + u.acc_off, sums, ts, trs, dw5_choose(dt, true, u.g), st);
+                else dw3_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, bsums(s, sv) + u.acc_off, sums, ts, trs, dw3_choose(dt, true, u.g), st);
                 if (want_in) {
                     gi.state = G_OWNED;
                     gi.ptr = own(u.in);
@@ -984,7 +986,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                         float* ts = sv.stats + tv.stat_off;
                         red = BnRed{sv.base + tv.buf_off, ts + 2 * (size_t)tv.c, ts + 3 * (size_t)tv.c, ts, ts + tv.c, tu.act, nullptr, 0};
                         p.red = &red;
-                        p.so = BnSumsOut{sv.bsum + 2 * tu.sum_off, nullptr, nullptr};
+                        p.so = BnSumsOut{bsums(s, sv) + 2 * tu.sum_off, nullptr, nullptr};
                         pend.unit[tgt] = 1;
                         reduced[tgt] = 1;
                         s->bwd_sums_by[tgt] = ui;
@@ -1037,7 +1039,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                     const Val& tv = s->vals[tu.out];
                     float* ts = sv.stats + tv.stat_off;
                     fused = ew_relu_mask_bn_sums(dt, go.ptr, sv.base + o.buf_off, sv.base + tv.buf_off, o.elems / o.c, o.c, ts, ts + tv.c, own(u.out),
-                                                 sv.bsum + 2 * tu.sum_off, s->scratch_floats, st);
+                                                 bsums(s, sv) + 2 * tu.sum_off, s->scratch_floats, st);
                     if (fused) {
                         pend.unit[tgt] = 1;
                         reduced[tgt] = 1;
@@ -1079,12 +1081,12 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 }
                 if (want_in) se_backward_scale(dt, go.ptr, s->B, o.h * o.w, c, gate, wk.ds, addend, own(u.in), st);
             } else if (want_in) {
-                double* sums = nullptr;
+                ChanSums sums{};
                 const float* ts = nullptr;
                 const int tgt = s->vals[u.in].first_cons == ui && bn_reduce_target(s, u.in) == s->vals[u.in].unit ? s->vals[u.in].unit : -1;
-                if (tgt >= 0 && s->units[tgt].act == ACT_NONE) {
+                if (tgt >= 0 && s->units[tgt].act == ACT_NONE && s->B <= MAX_SUM_BLOCKS) {      // the pass has at least one block a sample
                     const Unit& tu = s->units[tgt];
-                    sums = sv.bsum + 2 * tu.sum_off;
+                    sums = bsums(s, sv) + 2 * tu.sum_off;
                     ts = sv.stats + s->vals[tu.out].stat_off;
                     pend.unit[tgt] = 1;
                     reduced[tgt] = 1;
@@ -1112,7 +1114,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
     }
     if (s->need_dx && gs[0].state == G_ALIAS)
         CU(cudaMemcpyAsync(dx, gs[0].ptr, s->vals[0].elems * s->esz, cudaMemcpyDeviceToDevice, st));
-    if (s->n_dw_weights) dw_settle(sv.bsum, s->dw_tab, s->n_dw, s->n_dw_weights, s->g, st);
+    if (s->n_dw_weights) dw_settle(bsums(s, sv), s->dw_tab, s->n_dw, s->n_dw_weights, s->g, st);
     if (side_used) {            // join: the call's work is complete, in the caller's stream order, when the second stream's is
         CU(cudaEventRecord(s->ev_join, s->side));
         CU(cudaStreamWaitEvent(st, s->ev_join, 0));
@@ -1211,7 +1213,7 @@ static int create_impl(const ast_layer* net, int n_layers, int first, int last, 
         if ((rc = arena_alloc(s, "padded weights", &s->wpad, s->n_wpad * 2, &mod))) return rc;
         if ((rc = arena_alloc(s, "padded weight gradient", &s->gpad, s->n_gpad * 4, &work))) return rc;
     }
-    if ((rc = arena_alloc(s, "forward channel sums", &s->fsum, s->n_bn_ch * 2 * sizeof(double), &work))) return rc;
+    if ((rc = arena_alloc(s, "forward channel sums", &s->fsum, chan_sums_bytes(2 * s->n_bn_ch), &work))) return rc;
     if (s->n_dw) {
         std::vector<DwSettle> tab;
         for (const auto& u : s->units)
@@ -1391,7 +1393,7 @@ int asteroid_stage_backward(asteroid_stage* s, int mb, const void* dy, void* dx,
     int slot = s->slot_of_mb[mb];
     if (slot < 0) return fail(AST_ERR_ORDER, "backward of micro-batch %d without a resident forward", mb);
     if (s->pending_g >= 0) return fail(AST_ERR_ORDER, "gradients of micro-batch %d have not been accumulated yet", s->pending_g);
-    if (s->sums_left[slot] && s->n_bsum) CU(cudaMemsetAsync(slot_view(s, slot).bsum, 0, s->n_bsum * sizeof(double), (cudaStream_t)stream));
+    if (s->sums_left[slot] && s->n_bsum) CU(cudaMemsetAsync(slot_view(s, slot).bsum, 0, chan_sums_bytes(s->n_bsum), (cudaStream_t)stream));
     int rc = run_call(s, true, slot, dy, dx, (cudaStream_t)stream, [&](cudaStream_t st) { return backward_impl(s, slot, dy, dx, st); });
     s->sums_left[slot] = rc != AST_OK;
     if (rc) return rc;
@@ -1406,7 +1408,7 @@ int asteroid_stage_accumulate(asteroid_stage* s, int mb, void* stream) {
     if (!s) return fail(AST_ERR_ARG, "null argument");
     if (s->pending_g != mb) return fail(AST_ERR_ORDER, "accumulate(%d): the last backward was of micro-batch %d", mb, s->pending_g);
     if (s->n_acc >= s->M) return fail(AST_ERR_ORDER, "already accumulated %d micro-batches this round", s->M);
-    accumulate(s->G, s->g, s->n_pad, slot_view(s, s->pending_slot).bsum, s->n_bsum, (cudaStream_t)stream);
+    accumulate(s->G, s->g, s->n_pad, bsums(s, slot_view(s, s->pending_slot)), s->n_bsum, (cudaStream_t)stream);
     CU(cudaGetLastError());
     s->pending_g = -1;
     s->n_acc++;

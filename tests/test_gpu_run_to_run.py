@@ -61,3 +61,72 @@ def test_gradients_do_not_depend_on_the_order_of_additions(kind, bf16):
                 np.testing.assert_array_equal(a, b, err_msg="run %d" % run)
     finally:
         P.asteroid_stage_destroy(hdl)
+
+
+@pytest.mark.parametrize("kind", ["own_pass", "pointwise", "depthwise3"])
+@pytest.mark.parametrize("exp", [-130, -80, -55, -33, -10, 10, 30, 60, 100])
+def test_sums_of_every_magnitude(kind, exp):
+    """beta's gradient against float64 for output gradients of about 2^exp, from where partial sums are subnormal to near the largest float.  A
+    block's partial sum is a chain of float32 additions, each off by 2^-24 of what it holds: 2^-16 of the sum of magnitudes covers chains of 256."""
+    import paper_2408_08015_b200 as P
+    c = 32
+    net = _net(kind, c)
+    last = len(net) - 1
+    gen = torch.Generator(device="cuda").manual_seed(12)
+    x = torch.randn(B, H, W, c, generator=gen, device="cuda")
+    dy = torch.randn(B, H, W, c, generator=gen, device="cuda") * torch.tensor(2.0, device="cuda").pow(exp / 2) * torch.tensor(2.0, device="cuda").pow(exp / 2)
+    params = np.ascontiguousarray(si.init_params(net, 0, last, 4), np.float32)
+    at = [i for i, name, _ in si.param_layout(net, 0, last) for _ in [0] if name == "beta"]
+    assert at == [1]
+    off, tail = {}, 0
+    for i, name, shape in si.param_layout(net, 0, last):
+        off[name, i] = (tail, shape)
+        tail += int(np.prod(shape))
+    y, dx = torch.empty_like(x), torch.empty_like(x)
+    hdl = P.asteroid_stage_create(net, 0, last, H, W, B, 1, dtype=P.AST_F32)
+    try:
+        P.asteroid_stage_import_state(hdl, params)
+        sp = torch.cuda.current_stream().cuda_stream
+        P.asteroid_stage_forward(hdl, 0, x.data_ptr(), y.data_ptr(), sp)
+        P.asteroid_stage_backward(hdl, 0, dy.data_ptr(), dx.data_ptr(), sp)
+        g = np.empty(tail, np.float32)
+        P.asteroid_stage_export_state(hdl, micro_grad=g)
+    finally:
+        P.asteroid_stage_destroy(hdl)
+    d = dy.double()
+    if kind != "own_pass":
+        o, shape = off["weight", last]
+        w = torch.from_numpy(params[o:o + int(np.prod(shape))].astype(np.float64)).cuda()
+        conv = torch.nn.grad.conv2d_input
+        if kind == "pointwise":
+            d = d.reshape(-1, c) @ w.reshape(c, c)
+        else:
+            d = conv((B, c, H, W), w.reshape(c, 1, 3, 3), d.permute(0, 3, 1, 2), padding=1, groups=c).permute(0, 2, 3, 1).reshape(-1, c)
+    d = d.reshape(-1, c)
+    o, _ = off["beta", 1]
+    err = np.abs(g[o:o + c] - d.sum(0).cpu().numpy())
+    # and a subnormal result is a multiple of 2^-149
+    assert (err <= 2.0 ** -16 * d.abs().sum(0).cpu().numpy() + B * H * W * 2.0 ** -150).all(), (err, d.sum(0))
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan")])
+def test_what_is_not_finite_stays_so(value):
+    import paper_2408_08015_b200 as P
+    c = 32
+    net = _net("own_pass", c)
+    x = torch.randn(B, H, W, c, device="cuda")
+    dy = torch.randn(B, H, W, c, device="cuda")
+    dy[3, 5, 7, 4] = value
+    y, dx = torch.empty_like(x), torch.empty_like(x)
+    hdl = P.asteroid_stage_create(net, 0, 1, H, W, B, 1, dtype=P.AST_F32)
+    try:
+        P.asteroid_stage_import_state(hdl, np.ascontiguousarray(si.init_params(net, 0, 1, 4), np.float32))
+        P.asteroid_stage_forward(hdl, 0, x.data_ptr(), y.data_ptr())
+        P.asteroid_stage_backward(hdl, 0, dy.data_ptr(), dx.data_ptr())
+        g = np.empty(si.param_count(net, 0, 1), np.float32)
+        P.asteroid_stage_export_state(hdl, micro_grad=g)
+    finally:
+        P.asteroid_stage_destroy(hdl)
+    beta = g[c * c + c:]
+    assert beta[4] == value or (np.isnan(value) and np.isnan(beta[4]))
+    assert np.isfinite(np.delete(beta, 4)).all()

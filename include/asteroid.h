@@ -158,7 +158,8 @@ int asteroid_stage_step(asteroid_stage* s, float lr, float momentum, void* strea
  * statistics and backward sums taken inside the neighbouring kernels wherever the round does so),
  * except that every kernel stays on one stream, so that a layer's time is that of its own kernels.
  * A BatchNorm whose sums were taken by another layer's kernel reports only its finishing kernel
- * (alg_bytes of a few kB, or 0) and names that layer in fused_into. */
+ * (alg_bytes of a few kB, or 0) and names that layer in fused_into.  A residual sum that the 1x1 conv behind it forms as it
+ * loads reports no FP time or bytes and names that conv, whose alg_bytes_f include the sum's. */
 int asteroid_stage_profile(asteroid_stage* s, int layer, int batch, ast_layer_profile* out);
 
 /* Loss heads (used by the last stage and by tests).  All pointers are DEVICE pointers.

@@ -158,6 +158,7 @@ struct asteroid_stage {
     // what the last forward / backward did, per unit: statistics partials written by the producing kernel (their count, 0 =
     // standalone pass); unit whose backward-data kernel took this unit's BatchNorm-backward sums (-1 = standalone pass)
     std::vector<int> fwd_stats_blocks, bwd_sums_by;
+    std::vector<char> add_deferred;                // ... residual sums that the pointwise layer behind formed
 };
 
 namespace ast {
@@ -635,10 +636,10 @@ static bool f32_unit(const asteroid_stage* s, const Unit& u, bool bwd, F32Tiling
 // A residual sum of two tensors without activations of their own, read next by a pointwise layer on the register-operand or float32
 // kernels: that layer forms it as it loads, and writes it out for the others.  Up to 4 M elements, where the sum is mostly a launch in the chain (a
 // round of a sixth of MobileNetV2 at batch 4 1681 -> 1647 us, of small images 1469 -> 1440); beyond, two operands to wait for cost the
-// pointwise layer more than the pass saves (ResNet stage at batch 32: 1 % slower).  Not while a profile times the units one by one.
+// pointwise layer more than the pass saves (ResNet stage at batch 32: 1 % slower).
 static bool defers_add(const asteroid_stage* s, size_t ui) {
     const Unit& u = s->units[ui];
-    if (s->tm.on || ui + 1 >= s->units.size() || s->vals[u.out].elems > (size_t)4 << 20) return false;
+    if (ui + 1 >= s->units.size() || s->vals[u.out].elems > (size_t)4 << 20) return false;
     const Unit& v = s->units[ui + 1];
     MmaTiling t;
     F32Tiling t32;
@@ -758,6 +759,7 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
             squeeze_splits = 0;
         } else if (u.kind == U_ADD && defers_add(s, ui)) {
             deferred = (int)ui;
+            s->add_deferred[ui] = 1;
         } else if (u.kind == U_ADD) {
             if (!ew_takes_pending(dt, o.c)) {
                 pend.settle_fwd(producer(u.in));
@@ -1250,6 +1252,7 @@ static int create_impl(const ast_layer* net, int n_layers, int first, int last, 
     s->sums_left.assign(s->slots, 0);
     s->fwd_stats_blocks.assign(s->units.size(), 0);
     s->bwd_sums_by.assign(s->units.size(), -1);
+    s->add_deferred.assign(s->units.size(), 0);
     return AST_OK;
 }
 
@@ -1547,9 +1550,15 @@ int asteroid_stage_profile(asteroid_stage* s, int layer, int batch, ast_layer_pr
                 out->alg_bytes_f = xin + zo + out->w_l_bytes;
                 // bwd-weight reads dy, z, x; bwd-data reads dy, z and writes dx
                 out->alg_bytes_b = 2 * (zo + zo) + xin + ((u.in != 0 || t->need_dx) ? xin : 0) + 2 * out->w_l_bytes;
+                if (ui > 0 && t->add_deferred[ui - 1]) out->alg_bytes_f += 2 * xin;    // the second operand of the sum in front, and the sum written
             } else if (u.kind == U_ADD) {
                 out->alg_bytes_f = 3 * zo;
                 out->alg_bytes_b = u.act == ACT_RELU ? 3 * zo : 0;
+                if (t->add_deferred[ui]) {             // formed by the pointwise layer behind
+                    out->t_f_ms = 0;
+                    out->alg_bytes_f = 0;
+                    out->fused_into = t->units[ui + 1].l_main;
+                }
             } else if (u.kind == U_SILU) {
                 out->alg_bytes_f = xin + zo;
                 out->alg_bytes_b = 3 * zo;              // dy, x -> dx

@@ -150,7 +150,7 @@ void conv_pad_weights(const float* w, int co, int K, int Kp, __nv_bfloat16* wpad
 void conv_unpad_grad(const float* gpad, int co, int K, int Kp, float* gw, cudaStream_t st);
 
 // ---- pointwise conv on tcgen05 tensor cores (bf16 storage, channel counts multiples of 8) ----
-bool pw_tc_supported(int dtype, const ConvGeom& g, bool bwd_data);
+bool pw_tc_supported(int dtype, const ConvGeom& g);
 // wb: bf16 weights [co][ci]; wtb: bf16 transposed weights [ci][co]; err: device error word
 // With `pivot` and `partial` given, the pipelined kernel also writes the BatchNorm statistics partials of its output,
 // partial[cta][2][co] = sums of (z - pivot[c]) and (z - pivot[c])^2 over the CTA's pixels (z as stored, after rounding),
@@ -163,7 +163,7 @@ int pw_fwd_tc(const ConvGeom& g, const ValSrc& x, const __nv_bfloat16* wb, const
 // of the unit that produced this conv's input.  Returns the number of CTAs (for bn_bwd_finish_partials); 0 = none written.
 int pw_bwd_data_tc(const ConvGeom& g, const GradSrc& dz, const __nv_bfloat16* wtb, const void* addend, void* dx, const BnRed* red, int* err,
                    cudaStream_t st);
-// streaming form (pw_stream.cu) for stride-1 layers with more than 256 channels on a side (channel counts multiples of 64): forward
+// streaming form (pw_stream.cu) for stride-1 layers the pipeline has no room for (channel counts multiples of 64): forward
 // (bwd == false: x [P][K], w = [N][K]) or backward-data (bwd == true: dz [P][K], w = transposed weights [N][K]); false = does not fit
 bool pw_stream(bool bwd, int P, int K, int N, const ValSrc& x, const GradSrc& dz, const __nv_bfloat16* w, const void* addend, void* out, int* err,
                int kind, double bytes, cudaStream_t st);

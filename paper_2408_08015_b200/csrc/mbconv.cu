@@ -918,51 +918,46 @@ void se_backward_scale(int dtype, const void* dout, int n, int hw, int c, const 
         if ((dtype) == 0) { using T = float; constexpr int V = 4; __VA_ARGS__ }     \
         else { using T = __nv_bfloat16; constexpr int V = 4; __VA_ARGS__ }          \
     } while (0)
-// ... and with the compile-time kernel size (3x3: dw3.cu, 5x5: dw5.cu)
-#define DISPATCH_K(k, ...)       \
-    do {                         \
-        constexpr int K = 7;     \
-        __VA_ARGS__              \
-    } while (0)
+constexpr int DWK = 7;         // the kernel size of the functions below (3x3: dw3.cu, 5x5: dw5.cu)
 
 void dwk_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const float* wkc, void* z, cudaStream_t st) {
     const size_t out_e = (size_t)g.n * g.ho * g.wo * g.ci, in_e = (size_t)g.n * g.hi * g.wi * g.ci;
     LaunchScope ls(K_DW_FWD, ((double)in_e + out_e) * esz_(dtype) + 4.0 * g.k * g.k * g.ci, 2.0 * g.k * g.k * out_e, st);
-    DISPATCH_T16(dtype, DISPATCH_K(g.k, {
+    DISPATCH_T16(dtype, {
         constexpr int TW = 4;
         const int strips = (g.wo + TW - 1) / TW, vpr = g.ci / V;
         const size_t items = (size_t)g.n * g.ho * strips * vpr;
         const VecGrid vg = vec_grid(items, vpr, 1);
         if (g.stride == 1)
-            launch_pdl(dwk_strip_kernel<T, V, K, 1, TW, false, ValCoef<V>, ValSrc>, vg.blocks, 256, 0, st, g.hi, g.wi, g.ho, g.wo, g.ci, x, wkc, (const T*)nullptr, items,
+            launch_pdl(dwk_strip_kernel<T, V, DWK, 1, TW, false, ValCoef<V>, ValSrc>, vg.blocks, 256, 0, st, g.hi, g.wi, g.ho, g.wo, g.ci, x, wkc, (const T*)nullptr, items,
                        strips, vg.stride, (T*)z);
         else
-            launch_pdl(dwk_strip_kernel<T, V, K, 2, TW, false, ValCoef<V>, ValSrc>, vg.blocks, 256, 0, st, g.hi, g.wi, g.ho, g.wo, g.ci, x, wkc, (const T*)nullptr, items,
+            launch_pdl(dwk_strip_kernel<T, V, DWK, 2, TW, false, ValCoef<V>, ValSrc>, vg.blocks, 256, 0, st, g.hi, g.wi, g.ho, g.wo, g.ci, x, wkc, (const T*)nullptr, items,
                        strips, vg.stride, (T*)z);
-    }););
+    });
 }
 
 void dwk_bwd_data(int dtype, const ConvGeom& g, const GradSrc& dz, const float* wkc, const void* addend, void* dx, cudaStream_t st) {
     const size_t out_e = (size_t)g.n * g.ho * g.wo * g.ci, in_e = (size_t)g.n * g.hi * g.wi * g.ci;
     LaunchScope ls(K_DW_BWD_DATA, ((double)out_e * (grad_needs_z(dz) ? 2 : 1) + (double)in_e * (addend ? 2 : 1)) * esz_(dtype), 2.0 * g.k * g.k * out_e, st);
-    DISPATCH_T16(dtype, DISPATCH_K(g.k, {
+    DISPATCH_T16(dtype, {
         constexpr int TW = 4;
         const int strips = (g.wi + TW - 1) / TW, vpr = g.ci / V;
         const size_t items = (size_t)g.n * g.hi * strips * vpr;
         const VecGrid vg = vec_grid(items, vpr, 1);
         if (g.stride == 1)
-            launch_pdl(dwk_strip_kernel<T, V, K, 1, TW, true, GradCoef<V>, GradSrc>, vg.blocks, 256, 0, st, g.ho, g.wo, g.hi, g.wi, g.ci, dz, wkc, (const T*)addend, items,
+            launch_pdl(dwk_strip_kernel<T, V, DWK, 1, TW, true, GradCoef<V>, GradSrc>, vg.blocks, 256, 0, st, g.ho, g.wo, g.hi, g.wi, g.ci, dz, wkc, (const T*)addend, items,
                        strips, vg.stride, (T*)dx);
         else
-            launch_pdl(dwk_bwd_data_s2_kernel<T, V, K, TW>, vg.blocks, 256, 0, st, g, dz, wkc, (const T*)addend, items, strips, vg.stride, (T*)dx);
-    }););
+            launch_pdl(dwk_bwd_data_s2_kernel<T, V, DWK, TW>, vg.blocks, 256, 0, st, g, dz, wkc, (const T*)addend, items, strips, vg.stride, (T*)dx);
+    });
 }
 
 void dwk_bwd_weight(int dtype, const ConvGeom& g, const GradSrc& dz, const ValSrc& x, float* scratch, size_t scratch_floats, float* gw, cudaStream_t st) {
     const size_t positions = (size_t)g.n * g.ho * g.wo, out_e = positions * g.ci, in_e = (size_t)g.n * g.hi * g.wi * g.ci;
     const int taps = g.k * g.k;
     int by = 0;
-    DISPATCH_T16(dtype, DISPATCH_K(g.k, {
+    DISPATCH_T16(dtype, {
         constexpr int TW = 4;
         const int strips = (g.wo + TW - 1) / TW;
         const size_t total = (size_t)g.n * g.ho * strips;
@@ -975,9 +970,9 @@ void dwk_bwd_weight(int dtype, const ConvGeom& g, const GradSrc& dz, const ValSr
         const size_t spb = (total + want - 1) / want;
         by = (int)((total + spb - 1) / spb);
         LaunchScope ls(K_DW_BWD_WEIGHT, ((double)out_e * (grad_needs_z(dz) ? 2 : 1) + in_e) * esz_(dtype) + 4.0 * taps * g.ci, 2.0 * taps * out_e, st);
-        if (g.stride == 1) launch_pdl(dwk_bwd_weight_kernel<T, V, K, 1, TW>, dim3(gx, by), 128, 0, st, g, dz, x, strips, spb, scratch);
-        else launch_pdl(dwk_bwd_weight_kernel<T, V, K, 2, TW>, dim3(gx, by), 128, 0, st, g, dz, x, strips, spb, scratch);
-    }););
+        if (g.stride == 1) launch_pdl(dwk_bwd_weight_kernel<T, V, DWK, 1, TW>, dim3(gx, by), 128, 0, st, g, dz, x, strips, spb, scratch);
+        else launch_pdl(dwk_bwd_weight_kernel<T, V, DWK, 2, TW>, dim3(gx, by), 128, 0, st, g, dz, x, strips, spb, scratch);
+    });
     LaunchScope ls(K_DW_BWD_WEIGHT_FINISH, 4.0 * taps * g.ci * (by + 1), (double)taps * g.ci * by, st);
     launch_pdl(dwk_weight_finish_kernel, (taps * g.ci + 255) / 256, 256, 0, st, (const float*)scratch, by, taps, g.ci, gw);
 }

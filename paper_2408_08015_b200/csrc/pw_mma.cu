@@ -65,7 +65,7 @@ bool bwd_choose(int P, int K, int N, MmaTiling* out) {
     const int KCH = (K + 31) / 32, sms = sm_count();
     double best = 0;
     auto offer = [&](int mi, int nj, int wm, int wk, int ctas) {
-        const MmaTiling c{mi, nj, wm, 1, wk, ctas};
+        const MmaTiling c{mi, nj, wm, wk, ctas};
         if (mma_smem(true, K, c) * (wk == 1 ? ctas : 1) > 200 * 1024) return;
         const int cols = (N + 8 * nj - 1) / (8 * nj);
         double t;
@@ -111,7 +111,7 @@ bool fwd_choose(int P, int K, int N, MmaTiling* out) {
     const int KCH = (K + 31) / 32, sms = sm_count();
     double best = 0;
     auto offer = [&](int mi, int nj, int wm, int wk, int ctas) {
-        const MmaTiling c{mi, nj, wm, 1, wk, ctas};
+        const MmaTiling c{mi, nj, wm, wk, ctas};
         if (mma_smem(false, K, c) * (wk == 1 ? ctas : 1) > 200 * 1024) return;
         const int cols = (N + 8 * nj - 1) / (8 * nj);
         double t;
@@ -153,6 +153,8 @@ bool fwd_choose(int P, int K, int N, MmaTiling* out) {
 // 256 channels a side.  There the arithmetic of mma.sync (and the shared-memory reads of its weights) is the bound and the tensor-memory
 // pipeline of pw_tc.cu is as fast or faster: 64 -> 256 at 100 352 pixels 26.3 us against 29.3, backward to 256 channels 71 against 77.  To at
 // most 64 channels it is not: 256 -> 64 30.6 against 24.0, backward 45 against 42.  (One layer with its BatchNorm sums in a captured chain.)
+// With 192 to 256 channels on both sides the pipeline does not fit and pw_stream.cu and the one-tile kernel take the layer: 256 -> 256 on 50 176
+// pixels forward 33 us with its pass for the sums (37 here), backward with a transform 49 (72), without 23 (49).
 bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {
     if (K % 8 || N % 8 || (double)P * (K > N ? K : N) * 2.0 >= 4.0e9) return false;
     if (P >= 50000 && K <= 256 && N <= 256 && K * N >= 256 * 64 && N > 64) return false;
@@ -160,7 +162,7 @@ bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {
 }
 
 size_t mma_smem(bool bwd, int K, const MmaTiling& c) {
-    const int Kp = (K + 31) / 32 * 32, BN = c.wk == 1 ? c.wn * c.nj * 8 : c.nj * 8;
+    const int Kp = (K + 31) / 32 * 32, BN = c.nj * 8;
     size_t b = (size_t)BN * w_pitch(K) + (size_t)(bwd ? 5 : 3) * Kp * 4 + (size_t)(bwd ? 4 : 1) * BN * 4;
     if (c.wk == 1) b += (size_t)c.wm * 2 * BN * 4;
     else {
@@ -195,9 +197,9 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
         }
     }
     a.w = (const __nv_bfloat16*)p.w; a.bias = p.bias; a.addend = p.addend; a.out = (__nv_bfloat16*)p.out;
-    a.WM = c.wm; a.WN = c.wn;
+    a.WM = c.wm;
     a.wpitch = w_pitch(p.K);
-    const int BN = c.wk == 1 ? c.wn * c.nj * 8 : c.nj * 8, BM = c.wk == 1 ? 16 * c.mi * c.wm : 16 * (8 / c.wk);
+    const int BN = c.nj * 8, BM = c.wk == 1 ? 16 * c.mi * c.wm : 16 * (8 / c.wk);
     a.m_tiles = (p.P + BM - 1) / BM;
     const int ny = (p.N + BN - 1) / BN;
     int gx = a.m_tiles;
@@ -216,7 +218,7 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
     else raise_limits<false>();
     const size_t smem = mma_smem(bwd, p.K, c);
     LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 2.0 * p.P * p.N : 0.0) + (p.sum_out ? 4.0 * p.P * p.K : 0.0), 2.0 * p.P * p.N * p.K, st);
-    launch_pdl(bwd ? kernel_for<true>(c, xf) : kernel_for<false>(c, xf), dim3(gx, ny), c.wk == 1 ? 32 * c.wm * c.wn : 256, smem, st, a);
+    launch_pdl(bwd ? kernel_for<true>(c, xf) : kernel_for<false>(c, xf), dim3(gx, ny), c.wk == 1 ? 32 * c.wm : 256, smem, st, a);
 }
 
 }  // namespace ast

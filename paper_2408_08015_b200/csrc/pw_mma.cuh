@@ -36,7 +36,7 @@ struct Args {
     __nv_bfloat16* out;        // [P][N]
     int P, K, N;
     int KCH;                   // 32-channel chunks of the reduction
-    int WM, WN;                // warps along the pixels / the columns
+    int WM;                    // warps, each with pixels of its own
     int m_tiles;
     uint32_t wpitch;           // bytes between rows of the staged weights
     BnPendFwd pf;              // pending coefficients of the operand (sums null: c0.. are final)
@@ -273,8 +273,8 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
     pdl_launch();
     extern __shared__ __align__(16) uint8_t sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-    const int wm = warp % a.WM, wn = warp / a.WM;
-    const int BN = a.WN * NJ * 8, n0 = blockIdx.y * BN, Kp = a.KCH * 32;
+    const int wm = warp;
+    const int BN = NJ * 8, n0 = blockIdx.y * BN, Kp = a.KCH * 32;
     uint8_t* sW = sm;
     float* sK = reinterpret_cast<float*>(sW + (size_t)BN * a.wpitch);
     float* sN = sK + (BWD ? 5 : 3) * Kp;
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
     __syncthreads();
 
     const float rlo = a.r_act == ACT_NONE ? -INFINITY : 0.f, rhi = a.r_act == ACT_RELU6 ? 6.f : INFINITY;
-    const uint8_t* wb = sW + (uint32_t)(wn * NJ * 8 + g) * a.wpitch + t * 16;
+    const uint8_t* wb = sW + (uint32_t)g * a.wpitch + t * 16;
     const bool sums = (bool)a.so.sums;
     float2 s1[NJ], s2[NJ];
 #pragma unroll
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
     auto fetch_z = [&](int tl) {
 #pragma unroll
         for (int gr = 0; gr < NG; ++gr) {
-            const uint32_t n = (uint32_t)min(n0 + wn * NJ * 8 + gr * 8 * G + C * t, a.N - C);
+            const uint32_t n = (uint32_t)min(n0 + gr * 8 * G + C * t, a.N - C);
 #pragma unroll
             for (int mi = 0; mi < MI; ++mi)
 #pragma unroll
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
     constexpr bool AHEAD = MI * NJ < 16;
     CVec<C> av[2][MI][2];
     auto fetch_add = [&](int gr, int row0, CVec<C> (*v)[2]) {
-        const uint32_t n = (uint32_t)min(n0 + wn * NJ * 8 + gr * 8 * G + C * t, a.N - C);
+        const uint32_t n = (uint32_t)min(n0 + gr * 8 * G + C * t, a.N - C);
 #pragma unroll
         for (int mi = 0; mi < MI; ++mi)
 #pragma unroll
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
             for (int mi = 0; mi < MI; ++mi)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) cu[mi][h] = xf.apply(nx[mi][h], nz[mi][h]);
-            if (!BWD && XF == XF_ADD && blockIdx.y == 0 && wn == 0 && kc * 64 + t * 16 < a.K * 2)
+            if (!BWD && XF == XF_ADD && blockIdx.y == 0 && kc * 64 + t * 16 < a.K * 2)
 #pragma unroll
                 for (int mi = 0; mi < MI; ++mi)
 #pragma unroll
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
         }
 #pragma unroll
         for (int gr = 0; gr < NG; ++gr) {
-            const int cl = wn * NJ * 8 + gr * 8 * G + C * t, n = n0 + cl;
+            const int cl = gr * 8 * G + C * t, n = n0 + cl;
             if (BWD && AHEAD && a.addend && gr + 1 < NG) fetch_add(gr + 1, row0, av[(gr + 1) & 1]);
             if (BWD && !AHEAD && a.addend) fetch_add(gr, row0, av[gr & 1]);
             if (n >= a.N) continue;
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
     if (g == 0) {
 #pragma unroll
         for (int i = 0; i < NJ; ++i) {
-            const int cl = wn * NJ * 8 + (i / G) * 8 * G + 2 * G * t + 2 * (i % G);
+            const int cl = (i / G) * 8 * G + 2 * G * t + 2 * (i % G);
             *reinterpret_cast<float2*>(red + (wm * 2 + 0) * BN + cl) = s1[i];
             *reinterpret_cast<float2*>(red + (wm * 2 + 1) * BN + cl) = s2[i];
         }

@@ -4,10 +4,10 @@
 
 namespace ast {
 
-// A tiling of the layer.  wk == 1: persistent CTAs of wm x wn warps, a warp owns 16*mi pixels x 8*nj columns and the whole reduction;
+// A tiling of the layer.  wk == 1: persistent CTAs of wm warps, a warp owns 16*mi pixels x 8*nj columns and the whole reduction;
 // wk > 1: one tile of 16*(8/wk) pixels x 8*nj columns per CTA, the reduction split over wk warps.
 struct MmaTiling {
-    int mi, nj, wm, wn, wk;
+    int mi, nj, wm, wk;
     int ctas;                  // wk == 1: CTAs per multiprocessor the grid is sized for
 };
 

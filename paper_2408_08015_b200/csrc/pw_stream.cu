@@ -1,6 +1,7 @@
-// Pointwise (1x1, stride 1) convolution, forward and backward-data, for layers with more than 256 channels
-// on one side (which the pointwise pipeline of pw_tc.cu cannot keep resident): a persistent warp-specialised
-// GEMM whose reduction streams through shared memory in 64-channel blocks.
+// Pointwise (1x1, stride 1) convolution, forward and backward-data, for large maps with 192 to 256 channels on both
+// sides (which the pointwise pipeline of pw_tc.cu cannot keep resident; pw_mma.cu has the wider layers): a persistent
+// warp-specialised GEMM whose reduction streams through shared memory in 64-channel blocks.  256 -> 256 on 50 176 pixels
+// 21 us forward and 23 us backward without a transform (register-operand kernels 36 and 49).
 //
 //   out[p][n] = sum_k A[p][k] * W[n][k]      A = act(x*scale + shift) (forward) or the BatchNorm-backward
 //                                            transform of (dy, z) (backward-data), W = [N][K] bf16

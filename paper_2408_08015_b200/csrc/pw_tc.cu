@@ -1419,8 +1419,7 @@ template <bool BWD> void launch(const PwArgs& a0, const Tiling& t, int kind, dou
 
 }  // namespace
 
-bool pw_tc_supported(int dtype, const ConvGeom& g, bool bwd_data) {
-    (void)bwd_data;
+bool pw_tc_supported(int dtype, const ConvGeom& g) {
     return dtype == 1 && g.k == 1 && g.pad == 0 && g.ci % 8 == 0 && g.co % 8 == 0 && g.ci >= 8 && g.co >= 8;
 }
 
@@ -1443,7 +1442,7 @@ int pw_fwd_tc(const ConvGeom& g, const ValSrc& x, const __nv_bfloat16* wb, const
         alignas(64) CUtensorMap tm_out;
         if (plan_pipe(pa, &smem) && make_out_map(z, pa.P, pa.N, &tm_out)) return launch_pipe<false>(pa, tm_out, smem, K_PW_FWD_TC, bytes, partial_floats, st);
     }
-    // more than 256 channels on a side: the streaming kernel, where the layer fits it
+    // 192 to 256 channels on both sides, whose weights leave the pipeline no room: the streaming kernel, where the layer fits it
     if (g.stride == 1 && !bias && pw_stream(false, a.P, a.K, a.N, x, GradSrc{}, wb, nullptr, z, err, K_PW_FWD_TC, bytes, st)) return 0;
     Tiling t = pick_tiling(a.K, a.N);
     launch<false>(a, t, K_PW_FWD_TC, bytes, st);

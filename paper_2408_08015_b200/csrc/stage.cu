@@ -620,9 +620,8 @@ struct Pending {
 };
 
 // Pointwise problem of a unit on the register-operand kernels; false: it does not run there.
-static bool mma_unit(const asteroid_stage* s, const Unit& u, const ConvGeom& g, bool bwd, MmaTiling* t) {
+static bool mma_unit(const asteroid_stage* s, const ConvGeom& g, bool bwd, MmaTiling* t) {
     if (s->dtype != AST_BF16 || g.k != 1 || g.stride != 1 || g.pad != 0) return false;
-    (void)u;
     return bwd ? mma_choose(true, g.n * g.ho * g.wo, g.co, g.ci, t) : mma_choose(false, g.n * g.ho * g.wo, g.ci, g.co, t);
 }
 
@@ -645,7 +644,7 @@ static bool defers_add(const asteroid_stage* s, size_t ui) {
     F32Tiling t32;
     if (v.kind != U_CONV || v.in != u.out || v.col_kp || v.sub_off >= 0) return false;
     if (u.in == u.in2 || s->vals[u.in].act != ACT_NONE || s->vals[u.in2].act != ACT_NONE) return false;
-    return mma_unit(s, v, v.g, false, &t) || f32_unit(s, v, false, &t32);
+    return mma_unit(s, v.g, false, &t) || f32_unit(s, v, false, &t32);
 }
 
 static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cudaStream_t st) {
@@ -697,7 +696,7 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
             else mma_launch(false, p, til, K_PW_FWD_TC, 2.0 * elems, st);
             fused_stats = bn ? -1 : 0;
         };
-        if (u.kind == U_CONV && !u.col_kp && u.sub_off < 0 && mma_unit(s, u, u.g, false, &til)) {
+        if (u.kind == U_CONV && !u.col_kp && u.sub_off < 0 && mma_unit(s, u.g, false, &til)) {
             const int from = deferred >= 0 ? s->units[deferred].in : u.in;
             on_mma(u.g, val_src(s, sv, from), producer(from), s->wb + u.w_off);
         } else if (f32_unit(s, u, false, &til32)) {
@@ -710,7 +709,7 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
                 void* col = sv.base + u.col_off;
                 conv_im2col(u.g, val_src(s, sv, u.in), u.col_kp, col, st);
                 const ValSrc cs{col, nullptr, nullptr, ACT_NONE};
-                if (mma_unit(s, u, col_geom(u), false, &til)) on_mma(col_geom(u), cs, -1, s->wpad + u.wpad_off);
+                if (mma_unit(s, col_geom(u), false, &til)) on_mma(col_geom(u), cs, -1, s->wpad + u.wpad_off);
                 else
                 fused_stats = pw_fwd_tc(col_geom(u), cs, s->wpad + u.wpad_off, nullptr, obuf,
                                         bn ? s->run + u.run_off : nullptr, bn ? s->scratch : nullptr, s->scratch_floats, s->err, st);
@@ -719,11 +718,11 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
                 void* sub = sv.base + u.sub_off;
                 ew_subsample2(xs.p, u.g.n, u.g.hi, u.g.wi, u.g.ho, u.g.wo, u.g.ci, sub, st);
                 xs.p = sub;                                  // the producer's BatchNorm / activation is per channel: applied on load as before
-                if (mma_unit(s, u, sub_geom(u), false, &til)) on_mma(sub_geom(u), xs, -1, s->wb + u.w_off);
+                if (mma_unit(s, sub_geom(u), false, &til)) on_mma(sub_geom(u), xs, -1, s->wb + u.w_off);
                 else
                 fused_stats = pw_fwd_tc(sub_geom(u), xs, s->wb + u.w_off, bias, obuf, bn ? s->run + u.run_off : nullptr,
                                         bn ? s->scratch : nullptr, s->scratch_floats, s->err, st);
-            } else if (pw_tc_supported(dt, u.g, false))
+            } else if (pw_tc_supported(dt, u.g))
                 fused_stats = pw_fwd_tc(u.g, val_src(s, sv, u.in), s->wb + u.w_off, bias, obuf, bn ? s->run + u.run_off : nullptr,
                                         bn ? s->scratch : nullptr, s->scratch_floats, s->err, st);
             else if (conv3_tc_supported(dt, u.g)) conv3_fwd_tc(u.g, val_src(s, sv, u.in), s->wb + u.w_off, obuf, s->err, st);
@@ -898,7 +897,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             const bool pw = u.kind == U_CONV && dt == AST_BF16 && wg.k == 1 && wg.stride == 1 && wg.pad == 0;
             const bool mma_w = pw && wgrad_mma_choose(wg.n * wg.ho * wg.wo, wg.co, wg.ci, pw_wgrad_pipeline_fits(wg, grad_needs_z(d), s->scratch_floats),
                                                       s->scratch_floats, &til_w);
-            const bool mma_d = want_in && u.kind == U_CONV && !u.col_kp && mma_unit(s, u, u.g, true, &til_d);
+            const bool mma_d = want_in && u.kind == U_CONV && !u.col_kp && mma_unit(s, u.g, true, &til_d);
             F32Tiling til_d32{};
             F32WgradTiling til_w32{};
             const bool f32_d = want_in && f32_unit(s, u, true, &til_d32);
@@ -965,7 +964,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 ValSrc xs = xin;
                 xs.p = sv.base + u.sub_off;                  // written by the forward of this micro-batch
                 pw_bwd_weight_tc(sub_geom(u), d, xs, wscratch, s->scratch_floats, s->g + u.w_off, s->err, wst);
-            } else if (u.kind == U_CONV && pw_tc_supported(dt, u.g, false))
+            } else if (u.kind == U_CONV && pw_tc_supported(dt, u.g))
                 pw_bwd_weight_tc(u.g, d, xin, wscratch, s->scratch_floats, s->g + u.w_off, s->err, wst);
             else if (u.kind == U_CONV && conv3_wgrad_tc_supported(dt, u.g))
                 conv3_bwd_weight_tc(u.g, d, xin, wscratch, s->scratch_floats, s->g + u.w_off, s->err, wst);
@@ -996,7 +995,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                     const double elems = (double)p.P * p.K * (grad_needs_z(d) ? 2.0 : 1.0) + (double)p.P * p.N * (addend ? 2.0 : 1.0) + (double)p.N * p.K;
                     if (f32_d) f32_launch(true, p, til_d32, K_CONV_BWD_DATA, 4.0 * elems, st);
                     else mma_launch(true, p, til_d, K_PW_BWD_DATA_TC, 2.0 * elems, st);
-                } else if (u.kind == U_CONV && pw_tc_supported(dt, u.g, true)) {
+                } else if (u.kind == U_CONV && pw_tc_supported(dt, u.g)) {
                     BnRed red{};
                     if (tgt >= 0) {
                         const Unit& tu = s->units[tgt];

@@ -18,7 +18,21 @@
  *    and profile synchronise the device.  backward also enqueues the weight-gradient kernels on a
  *    stream of the stage that forks from `stream` and joins it before backward returns, so a whole
  *    round of these calls (after one plain round, in which first-use set-up happens) may be
- *    captured into a CUDA graph on `stream` and replayed.
+ *    captured into a CUDA graph on `stream` and replayed.  The calls of one stage come from one
+ *    thread at a time and on streams that are ordered among themselves: all use its workspaces.
+ *  - A captured round depends on nothing but the stage's state: calls that were made, and dropped
+ *    again by import, between the capture and a replay leave no trace in it.
+ *  - Graphs of the library's own.  The third forward or backward with the same slot and the same two
+ *    buffers captures itself (host work of about as much as a call; the first such call creates a
+ *    stream) and is launched as a graph from then on: 20 to 190 launches of 2.5 us on the host become
+ *    one.  A caller that hands in other buffers on every call does not get this.  A stage keeps at most
+ *    64 such calls; one that was not made for 64 rounds makes room, and a round of more than 32
+ *    micro-batches has the rest launched directly.  Nothing is captured while `stream` is
+ *    being captured, and captures open elsewhere are left alone.  The graphs take device memory that
+ *    no mem_* term of the profile counts (2 MB for up to 1 300 launches, from the driver's pool).
+ *  - Results do not depend on the order in which blocks finish: the same calls on the same state
+ *    and inputs give the same bits on every run of the same build on the same device, whether launched
+ *    directly or replayed.
  *  - The library has no CPU fallback: without a CUDA device every compute call fails.
  *
  * Flat parameter order (import/export): layers in list order; per layer

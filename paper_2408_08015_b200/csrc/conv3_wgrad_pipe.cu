@@ -13,7 +13,8 @@
 // columns in tensor memory; nine taps do not fit the 512 columns, so the taps are split over
 // groups of CTAs (each group stages the same windows), and a CTA accumulates over all its tiles
 // and writes one partial in the gradient's own layout; the partials are summed in index order by
-// the split-sum kernel.
+// the split-sum kernel.  From 64 to 64 channels the roles are swapped: the 128 accumulator rows are the
+// input channels of two taps, so five accumulators of 64 columns hold all nine taps and no group is needed.
 //
 //   warp 0        producer: per tile the tensor copies of x and dy (one ring) and of z (a second ring)
 //   warps 1-2     MMA issuers: each owns a share of the CTA's taps (disjoint accumulator columns) and

@@ -139,10 +139,10 @@ class ClockSampler:
 
 def ncu_traffic(cfg, kernel):
     """DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of a kernel kind from the committed ncu
-    summary, or None when there is no capture of the kernel's current source."""
+    summary, or None when there is no capture of the kernels' current sources."""
     try:
         rec = json.load(open(os.path.join(ROOT, "profiles", "ncu_traffic.json")))["config%d" % cfg][kernel]
-        cur = hashlib.sha256(open(os.path.join(ROOT, rec["file"]), "rb").read()).hexdigest()[:16]
+        cur = hashlib.sha256(b"".join(open(os.path.join(ROOT, f), "rb").read() for f in rec["files"])).hexdigest()[:16]
         return rec["bytes_per_launch"] if cur == rec["sha"] else None
     except (OSError, KeyError, ValueError):
         return None

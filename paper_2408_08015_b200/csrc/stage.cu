@@ -1408,7 +1408,7 @@ int asteroid_stage_backward(asteroid_stage* s, int mb, const void* dy, void* dx,
 
 int asteroid_stage_accumulate(asteroid_stage* s, int mb, void* stream) {
     if (!s) return fail(AST_ERR_ARG, "null argument");
-    if (s->pending_g != mb) return fail(AST_ERR_ORDER, "accumulate(%d): the last backward was of micro-batch %d", mb, s->pending_g);
+    if (s->pending_g < 0 || s->pending_g != mb) return fail(AST_ERR_ORDER, "accumulate(%d): the last backward was of micro-batch %d", mb, s->pending_g);
     if (s->n_acc >= s->M) return fail(AST_ERR_ORDER, "already accumulated %d micro-batches this round", s->M);
     accumulate(s->G, s->g, s->n_pad, bsums(s, slot_view(s, s->pending_slot)), s->n_bsum, (cudaStream_t)stream);
     CU(cudaGetLastError());

@@ -61,3 +61,28 @@ def test_replay_after_an_import_that_drops_calls(bf16, dropped):
             np.testing.assert_array_equal(a, b)
     finally:
         P.asteroid_stage_destroy(hdl)
+
+
+def test_accumulate_without_a_backward_is_refused():
+    """... whatever micro-batch it names: -1 is also what stands for none."""
+    import paper_2408_08015_b200 as P
+    net = si.block_net(16, 6)
+    last = len(net) - 1
+    x = torch.randn(B, H, W, 16, device="cuda")
+    y, dx = torch.empty_like(x), torch.empty_like(x)
+    hdl = P.asteroid_stage_create(net, 0, last, H, W, B, M)
+    try:
+        P.asteroid_stage_import_state(hdl, np.ascontiguousarray(si.init_params(net, 0, last, 3), np.float32))
+        for mb in (-1, 0, M):
+            with pytest.raises(P.binding.AsteroidError) as e:
+                P.asteroid_stage_accumulate(hdl, mb)
+            assert e.value.code == P.AST_ERR_ORDER
+        P.asteroid_stage_forward(hdl, 0, x.data_ptr(), y.data_ptr())
+        P.asteroid_stage_backward(hdl, 0, y.data_ptr(), dx.data_ptr())
+        P.asteroid_stage_accumulate(hdl, 0)
+        for mb in (-1, 0, 1):
+            with pytest.raises(P.binding.AsteroidError) as e:
+                P.asteroid_stage_accumulate(hdl, mb)
+            assert e.value.code == P.AST_ERR_ORDER
+    finally:
+        P.asteroid_stage_destroy(hdl)

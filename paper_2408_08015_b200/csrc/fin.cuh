@@ -13,7 +13,7 @@
 // accumulator has something in the words for the rest, from subnormal numbers to the largest float, and what is not finite.  There is
 // room for MAX_SUM_BLOCKS partial sums a channel: a launch has at most some 2 000 blocks a channel, the SiLU backward at least one a sample.
 // Before, an accumulator was a double, whose additions are exact only as long as the partial sums lie within 2^-30 of the sum of their
-// magnitudes.  A round of a sixth of MobileNetV2 at batch 4 takes 1635 us, with doubles 1581.  Also exact and slower: two-sums, each addition's rounding
+// magnitudes.  A round of a sixth of MobileNetV2 at batch 4 takes 1639 us, with doubles 1581.  Also exact and slower: two-sums, each addition's rounding
 // taken from the value the atomic addition returns (1743: the kernels wait for it); a second atomic addition for every partial sum, as a
 // checksum beside a double (1753) or as the upper half of a word (1768); four words (1684) or a conversion for each of two (1649).
 #pragma once
@@ -47,10 +47,11 @@ __device__ __forceinline__ void zero_sum(const ChanSums& a, size_t i) {
     a.near[i] = make_longlong2(0, 0);
 }
 __device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
-// The two words as one number: exact where it fits one, else less the last 26 bits of more than 61.  One conversion: each costs 2 % of a round of small maps.
+// The two words as one number, less as many of its last bits as it has beyond 61, rounded to double.  One conversion: each costs 2 % of a round of
+// small maps.
 __device__ __forceinline__ double near_total(const longlong2& n, int shift) {
-    const bool fits = (unsigned long long)(n.y + (1ll << 35)) < (1ull << 36);
-    return (double)(fits ? n.x + (n.y << SUM_STEP) : (n.x >> SUM_STEP) + n.y) * pow2(NEAR_WORD * SUM_STEP - 150 - shift + (fits ? 0 : SUM_STEP));
+    const int top = (int)(n.y >> 32), drop = min(max(29 - __clz(top ^ (top >> 31)), 0), SUM_STEP);       // |n.y| < 2^(35 + drop)
+    return (double)((n.x >> drop) + (n.y << (SUM_STEP - drop))) * pow2(NEAR_WORD * SUM_STEP - 150 - shift + drop);
 }
 // Sums i and j with all their words.
 static __device__ __noinline__ double2 full_totals(longlong2* near, const FarSum* far, int shift, int i, int j) {

@@ -6,7 +6,7 @@ bfloat16 storage with float32 accumulation must meet the stated tolerance agains
 directly: max|gpu-ref| / max|ref| <= 2e-2 (1e-4 in float32 storage) on the stage output, the input gradient,
 every accumulated parameter gradient and every updated parameter, with no outlier allowance and no
 diagnostic criterion.  Sizes cover partial tiles and, for the persistent kernels, more than one tile per CTA
-(more than 148 x 128 pixels).  The kernel trace shows that the intended kernel is the one that ran."""
+(more than 148 x 128 pixels).  The kernel trace shows that the intended kind of kernel ran."""
 import numpy as np
 import pytest
 
@@ -20,7 +20,8 @@ PW = ("pw_fwd_tcgen05", "pw_bwd_data_tcgen05", "pw_bwd_weight_tcgen05")
 C3 = ("conv3x3_fwd_tcgen05", "conv3x3_bwd_data_tcgen05", "conv3x3_bwd_weight_tcgen05")
 DW = ("dw_fwd",)
 CASES = {
-    # pointwise, K and N <= 256: the persistent pipelines; 2 x 101 x 97 = 19 594 pixels = 153.1 tiles of 128
+    # pointwise, K and N <= 256; 2 x 101 x 97 = 19 594 pixels = 153.1 tiles of 128 (the tensor-memory kernels begin at 50 000 pixels:
+    # test_gpu_pointwise_large_maps.py)
     "pw_24_144": (si.single_unit_net("conv", 24, 144), 101, 97, 2, 2, "mse", PW),
     "pw_144_24": (si.single_unit_net("conv", 144, 24), 101, 97, 2, 2, "mse", PW),
     "pw_64_256": (si.single_unit_net("conv", 64, 256), 57, 43, 2, 1, "mse", PW),
@@ -32,8 +33,8 @@ CASES = {
     "pw_512_128": (si.single_unit_net("conv", 512, 128), 29, 27, 3, 1, "mse", PW),
     "pw_512_128_bn": (si.single_unit_net("conv", 512, 128, bn=True), 29, 27, 3, 1, "mse", PW),
     "pw_320_1280_bn": (si.single_unit_net("conv", 320, 1280, bn=True), 7, 7, 5, 1, "mse", PW),
-    # weight gradient on channel sub-ranges with the BatchNorm-backward transform on the wide side: four sub-ranges of 128
-    # (512 channels), two of 192 (384 channels, where a quarter is no multiple of 64)
+    # weight gradient with the BatchNorm-backward transform on the wide side, 512 and 384 channels (its pipeline on channel sub-ranges begins
+    # beyond 4 096 pixels: test_gpu_pointwise_large_maps.py)
     "pw_128_512_bn": (si.single_unit_net("conv", 128, 512, bn=True), 29, 27, 3, 1, "mse", PW),
     "pw_128_384_bn": (si.single_unit_net("conv", 128, 384, bn=True), 23, 21, 3, 1, "mse", PW),
     # strided 1x1 (projection shortcut) on an odd-sized map

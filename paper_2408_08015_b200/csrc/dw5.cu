@@ -73,13 +73,12 @@ __global__ void __launch_bounds__(BT) dw5_fwd_kernel(const DwFwdArgs a) {
         place();
         fetch(oh0 * S - 2);
     }
+    const bool stats = (bool)a.so.sums;
+    float2 piv = stats && live ? ld2(a.so.pivot + c0) : zero2();
     stage_val(a.x, a.pf, cb, width, g.c, a.first && blockIdx.x == 0, sm);
     __syncthreads();
     const float2 sc = ld2(sm + 2 * jl), sh = ld2(sm + width + 2 * jl);
-    float2 piv = zero2();
-    const bool stats = (bool)a.so.sums;
     if (stats && live) {
-        piv = ld2(a.so.pivot + c0);
         if (blockIdx.x == 0 && row == 0) *reinterpret_cast<float2*>(a.so.pivot_copy + c0) = piv;
         piv = make_float2(-piv.x, -piv.y);
     }
@@ -200,15 +199,7 @@ template <typename T, int XF> struct Coef1 {
     }
 };
 template <typename T, int XF> __device__ __forceinline__ Coef1<T, XF> coefs1(const DwBwdArgs& a, int cb, int width, int jl, float* sm) {
-    stage_grad(a.dz, a.pb, cb, width, a.g.c, a.first && blockIdx.x == 0, sm);
-    float* s = sm + 5 * width;
-    stage_val(a.x, BnPendFwd{}, cb, width, a.g.c, false, s);
-    for (int i = threadIdx.x; i < width; i += blockDim.x) {
-        const bool ok = a.sums && cb + i < a.g.c;
-        const float r = ok ? a.rstd[cb + i] : 0.f;
-        s[2 * width + i] = r;
-        s[3 * width + i] = ok ? -a.mean[cb + i] * r : 0.f;
-    }
+    stage_bwd(a.dz, a.pb, a.x, a.sums ? a.mean : nullptr, a.sums ? a.rstd : nullptr, cb, width, a.g.c, a.first && blockIdx.x == 0, sm);
     __syncthreads();
     const float* p = sm + jl;
     Coef1<T, XF> k;

@@ -94,12 +94,18 @@ struct TwoSums {
 // estimates keep.  Arithmetic in double, as the standalone finishing kernels of bn_ew.cu.
 struct BnFwdIn {
     TwoSums s;
-    float pivot, gamma, beta;
-    __device__ __forceinline__ void load(const BnPendFwd& b, int ch) {
+    float pivot, gamma, beta, run_mean, run_var;
+    // everything `coef` needs, the running estimates too: read there they are another trip to memory, and the CTA that writes is the one the
+    // kernel behind waits for
+    __device__ __forceinline__ void load(const BnPendFwd& b, int ch, bool write) {
         s.load(b.sums, ch, b.c + ch);
         pivot = b.pivot[ch];
         gamma = b.gamma[ch];
         beta = b.beta[ch];
+        if (write) {
+            run_mean = b.o.run_mean[ch];
+            run_var = b.o.run_var[ch];
+        }
     }
     __device__ __forceinline__ float2 coef(const BnPendFwd& b, int ch, bool write) const {
         double s1, s2;
@@ -114,15 +120,15 @@ struct BnFwdIn {
             b.o.rstd[ch] = (float)rstd;
             b.o.scale[ch] = r.x;
             b.o.shift[ch] = r.y;
-            b.o.run_mean[ch] = (float)((1.0 - b.momentum) * b.o.run_mean[ch] + b.momentum * mean);
-            b.o.run_var[ch] = (float)((1.0 - b.momentum) * b.o.run_var[ch] + b.momentum * (var * b.unbias));
+            b.o.run_mean[ch] = (float)((1.0 - b.momentum) * run_mean + b.momentum * mean);
+            b.o.run_var[ch] = (float)((1.0 - b.momentum) * run_var + b.momentum * (var * b.unbias));
         }
         return r;
     }
 };
 __device__ __forceinline__ float2 bn_fwd_coef(const BnPendFwd& b, int ch, bool write) {
     BnFwdIn in;
-    in.load(b, ch);
+    in.load(b, ch, write);
     return in.coef(b, ch, write);
 }
 

@@ -96,48 +96,65 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
     int tile = blockIdx.x;
     fetch(tile, 0);
     const bool first = blockIdx.x == 0 && blockIdx.y == 0;
+    // everything a thread reads from memory is requested before it uses anything; BN <= NT: a column a thread
+    const bool sums = (bool)a.so.sums, col = sums && tid < BN && n0 + tid < a.N;
+    float nr = 0.f, ns = 0.f, nh = 0.f, nm = 0.f;
+    if (col) {
+        if (BWD) {
+            nr = a.r_rstd[n0 + tid];
+            ns = a.r_scale[n0 + tid];
+            nh = a.r_shift[n0 + tid];
+            nm = a.r_mean[n0 + tid];
+        } else nm = a.so.pivot[n0 + tid];
+    }
     if (XF)
         for (int c = tid; c < a.K; c += NT) {
             if (BWD) {
                 float3 k = make_float3(1.f, 0.f, 0.f);
-                if (a.pb.sums) k = bn_bwd_coef(a.pb, c, first);
+                float s = 1.f, h = 0.f;
+                BnBwdIn in;
+                if (a.pb.sums) in.load(a.pb, c);
                 else if (a.c0) k = make_float3(a.c0[c], a.c1[c], a.c2[c]);
+                if (a.c3) {
+                    s = a.c3[c];
+                    h = a.c4[c];
+                }
+                if (a.pb.sums) k = in.coef(a.pb, c, first);
                 sK[c] = k.x;
                 sK[Kp + c] = k.y;
                 sK[2 * Kp + c] = k.z;
-                sK[3 * Kp + c] = a.c3 ? a.c3[c] : 1.f;
-                sK[4 * Kp + c] = a.c3 ? a.c4[c] : 0.f;
+                sK[3 * Kp + c] = s;
+                sK[4 * Kp + c] = h;
             } else {
-                float2 k = make_float2(1.f, 0.f);
-                if (a.pf.sums) k = bn_fwd_coef(a.pf, c, first);
+                float2 k = make_float2(1.f, 0.f), k2 = k;
+                BnFwdIn in, in2;
+                if (a.pf.sums) in.load(a.pf, c, first);
                 else if (a.c0) k = make_float2(a.c0[c], a.c1[c]);
+                if (XF == XF_ADD) {
+                    if (a.pf2.sums) in2.load(a.pf2, c, first);
+                    else if (a.d0) k2 = make_float2(a.d0[c], a.d1[c]);
+                }
+                if (a.pf.sums) k = in.coef(a.pf, c, first);
                 sK[c] = k.x;
                 if (XF == XF_ADD) {
-                    float2 k2 = make_float2(1.f, 0.f);
-                    if (a.pf2.sums) k2 = bn_fwd_coef(a.pf2, c, first);
-                    else if (a.d0) k2 = make_float2(a.d0[c], a.d1[c]);
+                    if (a.pf2.sums) k2 = in2.coef(a.pf2, c, first);
                     sK[2 * Kp + c] = k2.x;
                     k.y += k2.y;
                 }
                 sK[Kp + c] = k.y;
             }
         }
-    const bool sums = (bool)a.so.sums;
-    if (sums)
-        for (int c = tid; c < BN; c += NT) {
-            const bool ok = n0 + c < a.N;
-            if (BWD) {
-                const float rs = ok ? a.r_rstd[n0 + c] : 0.f;
-                sN[c] = ok ? a.r_scale[n0 + c] : 0.f;
-                sN[BN + c] = ok ? a.r_shift[n0 + c] : 0.f;
-                sN[2 * BN + c] = rs;
-                sN[3 * BN + c] = ok ? -a.r_mean[n0 + c] * rs : 0.f;
-            } else {
-                const float p = ok ? a.so.pivot[n0 + c] : 0.f;
-                sN[c] = p;
-                if (ok && blockIdx.x == 0) a.so.pivot_copy[n0 + c] = p;
-            }
+    if (sums && tid < BN) {
+        if (BWD) {
+            sN[tid] = ns;
+            sN[BN + tid] = nh;
+            sN[2 * BN + tid] = nr;
+            sN[3 * BN + tid] = -nm * nr;
+        } else {
+            sN[tid] = nm;
+            if (col && blockIdx.x == 0) a.so.pivot_copy[n0 + tid] = nm;
         }
+    }
     cp_wait<0>();
     __syncthreads();
 

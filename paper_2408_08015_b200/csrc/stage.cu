@@ -885,8 +885,10 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 }
                 d.k1 = kc; d.k2 = kc + o.c; d.k3 = kc + 2 * (size_t)o.c;
             }
-            if (u.b_off >= 0) {
-                bias_grad(dt, d.dy, d.z, o.elems / o.c, o.c, u.act, s->scratch, s->scratch_floats, s->g + u.b_off, st);
+            if (u.b_off >= 0) {                    // nothing of the pass depends on it: on the second stream, 14 us in front of everything else otherwise
+                int frc = fork();
+                if (frc) return frc;
+                bias_grad(dt, d.dy, d.z, o.elems / o.c, o.c, u.act, wscratch, s->scratch_floats, s->g + u.b_off, wst);
             }
             // pending coefficients stay pending where both kernels of the unit can form them
             MmaTiling til_d{};

@@ -149,6 +149,7 @@ struct DwBwdArgs {
     ChanSums gw;                 // [taps][c] accumulators of the weight gradient
     ChanSums sums;               // [2][c] of the unit that produced x, or none
     const float *mean, *rstd;    // of that unit
+    bool mask;                   // dx is stored as that unit's activation lets it through
     bool first;
 };
 

@@ -160,33 +160,39 @@ __global__ void __launch_bounds__(BT) dw3_fwd_kernel(const DwFwdArgs a) {
 // ------------------------------------------------------------------------------------------ backward
 // Coefficients of a thread's two channels, in registers for the kernel's life: the gradient's transform, the input's, and what the sums
 // of the unit in front need.  Two pixels of two channels at a time go through packed arithmetic.
-template <typename T, bool XF> struct BwdCoef {
+enum { Z_PLAIN = 0, Z_AFFINE = 1, Z_ACT = 2 };          // the gradient's transform: none, BatchNorm's, BatchNorm's behind an activation
+template <typename T, int XF> struct BwdCoef {
     float2 k1, k2, k3, zs, zh, sc, sh, rs, rm;
     float zlo, zhi, xlo, xhi;
     // dz = k1*dy*[lo < pre < hi] + k2 + k3*z
     __device__ __forceinline__ float2 grad(const P2<T>& rd, const P2<T>& rz) const {
         float2 o = rd.get();
-        if (XF) {
-            const float2 z = rz.get(), pre = __ffma2_rn(z, zs, zh);
-            float2 d;
-            d.x = pre.x > zlo && pre.x < zhi ? o.x : 0.f;
-            d.y = pre.y > zlo && pre.y < zhi ? o.y : 0.f;
-            o = __ffma2_rn(k1, d, __ffma2_rn(k3, z, k2));
+        if (XF != Z_PLAIN) {
+            const float2 z = rz.get();
+            if (XF == Z_ACT) {
+                const float2 pre = __ffma2_rn(z, zs, zh);
+                o.x = pre.x > zlo && pre.x < zhi ? o.x : 0.f;
+                o.y = pre.y > zlo && pre.y < zhi ? o.y : 0.f;
+            }
+            o = __ffma2_rn(k1, o, __ffma2_rn(k3, z, k2));
         }
         return o;
     }
-    // dx as stored and the raw input of its position -> the sums
-    __device__ __forceinline__ void add(const float2& dx, const float2& raw, float2* s) const {
+    // dx of a position whose raw input is given: stored, and as stored into the sums
+    __device__ __forceinline__ void put(void* p, uint32_t e, float2 dx, const float2& raw, bool mask, float2* s) const {
         const float2 pre = __ffma2_rn(raw, sc, sh), xh = __ffma2_rn(raw, rs, rm);
+        const bool mx = pre.x > xlo && pre.x < xhi, my = pre.y > xlo && pre.y < xhi;
+        if (mask) dx = make_float2(mx ? dx.x : 0.f, my ? dx.y : 0.f);
+        const float2 v = P2<T>::put(p, e, dx);
         float2 d;
-        d.x = pre.x > xlo && pre.x < xhi ? dx.x : 0.f;
-        d.y = pre.y > xlo && pre.y < xhi ? dx.y : 0.f;
+        d.x = mx ? v.x : 0.f;
+        d.y = my ? v.y : 0.f;
         s[0] = __fadd2_rn(s[0], d);
         s[1] = __ffma2_rn(d, xh, s[1]);
     }
 };
 // shared memory of a backward block until its sums: gradient coefficients [5][width], input coefficients [4][width]
-template <typename T, bool XF>
+template <typename T, int XF>
 __device__ __forceinline__ BwdCoef<T, XF> bwd_coefs(const DwBwdArgs& a, int cb, int width, int jl, float* sm) {
     stage_bwd(a.dz, a.pb, a.x, a.sums ? a.mean : nullptr, a.sums ? a.rstd : nullptr, cb, width, a.g.c, a.first && blockIdx.x == 0, sm);
     __syncthreads();
@@ -208,7 +214,7 @@ __device__ __forceinline__ BwdCoef<T, XF> bwd_coefs(const DwBwdArgs& a, int cb, 
     return k;
 }
 
-template <typename T, int TW, bool XF, bool EX>
+template <typename T, int TW, int XF, bool EX>
 __global__ void __launch_bounds__(BT, 3) dw3_bwd_s1_kernel(const DwBwdArgs a) {
     pdl_launch();
     constexpr int NZ = TW + 2;
@@ -237,7 +243,7 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s1_kernel(const DwBwdArgs a) {
 #pragma unroll
         for (int q = 0; q < NZ; ++q) {
             nd[q].load(a.dz.dy, rb + col[q]);
-            if (XF) nz[q].load(a.dz.z, rb + col[q]);
+            if (XF != Z_PLAIN) nz[q].load(a.dz.z, rb + col[q]);
         }
     };
     auto fetch_x = [&](int r) {
@@ -308,8 +314,7 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s1_kernel(const DwBwdArgs a) {
 #pragma unroll
                 for (int t = 0; t < TW; ++t)
                     if (EX || wo0 + t < g.wi) {
-                        const float2 v = P2<T>::put(a.dx, rb + col[t + 1], o[t]);
-                        k.add(v, raw[t], fs);
+                        k.put(a.dx, rb + col[t + 1], o[t], raw[t], a.mask, fs);
                     }
             };
             for (int ih = r0;;) {
@@ -331,7 +336,7 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s1_kernel(const DwBwdArgs a) {
 
 // Stride 2: dz(i, j) meets input rows 2i-1..2i+1 and columns 2j-1..2j+1, so the 2x2 input positions (2i + a, 2j + b) need dz(i, j), and where
 // a or b is 1 also dz(i+1, .) and dz(., j+1).  A thread owns TZ columns of dz = 2*TZ input columns and walks down the rows of dz.
-template <typename T, int TZ, bool XF, bool EX>
+template <typename T, int TZ, int XF, bool EX>
 __global__ void __launch_bounds__(BT, 3) dw3_bwd_s2_kernel(const DwBwdArgs a) {
     pdl_launch();
     extern __shared__ __align__(16) float sm[];
@@ -362,7 +367,7 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s2_kernel(const DwBwdArgs a) {
 #pragma unroll
         for (int q = 0; q <= TZ; ++q) {
             nd[q].load(a.dz.dy, rb + zcol[q]);
-            if (XF) nz[q].load(a.dz.z, rb + zcol[q]);
+            if (XF != Z_PLAIN) nz[q].load(a.dz.z, rb + zcol[q]);
         }
     };
     auto fetch_x = [&](int i) {
@@ -451,8 +456,7 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s2_kernel(const DwBwdArgs a) {
 #pragma unroll
                     for (int q = 0; q < 2 * TZ; ++q)
                         if (ok[q]) {
-                            const float2 v = P2<T>::put(a.dx, rb + xcol[q], o[q]);
-                            k.add(v, raw[h][q], fs);
+                            k.put(a.dx, rb + xcol[q], o[q], raw[h][q], a.mask, fs);
                         }
                 }
             };
@@ -519,16 +523,18 @@ void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf,
 }
 
 void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* wkc, const void* addend, void* dx, const ChanSums& gw,
-             const ChanSums& sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st) {
+             const ChanSums& sums, const float* mean, const float* rstd, bool mask, const DwTiling& t, cudaStream_t st) {
     typedef void (*Fn)(const DwBwdArgs);
     using B = __nv_bfloat16;
-    const bool xf = grad_needs_z(dz) || pb.sums;
+    const int xf = dz.act != ACT_NONE ? Z_ACT : dz.k1 || pb.sums ? Z_AFFINE : Z_PLAIN;
     Fn f;
     const bool ex = (g.stride == 1 ? g.wi : g.wo) % t.tw == 0;
-#define DW3_BWD(K, T, TW) (xf ? ex ? (Fn)K<T, TW, true, true> : (Fn)K<T, TW, true, false> : ex ? (Fn)K<T, TW, false, true> : (Fn)K<T, TW, false, false>)
+#define DW3_X(K, T, TW, XF) (ex ? (Fn)K<T, TW, XF, true> : (Fn)K<T, TW, XF, false>)
+#define DW3_BWD(K, T, TW) (xf == Z_ACT ? DW3_X(K, T, TW, Z_ACT) : xf == Z_AFFINE ? DW3_X(K, T, TW, Z_AFFINE) : DW3_X(K, T, TW, Z_PLAIN))
     if (g.stride == 1) f = dtype == 0 ? DW3_BWD(dw3_bwd_s1_kernel, float, 2) : t.tw == 4 ? DW3_BWD(dw3_bwd_s1_kernel, B, 4) : DW3_BWD(dw3_bwd_s1_kernel, B, 2);
     else f = dtype == 0 ? DW3_BWD(dw3_bwd_s2_kernel, float, 2) : DW3_BWD(dw3_bwd_s2_kernel, B, 2);
 #undef DW3_BWD
+#undef DW3_X
     const int rows_out = g.stride == 1 ? g.hi : g.ho, cols_out = g.stride == 1 ? g.wi : g.wo;
     const double in_e = (double)g.hi * g.wi * g.ci, out_e = (double)g.ho * g.wo * g.ci;
     const int chunk = image_chunk(dtype, g), launches = (g.n + chunk - 1) / chunk;
@@ -536,7 +542,7 @@ void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& p
         const int n = g.n - n0 < chunk ? g.n - n0 : chunk;
         const size_t ie = (size_t)n0 * g.hi * g.wi * g.ci, oe = (size_t)n0 * g.ho * g.wo * g.ci;
         DwBwdArgs a{};
-        a.dz = dz; a.pb = pb; a.x = x; a.wkc = wkc; a.gw = gw; a.sums = dx ? sums : ChanSums{}; a.mean = mean; a.rstd = rstd; a.first = n0 == 0;
+        a.dz = dz; a.pb = pb; a.x = x; a.wkc = wkc; a.gw = gw; a.sums = dx ? sums : ChanSums{}; a.mean = mean; a.rstd = rstd; a.mask = mask; a.first = n0 == 0;
         a.dz.dy = at(dz.dy, oe, dtype);
         a.dz.z = at(dz.z, oe, dtype);
         a.x.p = at(x.p, ie, dtype);

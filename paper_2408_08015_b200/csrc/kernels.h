@@ -132,6 +132,7 @@ struct BnRed {
     int act;
     float* partial;          // [blocks][2][c]
     size_t partial_floats;
+    bool mask;               // register-operand and float32 kernels: dy is stored with zeros where the activation passes none of it on
 };
 
 // ---- dense convolution as implicit GEMM (plain FFMA tiles; float and bfloat16 storage) ----
@@ -205,9 +206,10 @@ struct DwSettle {
 };
 DwTiling dw3_choose(int dtype, bool bwd, const ConvGeom& g);
 void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf, const float* w9c, void* z, const BnSumsOut& so, const DwTiling& t, cudaStream_t st);
-// dx may be null (weight gradient only); gw: [9][c] accumulators; sums [2][c] (may be null), mean, rstd: of the unit that produced x
+// dx may be null (weight gradient only); gw: [9][c] accumulators; sums [2][c] (may be null), mean, rstd: of the unit that produced x; mask: dx is
+// stored with zeros where that unit's activation passes none of it on
 void dw3_bwd(int dtype, const ConvGeom& g, const GradSrc& dz, const BnPendBwd& pb, const ValSrc& x, const float* w9c, const void* addend, void* dx, const ChanSums& gw,
-             const ChanSums& sums, const float* mean, const float* rstd, const DwTiling& t, cudaStream_t st);
+             const ChanSums& sums, const float* mean, const float* rstd, bool mask, const DwTiling& t, cudaStream_t st);
 // the same for 5x5 layers (dw5.cu)
 DwTiling dw5_choose(int dtype, bool bwd, const ConvGeom& g);
 void dw5_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf, const float* wkc, void* z, const BnSumsOut& so, const DwTiling& t, cudaStream_t st);

@@ -42,6 +42,7 @@ struct F32Args {
     const float* rz;           // backward sums: raw output of the unit whose gradient this is
     const float *r_scale, *r_shift, *r_mean, *r_rstd;
     float r_lo, r_hi;
+    bool r_mask;               // the output is stored as that unit's activation lets it through
 };
 
 __device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
@@ -55,7 +56,8 @@ __device__ __forceinline__ float grad1(float d, float z, float k1, float k2, flo
 // that the float4 fragments of both operands (four k of one row) feed packed FMAs as they are: 4 + TN shared-memory reads for 8*TN of them.
 // WK warps share a tile's reduction where the map is small.  The operand goes global -> registers (one chunk ahead) -> transform -> shared memory;
 // the weights of the CTA's columns stay in shared memory, row order permuted so that a lane's columns come in groups of G consecutive ones.
-enum { XF_NONE = 0, XF_VALUE = 1, XF_ADD = 2 };
+// Operand transform: XF_VALUE BatchNorm and activation, XF_ADD (forward) a residual sum, XF_AFFINE (backward) BatchNorm of a gradient stored masked
+enum { XF_NONE = 0, XF_VALUE = 1, XF_ADD = 2, XF_AFFINE = 2 };
 template <bool BWD, int TN, int WK, int XF>
 __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
     pdl_launch();
@@ -123,8 +125,10 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
                 sK[c] = k.x;
                 sK[Kp + c] = k.y;
                 sK[2 * Kp + c] = k.z;
-                sK[3 * Kp + c] = s;
-                sK[4 * Kp + c] = h;
+                if (XF == XF_VALUE) {
+                    sK[3 * Kp + c] = s;
+                    sK[4 * Kp + c] = h;
+                }
             } else {
                 float2 k = make_float2(1.f, 0.f), k2 = k;
                 BnFwdIn in, in2;
@@ -176,12 +180,20 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
                 if (BWD) {
                     float4 k1, k2, k3, s, h;
                     if (XF) {
-                        k1 = ld4(sK + k); k2 = ld4(sK + Kp + k); k3 = ld4(sK + 2 * Kp + k); s = ld4(sK + 3 * Kp + k); h = ld4(sK + 4 * Kp + k);
+                        k1 = ld4(sK + k); k2 = ld4(sK + Kp + k); k3 = ld4(sK + 2 * Kp + k);
+                    }
+                    if (XF == XF_VALUE) {
+                        s = ld4(sK + 3 * Kp + k); h = ld4(sK + 4 * Kp + k);
                     }
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         float4 v = nx[j];
-                        if (XF) {
+                        if (XF == XF_AFFINE) {
+                            v.x = fmaf(k1.x, v.x, fmaf(k3.x, nz[j].x, k2.x));
+                            v.y = fmaf(k1.y, v.y, fmaf(k3.y, nz[j].y, k2.y));
+                            v.z = fmaf(k1.z, v.z, fmaf(k3.z, nz[j].z, k2.z));
+                            v.w = fmaf(k1.w, v.w, fmaf(k3.w, nz[j].w, k2.w));
+                        } else if (XF) {
                             v.x = grad1(v.x, nz[j].x, k1.x, k2.x, k3.x, s.x, h.x, a.lo, a.hi);
                             v.y = grad1(v.y, nz[j].y, k1.y, k2.y, k3.y, s.y, h.y, a.lo, a.hi);
                             v.z = grad1(v.z, nz[j].z, k1.z, k2.z, k3.z, s.z, h.z, a.lo, a.hi);
@@ -304,6 +316,7 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
                             const float pre = fmaf(rz[i][q], c0, c1), xh = fmaf(rz[i][q], c2, c3), g = pre > a.r_lo && pre < a.r_hi ? v[i][j] : 0.f;
                             s1[j] += g;
                             s2[j] = fmaf(g, xh, s2[j]);
+                            if (a.r_mask) v[i][j] = g;
                         } else {
                             const float dd = v[i][j] - c0;
                             s1[j] += dd;
@@ -561,7 +574,7 @@ typedef void (*Fn)(const F32Args);
 template <bool BWD, int TN, int XF> Fn by_wk(int wk) { return wk == 1 ? pw_f32_kernel<BWD, TN, 1, XF> : wk == 2 ? pw_f32_kernel<BWD, TN, 2, XF> : pw_f32_kernel<BWD, TN, 4, XF>; }
 template <bool BWD, int XF> Fn by_tn(const F32Tiling& c) { return c.tn == 4 ? by_wk<BWD, 4, XF>(c.wk) : c.tn == 6 ? by_wk<BWD, 6, XF>(c.wk) : by_wk<BWD, 8, XF>(c.wk); }
 Fn kernel_for(bool bwd, int xf, const F32Tiling& c) {
-    if (bwd) return xf ? by_tn<true, XF_VALUE>(c) : by_tn<true, XF_NONE>(c);
+    if (bwd) return xf == XF_AFFINE ? by_tn<true, XF_AFFINE>(c) : xf ? by_tn<true, XF_VALUE>(c) : by_tn<true, XF_NONE>(c);
     return xf == XF_ADD ? by_tn<false, XF_ADD>(c) : xf ? by_tn<false, XF_VALUE>(c) : by_tn<false, XF_NONE>(c);
 }
 
@@ -618,8 +631,8 @@ void f32_launch(bool bwd, const MmaProblem& p, const F32Tiling& c, int kind, dou
     if (!(done.load(std::memory_order_acquire) & bit)) {
         for (int tn : {4, 6, 8})
             for (int wk : {1, 2, 4})
-                for (int v = 0; v < 5; ++v)
-                    cudaFuncSetAttribute(kernel_for(v < 2, v < 2 ? v : v - 2, F32Tiling{tn, wk, 0}), cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+                for (int v = 0; v < 6; ++v)
+                    cudaFuncSetAttribute(kernel_for(v < 3, v % 3, F32Tiling{tn, wk, 0}), cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         done.fetch_or(bit, std::memory_order_release);
     }
     F32Args a;
@@ -631,7 +644,7 @@ void f32_launch(bool bwd, const MmaProblem& p, const F32Tiling& c, int kind, dou
         a.a = (const float*)p.dz.dy; a.az = (const float*)p.dz.z;
         a.c0 = p.dz.k1; a.c1 = p.dz.k2; a.c2 = p.dz.k3; a.c3 = p.dz.scale; a.c4 = p.dz.shift;
         a.pb = p.pb;
-        xf = act != ACT_NONE || p.dz.k1 || p.pb.sums ? XF_VALUE : XF_NONE;
+        xf = act != ACT_NONE ? XF_VALUE : p.dz.k1 || p.pb.sums ? XF_AFFINE : XF_NONE;
     } else {
         a.a = (const float*)p.x.p;
         a.c0 = p.x.scale; a.c1 = p.x.shift;
@@ -652,6 +665,7 @@ void f32_launch(bool bwd, const MmaProblem& p, const F32Tiling& c, int kind, dou
     if (p.red) {
         a.rz = (const float*)p.red->z;
         a.r_scale = p.red->scale; a.r_shift = p.red->shift; a.r_mean = p.red->mean; a.r_rstd = p.red->rstd;
+        a.r_mask = p.red->mask;
         a.r_lo = p.red->act == ACT_NONE ? -INFINITY : 0.f;
         a.r_hi = p.red->act == ACT_RELU6 ? 6.f : INFINITY;
     }

@@ -213,6 +213,7 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
         a.rz = (const __nv_bfloat16*)p.red->z;
         a.r_scale = p.red->scale; a.r_shift = p.red->shift; a.r_mean = p.red->mean; a.r_rstd = p.red->rstd;
         a.r_act = p.red->act;
+        a.r_mask = p.red->mask;
     }
     if (bwd) raise_limits<true>();
     else raise_limits<false>();

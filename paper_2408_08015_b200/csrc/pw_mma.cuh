@@ -48,6 +48,7 @@ struct Args {
     const __nv_bfloat16* rz;   // backward sums: raw output [P][N] of the unit whose gradient this is, its coefficients and activation
     const float *r_scale, *r_shift, *r_mean, *r_rstd;
     int r_act;
+    bool r_mask;               // the output is stored as that unit's activation lets it through
 };
 
 __device__ __forceinline__ void mma16816(float* c, const uint32_t a0, const uint32_t a1, const uint32_t a2, const uint32_t a3, const uint32_t b0, const uint32_t b1) {
@@ -270,15 +271,16 @@ template <int C> struct CVec {
         else *reinterpret_cast<uint32_t*>(q) = w[0];
     }
 };
-// the stored pair's contribution to the two sums of its channels
+// the pair's contribution to the two sums of its channels; returns the pair as it is to be stored
 template <bool BWD> struct SumCoef;
 template <> struct SumCoef<false> {
     float2 pv;
     __device__ __forceinline__ void load(const float* sN, int, int c) { pv = make_float2(-sN[c], -sN[c + 1]); }
-    __device__ __forceinline__ void add(uint32_t d, uint32_t, float, float, float2& s1, float2& s2) const {
+    __device__ __forceinline__ uint32_t add(uint32_t d, uint32_t, float, float, bool, float2& s1, float2& s2) const {
         const float2 q = __fadd2_rn(unpack2(d), pv);
         s1 = __fadd2_rn(s1, q);
         s2 = __ffma2_rn(q, q, s2);
+        return d;
     }
 };
 template <> struct SumCoef<true> {
@@ -289,13 +291,14 @@ template <> struct SumCoef<true> {
         rs = *reinterpret_cast<const float2*>(sN + 2 * BN + c);
         rm = *reinterpret_cast<const float2*>(sN + 3 * BN + c);
     }
-    __device__ __forceinline__ void add(uint32_t d, uint32_t z, float lo, float hi, float2& s1, float2& s2) const {
+    __device__ __forceinline__ uint32_t add(uint32_t d, uint32_t z, float lo, float hi, bool mask, float2& s1, float2& s2) const {
         const float2 zz = unpack2(z), pre = __ffma2_rn(zz, sc, sh), xh = __ffma2_rn(zz, rs, rm);
         float2 q = unpack2(d);
         if (!(pre.x > lo && pre.x < hi)) q.x = 0.f;
         if (!(pre.y > lo && pre.y < hi)) q.y = 0.f;
         s1 = __fadd2_rn(s1, q);
         s2 = __ffma2_rn(q, xh, s2);
+        return mask ? __byte_perm(__float_as_uint(q.x), __float_as_uint(q.y), 0x7632) : d;
     }
 };
 
@@ -445,7 +448,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
                         if (BWD && a.addend) v = __fadd2_rn(v, unpack2(av[gr & 1][mi][h].w[q]));
                         if (!BWD && a.bias) v = __fadd2_rn(v, make_float2(__ldg(a.bias + n + 2 * q), __ldg(a.bias + n + 2 * q + 1)));
                         ov.w[q] = pack2(v);
-                        if (sums) sc[q].add(ov.w[q], BWD ? zv[gr][mi][h].w[q] : 0u, rlo, rhi, s1[gr * G + q], s2[gr * G + q]);
+                        if (sums) ov.w[q] = sc[q].add(ov.w[q], BWD ? zv[gr][mi][h].w[q] : 0u, rlo, rhi, BWD && a.r_mask, s1[gr * G + q], s2[gr * G + q]);
                     }
                     ov.store(a.out, e);
                 }
@@ -602,7 +605,7 @@ __global__ void __launch_bounds__(256) pw_mma_split_kernel(const Args a) {
                 if (sums) {
                     SumCoef<BWD> sc;
                     sc.load(sN, BN, ej * 8 + 2 * q);
-                    sc.add(wo[q], wz[q], rlo, rhi, s1[q], s2[q]);
+                    wo[q] = sc.add(wo[q], wz[q], rlo, rhi, BWD && a.r_mask, s1[q], s2[q]);
                 }
             }
             reinterpret_cast<uint4*>(a.out)[e] = make_uint4(wo[0], wo[1], wo[2], wo[3]);

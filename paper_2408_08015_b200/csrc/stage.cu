@@ -847,6 +847,9 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
     GatedGrad gated;
     std::vector<char> reduced(s->units.size(), 0);   // BatchNorm-backward sums already taken by the kernel that wrote dy
     Pending pend(s, sv, st);                         // ... and not yet turned into coefficients
+    // The kernel that takes a unit's sums forms its activation's mask for them anyway.  Where it can it stores the gradient masked, and the two or three kernels
+    // that read it are spared the mask, a third of their transform.
+    std::vector<char> masked(s->units.size(), 0);
     std::fill(s->bwd_sums_by.begin(), s->bwd_sums_by.end(), -1);
     // weight gradients go to the second stream (not while a profile run times the units one by one, nor while a
     // per-launch trace brackets every kernel with events: a kernel's duration is then that of the kernel running alone)
@@ -875,10 +878,12 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             GradSrc d{};
             d.dy = go.ptr;
             d.z = sv.base + o.buf_off;
-            d.act = u.act;
+            d.act = masked[ui] ? ACT_NONE : u.act;
             if (u.l_bn >= 0) {
-                d.scale = stt + 2 * (size_t)o.c;
-                d.shift = stt + 3 * (size_t)o.c;
+                if (!masked[ui]) {
+                    d.scale = stt + 2 * (size_t)o.c;
+                    d.shift = stt + 3 * (size_t)o.c;
+                }
                 if (!reduced[ui]) {
                     bn_bwd_reduce(dt, d.dy, d.z, o.elems / o.c, o.c, d.scale, d.shift, u.act, stt, stt + o.c, bsums(s, sv) + 2 * u.sum_off, s->scratch_floats, st);
                     pend.unit[ui] = 1;
@@ -930,7 +935,10 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                 void* to = want_in ? own(u.in) : nullptr;
                 const float* trs = ts ? ts + u.g.ci : nullptr;
                 if (u.g.k == 5) dw5_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, bsums(s, sv) + u.acc_off, sums, ts, trs, dw5_choose(dt, true, u.g), st);
-                else dw3_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, bsums(s, sv) + u.acc_off, sums, ts, trs, dw3_choose(dt, true, u.g), st);
+                else {
+                    if (tgt >= 0) masked[tgt] = s->units[tgt].act != ACT_NONE;
+                    dw3_bwd(dt, u.g, d, pb, xin, s->derived + u.w_off, addend, to, bsums(s, sv) + u.acc_off, sums, ts, trs, tgt >= 0 && masked[tgt], dw3_choose(dt, true, u.g), st);
+                }
                 if (want_in) {
                     gi.state = G_OWNED;
                     gi.ptr = own(u.in);
@@ -987,7 +995,8 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                         const Unit& tu = s->units[tgt];
                         const Val& tv = s->vals[tu.out];
                         float* ts = sv.stats + tv.stat_off;
-                        red = BnRed{sv.base + tv.buf_off, ts + 2 * (size_t)tv.c, ts + 3 * (size_t)tv.c, ts, ts + tv.c, tu.act, nullptr, 0};
+                        masked[tgt] = tgt == s->vals[u.in].unit && tu.act != ACT_NONE;      // through an alias the gradient is another value's too
+                        red = BnRed{sv.base + tv.buf_off, ts + 2 * (size_t)tv.c, ts + 3 * (size_t)tv.c, ts, ts + tv.c, tu.act, nullptr, 0, masked[tgt] != 0};
                         p.red = &red;
                         p.so = BnSumsOut{bsums(s, sv) + 2 * tu.sum_off, nullptr, nullptr};
                         pend.unit[tgt] = 1;
@@ -1003,7 +1012,7 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
                         const Unit& tu = s->units[tgt];
                         const Val& tv = s->vals[tu.out];
                         float* ts = sv.stats + tv.stat_off;
-                        red = BnRed{sv.base + tv.buf_off, ts + 2 * (size_t)tv.c, ts + 3 * (size_t)tv.c, ts, ts + tv.c, tu.act, s->scratch, s->scratch_floats};
+                        red = BnRed{sv.base + tv.buf_off, ts + 2 * (size_t)tv.c, ts + 3 * (size_t)tv.c, ts, ts + tv.c, tu.act, s->scratch, s->scratch_floats, false};
                     }
                     const int blocks = pw_bwd_data_tc(u.g, d, s->wtb + u.w_off, addend, own(u.in), tgt >= 0 ? &red : nullptr, s->err, st);
                     if (blocks > 0) {

@@ -709,24 +709,25 @@ __global__ void __launch_bounds__(C3_THREADS) conv3_wgrad_tc_kernel(const W3Args
     (void)kbi; (void)kbo;
 }
 
-// out[i] = sum over splits of partial[split][i], n a multiple of 4.  A block finishes 128 consecutive outputs: warp kg adds
-// the splits kg, kg+32, ... (each lane four consecutive outputs: 512 contiguous bytes per split and warp, all of a
-// thread's loads issued before the additions), the 32 sub-sums are combined in index order through shared memory.
-__global__ void __launch_bounds__(1024) reduce_splits_c3(const float* __restrict__ partial, int splits, size_t n, float* __restrict__ out) {
+// out[i] = sum over splits of partial[split][i], n a multiple of 4.  A block of W warps finishes 128 consecutive outputs: warp kg adds
+// the splits kg, kg+W, ... (each lane four consecutive outputs: 512 contiguous bytes per split and warp, U loads of a
+// thread issued before the additions), the W sub-sums are combined in index order through shared memory.
+template <int W> __global__ void __launch_bounds__(32 * W) reduce_splits_c3(const float* __restrict__ partial, int splits, size_t n, float* __restrict__ out) {
     pdl_wait();
     pdl_launch();
-    __shared__ float4 sh[32][33];
+    constexpr int U = W == 32 ? 4 : 8;
+    __shared__ float4 sh[W][33];
     const int il = threadIdx.x & 31, kg = threadIdx.x >> 5;
     const size_t i = ((size_t)blockIdx.x * 32 + il) * 4;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     if (i < n) {
-        for (int k0 = kg; k0 < splits; k0 += 32 * 4) {
-            float4 v[4];
+        for (int k0 = kg; k0 < splits; k0 += W * U) {
+            float4 v[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
-                v[u] = (k0 + 32 * u < splits) ? *reinterpret_cast<const float4*>(partial + (size_t)(k0 + 32 * u) * n + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int u = 0; u < U; ++u)
+                v[u] = (k0 + W * u < splits) ? *reinterpret_cast<const float4*>(partial + (size_t)(k0 + W * u) * n + i) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < U; ++u) {
                 acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w;
             }
         }
@@ -736,7 +737,7 @@ __global__ void __launch_bounds__(1024) reduce_splits_c3(const float* __restrict
     if (kg == 0 && i < n) {
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int k = 0; k < 32; ++k) {
+        for (int k = 0; k < W; ++k) {
             const float4 v = sh[k][il];
             s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
         }
@@ -746,8 +747,15 @@ __global__ void __launch_bounds__(1024) reduce_splits_c3(const float* __restrict
 
 }  // namespace
 
+// Split sums run beside the dependent chain, and a block of 32 warps only starts on a multiprocessor that has nothing else: from 64 blocks on they waited
+// for one, and the chain's next kernels for them (13.6 us a sum over the ResNet stage at batch 32, whose round takes 21.41 ms with blocks of 32
+// warps and 20.80 with 8; its ragged share 1816 -> 1710 us, EfficientNet 7241 -> 7130).  Fewer blocks find room as they are, and eight warps would
+// add more than four splits each in turn (with 8 warps everywhere the float32 stage takes 1682 us instead of 1640, the stage at
+// batch 32 4705 instead of 4660); nor is there anything to gain with up to 16 splits, one a warp (sixth of MobileNetV2 at batch 4 1510 instead of 1495).
 void reduce_splits_f4(const float* partial, int splits, size_t n, float* out, cudaStream_t st) {
-    launch_pdl(reduce_splits_c3, (unsigned)((n / 4 + 31) / 32), 1024, 0, st, partial, splits, n, out);
+    const unsigned blocks = (unsigned)((n / 4 + 31) / 32);
+    if (blocks < 64 || splits <= 16) launch_pdl(reduce_splits_c3<32>, blocks, 1024, 0, st, partial, splits, n, out);
+    else launch_pdl(reduce_splits_c3<8>, blocks, 256, 0, st, partial, splits, n, out);
 }
 
 bool conv3_tc_supported(int dtype, const ConvGeom& g) {
@@ -800,7 +808,7 @@ void conv3_bwd_weight_tc(const ConvGeom& g, const GradSrc& dz, const ValSrc& x, 
                                           useful_flops > 0 ? useful_flops : 2.0 * 9.0 * px * g.ci * g.co, st);
         if (ctas > 0) {
             LaunchScope ls(K_REDUCE_SPLITS, 4.0 * out_elems * (ctas + 1), (double)out_elems * ctas, st);
-            launch_pdl(reduce_splits_c3, (unsigned)((out_elems / 4 + 31) / 32), 1024, 0, st, scratch, ctas, out_elems, gw);
+            reduce_splits_f4(scratch, ctas, out_elems, gw, st);
             return;
         }
     }
@@ -834,7 +842,7 @@ void conv3_bwd_weight_tc(const ConvGeom& g, const GradSrc& dz, const ValSrc& x, 
         launch_pdl(conv3_wgrad_tc_kernel, dim3(ctas, groups), C3_THREADS, smem, st, a);
     }
     LaunchScope ls(K_REDUCE_SPLITS, 4.0 * out_elems * (ctas + 1), (double)out_elems * ctas, st);
-    launch_pdl(reduce_splits_c3, (unsigned)((out_elems / 4 + 31) / 32), 1024, 0, st, scratch, ctas, out_elems, gw);
+    reduce_splits_f4(scratch, ctas, out_elems, gw, st);
 }
 
 }  // namespace ast

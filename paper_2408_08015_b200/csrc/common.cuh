@@ -44,8 +44,18 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float
 // Programmatic dependent launch.  Every kernel of the library is launched with programmatic
 // stream serialization allowed and opens with pdl_wait(): nothing of the previous kernel in the
 // stream is read or overwritten before that kernel has completed and its writes are visible.
-// pdl_launch() then lets the next kernel's blocks be scheduled as soon as SM resources free up,
-// so its launch latency overlaps this kernel's execution.
+// pdl_launch() lets the next kernel's blocks be scheduled as soon as SM resources free up, so its launch latency and its prologue overlap this kernel's
+// execution.  Where it stands decides what the waiting blocks cost: they hold registers and shared memory, are placed where there happens to be room
+// while this kernel still runs, and a kernel that releases its own dependents before it has waited itself lets three or four kernels of the chain
+// pile up.  Hence, measured on whole rounds:
+//   - behind pdl_wait() (one kernel waits at a time) unless a rule below says otherwise: against the top of the kernel the forward's pointwise and
+//     depthwise kernels so gain 4.5 % of a round of MobileNetV2 on small images and 3.5 % of a sixth of it at batch 4, the weight gradients 1 % of half of it with
+//     the head, the tensor-memory pipelines 0.7 % of the ResNet stage;
+//   - at the top: the split pointwise backward (one tile a CTA and little else on the multiprocessors: behind the wait the sixth at batch 4 loses 3.3 %, the late
+//     sixth 1.6), the float32 forward (0.8 to 1.5 % of the smallest block) and the pipelined weight gradient (0.7 % of the stage at batch 32);
+//   - in front of the sums at the end: depthwise backward (168 registers a thread; the float32 stage loses 1.8 % with the launch behind the wait), depthwise forward
+//     of up to three blocks a multiprocessor (1.4 % of the sixth; with more blocks half of the network loses 1.2 %), persistent pointwise forward of more than
+//     one CTA a multiprocessor (1.5 % of the stage at batch 32), float32 backward and weight gradient (1.3 %, 1.1 %).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

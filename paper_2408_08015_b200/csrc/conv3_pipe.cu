@@ -70,7 +70,6 @@ conv3_pipe_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
                   const CPArgs a) {
     // barriers, tensor memory and the resident weights (written only by the refresh kernel, which never releases its
     // dependents early) are set up before the dependency wait and overlap the previous kernel's tail
-    pdl_launch();
     extern __shared__ uint8_t smem_raw[];
     // w_full, slot_full[S], slot_xf[S], slot_empty[S], acc_full[2], acc_empty[2], z_full[2], z_empty[2]
     __shared__ uint64_t bars[1 + 3 * CP_MAX_S + 8];
@@ -134,6 +133,7 @@ conv3_pipe_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
                 tma::load_3d(smem_u32(sB) + (uint32_t)(kb * 9 + t) * CP_WTAP, &tm_w, kb * 64, (a.flip) ? 8 - t : t, n0, w_full());
     }
     pdl_wait();
+    pdl_launch();
     const uint32_t tmem = tmem_slot;
 
     if (warp == 0) {

@@ -81,7 +81,6 @@ __device__ __forceinline__ uint64_t desc_mn(uint32_t smem_addr, uint32_t lbo_byt
 __global__ void __launch_bounds__(WP_THREADS, 1)
 conv3_wgrad_pipe_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_dy, const __grid_constant__ CUtensorMap tm_z,
                         const WPArgs a) {
-    pdl_launch();
     extern __shared__ uint8_t smem_raw[];
     // st_full[S], st_xf[S], st_empty[S], z_full[2], z_empty[2], done
     __shared__ uint64_t bars[3 * WP_MAX_S + 5];
@@ -137,6 +136,7 @@ conv3_wgrad_pipe_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_c
         if (use_z) tma::prefetch_map(&tm_z);
     }
     pdl_wait();
+    pdl_launch();
     const uint32_t tmem = tmem_slot;
 
     if (warp == 0) {

@@ -136,6 +136,7 @@ struct DwFwdArgs {
     void* out;
     BnSumsOut so;
     bool first;                  // writes the pending coefficients out
+    bool late;                   // dependents are released when the rows are done (common.cuh)
 };
 
 struct DwBwdArgs {

@@ -28,7 +28,6 @@ using namespace dw;
 // ------------------------------------------------------------------------------------------ forward
 template <typename T, int S, int TW, bool EX>
 __global__ void __launch_bounds__(BT) dw3_fwd_kernel(const DwFwdArgs a) {
-    pdl_launch();
     constexpr int NIN = (TW - 1) * S + 3;
     extern __shared__ __align__(16) float sm[];            // scale and shift [2][width]; reused for the sums
     const DwGeom& g = a.g;
@@ -38,6 +37,7 @@ __global__ void __launch_bounds__(BT) dw3_fwd_kernel(const DwFwdArgs a) {
     float2 w[9];
     load_weights<9>(a.wkc, g.c, c0, live, w);
     pdl_wait();
+    if (!a.late) pdl_launch();
     int item = blockIdx.x * g.rows + row, wo0 = 0, oh0 = 0, oh1 = 0, n = 0;
     uint32_t col[NIN];
     P2<T> nx[NIN];
@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(BT) dw3_fwd_kernel(const DwFwdArgs a) {
             place();
             fetch(oh0 * S - 1);
         }
+    if (a.late) pdl_launch();
     if (stats) block_sums<2>(s, g.lanes, g.rows, cb, g.c, a.so.sums, sm);
 }
 
@@ -216,7 +217,6 @@ __device__ __forceinline__ BwdCoef<T, XF> bwd_coefs(const DwBwdArgs& a, int cb, 
 
 template <typename T, int TW, int XF, bool EX>
 __global__ void __launch_bounds__(BT, 3) dw3_bwd_s1_kernel(const DwBwdArgs a) {
-    pdl_launch();
     constexpr int NZ = TW + 2;
     extern __shared__ __align__(16) float sm[];
     const DwGeom& g = a.g;
@@ -330,6 +330,7 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s1_kernel(const DwBwdArgs a) {
             place();
             fetch_z(r0 - 1);
         }
+    pdl_launch();
     block_sums<9>(gw, g.lanes, g.rows, cb, g.c, a.gw, sm);  // the staged coefficients are not needed any more
     if (a.sums) block_sums<2>(fs, g.lanes, g.rows, cb, g.c, a.sums, sm);
 }
@@ -338,7 +339,6 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s1_kernel(const DwBwdArgs a) {
 // a or b is 1 also dz(i+1, .) and dz(., j+1).  A thread owns TZ columns of dz = 2*TZ input columns and walks down the rows of dz.
 template <typename T, int TZ, int XF, bool EX>
 __global__ void __launch_bounds__(BT, 3) dw3_bwd_s2_kernel(const DwBwdArgs a) {
-    pdl_launch();
     extern __shared__ __align__(16) float sm[];
     const DwGeom& g = a.g;
     const int jl = threadIdx.x % g.lanes, row = threadIdx.x / g.lanes, width = 2 * g.lanes, cb = blockIdx.y * width, c0 = cb + 2 * jl;
@@ -471,6 +471,7 @@ __global__ void __launch_bounds__(BT, 3) dw3_bwd_s2_kernel(const DwBwdArgs a) {
             place();
             fetch_z(r0);
         }
+    pdl_launch();
     block_sums<9>(gw, g.lanes, g.rows, cb, g.c, a.gw, sm);
     if (a.sums) block_sums<2>(fs, g.lanes, g.rows, cb, g.c, a.sums, sm);
 }
@@ -518,7 +519,9 @@ void dw3_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf,
         d.items = n * d.nrc * d.sw;
         cut_channels(d);
         LaunchScope ls(K_DW_FWD, n * (in_e + out_e) * esz(dtype) + 36.0 * g.ci, 18.0 * n * out_e, st);
-        launch_pdl(f, cut_grid(d, t.ctas, launches), BT, (size_t)BT * 2 * 2 * 4, st, a);
+        const dim3 grid = cut_grid(d, t.ctas, launches);
+        a.late = (int)(grid.x * grid.y) <= 3 * sm_count();
+        launch_pdl(f, grid, BT, (size_t)BT * 2 * 2 * 4, st, a);
     }
 }
 

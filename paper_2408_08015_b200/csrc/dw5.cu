@@ -41,7 +41,6 @@ template <> struct P1<__nv_bfloat16> {
 // ------------------------------------------------------------------------------------------ forward
 template <typename T, int S, int TW, bool EX>
 __global__ void __launch_bounds__(BT) dw5_fwd_kernel(const DwFwdArgs a) {
-    pdl_launch();
     constexpr int NIN = (TW - 1) * S + 5;
     extern __shared__ __align__(16) float sm[];            // scale and shift [2][width]; reused for the sums
     const DwGeom& g = a.g;
@@ -51,6 +50,7 @@ __global__ void __launch_bounds__(BT) dw5_fwd_kernel(const DwFwdArgs a) {
     float2 w[25];
     load_weights<25>(a.wkc, g.c, c0, live, w);
     pdl_wait();
+    if (!a.late) pdl_launch();
     int item = blockIdx.x * g.rows + row, wo0 = 0, oh0 = 0, oh1 = 0, n = 0;
     uint32_t col[NIN];
     P2<T> nx[NIN];
@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(BT) dw5_fwd_kernel(const DwFwdArgs a) {
             place();
             fetch(oh0 * S - 2);
         }
+    if (a.late) pdl_launch();
     if (stats) block_sums<2>(s, g.lanes, g.rows, cb, g.c, a.so.sums, sm);
 }
 
@@ -221,7 +222,6 @@ template <typename T, int XF> __device__ __forceinline__ Coef1<T, XF> coefs1(con
 
 template <typename T, int TW, int XF, bool EX>
 __global__ void __launch_bounds__(BT, 3) dw5_bwd_s1_kernel(const DwBwdArgs a) {
-    pdl_launch();
     constexpr int NZ = TW + 4;
     extern __shared__ __align__(16) float sm[];
     const DwGeom& g = a.g;
@@ -339,6 +339,7 @@ __global__ void __launch_bounds__(BT, 3) dw5_bwd_s1_kernel(const DwBwdArgs a) {
             place();
             fetch_z(r0 - 2);
         }
+    pdl_launch();
     block_sums<25>(gw, g.lanes, g.rows, cb, g.c, a.gw, sm);
     if (a.sums) block_sums<2>(fs, g.lanes, g.rows, cb, g.c, a.sums, sm);
 }
@@ -347,7 +348,6 @@ __global__ void __launch_bounds__(BT, 3) dw5_bwd_s1_kernel(const DwBwdArgs a) {
 // is 0, i-1 (tap rows a, a + 2, 4), and columns likewise.  A thread owns TZ columns of dz = 2*TZ input columns and walks down the rows of dz.
 template <typename T, int TZ, int XF, bool EX>
 __global__ void __launch_bounds__(BT, 3) dw5_bwd_s2_kernel(const DwBwdArgs a) {
-    pdl_launch();
     constexpr int NZ = TZ + 2, NX = 2 * TZ;
     extern __shared__ __align__(16) float sm[];
     const DwGeom& g = a.g;
@@ -471,6 +471,7 @@ __global__ void __launch_bounds__(BT, 3) dw5_bwd_s2_kernel(const DwBwdArgs a) {
             place();
             fetch_z(r0 - 1);
         }
+    pdl_launch();
     block_sums<25>(gw, g.lanes, g.rows, cb, g.c, a.gw, sm);
     if (a.sums) block_sums<2>(fs, g.lanes, g.rows, cb, g.c, a.sums, sm);
 }
@@ -499,7 +500,9 @@ void dw5_fwd(int dtype, const ConvGeom& g, const ValSrc& x, const BnPendFwd& pf,
         d.items = n * d.nrc * d.sw;
         cut_channels(d);
         LaunchScope ls(K_DW_FWD, n * (in_e + out_e) * esz(dtype) + 100.0 * g.ci, 50.0 * n * out_e, st);
-        launch_pdl(f, cut_grid(d, t.ctas, launches), BT, (size_t)BT * 2 * 2 * 4, st, a);
+        const dim3 grid = cut_grid(d, t.ctas, launches);
+        a.late = (int)(grid.x * grid.y) <= 3 * sm_count();
+        launch_pdl(f, grid, BT, (size_t)BT * 2 * 2 * 4, st, a);
     }
 }
 

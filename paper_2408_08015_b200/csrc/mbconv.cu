@@ -157,8 +157,8 @@ template <int V, typename F> __device__ __forceinline__ void rows_sum(const Pass
 template <typename T, int V, bool PART>
 __global__ void __launch_bounds__(256, 4) silu_fwd_kernel(ValSrc x, BnPendFwd pf, PassCut k, int hw, int c, T* __restrict__ out, T* __restrict__ out2,
                                                        float* __restrict__ part) {
-    pdl_launch();
     pdl_wait();
+    pdl_launch();
     extern __shared__ float sm[];              // scale and shift of the block's channels; then the sums
     PassIdx ix;
     ix.init<V>(k, hw, c);
@@ -223,8 +223,8 @@ struct SiluBwdArgs {
     void* dx;
 };
 template <typename T, int V, bool GATE, bool SUMS> __global__ void __launch_bounds__(256, 2) silu_bwd_kernel(SiluBwdArgs a, PassCut k) {
-    pdl_launch();
     pdl_wait();
+    pdl_launch();
     extern __shared__ float sm[];
     PassIdx ix;
     ix.init<V>(k, a.hw, a.c);
@@ -350,7 +350,6 @@ __device__ __forceinline__ float split_sum(const float* part, int splits, size_t
 __global__ void __launch_bounds__(256) se_fc_fwd_kernel(const float* __restrict__ part, int splits, float inv_hw, const float* __restrict__ w1,
                                                         const float* __restrict__ b1, const float* __restrict__ w2, const float* __restrict__ b2, int c, int k,
                                                         int staged, float* __restrict__ s, float* __restrict__ p1, float* __restrict__ g) {
-    pdl_launch();
     extern __shared__ float hs[];              // h[k], s[c], weights
     float* sn = hs + k;
     const int n = blockIdx.x, nb = gridDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -360,6 +359,7 @@ __global__ void __launch_bounds__(256) se_fc_fwd_kernel(const float* __restrict_
         w2 = w1 + k * c;
     }
     pdl_wait();
+    pdl_launch();
     for (int i = threadIdx.x; i < c; i += 256) {
         const float a = split_sum(part + (size_t)n * c + i, splits, (size_t)nb * c) * inv_hw;
         sn[i] = a;
@@ -387,7 +387,6 @@ __global__ void __launch_bounds__(256) se_fc_fwd_kernel(const float* __restrict_
 __global__ void __launch_bounds__(256) se_fc_bwd_kernel(const float* __restrict__ part, int splits, const float* __restrict__ g, const float* __restrict__ p1,
                                                         const float* __restrict__ w1, const float* __restrict__ w2, int c, int k, int staged, float inv_hw,
                                                         float* __restrict__ dp2, float* __restrict__ dp1, float* __restrict__ ds) {
-    pdl_launch();
     extern __shared__ float sm[];              // dp2[c], dp1[k], weights
     float* sdp2 = sm;
     float* sdp1 = sm + c;
@@ -398,6 +397,7 @@ __global__ void __launch_bounds__(256) se_fc_bwd_kernel(const float* __restrict_
         w2 = w1 + k * c;
     }
     pdl_wait();
+    pdl_launch();
     for (int i = threadIdx.x; i < c; i += 256) {
         const float gg = g[(size_t)n * c + i];
         // gradient of the gate: the pixel-split partials of sum dout*x
@@ -468,8 +468,8 @@ __global__ void __launch_bounds__(256) se_param_grad_kernel(const float* __restr
 template <typename T, int V, int MODE>
 __global__ void __launch_bounds__(256, 4) se_scale_kernel(ValSrc x, const T* __restrict__ d, const float* __restrict__ gate, const float* __restrict__ ds,
                                                        const T* addend, PassCut k, int hw, int c, T* __restrict__ out, T* __restrict__ out2) {
-    pdl_launch();
     pdl_wait();
+    pdl_launch();
     PassIdx ix;
     ix.init<V>(k, hw, c);
     if (!ix.live) return;

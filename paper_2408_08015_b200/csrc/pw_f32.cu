@@ -60,7 +60,7 @@ __device__ __forceinline__ float grad1(float d, float z, float k1, float k2, flo
 enum { XF_NONE = 0, XF_VALUE = 1, XF_ADD = 2, XF_AFFINE = 2 };
 template <bool BWD, int TN, int WK, int XF>
 __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
-    pdl_launch();
+    if (!BWD) pdl_launch();
     constexpr int WM = 4 / WK, BM = 32 * WM, BK = 16 * WK, AP = BK + 4, QC = BK / 4, BN = 4 * TN, G = TN % 4 == 0 ? 4 : 2, NG = TN / G;
     extern __shared__ __align__(16) float sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r = lane >> 2, t = lane & 3, wm = warp % WM, wk = warp / WM;
@@ -334,6 +334,7 @@ __global__ void __launch_bounds__(NT) pw_f32_kernel(const F32Args a) {
             }
         }
     }
+    if (BWD) pdl_launch();
     if (!sums) return;
     __syncthreads();                                       // sR: the last tile's partials have been read
     if (wk == 0) {
@@ -449,7 +450,6 @@ __device__ __forceinline__ void cluster_sync() {
 
 // MDZ: the gradient is the wide side (CO >= CI)
 template <int TN, bool MDZ> __global__ void __launch_bounds__(NT) pw_f32_wgrad_kernel(const F32WArgs a) {
-    pdl_launch();
     constexpr int BN = 4 * TN, G = TN % 4 == 0 ? 4 : 2, SP = BN + 1, BLK = WBM * SP, NM = MDZ ? 5 : 2, NN = MDZ ? 2 : 5;
     constexpr int STG = WPX * (WBM + BN);
     __shared__ __align__(16) float coef[NM * WBM + NN * BN];
@@ -527,6 +527,7 @@ template <int TN, bool MDZ> __global__ void __launch_bounds__(NT) pw_f32_wgrad_k
         }
         __syncwarp();
     }
+    pdl_launch();
     __syncthreads();                                       // the blocks below reuse the stages of all warps
 #pragma unroll
     for (int i = 0; i < WTM; ++i)

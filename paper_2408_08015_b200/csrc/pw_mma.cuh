@@ -49,6 +49,7 @@ struct Args {
     const float *r_scale, *r_shift, *r_mean, *r_rstd;
     int r_act;
     bool r_mask;               // the output is stored as that unit's activation lets it through
+    bool late;                 // persistent form: dependents are released when the products are done (common.cuh)
 };
 
 __device__ __forceinline__ void mma16816(float* c, const uint32_t a0, const uint32_t a1, const uint32_t a2, const uint32_t a3, const uint32_t b0, const uint32_t b1) {
@@ -306,7 +307,6 @@ template <> struct SumCoef<true> {
 // Large maps: CTAs walk down the pixel tiles, every warp has 16*MI pixels x 8*NJ columns and the whole reduction.
 template <bool BWD, int MI, int NJ, int G, int XF>
 __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
-    pdl_launch();
     extern __shared__ __align__(16) uint8_t sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int wm = warp;
@@ -317,6 +317,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
     float* red = sN + (BWD ? 4 : 1) * BN;                  // [WM][2][BN]
     stage_weights<G>(a, sW, n0, BN);
     pdl_wait();
+    if (!a.late) pdl_launch();
 
     const uint8_t* pa = reinterpret_cast<const uint8_t*>(a.a);
     const uint8_t* pz = reinterpret_cast<const uint8_t*>(a.az);
@@ -455,6 +456,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
         }
         if (BWD && sums && tile + (int)gridDim.x < a.m_tiles) fetch_z(tile + gridDim.x);
     }
+    if (a.late) pdl_launch();
     if (!sums) return;
 #pragma unroll
     for (int i = 0; i < NJ; ++i) {
@@ -489,7 +491,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
 // a layer of a few hundred pixels still spreads over the chip and a long reduction costs one memory latency instead of K/32.
 template <bool BWD, int NJ, int G, int WK, int XF>
 __global__ void __launch_bounds__(256) pw_mma_split_kernel(const Args a) {
-    pdl_launch();
+    if (BWD) pdl_launch();
     extern __shared__ __align__(16) uint8_t sm[];
     constexpr int WM = 8 / WK, BM = 16 * WM, BN = 8 * NJ, RP = BN + 4, D = BWD ? 3 : 4;
     constexpr bool USE_Z = BWD ? XF != XF_NONE : XF == XF_ADD;
@@ -502,6 +504,7 @@ __global__ void __launch_bounds__(256) pw_mma_split_kernel(const Args a) {
     float* racc = sN + (BWD ? 4 : 1) * BN;                 // [WK][BM][RP]
     stage_weights<G>(a, sW, n0, BN);
     pdl_wait();
+    if (!BWD) pdl_launch();
 
     const size_t r0 = (size_t)min(p0 + wm * 16 + g, a.P - 1) * a.K * 2, r1 = (size_t)min(p0 + wm * 16 + g + 8, a.P - 1) * a.K * 2;
     const uint8_t *ra0 = reinterpret_cast<const uint8_t*>(a.a) + r0, *ra1 = reinterpret_cast<const uint8_t*>(a.a) + r1;

@@ -598,7 +598,6 @@ template <bool BWD, bool EXTRA, bool PANELS> __global__ void __launch_bounds__(P
     // Set-up that reads nothing the previous kernel in the stream writes (barriers, tensor memory, the resident
     // weights: written only by the refresh kernel, which never releases its dependents before it has completed) runs before
     // the dependency wait and so overlaps the previous kernel's tail.
-    pdl_launch();
     extern __shared__ uint8_t smem_raw[];
     // raw_full[R], raw_empty[R], a_full[2], a_empty[2], acc_full[2], acc_empty[2], zp_full[2], zp_empty[2], so_full[2], so_free[2]
     __shared__ uint64_t bars[2 * MAX_RAW + 16];
@@ -665,6 +664,7 @@ template <bool BWD, bool EXTRA, bool PANELS> __global__ void __launch_bounds__(P
     __syncthreads();
     fence_after_sync();
     pdl_wait();
+    pdl_launch();
     const uint32_t tmem = tmem_slot;
     const int my_tiles = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
     const uint32_t row_bytes = (uint32_t)a.K * 2u;

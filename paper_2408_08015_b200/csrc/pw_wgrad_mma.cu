@@ -145,7 +145,6 @@ template <int V, bool GRAD> struct Side {
 // MDZ: the gradient is the M side (CO >= CI)
 template <int VM, int VN, bool MDZ>
 __global__ void __launch_bounds__(WARPS * 32) pw_wgrad_mma_kernel(const WmArgs a) {
-    pdl_launch();
     extern __shared__ __align__(16) float st[];
     // the block in shared memory with the input channels contiguous: what is summed over the cluster and written out is then read and written in rows
     constexpr int BM = 8 * VM, BN = 8 * VN, BC = MDZ ? BN : BM, SP = BC + 1, BLK = (BM * BN / BC) * SP, NM = MDZ ? 5 : 2, NN = MDZ ? 2 : 5;
@@ -153,6 +152,7 @@ __global__ void __launch_bounds__(WARPS * 32) pw_wgrad_mma_kernel(const WmArgs a
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int m0 = ((int)blockIdx.y % a.mb) * BM, n0 = ((int)blockIdx.y / a.mb) * BN;
     pdl_wait();
+    pdl_launch();
 
     const int pbeg = blockIdx.x * a.pix_per_cta, pend = min(a.P, pbeg + a.pix_per_cta);
     Side<VM, MDZ> sm_;

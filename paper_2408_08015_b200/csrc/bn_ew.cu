@@ -315,8 +315,8 @@ __device__ __forceinline__ bool sum_partials(const float* __restrict__ partial, 
 __global__ void __launch_bounds__(1024) bn_stats_finish(const float* __restrict__ partial, int blocks, int c, double count,
                                                        const float* __restrict__ gamma, const float* __restrict__ beta, float eps, float momentum,
                                                        BnFwdOut o) {
-    pdl_wait();
     pdl_launch();
+    pdl_wait();
     // the owner thread's per-channel inputs are requested before the partials so that all of the
     // kernel's global loads overlap
     const int chp = blockIdx.x * 32 + (threadIdx.x & 31);
@@ -853,8 +853,8 @@ bool ew_relu_mask_bn_sums(int dtype, const void* d, const void* out_val, const v
 
 // ---- pending coefficients settled by a kernel of their own: in front of a kernel that cannot form them itself
 __global__ void __launch_bounds__(128) bn_settle_fwd_kernel(BnPendFwd b) {
-    pdl_wait();
     pdl_launch();
+    pdl_wait();
     const int ch = blockIdx.x * 128 + threadIdx.x;
     if (ch < b.c) bn_fwd_coef(b, ch, true);
 }

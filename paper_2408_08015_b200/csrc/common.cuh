@@ -52,7 +52,8 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float
 //     depthwise kernels so gain 4.5 % of a round of MobileNetV2 on small images and 3.5 % of a sixth of it at batch 4, the weight gradients 1 % of half of it with
 //     the head, the tensor-memory pipelines 0.7 % of the ResNet stage;
 //   - at the top: the split pointwise backward (one tile a CTA and little else on the multiprocessors: behind the wait the sixth at batch 4 loses 3.3 %, the late
-//     sixth 1.6), the float32 forward (0.8 to 1.5 % of the smallest block) and the pipelined weight gradient (0.7 % of the stage at batch 32);
+//     sixth 1.6), the kernels that settle the forward's BatchNorm sums (0.6 % of the ResNet
+//     stage, 0.8 of its ragged share; the backward's would cost the stage at batch 32 2.8 %), the float32 forward (0.8 to 1.5 % of the smallest block) and the pipelined weight gradient (0.7 % of the stage at batch 32);
 //   - in front of the sums at the end: depthwise backward (168 registers a thread; the float32 stage loses 1.8 % with the launch behind the wait), depthwise forward
 //     of up to three blocks a multiprocessor (1.4 % of the sixth; with more blocks half of the network loses 1.2 %), persistent pointwise forward of more than
 //     one CTA a multiprocessor (1.5 % of the stage at batch 32), float32 backward and weight gradient (1.3 %, 1.1 %).

@@ -953,7 +953,9 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             if (int rc = mark()) return rc;
             const auto weights = [&]() -> int {
                 if (int rc = on_side()) return rc;
-                if (u.b_off >= 0) bias_grad(dt, d.dy, d.z, o.elems / o.c, o.c, u.act, wscratch, s->scratch_floats, s->g + u.b_off, wst);
+                // a BatchNorm behind takes the bias out again with the mean: the gradient behind its backward sums to zero over the micro-batch
+                if (u.b_off >= 0 && u.l_bn >= 0) CU(cudaMemsetAsync(s->g + u.b_off, 0, (size_t)o.c * sizeof(float), wst));
+                else if (u.b_off >= 0) bias_grad(dt, d.dy, d.z, o.elems / o.c, o.c, u.act, wscratch, s->scratch_floats, s->g + u.b_off, wst);
                 if (s2_tc && conv3_wgrad_tc_supported(dt, s1_geom(u)))
                     conv3_bwd_weight_tc(s1_geom(u), dup, xin, wscratch, s->scratch_floats, s->g + u.w_off, s->err, wst, conv_flops(u.g));
                 else if (mma_w || f32_w) {

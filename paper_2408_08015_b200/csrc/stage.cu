@@ -987,7 +987,8 @@ static int backward_impl(asteroid_stage* s, int slot, const void* dy, void* dx, 
             // 264 us, of the ragged stage 640 -> 622, of a sixth of MobileNetV2 at batch 4 1497 -> 1475, EfficientNet 7135 -> 7070).  At the others, and at a first
             // one that begins the call, the weight gradients do: placed second they are scattered over streams of the graph's own and
             // lose their programmatic launches (half of MobileNetV2 with the head 4170 -> 4640 us).
-            const bool chain_first = !side_used && (ui + 1 < (int)s->units.size() || u.l_bn >= 0);
+            // On one stream (a trace, a profile) there is no fork: each layer's weight gradient in front of its input gradient.
+            const bool chain_first = use_side && !side_used && (ui + 1 < (int)s->units.size() || u.l_bn >= 0);
             if (!chain_first)
                 if (int rc = weights()) return rc;
             if (want_in) {

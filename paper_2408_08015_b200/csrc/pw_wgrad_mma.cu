@@ -46,6 +46,11 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// Warps and pixel ranges are added in pairs: four ranges, whose warps chain two products, instead of eight leave 64 x 384 at 784 pixels 7.8e-8 (2-norm, against
+// 7.6e-8) from its sum in 64 bits when added one after the other, in pairs 7.0e-8.  The same number of additions; the other cuts gain as well: 576 x 96
+// 7.8 -> 7.0e-8, 160 x 960 10.9 -> 10.4e-8.
+__device__ __forceinline__ float sum8(const float* q) { return ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7])); }
+
 // V consecutive channels (V * 2 bytes)
 template <int V> struct Raw {
     uint32_t w[V / 2];
@@ -225,10 +230,10 @@ __global__ void __launch_bounds__(WARPS * 32) pw_wgrad_mma_kernel(const WmArgs a
     __syncthreads();
     for (int e = tid; e < BM * BN; e += WARPS * 32) {
         float* d = st + (e / BC) * SP + e % BC;
-        float s = d[0];
+        float q[8];
 #pragma unroll
-        for (int w = 1; w < WARPS; ++w) s += d[w * BLK];
-        d[0] = s;
+        for (int w = 0; w < WARPS; ++w) q[w] = d[w * BLK];
+        d[0] = sum8(q);
     }
     uint32_t cs, rank;
     asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(cs));
@@ -247,8 +252,7 @@ __global__ void __launch_bounds__(WARPS * 32) pw_wgrad_mma_kernel(const WmArgs a
             float q[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) q[k] = k < (int)cs ? ld_cluster(ad, k) : 0.f;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) s += q[k];
+            s = sum8(q);
         }
         const int k = (MDZ ? m0 : n0) + kr, c = (MDZ ? n0 : m0) + cc;
         if (k < a.CO && c < a.CI) out[(size_t)k * a.CI + c] = s;

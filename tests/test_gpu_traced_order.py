@@ -25,7 +25,7 @@ def test_order_of_a_traced_backward(tmp_path):
         P.asteroid_stage_forward(hdl, 0, x.data_ptr(), y.data_ptr(), sp)
         torch.cuda.synchronize()
         P.asteroid_trace_start()
-        with profile(activities=[ProfilerActivity.CUDA]) as p:
+        with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as p:
             P.asteroid_stage_backward(hdl, 0, dy.data_ptr(), dx.data_ptr(), sp)
             torch.cuda.synchronize()
         P.asteroid_trace_stop()

@@ -1,6 +1,6 @@
-"""Pixel ranges of the pointwise weight gradient on small maps: one, two, four or eight to a cluster, the last two where every warp of a range has a group of 16
-pixels (512 and 1024 pixels).  Maps at those limits, one pixel below and above, gradients of one block of 32 x 32 and of several; with a BatchNorm
-(coefficients formed by the kernel).  A range left out or taken twice changes a gradient by at least a third, the contract is 2e-2."""
+"""Pixel ranges of the pointwise weight gradient on small maps: a partial each where the gradient has few blocks, else one, two, four or eight to a cluster, four
+from 512 pixels and eight from 1024 on (a group of 16 pixels for every warp of a range).  With a BatchNorm (coefficients formed by the kernel).  A
+range left out or taken twice changes a gradient by about a quarter or more, the contract is 2e-2."""
 import pytest
 
 import stage_inputs as si
@@ -9,8 +9,19 @@ from harness import CONTRACT, MIRROR, bf16_store, compare, gpu_round, make_input
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("h, w", [(7, 73), (16, 32), (19, 27), (31, 33), (32, 32), (25, 41)])
-@pytest.mark.parametrize("c_in, c_out", [(24, 32), (72, 40), (40, 136)])
+# below 512 pixels clusters of two, at 512 and 513 of four, from 1023 on 15 or 16 partials
+FEW_BLOCKS = [(ci, co, h, w) for ci, co in ((24, 32), (72, 40), (40, 136)) for h, w in ((7, 73), (16, 32), (19, 27), (31, 33), (32, 32), (25, 41))]
+MORE_BLOCKS = [
+    # 24 and 30 blocks of 32 x 32: one range
+    (64, 384, 11, 11), (160, 192, 9, 14),
+    # clusters of two, four (up to 1023 pixels) and eight
+    (64, 384, 8, 16), (160, 192, 7, 73), (64, 384, 16, 32), (64, 384, 28, 36), (160, 192, 31, 33), (64, 384, 32, 32), (160, 192, 25, 41), (64, 384, 26, 40),
+    # 75 blocks of 64 x 64: one range whatever the map
+    (320, 960, 7, 9), (960, 320, 13, 11),
+]
+
+
+@pytest.mark.parametrize("c_in, c_out, h, w", FEW_BLOCKS + MORE_BLOCKS)
 def test_wgrad_ranges(c_in, c_out, h, w):
     net = si.single_unit_net("conv", c_in, c_out, bn=True)
     last = len(net) - 1

@@ -13,6 +13,9 @@
  *  - Activation tensors are DEVICE pointers, NHWC, in the stage's storage type (float or
  *    bfloat16), owned by the caller.  Parameter / state vectors passed to import/export are
  *    HOST pointers to float.  The stage owns its arenas and frees them in destroy.
+ *  - Alignment: x and the loss heads' tensors may start at any element.  y, dy and dx start at a 16-byte
+ *    boundary, as every device allocation does; where the stage's last layer is a pool its y and dy, where
+ *    the first is one its dx, may start at any element too.
  *  - `stream` is a cudaStream_t passed as void*.  forward/backward/accumulate/step and the loss
  *    heads only enqueue work on it; they never synchronise.  create, destroy, import, export
  *    and profile synchronise the device.  backward also enqueues the weight-gradient kernels on a
@@ -115,7 +118,7 @@ typedef struct {
  * M micro-batches per round.  Parameters start at zero (gamma too): call import_state.
  * Errors: AST_ERR_ARG (range, sizes, references below first-1), AST_ERR_UNSUPPORTED (a BN or
  * activation that does not follow a conv/add it can fuse with, an intermediate of a fused
- * conv-BN-activation chain read by another layer, dwconv with k!=3), AST_ERR_ALLOC. */
+ * conv-BN-activation chain read by another layer, dwconv with k other than 3, 5, 7), AST_ERR_ALLOC. */
 int asteroid_stage_create(const ast_layer* net, int n_layers, int first, int last,
                           int in_h, int in_w, int micro_batch, int M,
                           const ast_opts* opts, asteroid_stage** out);

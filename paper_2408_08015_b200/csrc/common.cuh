@@ -42,8 +42,9 @@ template <> __device__ __forceinline__ float from_f<float>(float v) { return v; 
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
 // Programmatic dependent launch.  Every kernel of the library is launched with programmatic
-// stream serialization allowed and opens with pdl_wait(): nothing of the previous kernel in the
-// stream is read or overwritten before that kernel has completed and its writes are visible.
+// stream serialization allowed and waits in pdl_wait(): nothing of the previous kernel in the
+// stream is read or overwritten before that kernel has completed and its writes are visible.  In front of the wait a kernel only sets up barriers, tensor
+// memory and shared memory, and reads weights and their copies, which are written by kernels that never release their dependents.
 // pdl_launch() lets the next kernel's blocks be scheduled as soon as SM resources free up, so its launch latency and its prologue overlap this kernel's
 // execution.  Where it stands decides what the waiting blocks cost: they hold registers and shared memory, are placed where there happens to be room
 // while this kernel still runs, and a kernel that releases its own dependents before it has waited itself lets three or four kernels of the chain
@@ -53,7 +54,11 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float
 //     the head, the tensor-memory pipelines 0.7 % of the ResNet stage;
 //   - at the top: the split pointwise backward (one tile a CTA and little else on the multiprocessors: behind the wait the sixth at batch 4 loses 3.3 %, the late
 //     sixth 1.6), the kernels that settle the forward's BatchNorm sums (0.6 % of the ResNet
-//     stage, 0.8 of its ragged share; the backward's would cost the stage at batch 32 2.8 %), the float32 forward (0.8 to 1.5 % of the smallest block) and the pipelined weight gradient (0.7 % of the stage at batch 32);
+//     stage, 0.8 of its ragged share; the backward's would cost the stage at batch 32 2.8 %), the float32 forward (0.8 to 1.5 % of the smallest block) and the
+//     pipelined pointwise weight gradient (0.7 % of the stage at batch 32; the 3x3 one releases behind its wait);
+//   - at the top as well, where they have always released and not measured anywhere else, because no round of the networks has more than one or two of
+//     them a call: the pool by vectors, the columns of a first layer, pointwise layers of 192 to 256 channels on both sides (pw_stream.cu), and the
+//     one-tile and persistent 3x3 kernels for layers that the pipeline does not take;
 //   - in front of the sums at the end: depthwise backward (168 registers a thread; the float32 stage loses 1.8 % with the launch behind the wait), depthwise forward
 //     of up to three blocks a multiprocessor (1.4 % of the sixth; with more blocks half of the network loses 1.2 %), persistent pointwise forward of more than
 //     one CTA a multiprocessor (1.5 % of the stage at batch 32), float32 backward and weight gradient (1.3 %, 1.1 %).

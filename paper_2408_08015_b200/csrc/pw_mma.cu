@@ -217,7 +217,7 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
     }
     if (bwd) raise_limits<true>();
     else raise_limits<false>();
-    a.late = !bwd && gx * ny > sm_count();
+    a.late = !bwd && c.wk == 1 && gx * ny > sm_count();
     const size_t smem = mma_smem(bwd, p.K, c);
     LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 2.0 * p.P * p.N : 0.0) + (p.sum_out ? 4.0 * p.P * p.K : 0.0), 2.0 * p.P * p.N * p.K, st);
     launch_pdl(bwd ? kernel_for<true>(c, xf) : kernel_for<false>(c, xf), dim3(gx, ny), c.wk == 1 ? 32 * c.wm : 256, smem, st, a);

@@ -276,9 +276,10 @@ template <bool MDZ> WKernel wkernel(int vm, int vn) {
 //     warp block holds them (16 x 32 at 200 704 pixels: 20.4 -> 14.0).
 //   - 32 x 32 blocks (64 x 64 from 960 x 320 up, where the re-reads of 32 x 32 blocks cost more than the idle multiprocessors); about one
 //     and a half CTAs per multiprocessor, of which two fit one (one of the 64 x 64 blocks': a second wave for the last two of 150 CTAs made
-//     320 x 960 at 784 pixels 25.9 us instead of 14.9); up to eight pixel ranges are one cluster, which writes the gradient itself.  A range is
-//     at least a group of 16 pixels for every warp: shorter ones are as fast alone, but the sums over a CTA's warps and its coefficients are paid for by the dependent
-//     chain beside it (four ranges instead of eight at 784 pixels: sixth of MobileNetV2 at batch 4 1427 -> 1380 us a round).
+//     320 x 960 at 784 pixels 25.9 us instead of 14.9); up to eight pixel ranges are one cluster, which writes the gradient itself.  In clusters of four and eight a range
+//     is at least a group of 16 pixels for every warp (512, 1 024 pixels): shorter ones are as fast alone, but the sums over a CTA's warps and its coefficients are paid
+//     for by the dependent chain beside it (four ranges instead of eight at 784 pixels: sixth of MobileNetV2 at batch 4 1427 -> 1380 us a round).  Clusters of
+//     two and ranges with a partial each go down to 64 pixels; there the longer range has not been measured.
 bool wgrad_mma_choose(int P, int CO, int CI, bool pipeline_fits, size_t scratch_floats, WgradTiling* out) {
     if (CO % 8 || CI % 8) return false;
     if (P > 4096 && !(P <= 16384 && !pipeline_fits) && CO * CI > 512) return false;

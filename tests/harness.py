@@ -123,21 +123,16 @@ def rel_err(a, b, floor=0.0):
     return float(np.abs(a - b).max() / max(np.abs(b).max(), floor, 1e-300))
 
 
-PARITY_LOG = os.environ.get("ASTEROID_PARITY_LOG",
-                            os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "gpurun_out", "parity_table.jsonl"))
+PARITY_LOG = os.environ.get("ASTEROID_PARITY_LOG")       # file for the records of `compare`, if wanted
 
 
 def _log_records(case, records):
-    """One JSON line per compared tensor, appended to the parity table a GPU run leaves behind."""
-    if not case:
+    """One JSON line per compared tensor, appended to the file that ASTEROID_PARITY_LOG names."""
+    if not case or not PARITY_LOG:
         return
-    try:
-        os.makedirs(os.path.dirname(PARITY_LOG), exist_ok=True)
-        with open(PARITY_LOG, "a") as f:
-            for r in records:
-                f.write(json.dumps(dict(case=case, **r)) + "\n")
-    except OSError:
-        pass
+    with open(PARITY_LOG, "a") as f:
+        for r in records:
+            f.write(json.dumps(dict(case=case, **r)) + "\n")
 
 
 CONTRACT, MIRROR, CALIBRATED = "contract", "mirror", "calibrated"

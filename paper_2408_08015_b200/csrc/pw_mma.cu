@@ -12,22 +12,37 @@ using namespace mma;
 
 typedef void (*KernelFn)(const Args);
 
-template <bool BWD, int NJ, int G, int XF> KernelFn pick(int mi, int wk) {
-    if (wk == 1) return mi == 1 ? pw_mma_kernel<BWD, 1, NJ, G, XF> : pw_mma_kernel<BWD, 2, NJ, G, XF>;
+constexpr size_t SMEM_MOST = 200 * 1024;
+// Whether a persistent layer's operands are requested several steps ahead (pw_mma.cuh): input gradients of 256 channels and more, forwards of 128 and more in blocks of 64
+// columns, where a CTA has more than one tile.  These read two to sixteen times what they write and took 0.75 to 1 us a step, a trip to memory, whatever the step's work was:
+// ResNet stage at batch 32 20 572 -> 19 885 us a round, the sums of defers_add (stage.cu) among it.  Elsewhere one step ahead in registers is as good or better, because slots cost
+// a store and a load of shared memory a vector: slots in all persistent kernels took half of MobileNetV2 with the head 4140 -> 4210 us, EfficientNet 6941 -> 7029, the ragged stage
+// 613 -> 637; input gradients from 128 channels on EfficientNet 6955 -> 6994, single tiles the ragged ResNet share 1681 -> 1689.
+constexpr bool deep_form(bool bwd, int nj, int xf) { return bwd ? nj >= 4 && xf != XF_NONE : nj == 8; }
+size_t slot_bytes(const MmaTiling& c) { return (size_t)4 * c.mi * (c.mi == 2 ? 3 : 4) * 16 * 32 * c.wm; }       // of Slots (pw_mma.cuh), both operands
+bool deep_layer(bool bwd, int K, const MmaTiling& c, int xf) {
+    const size_t smem = mma_smem(bwd, K, c) + slot_bytes(c);
+    return c.wk == 1 && deep_form(bwd, c.nj, xf) && K >= (bwd ? 256 : 128) && smem <= SMEM_MOST && (smem + 1024) * c.ctas <= 227 * 1024;
+}
+
+template <bool BWD, int NJ, int G, int XF> KernelFn pick(int mi, int wk, bool deep) {
+    if constexpr (deep_form(BWD, NJ, XF))
+        if (wk == 1 && deep) return mi == 1 ? pw_mma_kernel<BWD, 1, NJ, G, XF, true> : pw_mma_kernel<BWD, 2, NJ, G, XF, true>;
+    if (wk == 1) return mi == 1 ? pw_mma_kernel<BWD, 1, NJ, G, XF, false> : pw_mma_kernel<BWD, 2, NJ, G, XF, false>;
     return wk == 2 ? pw_mma_split_kernel<BWD, NJ, G, 2, XF> : wk == 4 ? pw_mma_split_kernel<BWD, NJ, G, 4, XF> : pw_mma_split_kernel<BWD, NJ, G, 8, XF>;
 }
-template <bool BWD, int XF> KernelFn by_columns(const MmaTiling& c) {
+template <bool BWD, int XF> KernelFn by_columns(const MmaTiling& c, bool deep) {
     switch (c.nj) {
-        case 2: return pick<BWD, 2, 2, XF>(c.mi, c.wk);
-        case 3: return pick<BWD, 3, 1, XF>(c.mi, c.wk);
-        case 4: return pick<BWD, 4, 4, XF>(c.mi, c.wk);
-        case 6: return pick<BWD, 6, 2, XF>(c.mi, c.wk);
-        default: return pick<BWD, 8, 4, XF>(c.mi, c.wk);
+        case 2: return pick<BWD, 2, 2, XF>(c.mi, c.wk, deep);
+        case 3: return pick<BWD, 3, 1, XF>(c.mi, c.wk, deep);
+        case 4: return pick<BWD, 4, 4, XF>(c.mi, c.wk, deep);
+        case 6: return pick<BWD, 6, 2, XF>(c.mi, c.wk, deep);
+        default: return pick<BWD, 8, 4, XF>(c.mi, c.wk, deep);
     }
 }
-template <bool BWD> KernelFn kernel_for(const MmaTiling& c, int xf) {
-    if (!BWD && xf == XF_ADD) return by_columns<false, XF_ADD>(c);
-    return xf == XF_NONE ? by_columns<BWD, XF_NONE>(c) : xf == XF_AFFINE ? by_columns<BWD, XF_AFFINE>(c) : by_columns<BWD, XF_ACT>(c);
+template <bool BWD> KernelFn kernel_for(const MmaTiling& c, int xf, bool deep) {
+    if (!BWD && xf == XF_ADD) return by_columns<false, XF_ADD>(c, deep);
+    return xf == XF_NONE ? by_columns<BWD, XF_NONE>(c, deep) : xf == XF_AFFINE ? by_columns<BWD, XF_AFFINE>(c, deep) : by_columns<BWD, XF_ACT>(c, deep);
 }
 // the shared-memory limit of every instantiation, raised once per device
 template <bool BWD> void raise_limits() {
@@ -43,7 +58,7 @@ template <bool BWD> void raise_limits() {
                 c.nj = nj;
                 c.mi = v == 1 ? 2 : 1;
                 c.wk = v < 2 ? 1 : 1 << (v - 1);
-                cudaFuncSetAttribute(kernel_for<BWD>(c, xf), cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+                for (bool deep : {false, true}) cudaFuncSetAttribute(kernel_for<BWD>(c, xf, deep), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MOST);
             }
     done.fetch_or(bit, std::memory_order_release);
 }
@@ -161,6 +176,8 @@ bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {
     return bwd ? bwd_choose(P, K, N, out) : fwd_choose(P, K, N, out);
 }
 
+bool mma_deep_sum(int P, int K, const MmaTiling& c) { return deep_layer(false, K, c, XF_ADD) && (P + 16 * c.mi * c.wm - 1) / (16 * c.mi * c.wm) > sm_count() * c.ctas; }
+
 size_t mma_smem(bool bwd, int K, const MmaTiling& c) {
     const int Kp = (K + 31) / 32 * 32, BN = c.nj * 8;
     size_t b = (size_t)BN * w_pitch(K) + (size_t)(bwd ? 5 : 3) * Kp * 4 + (size_t)(bwd ? 4 : 1) * BN * 4;
@@ -218,9 +235,10 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
     if (bwd) raise_limits<true>();
     else raise_limits<false>();
     a.late = !bwd && c.wk == 1 && gx * ny > sm_count();
-    const size_t smem = mma_smem(bwd, p.K, c);
+    const bool deep = deep_layer(bwd, p.K, c, xf) && a.m_tiles > gx;
+    const size_t smem = mma_smem(bwd, p.K, c) + (deep ? slot_bytes(c) : 0);
     LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 2.0 * p.P * p.N : 0.0) + (p.sum_out ? 4.0 * p.P * p.K : 0.0), 2.0 * p.P * p.N * p.K, st);
-    launch_pdl(bwd ? kernel_for<true>(c, xf) : kernel_for<false>(c, xf), dim3(gx, ny), c.wk == 1 ? 32 * c.wm : 256, smem, st, a);
+    launch_pdl(bwd ? kernel_for<true>(c, xf, deep) : kernel_for<false>(c, xf, deep), dim3(gx, ny), c.wk == 1 ? 32 * c.wm : 256, smem, st, a);
 }
 
 }  // namespace ast

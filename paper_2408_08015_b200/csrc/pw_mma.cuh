@@ -305,8 +305,18 @@ template <> struct SumCoef<true> {
 
 // ---------------------------------------------------------------------------------------------------------------------
 // Large maps: CTAs walk down the pixel tiles, every warp has 16*MI pixels x 8*NJ columns and the whole reduction.
-template <bool BWD, int MI, int NJ, int G, int XF>
+//
+// A chunk of 32 channels is a step, whose operands are requested one step ahead, in registers.  DEEP: two or three steps ahead, by asynchronous copies into shared-memory slots that no
+// other thread reads, so that no barrier is needed.
+template <bool BWD, int MI, int XF> struct Slots {
+    static constexpr bool USE_Z = BWD ? XF != XF_NONE : XF == XF_ADD;
+    static constexpr int VECS = MI * 2 * (USE_Z ? 2 : 1), STEPS = VECS >= 8 ? 3 : 4;      // 16-byte vectors a thread and step, steps there is room for
+};
+template <bool BWD, int MI, int NJ, int G, int XF, bool DEEP>
 __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
+    using S = Slots<BWD, MI, XF>;
+    constexpr bool USE_Z = S::USE_Z;
+    constexpr int D = S::STEPS;
     extern __shared__ __align__(16) uint8_t sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const int wm = warp;
@@ -321,7 +331,6 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
 
     const uint8_t* pa = reinterpret_cast<const uint8_t*>(a.a);
     const uint8_t* pz = reinterpret_cast<const uint8_t*>(a.az);
-    constexpr bool USE_Z = BWD ? XF != XF_NONE : XF == XF_ADD;
     const int warp_row = wm * (16 * MI) + g, BM = a.WM * 16 * MI;
     const uint32_t row_bytes = (uint32_t)a.K * 2u;
     const uint32_t last_off = (uint32_t)min((a.KCH - 1) * 64 + t * 16, a.K * 2 - 16);     // beyond K: any finite value, its weights are zero
@@ -333,21 +342,52 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
             for (int h = 0; h < 2; ++h) roff[mi][h] = (uint32_t)min(tile * BM + warp_row + mi * 16 + h * 8, a.P - 1) * row_bytes;
     };
     uint4 nx[MI][2], nz[MI][2];
+    const uint32_t pitch = blockDim.x * 16u;               // DEEP: from one vector of a thread to its next, [slot][vector][thread]
+    const uint8_t* slots = reinterpret_cast<const uint8_t*>(red + a.WM * 2 * BN) + tid * 16;
+    const uint32_t slots_s = (uint32_t)__cvta_generic_to_shared(slots);
+    int ftile = blockIdx.x, fkc = 0, fslot = 0, slot = 0;  // DEEP: the step requested next, its slot; the slot of the step at hand
     auto fetch = [&](int kc) {
         const uint32_t o = kc == a.KCH - 1 ? last_off : (uint32_t)(kc * 64 + t * 16);
+        uint32_t d = slots_s + (uint32_t)(fslot * S::VECS) * pitch;
 #pragma unroll
         for (int mi = 0; mi < MI; ++mi)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                nx[mi][h] = *reinterpret_cast<const uint4*>(pa + (size_t)(roff[mi][h] + o));
-                if (USE_Z) nz[mi][h] = *reinterpret_cast<const uint4*>(pz + (size_t)(roff[mi][h] + o));
+                if constexpr (DEEP) {
+                    cp_async16(d, pa + (size_t)(roff[mi][h] + o), true);
+                    d += pitch;
+                    if (USE_Z) {
+                        cp_async16(d, pz + (size_t)(roff[mi][h] + o), true);
+                        d += pitch;
+                    }
+                } else {
+                    nx[mi][h] = *reinterpret_cast<const uint4*>(pa + (size_t)(roff[mi][h] + o));
+                    if (USE_Z) nz[mi][h] = *reinterpret_cast<const uint4*>(pz + (size_t)(roff[mi][h] + o));
+                }
             }
+    };
+    auto fetch_next = [&] {                                // DEEP
+        if (ftile < a.m_tiles) {
+            fetch(fkc);
+            if (++fkc == a.KCH) {
+                fkc = 0;
+                ftile += gridDim.x;
+                set_rows(ftile);
+            }
+        }
+        cp_commit();
+        if (++fslot == D) fslot = 0;
     };
     int tile = blockIdx.x;
     set_rows(tile);
-    fetch(0);
+    if constexpr (DEEP) {
+#pragma unroll
+        for (int i = 0; i < D - 1; ++i) fetch_next();
+    } else {
+        fetch(0);
+    }
     stage_coefs<BWD, XF>(a, sK, sN, n0, BN);
-    cp_wait<0>();
+    cp_wait<DEEP ? D - 1 : 0>();
     __syncthreads();
 
     const float rlo = a.r_act == ACT_NONE ? -INFINITY : 0.f, rhi = a.r_act == ACT_RELU6 ? 6.f : INFINITY;
@@ -397,10 +437,24 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
         for (int kc = 0; kc < a.KCH; ++kc) {
             uint4 cu[MI][2];
             if (a.KCH > 1) xf.load(sK, Kp, kc * 32 + t * 8);
+            if constexpr (DEEP) {
+                cp_wait<D - 2>();
+                const uint8_t* q = slots + (uint32_t)(slot * S::VECS) * pitch;
+#pragma unroll
+                for (int mi = 0; mi < MI; ++mi)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        nx[mi][h] = *reinterpret_cast<const uint4*>(q);
+                        if (USE_Z) nz[mi][h] = *reinterpret_cast<const uint4*>(q + pitch);
+                        q += pitch * (USE_Z ? 2 : 1);
+                    }
+                if (++slot == D) slot = 0;
+            }
 #pragma unroll
             for (int mi = 0; mi < MI; ++mi)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) cu[mi][h] = xf.apply(nx[mi][h], nz[mi][h]);
+            if constexpr (DEEP) fetch_next();
             if (!BWD && XF == XF_ADD && blockIdx.y == 0 && kc * 64 + t * 16 < a.K * 2)
 #pragma unroll
                 for (int mi = 0; mi < MI; ++mi)
@@ -409,10 +463,12 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
                         const int p = row0 + mi * 16 + h * 8;
                         if (p < a.P) *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(a.sum_out) + (size_t)p * row_bytes + (uint32_t)(kc * 64 + t * 16)) = cu[mi][h];
                     }
-            if (kc + 1 < a.KCH) fetch(kc + 1);
-            else if (tile + (int)gridDim.x < a.m_tiles) {
-                set_rows(tile + gridDim.x);
-                fetch(0);
+            if constexpr (!DEEP) {
+                if (kc + 1 < a.KCH) fetch(kc + 1);
+                else if (tile + (int)gridDim.x < a.m_tiles) {
+                    set_rows(tile + gridDim.x);
+                    fetch(0);
+                }
             }
 #pragma unroll
             for (int j = 0; j < NJ; ++j) {

@@ -33,6 +33,8 @@ struct MmaProblem {
 
 // Chooses a tiling; false: the layer does not run here (pw_tc.cu has the kernels for it).
 bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out);
+// whether a forward of this tiling, one CTA to all of the layer's columns, requests the operands of a deferred sum several steps ahead
+bool mma_deep_sum(int P, int K, const MmaTiling& c);
 size_t mma_smem(bool bwd, int K, const MmaTiling& c);
 void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, double bytes, cudaStream_t st);
 

@@ -634,17 +634,19 @@ static bool f32_unit(const asteroid_stage* s, const Unit& u, bool bwd, F32Tiling
 
 // A residual sum of two tensors without activations of their own, read next by a pointwise layer on the register-operand or float32
 // kernels: that layer forms it as it loads, and writes it out for the others.  Up to 4 M elements, where the sum is mostly a launch in the chain (a
-// round of a sixth of MobileNetV2 at batch 4 1681 -> 1647 us, of small images 1469 -> 1440); beyond, two operands to wait for cost the
-// pointwise layer more than the pass saves (ResNet stage at batch 32: 1 % slower).
+// round of a sixth of MobileNetV2 at batch 4 1681 -> 1647 us, of small images 1469 -> 1440); beyond, where every CTA of that layer takes all of its columns and has a reduction
+// long enough to request several steps ahead (pw_mma.cu): each operand is then read once, and the sum not again.  ResNet stage at batch 32: the three sums of 25.7 M elements in front of
+// 256 -> 64 19 887 -> 19 467 us a round, all sums up to 16.8 M, those of 12.8 M in front of 512 -> 128 whose columns take three CTAs, 20 055.
 static bool defers_add(const asteroid_stage* s, size_t ui) {
     const Unit& u = s->units[ui];
-    if (ui + 1 >= s->units.size() || s->vals[u.out].elems > (size_t)4 << 20) return false;
+    if (ui + 1 >= s->units.size()) return false;
     const Unit& v = s->units[ui + 1];
-    MmaTiling t;
+    MmaTiling t{};
     F32Tiling t32;
     if (v.kind != U_CONV || v.in != u.out || v.col_kp || v.sub_off >= 0) return false;
     if (u.in == u.in2 || s->vals[u.in].act != ACT_NONE || s->vals[u.in2].act != ACT_NONE) return false;
-    return mma_unit(s, v.g, false, &t) || f32_unit(s, v, false, &t32);
+    const bool mma = mma_unit(s, v.g, false, &t), small = s->vals[u.out].elems <= (size_t)4 << 20;
+    return small ? mma || f32_unit(s, v, false, &t32) : mma && 8 * t.nj >= v.g.co && mma_deep_sum(v.g.n * v.g.ho * v.g.wo, v.g.ci, t);
 }
 
 static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cudaStream_t st) {

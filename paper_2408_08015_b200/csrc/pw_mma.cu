@@ -13,16 +13,17 @@ using namespace mma;
 typedef void (*KernelFn)(const Args);
 
 constexpr size_t SMEM_MOST = 200 * 1024;
-// Whether a persistent layer's operands are requested several steps ahead (pw_mma.cuh): input gradients of 256 channels and more, forwards of 128 and more in blocks of 64
-// columns, where a CTA has more than one tile.  These read two to sixteen times what they write and took 0.75 to 1 us a step, a trip to memory, whatever the step's work was:
-// ResNet stage at batch 32 20 572 -> 19 885 us a round, the sums of defers_add (stage.cu) among it.  Elsewhere one step ahead in registers is as good or better, because slots cost
-// a store and a load of shared memory a vector: slots in all persistent kernels took half of MobileNetV2 with the head 4140 -> 4210 us, EfficientNet 6941 -> 7029, the ragged stage
-// 613 -> 637; input gradients from 128 channels on EfficientNet 6955 -> 6994, single tiles the ragged ResNet share 1681 -> 1689.
+// Whether a persistent layer's operands are requested several steps ahead (pw_mma.cuh): reductions of 128 channels and more in blocks of 64 columns, input gradients of 256 and more
+// in blocks of 32 and 48 as well, where a CTA has more than one tile.  These read two to sixteen times what they write and took 0.75 to 1 us a step, a trip to memory, whatever the
+// step's work was: ResNet stage at batch 32 20 575 -> 19 842 us a round, the sums of defers_add (stage.cu) among it (19 885 with input gradients from 256 channels on only).  Elsewhere one
+// step ahead in registers is as good or better, because slots cost a store and a load of shared memory a vector: slots in all persistent kernels took half of MobileNetV2 with the head
+// 4140 -> 4210 us, EfficientNet 6941 -> 7029, the ragged stage 613 -> 637; input gradients from 128 channels on in narrow blocks EfficientNet 6955 -> 6994, single tiles the ragged
+// ResNet share 1681 -> 1689.
 constexpr bool deep_form(bool bwd, int nj, int xf) { return bwd ? nj >= 4 && xf != XF_NONE : nj == 8; }
 size_t slot_bytes(const MmaTiling& c) { return (size_t)4 * c.mi * (c.mi == 2 ? 3 : 4) * 16 * 32 * c.wm; }       // of Slots (pw_mma.cuh), both operands
 bool deep_layer(bool bwd, int K, const MmaTiling& c, int xf) {
     const size_t smem = mma_smem(bwd, K, c) + slot_bytes(c);
-    return c.wk == 1 && deep_form(bwd, c.nj, xf) && K >= (bwd ? 256 : 128) && smem <= SMEM_MOST && (smem + 1024) * c.ctas <= 227 * 1024;
+    return c.wk == 1 && deep_form(bwd, c.nj, xf) && K >= (c.nj == 8 ? 128 : 256) && smem <= SMEM_MOST && (smem + 1024) * c.ctas <= 227 * 1024;
 }
 
 template <bool BWD, int NJ, int G, int XF> KernelFn pick(int mi, int wk, bool deep) {

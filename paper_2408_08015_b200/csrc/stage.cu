@@ -635,8 +635,8 @@ static bool f32_unit(const asteroid_stage* s, const Unit& u, bool bwd, F32Tiling
 // A residual sum of two tensors without activations of their own, read next by a pointwise layer on the register-operand or float32
 // kernels: that layer forms it as it loads, and writes it out for the others.  Up to 4 M elements, where the sum is mostly a launch in the chain (a
 // round of a sixth of MobileNetV2 at batch 4 1681 -> 1647 us, of small images 1469 -> 1440); beyond, where every CTA of that layer takes all of its columns and has a reduction
-// long enough to request several steps ahead (pw_mma.cu): each operand is then read once, and the sum not again.  ResNet stage at batch 32: the three sums of 25.7 M elements in front of
-// 256 -> 64 19 887 -> 19 467 us a round, all sums up to 16.8 M, those of 12.8 M in front of 512 -> 128 whose columns take three CTAs, 20 055.
+// long enough to request several steps ahead (pw_mma.cu): each operand is then read once, and the sum not again.  ResNet stage at batch 32, with such requests in all persistent layers: no large
+// sum left to the layer behind 19 871 us a round, all of them 19 651, those of 12.8 M elements in front of 512 -> 128 alone, whose columns take three CTAs, 20 055.
 static bool defers_add(const asteroid_stage* s, size_t ui) {
     const Unit& u = s->units[ui];
     if (ui + 1 >= s->units.size()) return false;

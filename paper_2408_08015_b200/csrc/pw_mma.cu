@@ -13,17 +13,19 @@ using namespace mma;
 typedef void (*KernelFn)(const Args);
 
 constexpr size_t SMEM_MOST = 200 * 1024;
-// Whether a persistent layer's operands are requested several steps ahead (pw_mma.cuh): reductions of 128 channels and more in blocks of 64 columns, input gradients of 256 and more
-// in blocks of 32 and 48 as well, where a CTA has more than one tile.  These read two to sixteen times what they write and took 0.75 to 1 us a step, a trip to memory, whatever the
-// step's work was: ResNet stage at batch 32 20 575 -> 19 842 us a round, the sums of defers_add (stage.cu) among it (19 885 with input gradients from 256 channels on only).  Elsewhere one
-// step ahead in registers is as good or better, because slots cost a store and a load of shared memory a vector: slots in all persistent kernels took half of MobileNetV2 with the head
-// 4140 -> 4210 us, EfficientNet 6941 -> 7029, the ragged stage 613 -> 637; input gradients from 128 channels on in narrow blocks EfficientNet 6955 -> 6994, single tiles the ragged
-// ResNet share 1681 -> 1689.
-constexpr bool deep_form(bool bwd, int nj, int xf) { return bwd ? nj >= 4 && xf != XF_NONE : nj == 8; }
+// Whether a persistent layer's operands are requested several steps ahead (pw_mma.cuh): reductions of 128 channels and more in blocks of 64 columns, where a CTA has more than one
+// tile.  These read two to sixteen times what they write and took 0.75 to 1 us a step, a trip to memory, whatever the step's work was: ResNet stage at batch 32 20 566 -> 19 614 us a
+// round, the sums of defers_add (stage.cu) among it.  Elsewhere one step ahead in registers is as good or better, because slots cost a store and a load of shared memory a vector:
+// slots in all persistent kernels took half of MobileNetV2 with the head 4140 -> 4210 us, EfficientNet 6941 -> 7029, the ragged stage 613 -> 637; input gradients in narrower blocks
+// EfficientNet 6955 -> 6994 from 128 channels on, 6936 -> 6955 from 256; single tiles the ragged ResNet share 1681 -> 1689.
+constexpr bool deep_form(bool bwd, int nj, int xf) { return nj == 8 && !(bwd && xf == XF_NONE); }
 size_t slot_bytes(const MmaTiling& c) { return (size_t)4 * c.mi * (c.mi == 2 ? 3 : 4) * 16 * 32 * c.wm; }       // of Slots (pw_mma.cuh), both operands
+// The slots lie behind the coefficients that the transform has, not the most it could have: the 8 KB of two CTAs decide whether gradients of 512 channels in blocks of 64 columns fit two to a
+// multiprocessor (ResNet stage at batch 32 19 830 -> 19 636 us a round).  Five steps ahead instead of three: 19 855.
+size_t deep_smem(bool bwd, int K, const MmaTiling& c, int xf) { return mma_smem(bwd, K, c) - (bwd && xf != XF_ACT ? (size_t)(K + 31) / 32 * 32 * 8 : 0) + slot_bytes(c); }
 bool deep_layer(bool bwd, int K, const MmaTiling& c, int xf) {
-    const size_t smem = mma_smem(bwd, K, c) + slot_bytes(c);
-    return c.wk == 1 && deep_form(bwd, c.nj, xf) && K >= (c.nj == 8 ? 128 : 256) && smem <= SMEM_MOST && (smem + 1024) * c.ctas <= 227 * 1024;
+    const size_t smem = deep_smem(bwd, K, c, xf);
+    return c.wk == 1 && deep_form(bwd, c.nj, xf) && K >= 128 && smem <= SMEM_MOST && (smem + 1024) * c.ctas <= 227 * 1024;
 }
 
 template <bool BWD, int NJ, int G, int XF> KernelFn pick(int mi, int wk, bool deep) {
@@ -237,7 +239,7 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
     else raise_limits<false>();
     a.late = !bwd && c.wk == 1 && gx * ny > sm_count();
     const bool deep = deep_layer(bwd, p.K, c, xf) && a.m_tiles > gx;
-    const size_t smem = mma_smem(bwd, p.K, c) + (deep ? slot_bytes(c) : 0);
+    const size_t smem = deep ? deep_smem(bwd, p.K, c, xf) : mma_smem(bwd, p.K, c);
     LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 2.0 * p.P * p.N : 0.0) + (p.sum_out ? 4.0 * p.P * p.K : 0.0), 2.0 * p.P * p.N * p.K, st);
     launch_pdl(bwd ? kernel_for<true>(c, xf, deep) : kernel_for<false>(c, xf, deep), dim3(gx, ny), c.wk == 1 ? 32 * c.wm : 256, smem, st, a);
 }

@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
     const int BN = NJ * 8, n0 = blockIdx.y * BN, Kp = a.KCH * 32;
     uint8_t* sW = sm;
     float* sK = reinterpret_cast<float*>(sW + (size_t)BN * a.wpitch);
-    float* sN = sK + (BWD ? 5 : 3) * Kp;
+    float* sN = sK + (BWD && XF == XF_ACT ? 5 : 3) * Kp;
     float* red = sN + (BWD ? 4 : 1) * BN;                  // [WM][2][BN]
     stage_weights<G>(a, sW, n0, BN);
     pdl_wait();

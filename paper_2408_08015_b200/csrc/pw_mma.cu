@@ -170,7 +170,8 @@ bool fwd_choose(int P, int K, int N, MmaTiling* out) {
 // Which layers run here: all whose channel counts are whole vectors, but for more than 256 x 64 products per pixel on more than 50 000 pixels with at most
 // 256 channels a side.  There the arithmetic of mma.sync (and the shared-memory reads of its weights) is the bound and the tensor-memory
 // pipeline of pw_tc.cu is as fast or faster: 64 -> 256 at 100 352 pixels 26.3 us against 29.3, backward to 256 channels 71 against 77.  To at
-// most 64 channels it is not: 256 -> 64 30.6 against 24.0, backward 45 against 42.  (One layer with its BatchNorm sums in a captured chain.)
+// most 64 channels it is not: 256 -> 64 30.6 against 24.0, backward 45 against 42.  (One layer with its BatchNorm sums in a captured chain.)  Requests several steps ahead do not move the
+// line: with 256 -> 128 forward here the ResNet stage at batch 32 takes 19 660 us a round, with its backward 19 671, without 19 611.
 // With 192 to 256 channels on both sides the pipeline does not fit and pw_stream.cu and the one-tile kernel take the layer: 256 -> 256 on 50 176
 // pixels forward 33 us with its pass for the sums (37 here), backward with a transform 49 (72), without 23 (49).
 bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {

@@ -13,12 +13,13 @@ using namespace mma;
 typedef void (*KernelFn)(const Args);
 
 constexpr size_t SMEM_MOST = 200 * 1024;
-// Whether a persistent layer's operands are requested several steps ahead (pw_mma.cuh): reductions of 128 channels and more in blocks of 64 columns, where a CTA has more than one
-// tile.  These read two to sixteen times what they write and took 0.75 to 1 us a step, a trip to memory, whatever the step's work was: ResNet stage at batch 32 20 566 -> 19 614 us a
-// round, the sums of defers_add (stage.cu) among it.  Elsewhere one step ahead in registers is as good or better, because slots cost a store and a load of shared memory a vector:
-// slots in all persistent kernels took half of MobileNetV2 with the head 4140 -> 4210 us, EfficientNet 6941 -> 7029, the ragged stage 613 -> 637; input gradients in narrower blocks
-// EfficientNet 6955 -> 6994 from 128 channels on, 6936 -> 6955 from 256; single tiles the ragged ResNet share 1681 -> 1689.
-constexpr bool deep_form(bool bwd, int nj, int xf) { return nj == 8 && !(bwd && xf == XF_NONE); }
+// Whether a persistent layer's operands are requested several steps ahead (pw_mma.cuh): input gradients of 128 channels and more in blocks of 64 columns and the large residual sums of
+// defers_add (stage.cu), where a CTA has more than one tile.  Both read two operands, and a step took 0.75 to 1 us, a trip to memory, whatever its work was: ResNet stage at batch 32
+// 20 566 -> 19 614 us a round.  A forward of one operand has its steps in time, and slots only add a store and a load of shared memory a vector: 128 -> 512 at 25 088 pixels 27.3 -> 29.9 us,
+// 256 -> 512 39.3 -> 43.7, 256 -> 64 at 57 000 19.0 -> 21.0 (that stage with such forwards 19 735 instead of 19 622).  Only operands beyond L2 gain there: 512 -> 64 from 94 000 pixels on,
+// 49 -> 43.  In narrower blocks one step ahead is as good or better too: slots in all persistent kernels took half of MobileNetV2 with the head 4140 -> 4210 us, EfficientNet 6941 -> 7029,
+// the ragged stage 613 -> 637; input gradients in narrower blocks EfficientNet 6955 -> 6994 from 128 channels on, 6936 -> 6955 from 256; single tiles the ragged ResNet share 1681 -> 1689.
+constexpr bool deep_form(bool bwd, int nj, int xf) { return nj == 8 && (bwd ? xf != XF_NONE : xf == XF_ADD); }
 size_t slot_bytes(const MmaTiling& c) { return (size_t)4 * c.mi * (c.mi == 2 ? 3 : 4) * 16 * 32 * c.wm; }       // of Slots (pw_mma.cuh), both operands
 // The slots lie behind the coefficients that the transform has, not the most it could have: the 8 KB of two CTAs decide whether gradients of 512 channels in blocks of 64 columns fit two to a
 // multiprocessor (ResNet stage at batch 32 19 830 -> 19 636 us a round).  Five steps ahead instead of three: 19 855.

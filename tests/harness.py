@@ -1,7 +1,9 @@
 """Shared test harness: run one HPP-Round on the oracle and on the CUDA library from the same
 seeded inputs, and compare tensor by tensor.  Imported by tests and the smoke check only."""
+import contextlib
 import json
 import os
+import tempfile
 
 import numpy as np
 
@@ -115,6 +117,25 @@ def gpu_round(net, first, last, h, w, B, M, loss, xs, tg, params, bf16, lr=0.01,
                 "loss": lossd.cpu().numpy().tolist(), "G": G, "w": wv, "v": vv, "g": micro}
     finally:
         P.asteroid_stage_destroy(hdl)
+
+
+@contextlib.contextmanager
+def kernels():
+    """The kernels that run inside the block, in the order of their starts: a list of {"name", "grid", "block"} that is filled when the block ends (empty where the profiler has no records)."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    found = []
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as p:
+        yield found
+        torch.cuda.synchronize()
+    with tempfile.TemporaryDirectory() as d:
+        path = os.path.join(d, "trace.json")
+        p.export_chrome_trace(path)
+        with open(path) as f:
+            events = [e for e in json.load(f)["traceEvents"] if e.get("cat") == "kernel"]
+    for e in sorted(events, key=lambda e: e["ts"]):
+        found.append({"name": e["name"], "grid": e["args"]["grid"], "block": e["args"]["block"]})
 
 
 def rel_err(a, b, floor=0.0):

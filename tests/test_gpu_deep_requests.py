@@ -4,7 +4,7 @@ elements that the layer behind forms as it loads, and ones that it does not (thr
 import pytest
 
 import stage_inputs as si
-from harness import ALL, CONTRACT, bf16_store, compare, gpu_round, make_inputs, oracle_round
+from harness import ALL, CONTRACT, bf16_store, compare, gpu_round, kernels, make_inputs, oracle_round
 
 pytestmark = pytest.mark.gpu
 
@@ -19,6 +19,24 @@ def _check(net, h, w, B, case, act):
     mirror = oracle_round(net, 0, last, B, 1, "mse", xs, tg, params, store=bf16_store) if act else None
     gpu = gpu_round(net, 0, last, h, w, B, 1, "mse", xs, tg, params, True)
     compare(gpu, plain, net, 0, last, 2e-2, mirror=mirror, allow=ALL if act else (CONTRACT,), case="deep/%s" % case)
+
+
+def _ahead(found, bwd):
+    """Of the register-operand pointwise kernels of one direction: which request several steps ahead (their last template argument)."""
+    if not found:
+        pytest.skip("no kernel records from the profiler")
+    names = [k["name"] for k in found if "pw_mma_kernel<%s," % ("true" if bwd else "false") in k["name"]]
+    return [n.split("pw_mma_kernel<")[1].split(">")[0].endswith("true") for n in names]
+
+
+# several column blocks, and one: forwards of long reductions and several tiles a CTA, whose operand the layer before has just written
+@pytest.mark.parametrize("c, c_out, h, w, B", [(128, 512, 28, 28, 32), (256, 512, 25, 20, 40), (256, 64, 95, 100, 6)])
+def test_forwards_request_one_step_ahead(c, c_out, h, w, B):
+    net = [L("conv", 16, c, 1, 1, 0, -1, -1), L("bn", c, c, 0, 1, 0, 0, -1), L("relu", c, c, 0, 1, 0, 1, -1), L("conv", c, c_out, 1, 1, 0, 2, -1), L("bn", c_out, c_out, 0, 1, 0, 3, -1)]
+    xs, tg, params, _ = make_inputs(net, 0, 4, h, w, B, 1, "mse", 59, True)
+    with kernels() as found:
+        gpu_round(net, 0, 4, h, w, B, 1, "mse", xs, tg, params, True)
+    assert _ahead(found, False) == [False, False]
 
 
 # 5 pixels: one tile; 1 000: single and partly filled ones; 19 594: several a CTA

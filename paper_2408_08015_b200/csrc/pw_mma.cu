@@ -19,11 +19,14 @@ constexpr size_t SMEM_MOST = 200 * 1024;
 // 256 -> 512 39.3 -> 43.7, 256 -> 64 at 57 000 19.0 -> 21.0 (that stage with such forwards 19 735 instead of 19 622).  Only operands beyond L2 gain there: 512 -> 64 from 94 000 pixels on,
 // 49 -> 43.  In narrower blocks one step ahead is as good or better too: slots in all persistent kernels took half of MobileNetV2 with the head 4140 -> 4210 us, EfficientNet 6941 -> 7029,
 // the ragged stage 613 -> 637; input gradients in narrower blocks EfficientNet 6955 -> 6994 from 128 channels on, 6936 -> 6955 from 256; single tiles the ragged ResNet share 1681 -> 1689.
-constexpr bool deep_form(bool bwd, int nj, int xf) { return nj == 8 && (bwd ? xf != XF_NONE : xf == XF_ADD); }
+constexpr bool deep_form(bool bwd, int nj, int xf) { return nj == 8 && (bwd ? xf != XF_NONE : xf == XF_SUM); }
 size_t slot_bytes(const MmaTiling& c) { return (size_t)4 * c.mi * (c.mi == 2 ? 3 : 4) * 16 * 32 * c.wm; }       // of Slots (pw_mma.cuh), both operands
 // The slots lie behind the coefficients that the transform has, not the most it could have: the 8 KB of two CTAs decide whether gradients of 512 channels in blocks of 64 columns fit two to a
 // multiprocessor (ResNet stage at batch 32 19 830 -> 19 636 us a round).  Five steps ahead instead of three: 19 855.
-size_t deep_smem(bool bwd, int K, const MmaTiling& c, int xf) { return mma_smem(bwd, K, c) - (bwd && xf != XF_ACT ? (size_t)(K + 31) / 32 * 32 * 8 : 0) + slot_bytes(c); }
+size_t deep_smem(bool bwd, int K, const MmaTiling& c, int xf) {
+    const size_t Kp = (size_t)(K + 31) / 32 * 32;
+    return mma_smem(bwd, K, c) - (bwd && xf != XF_ACT ? 8 * Kp : 0) + (xf == XF_SUM ? 4 * Kp : 0) + slot_bytes(c);
+}
 bool deep_layer(bool bwd, int K, const MmaTiling& c, int xf) {
     const size_t smem = deep_smem(bwd, K, c, xf);
     return c.wk == 1 && deep_form(bwd, c.nj, xf) && K >= 128 && smem <= SMEM_MOST && (smem + 1024) * c.ctas <= 227 * 1024;
@@ -45,6 +48,7 @@ template <bool BWD, int XF> KernelFn by_columns(const MmaTiling& c, bool deep) {
     }
 }
 template <bool BWD> KernelFn kernel_for(const MmaTiling& c, int xf, bool deep) {
+    if (!BWD && xf == XF_SUM) return c.mi == 1 ? pw_mma_kernel<false, 1, 8, 4, XF_SUM, true> : pw_mma_kernel<false, 2, 8, 4, XF_SUM, true>;
     if (!BWD && xf == XF_ADD) return by_columns<false, XF_ADD>(c, deep);
     return xf == XF_NONE ? by_columns<BWD, XF_NONE>(c, deep) : xf == XF_AFFINE ? by_columns<BWD, XF_AFFINE>(c, deep) : by_columns<BWD, XF_ACT>(c, deep);
 }
@@ -57,7 +61,7 @@ template <bool BWD> void raise_limits() {
     if (done.load(std::memory_order_acquire) & bit) return;
     for (int nj : {2, 3, 4, 6, 8})
         for (int v = 0; v < 5; ++v)
-            for (int xf = XF_NONE; xf <= (BWD ? XF_ACT : XF_ADD); ++xf) {
+            for (int xf = XF_NONE; xf <= (BWD ? XF_ACT : XF_SUM); ++xf) {
                 MmaTiling c{};
                 c.nj = nj;
                 c.mi = v == 1 ? 2 : 1;
@@ -181,7 +185,7 @@ bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {
     return bwd ? bwd_choose(P, K, N, out) : fwd_choose(P, K, N, out);
 }
 
-bool mma_deep_sum(int P, int K, const MmaTiling& c) { return deep_layer(false, K, c, XF_ADD) && (P + 16 * c.mi * c.wm - 1) / (16 * c.mi * c.wm) > sm_count() * c.ctas; }
+bool mma_deep_sum(int P, int K, const MmaTiling& c) { return deep_layer(false, K, c, XF_SUM) && (P + 16 * c.mi * c.wm - 1) / (16 * c.mi * c.wm) > sm_count() * c.ctas; }
 
 size_t mma_smem(bool bwd, int K, const MmaTiling& c) {
     const int Kp = (K + 31) / 32 * 32, BN = c.nj * 8;
@@ -211,7 +215,7 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
         a.pf = p.pf;
         xf = p.x.act != ACT_NONE ? XF_ACT : (p.x.scale || p.pf.sums) ? XF_AFFINE : XF_NONE;
         if (p.sum_out) {
-            xf = XF_ADD;
+            xf = p.sum_large ? XF_SUM : XF_ADD;
             a.az = p.x2.p; a.d0 = p.x2.scale; a.d1 = p.x2.shift;
             a.pf2 = p.pf2;
             a.sum_out = (__nv_bfloat16*)p.sum_out;
@@ -240,7 +244,7 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
     if (bwd) raise_limits<true>();
     else raise_limits<false>();
     a.late = !bwd && c.wk == 1 && gx * ny > sm_count();
-    const bool deep = deep_layer(bwd, p.K, c, xf) && a.m_tiles > gx;
+    const bool deep = xf == XF_SUM || (deep_layer(bwd, p.K, c, xf) && a.m_tiles > gx);
     const size_t smem = deep ? deep_smem(bwd, p.K, c, xf) : mma_smem(bwd, p.K, c);
     LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 2.0 * p.P * p.N : 0.0) + (p.sum_out ? 4.0 * p.P * p.K : 0.0), 2.0 * p.P * p.N * p.K, st);
     launch_pdl(bwd ? kernel_for<true>(c, xf, deep) : kernel_for<false>(c, xf, deep), dim3(gx, ny), c.wk == 1 ? 32 * c.wm : 256, smem, st, a);

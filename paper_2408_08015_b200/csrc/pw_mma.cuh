@@ -77,21 +77,26 @@ __device__ __forceinline__ uint32_t pack2(float2 f) {
 // Operand transforms of 8 channels.  Forward: the activation is applied after rounding on packed pairs, as one integer
 // min-then-max-with-0 (the bit patterns of non-negative bfloat16 numbers order like integers and negative ones are negative
 // integers; rounding is monotonic and 0 and 6 are bfloat16 numbers, so clamping before or after it is the same).
-// XF_ADD (forward): the operand is a residual sum that has not been formed yet, act(x*s + z*s2 + h) of two tensors.
-enum { XF_NONE = 0, XF_AFFINE = 1, XF_ACT = 2, XF_ADD = 3 };
+// XF_ADD, XF_SUM (forward): the operand is a residual sum that has not been formed yet, act(x*s + z*s2 + h) of two tensors with their shifts added first, or
+// act((x*s + h) + (z*s2 + h2)), the roundings of the elementwise pass (bn_ew.cu).  Only a ReLU may follow a sum.  Either applies it before rounding by that pass's fmaxf, so that what is
+// not a number leaves as it does there, as the activation's lower end.
+enum { XF_NONE = 0, XF_AFFINE = 1, XF_ACT = 2, XF_ADD = 3, XF_SUM = 4 };
+__host__ __device__ constexpr bool xf_sum(int xf) { return xf == XF_ADD || xf == XF_SUM; }
 template <int XF> struct XfFwd {
-    float s[8], h[8], s2[8];
-    uint32_t top;
-    bool relu;
+    float s[8], h[8], s2[8], h2[8];
+    float lo;                  // of a sum
+    uint32_t top;              // of a value
     __device__ __forceinline__ void load(const float* sm, int Kp, int c) {
         if (XF == XF_NONE) return;
         lds8(sm + c, s);
         lds8(sm + Kp + c, h);
-        if (XF == XF_ADD) lds8(sm + 2 * Kp + c, s2);
+        if (xf_sum(XF)) lds8(sm + 2 * Kp + c, s2);
+        if (XF == XF_SUM) lds8(sm + 3 * Kp + c, h2);
     }
     __device__ __forceinline__ uint32_t sum(uint32_t w, uint32_t z, int q) const {
-        const uint32_t r = pack2(__ffma2_rn(unpack2(w), make_float2(s[q], s[q + 1]), __ffma2_rn(unpack2(z), make_float2(s2[q], s2[q + 1]), make_float2(h[q], h[q + 1]))));
-        return relu ? __vimin_s16x2_relu(r, top) : r;
+        const float2 x = unpack2(w), y = unpack2(z), sx = make_float2(s[q], s[q + 1]), hx = make_float2(h[q], h[q + 1]), sy = make_float2(s2[q], s2[q + 1]);
+        const float2 r = XF == XF_SUM ? __fadd2_rn(__ffma2_rn(x, sx, hx), __ffma2_rn(y, sy, make_float2(h2[q], h2[q + 1]))) : __ffma2_rn(x, sx, __ffma2_rn(y, sy, hx));
+        return pack2(make_float2(fmaxf(r.x, lo), fmaxf(r.y, lo)));
     }
     __device__ __forceinline__ uint32_t two(uint32_t w, int q) const {
         const uint32_t r = pack2(__ffma2_rn(unpack2(w), make_float2(s[q], s[q + 1]), make_float2(h[q], h[q + 1])));
@@ -99,7 +104,7 @@ template <int XF> struct XfFwd {
     }
     __device__ __forceinline__ uint4 apply(const uint4& v, const uint4& z) const {
         if (XF == XF_NONE) return v;
-        if (XF == XF_ADD) return make_uint4(sum(v.x, z.x, 0), sum(v.y, z.y, 2), sum(v.z, z.z, 4), sum(v.w, z.w, 6));
+        if (xf_sum(XF)) return make_uint4(sum(v.x, z.x, 0), sum(v.y, z.y, 2), sum(v.z, z.z, 4), sum(v.w, z.w, 6));
         return make_uint4(two(v.x, 0), two(v.y, 2), two(v.z, 4), two(v.w, 6));
     }
 };
@@ -137,7 +142,7 @@ template <bool BWD, int XF> struct Xf;
 template <int XF> struct Xf<false, XF> : XfFwd<XF> {
     __device__ __forceinline__ void set_act(int act) {
         this->top = act == ACT_RELU6 ? 0x40C040C0u : 0x7F807F80u;
-        this->relu = act != ACT_NONE;
+        this->lo = act == ACT_NONE ? -INFINITY : 0.f;
     }
 };
 template <int XF> struct Xf<true, XF> : XfBwd<XF> {
@@ -200,7 +205,7 @@ template <bool BWD, int XF> __device__ __forceinline__ void stage_coefs(const Ar
                     to.k1 = a.c0[ch];
                     to.k2 = a.c1[ch];
                 }
-                if (XF == XF_ADD) {
+                if (xf_sum(XF)) {
                     if (a.pf2.sums) to.in2.load(a.pf2, ch, first);
                     else if (a.d0) {
                         to.s = a.d0[ch];
@@ -231,12 +236,13 @@ template <bool BWD, int XF> __device__ __forceinline__ void stage_coefs(const Ar
                 if (ok && a.pf.sums) k = in.in.coef(a.pf, c, first);
                 else if (ok && a.c0) k = make_float2(in.k1, in.k2);
                 sK[c] = k.x;
-                if (XF == XF_ADD) {
+                if (xf_sum(XF)) {
                     float2 k2 = make_float2(1.f, 0.f);
                     if (ok && a.pf2.sums) k2 = in.in2.coef(a.pf2, c, first);
                     else if (ok && a.d0) k2 = make_float2(in.s, in.h);
                     sK[2 * Kp + c] = k2.x;
-                    k.y += k2.y;
+                    if (XF == XF_SUM) sK[3 * Kp + c] = k2.y;
+                    else k.y += k2.y;
                 }
                 sK[Kp + c] = k.y;
             }
@@ -309,7 +315,7 @@ template <> struct SumCoef<true> {
 // A chunk of 32 channels is a step, whose operands are requested one step ahead, in registers.  DEEP: two or three steps ahead, by asynchronous copies into shared-memory slots that no
 // other thread reads, so that no barrier is needed.
 template <bool BWD, int MI, int XF> struct Slots {
-    static constexpr bool USE_Z = BWD ? XF != XF_NONE : XF == XF_ADD;
+    static constexpr bool USE_Z = BWD ? XF != XF_NONE : xf_sum(XF);
     static constexpr int VECS = MI * 2 * (USE_Z ? 2 : 1), STEPS = VECS >= 8 ? 3 : 4;      // 16-byte vectors a thread and step, steps there is room for
 };
 template <bool BWD, int MI, int NJ, int G, int XF, bool DEEP>
@@ -323,7 +329,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
     const int BN = NJ * 8, n0 = blockIdx.y * BN, Kp = a.KCH * 32;
     uint8_t* sW = sm;
     float* sK = reinterpret_cast<float*>(sW + (size_t)BN * a.wpitch);
-    float* sN = sK + (BWD && XF == XF_ACT ? 5 : 3) * Kp;
+    float* sN = sK + (BWD && XF == XF_ACT ? 5 : XF == XF_SUM ? 4 : 3) * Kp;
     float* red = sN + (BWD ? 4 : 1) * BN;                  // [WM][2][BN]
     stage_weights<G>(a, sW, n0, BN);
     pdl_wait();
@@ -455,7 +461,7 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) cu[mi][h] = xf.apply(nx[mi][h], nz[mi][h]);
             if constexpr (DEEP) fetch_next();
-            if (!BWD && XF == XF_ADD && blockIdx.y == 0 && kc * 64 + t * 16 < a.K * 2)
+            if (!BWD && xf_sum(XF) && blockIdx.y == 0 && kc * 64 + t * 16 < a.K * 2)
 #pragma unroll
                 for (int mi = 0; mi < MI; ++mi)
 #pragma unroll

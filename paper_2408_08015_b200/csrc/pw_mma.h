@@ -22,6 +22,7 @@ struct MmaProblem {
     BnPendFwd pf2;
     void* sum_out;
     int sum_act;
+    bool sum_large;            // mma_deep_sum said so: the roundings of the elementwise pass, operands requested several steps ahead
     BnPendBwd pb;              // pending coefficients of dz
     const void* w;             // [N][K]
     const float* bias;
@@ -33,7 +34,7 @@ struct MmaProblem {
 
 // Chooses a tiling; false: the layer does not run here (pw_tc.cu has the kernels for it).
 bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out);
-// whether a forward of this tiling, one CTA to all of the layer's columns, requests the operands of a deferred sum several steps ahead
+// whether a forward of this tiling, one CTA to all of the layer's columns, can request the operands of a deferred sum several steps ahead
 bool mma_deep_sum(int P, int K, const MmaTiling& c);
 size_t mma_smem(bool bwd, int K, const MmaTiling& c);
 void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, double bytes, cudaStream_t st);

@@ -637,6 +637,8 @@ static bool f32_unit(const asteroid_stage* s, const Unit& u, bool bwd, F32Tiling
 // round of a sixth of MobileNetV2 at batch 4 1681 -> 1647 us, of small images 1469 -> 1440); beyond, where every CTA of that layer takes all of its columns and has a reduction
 // long enough to request several steps ahead (pw_mma.cu): each operand is then read once, and the sum not again.  ResNet stage at batch 32, with such requests in all persistent layers: no large
 // sum left to the layer behind 19 871 us a round, all of them 19 651, those of 12.8 M elements in front of 512 -> 128 alone, whose columns take three CTAs, 20 055.
+// The value is the elementwise pass's: beyond 4 M elements to the bit, up to there but for the shifts, which are added first.
+static bool small_sum(const Val& sum) { return sum.elems <= (size_t)4 << 20; }
 static bool defers_add(const asteroid_stage* s, size_t ui) {
     const Unit& u = s->units[ui];
     if (ui + 1 >= s->units.size()) return false;
@@ -645,8 +647,8 @@ static bool defers_add(const asteroid_stage* s, size_t ui) {
     F32Tiling t32;
     if (v.kind != U_CONV || v.in != u.out || v.col_kp || v.sub_off >= 0) return false;
     if (u.in == u.in2 || s->vals[u.in].act != ACT_NONE || s->vals[u.in2].act != ACT_NONE) return false;
-    const bool mma = mma_unit(s, v.g, false, &t), small = s->vals[u.out].elems <= (size_t)4 << 20;
-    return small ? mma || f32_unit(s, v, false, &t32) : mma && 8 * t.nj >= v.g.co && mma_deep_sum(v.g.n * v.g.ho * v.g.wo, v.g.ci, t);
+    const bool mma = mma_unit(s, v.g, false, &t);
+    return small_sum(s->vals[u.out]) ? mma || f32_unit(s, v, false, &t32) : mma && 8 * t.nj >= v.g.co && mma_deep_sum(v.g.n * v.g.ho * v.g.wo, v.g.ci, t);
 }
 
 static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cudaStream_t st) {
@@ -690,6 +692,7 @@ static int forward_impl(asteroid_stage* s, int slot, const void* x, void* y, cud
                 p.pf2 = pend.take_fwd(producer(au.in2));
                 p.sum_out = sv.base + s->vals[au.out].buf_off;
                 p.sum_act = au.act;
+                p.sum_large = !small_sum(s->vals[au.out]);
                 deferred = -1;
             }
             if (bn) p.so = sums_fwd(s, u);

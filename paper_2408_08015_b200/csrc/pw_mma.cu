@@ -27,9 +27,14 @@ size_t deep_smem(bool bwd, int K, const MmaTiling& c, int xf) {
     const size_t Kp = (size_t)(K + 31) / 32 * 32;
     return mma_smem(bwd, K, c) - (bwd && xf != XF_ACT ? 8 * Kp : 0) + (xf == XF_SUM ? 4 * Kp : 0) + slot_bytes(c);
 }
-bool deep_layer(bool bwd, int K, const MmaTiling& c, int xf) {
+// Gradients behind an activation that is not in them yet have more arithmetic to a step, and rows that are no whole 32-byte sectors (the copies pass L1 by, where a load in registers finds the
+// sector it shares with the row before): both gain only where the two operands, 32 MB and more, come from beyond L2 in good part.  A unit's forward and backward, one step ahead against several
+// (reduction -> columns of the gradient): with a ReLU 136 -> 256 at 10 000 pixels 52.0 us against 53.0, 136 -> 64 at 57 000 71.5 against 72.6, but 384 -> 512 there 524 against 495; 136 -> 256
+// without at 10 000 pixels 49.8 against 50.2, 264 -> 512 at 57 000 410 against 377.  All others gain from 5 000 pixels on (512 -> 512 104.2 against 101.8) or stay (128 -> 64 at 25 088 44.5 against 44.6).
+bool deep_layer(bool bwd, int P, int K, const MmaTiling& c, int xf) {
     const size_t smem = deep_smem(bwd, K, c, xf);
-    return c.wk == 1 && deep_form(bwd, c.nj, xf) && K >= 128 && smem <= SMEM_MOST && (smem + 1024) * c.ctas <= 227 * 1024;
+    return c.wk == 1 && deep_form(bwd, c.nj, xf) && K >= 128 && (!bwd || (xf == XF_AFFINE && K % 16 == 0) || (size_t)P * K >= (size_t)8 << 20) && smem <= SMEM_MOST &&
+           (smem + 1024) * c.ctas <= 227 * 1024;
 }
 
 template <bool BWD, int NJ, int G, int XF> KernelFn pick(int mi, int wk, bool deep) {
@@ -185,7 +190,7 @@ bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {
     return bwd ? bwd_choose(P, K, N, out) : fwd_choose(P, K, N, out);
 }
 
-bool mma_deep_sum(int P, int K, const MmaTiling& c) { return deep_layer(false, K, c, XF_SUM) && (P + 16 * c.mi * c.wm - 1) / (16 * c.mi * c.wm) > sm_count() * c.ctas; }
+bool mma_deep_sum(int P, int K, const MmaTiling& c) { return deep_layer(false, P, K, c, XF_SUM) && (P + 16 * c.mi * c.wm - 1) / (16 * c.mi * c.wm) > sm_count() * c.ctas; }
 
 size_t mma_smem(bool bwd, int K, const MmaTiling& c) {
     const int Kp = (K + 31) / 32 * 32, BN = c.nj * 8;
@@ -244,7 +249,7 @@ void mma_launch(bool bwd, const MmaProblem& p, const MmaTiling& c, int kind, dou
     if (bwd) raise_limits<true>();
     else raise_limits<false>();
     a.late = !bwd && c.wk == 1 && gx * ny > sm_count();
-    const bool deep = xf == XF_SUM || (deep_layer(bwd, p.K, c, xf) && a.m_tiles > gx);
+    const bool deep = xf == XF_SUM || (deep_layer(bwd, p.P, p.K, c, xf) && a.m_tiles > gx);
     const size_t smem = deep ? deep_smem(bwd, p.K, c, xf) : mma_smem(bwd, p.K, c);
     LaunchScope ls(kind, bytes + (bwd && p.so.sums ? 2.0 * p.P * p.N : 0.0) + (p.sum_out ? 4.0 * p.P * p.K : 0.0), 2.0 * p.P * p.N * p.K, st);
     launch_pdl(bwd ? kernel_for<true>(c, xf, deep) : kernel_for<false>(c, xf, deep), dim3(gx, ny), c.wk == 1 ? 32 * c.wm : 256, smem, st, a);

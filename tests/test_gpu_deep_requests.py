@@ -39,15 +39,54 @@ def test_forwards_request_one_step_ahead(c, c_out, h, w, B):
     assert _ahead(found, False) == [False, False]
 
 
-# 5 pixels: one tile; 1 000: single and partly filled ones; 19 594: several a CTA
-@pytest.mark.parametrize("h, w, B", [(1, 5, 1), (25, 20, 2), (101, 97, 2)])
-@pytest.mark.parametrize("c_in, c_out", [(32, 128), (64, 136), (72, 168), (64, 264), (48, 520)])
-@pytest.mark.parametrize("act", [None, "relu6"])
-def test_input_gradients(c_in, c_out, h, w, B, act):
-    net = [L("conv", c_in, c_out, 1, 1, 0, -1, -1), L("bn", c_out, c_out, 0, 1, 0, 0, -1)] + ([L(act, c_out, c_out, 0, 1, 0, 1, -1)] if act else [])
-    if act and h * w * B < 50:
-        pytest.skip("masks of five values a channel")
-    _check(net, h, w, B, "%d_%d_%d_%s" % (c_in, c_out, h * w * B, act), act)
+def _net(c_in, c_out, act, where):
+    """A 1x1 layer with BatchNorm [and an activation]; "behind" another one, whose BatchNorm sums its input gradient takes; in a "block", whose residual gradient it adds as well."""
+    net = []
+
+    def unit(ci, co, src, op):
+        net.extend([L("conv", ci, co, 1, 1, 0, src, -1), L("bn", co, co, 0, 1, 0, len(net), -1)])
+        if op:
+            net.append(L(op, co, co, 0, 1, 0, len(net) - 1, -1))
+        return len(net) - 1
+
+    top = unit(16, c_in, -1, "relu") if where else -1
+    last = unit(c_in, c_out, top, act)
+    if where == "block":
+        last = unit(c_out, c_in, last, None)
+        net.append(L("add", c_in, c_in, 0, 1, 0, last, top))
+    return net
+
+
+GRADIENTS = {
+    # columns (c_in), reduction (c_out), activation, where, h, w, micro-batch: several steps ahead?, threads of a CTA, column blocks, fewest tiles of a CTA
+    "eight_warps": (256, 144, None, None, 209, 79, 1, True, 256, 4, 3),
+    "eight_warps_long": (128, 528, None, "behind", 53, 67, 5, True, 256, 2, 1),
+    "four_warps": (64, 176, None, None, 57013, 1, 1, True, 128, 1, 3),
+    "four_warps_chunk_tail": (64, 152, None, "behind", 57013, 1, 1, True, 128, 1, 3),
+    "four_warps_blocks": (192, 528, None, "behind", 20011, 1, 1, True, 128, 3, 3),
+    "column_tail": (184, 272, None, None, 20011, 1, 1, True, 128, 3, 3),
+    "one_block_column_tail": (56, 128, None, "behind", 101, 113, 5, True, 128, 1, 3),
+    "addend": (64, 144, "relu", "block", 101, 113, 5, True, 128, 1, 3),
+    "activation": (256, 264, "relu", None, 171, 193, 1, True, 128, 4, 6),
+    "activation_relu6": (320, 272, "relu6", "behind", 171, 193, 1, True, 128, 5, 8),
+    # one step ahead: an activation or split sectors on smaller maps, short reductions, one tile a CTA
+    "activation_small": (256, 136, "relu", None, 109, 92, 1, False, 256, 4, 2),
+    "split_sectors_small": (256, 136, None, None, 25, 1000, 1, False, 128, 4, 5),
+    "short": (64, 120, None, None, 57013, 1, 1, False, 128, 1, 3),
+    "one_tile": (64, 128, None, None, 13, 1000, 1, False, 256, 1, 1),
+}
+
+
+@pytest.mark.parametrize("name", list(GRADIENTS))
+def test_input_gradients(name):
+    c_in, c_out, act, where, h, w, B, ahead, threads, blocks, tiles = GRADIENTS[name]
+    net = _net(c_in, c_out, act, where)
+    with kernels() as found:
+        _check(net, h, w, B, name, bool(act or where))
+    got = [k for k in found if "pw_mma_kernel<true," in k["name"] and k["grid"][1] == blocks and ", 8, 4, " in k["name"]]
+    assert _ahead(found, True).count(True) == int(ahead)
+    mine = next(k for k in got if _ahead([k], True) == [ahead])
+    assert mine["block"][0] == threads and -(-h * w * B // (threads // 2)) >= tiles * mine["grid"][0]
 
 
 # formed by the layer: 256 -> 64 and 264 -> 40 on 16 510 pixels; not: 256 -> 136 (more columns than a CTA takes), 128 -> 64 on 33 020

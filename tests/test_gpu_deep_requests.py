@@ -69,6 +69,7 @@ GRADIENTS = {
     "addend": (64, 144, "relu", "block", 101, 113, 5, True, 128, 1, 3),
     "activation": (256, 264, "relu", None, 171, 193, 1, True, 128, 4, 6),
     "activation_relu6": (320, 272, "relu6", "behind", 171, 193, 1, True, 128, 5, 8),
+    "activation_short": (512, 128, "relu", None, 28, 28, 32, True, 128, 8, 10),
     # one step ahead: an activation or split sectors on smaller maps, short reductions, one tile a CTA
     "activation_small": (256, 136, "relu", None, 109, 92, 1, False, 256, 4, 2),
     "split_sectors_small": (256, 136, None, None, 25, 1000, 1, False, 128, 4, 5),

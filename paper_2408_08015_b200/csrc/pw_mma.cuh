@@ -78,13 +78,13 @@ __device__ __forceinline__ uint32_t pack2(float2 f) {
 // min-then-max-with-0 (the bit patterns of non-negative bfloat16 numbers order like integers and negative ones are negative
 // integers; rounding is monotonic and 0 and 6 are bfloat16 numbers, so clamping before or after it is the same).
 // XF_ADD, XF_SUM (forward): the operand is a residual sum that has not been formed yet, act(x*s + z*s2 + h) of two tensors with their shifts added first, or
-// act((x*s + h) + (z*s2 + h2)), the roundings of the elementwise pass (bn_ew.cu).  Only a ReLU may follow a sum.  Either applies it before rounding by that pass's fmaxf, so that what is
-// not a number leaves as it does there, as the activation's lower end.
+// act((x*s + h) + (z*s2 + h2)), the roundings of the elementwise pass (bn_ew.cu).  Only a ReLU may follow a sum.  Either applies it as a maximum of packed pairs, by which what is not a number
+// leaves as it does there by fmaxf, as the activation's lower end.
 enum { XF_NONE = 0, XF_AFFINE = 1, XF_ACT = 2, XF_ADD = 3, XF_SUM = 4 };
 __host__ __device__ constexpr bool xf_sum(int xf) { return xf == XF_ADD || xf == XF_SUM; }
 template <int XF> struct XfFwd {
     float s[8], h[8], s2[8], h2[8];
-    float lo;                  // of a sum
+    __nv_bfloat162 lo;         // of a sum
     uint32_t top;              // of a value
     __device__ __forceinline__ void load(const float* sm, int Kp, int c) {
         if (XF == XF_NONE) return;
@@ -96,7 +96,8 @@ template <int XF> struct XfFwd {
     __device__ __forceinline__ uint32_t sum(uint32_t w, uint32_t z, int q) const {
         const float2 x = unpack2(w), y = unpack2(z), sx = make_float2(s[q], s[q + 1]), hx = make_float2(h[q], h[q + 1]), sy = make_float2(s2[q], s2[q + 1]);
         const float2 r = XF == XF_SUM ? __fadd2_rn(__ffma2_rn(x, sx, hx), __ffma2_rn(y, sy, make_float2(h2[q], h2[q + 1]))) : __ffma2_rn(x, sx, __ffma2_rn(y, sy, hx));
-        return pack2(make_float2(fmaxf(r.x, lo), fmaxf(r.y, lo)));
+        const __nv_bfloat162 o = __hmax2(__floats2bfloat162_rn(r.x, r.y), lo);
+        return *reinterpret_cast<const uint32_t*>(&o);
     }
     __device__ __forceinline__ uint32_t two(uint32_t w, int q) const {
         const uint32_t r = pack2(__ffma2_rn(unpack2(w), make_float2(s[q], s[q + 1]), make_float2(h[q], h[q + 1])));
@@ -142,7 +143,7 @@ template <bool BWD, int XF> struct Xf;
 template <int XF> struct Xf<false, XF> : XfFwd<XF> {
     __device__ __forceinline__ void set_act(int act) {
         this->top = act == ACT_RELU6 ? 0x40C040C0u : 0x7F807F80u;
-        this->lo = act == ACT_NONE ? -INFINITY : 0.f;
+        this->lo = __float2bfloat162_rn(act == ACT_NONE ? -INFINITY : 0.f);
     }
 };
 template <int XF> struct Xf<true, XF> : XfBwd<XF> {

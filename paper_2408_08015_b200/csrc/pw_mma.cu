@@ -19,13 +19,13 @@ constexpr size_t SMEM_MOST = 200 * 1024;
 // 256 -> 512 39.3 -> 43.7, 256 -> 64 at 57 000 19.0 -> 21.0 (that stage with such forwards 19 735 instead of 19 622).  Only operands beyond L2 gain there: 512 -> 64 from 94 000 pixels on,
 // 49 -> 43.  In narrower blocks one step ahead is as good or better too: slots in all persistent kernels took half of MobileNetV2 with the head 4140 -> 4210 us, EfficientNet 6941 -> 7029,
 // the ragged stage 613 -> 637; input gradients in narrower blocks EfficientNet 6955 -> 6994 from 128 channels on, 6936 -> 6955 from 256; single tiles the ragged ResNet share 1681 -> 1689.
-constexpr bool deep_form(bool bwd, int nj, int xf) { return nj == 8 && (bwd ? xf != XF_NONE : xf == XF_SUM); }
-size_t slot_bytes(const MmaTiling& c) { return (size_t)4 * c.mi * (c.mi == 2 ? 3 : 4) * 16 * 32 * c.wm; }       // of Slots (pw_mma.cuh), both operands
+// The form is built for what is launched: gradients with a transform, whose blocks of 64 columns bwd_choose offers one pixel tile a warp, and large sums, for which fwd_choose takes two.
+constexpr bool deep_form(bool bwd, int mi, int nj, int xf) { return nj == 8 && (bwd ? mi == 1 && xf != XF_NONE : mi == 2 && xf == XF_SUM); }
 // The slots lie behind the coefficients that the transform has, not the most it could have: the 8 KB of two CTAs decide whether gradients of 512 channels in blocks of 64 columns fit two to a
 // multiprocessor (ResNet stage at batch 32 19 830 -> 19 636 us a round).  Five steps ahead instead of three: 19 855.
 size_t deep_smem(bool bwd, int K, const MmaTiling& c, int xf) {
     const size_t Kp = (size_t)(K + 31) / 32 * 32;
-    return mma_smem(bwd, K, c) - (bwd && xf != XF_ACT ? 8 * Kp : 0) + (xf == XF_SUM ? 4 * Kp : 0) + slot_bytes(c);
+    return mma_smem(bwd, K, c) - (bwd && xf != XF_ACT ? 8 * Kp : 0) + (xf == XF_SUM ? 4 * Kp : 0) + (size_t)(c.mi == 1 ? Slots<1>::BYTES : Slots<2>::BYTES) * 32 * c.wm;
 }
 // Two kinds of gradients gain only where their operands, 32 MB and more, come from beyond L2 in good part: rows that are no whole 32-byte sectors (the copies pass L1 by, where a load in
 // registers finds the sector it shares with the row before), and, on the small maps of one CTA of eight warps, those behind an activation that is not in them yet.  A unit's forward and backward,
@@ -35,13 +35,13 @@ size_t deep_smem(bool bwd, int K, const MmaTiling& c, int xf) {
 // at 25 088 44.5 against 44.6).
 bool deep_layer(bool bwd, int P, int K, const MmaTiling& c, int xf) {
     const size_t smem = deep_smem(bwd, K, c, xf);
-    return c.wk == 1 && deep_form(bwd, c.nj, xf) && K >= 128 && (!bwd || (K % 16 == 0 && (xf == XF_AFFINE || P >= 20000)) || (size_t)P * K >= (size_t)8 << 20) && smem <= SMEM_MOST &&
+    return c.wk == 1 && deep_form(bwd, c.mi, c.nj, xf) && K >= 128 && (!bwd || (K % 16 == 0 && (xf == XF_AFFINE || P >= 20000)) || (size_t)P * K >= (size_t)8 << 20) && smem <= SMEM_MOST &&
            (smem + 1024) * c.ctas <= 227 * 1024;
 }
 
 template <bool BWD, int NJ, int G, int XF> KernelFn pick(int mi, int wk, bool deep) {
-    if constexpr (deep_form(BWD, NJ, XF))
-        if (wk == 1 && deep) return mi == 1 ? pw_mma_kernel<BWD, 1, NJ, G, XF, true> : pw_mma_kernel<BWD, 2, NJ, G, XF, true>;
+    if constexpr (deep_form(BWD, 1, NJ, XF))
+        if (deep && mi == 1 && wk == 1) return pw_mma_kernel<BWD, 1, NJ, G, XF, true>;
     if (wk == 1) return mi == 1 ? pw_mma_kernel<BWD, 1, NJ, G, XF, false> : pw_mma_kernel<BWD, 2, NJ, G, XF, false>;
     return wk == 2 ? pw_mma_split_kernel<BWD, NJ, G, 2, XF> : wk == 4 ? pw_mma_split_kernel<BWD, NJ, G, 4, XF> : pw_mma_split_kernel<BWD, NJ, G, 8, XF>;
 }
@@ -55,7 +55,7 @@ template <bool BWD, int XF> KernelFn by_columns(const MmaTiling& c, bool deep) {
     }
 }
 template <bool BWD> KernelFn kernel_for(const MmaTiling& c, int xf, bool deep) {
-    if (!BWD && xf == XF_SUM) return c.mi == 1 ? pw_mma_kernel<false, 1, 8, 4, XF_SUM, true> : pw_mma_kernel<false, 2, 8, 4, XF_SUM, true>;
+    if (!BWD && xf == XF_SUM) return pw_mma_kernel<false, 2, 8, 4, XF_SUM, true>;
     if (!BWD && xf == XF_ADD) return by_columns<false, XF_ADD>(c, deep);
     return xf == XF_NONE ? by_columns<BWD, XF_NONE>(c, deep) : xf == XF_AFFINE ? by_columns<BWD, XF_AFFINE>(c, deep) : by_columns<BWD, XF_ACT>(c, deep);
 }

@@ -313,16 +313,17 @@ template <> struct SumCoef<true> {
 // ---------------------------------------------------------------------------------------------------------------------
 // Large maps: CTAs walk down the pixel tiles, every warp has 16*MI pixels x 8*NJ columns and the whole reduction.
 //
-// A chunk of 32 channels is a step, whose operands are requested one step ahead, in registers.  DEEP: two or three steps ahead, by asynchronous copies into shared-memory slots that no
-// other thread reads, so that no barrier is needed.
-template <bool BWD, int MI, int XF> struct Slots {
-    static constexpr bool USE_Z = BWD ? XF != XF_NONE : xf_sum(XF);
-    static constexpr int VECS = MI * 2 * (USE_Z ? 2 : 1), STEPS = VECS >= 8 ? 3 : 4;      // 16-byte vectors a thread and step, steps there is room for
+// A chunk of 32 channels is a step, whose operands are requested one step ahead, in registers.  DEEP (two operands): two or three steps ahead, by asynchronous copies into shared-memory slots that
+// no other thread reads, so that no barrier is needed.
+template <int MI> struct Slots {
+    static constexpr int VECS = MI * 4, STEPS = VECS >= 8 ? 3 : 4;      // 16-byte vectors a thread and step, steps there is room for
+    static constexpr int BYTES = VECS * STEPS * 16;                     // of a thread
 };
 template <bool BWD, int MI, int NJ, int G, int XF, bool DEEP>
 __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
-    using S = Slots<BWD, MI, XF>;
-    constexpr bool USE_Z = S::USE_Z;
+    using S = Slots<MI>;
+    constexpr bool USE_Z = BWD ? XF != XF_NONE : xf_sum(XF);
+    static_assert(USE_Z || !DEEP, "slots are laid out for two operands");
     constexpr int D = S::STEPS;
     extern __shared__ __align__(16) uint8_t sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -362,11 +363,8 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
             for (int h = 0; h < 2; ++h) {
                 if constexpr (DEEP) {
                     cp_async16(d, pa + (size_t)(roff[mi][h] + o), true);
-                    d += pitch;
-                    if (USE_Z) {
-                        cp_async16(d, pz + (size_t)(roff[mi][h] + o), true);
-                        d += pitch;
-                    }
+                    cp_async16(d + pitch, pz + (size_t)(roff[mi][h] + o), true);
+                    d += 2 * pitch;
                 } else {
                     nx[mi][h] = *reinterpret_cast<const uint4*>(pa + (size_t)(roff[mi][h] + o));
                     if (USE_Z) nz[mi][h] = *reinterpret_cast<const uint4*>(pz + (size_t)(roff[mi][h] + o));
@@ -452,8 +450,8 @@ __global__ void __launch_bounds__(256) pw_mma_kernel(const Args a) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         nx[mi][h] = *reinterpret_cast<const uint4*>(q);
-                        if (USE_Z) nz[mi][h] = *reinterpret_cast<const uint4*>(q + pitch);
-                        q += pitch * (USE_Z ? 2 : 1);
+                        nz[mi][h] = *reinterpret_cast<const uint4*>(q + pitch);
+                        q += 2 * pitch;
                     }
                 if (++slot == D) slot = 0;
             }

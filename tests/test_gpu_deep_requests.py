@@ -1,6 +1,6 @@
-"""Pointwise layers whose operands are requested several steps ahead: input gradients of 128 channels and more at reductions that end inside a 32-channel chunk, with fewer steps than
-slots, several tiles a CTA and a last one partly filled, with and without an activation behind the BatchNorm (whose gradient then is not stored masked: the layer is the last); residual sums of more than 4 M
-elements that the layer behind forms as it loads, and ones that it does not (three column tiles, a short reduction)."""
+"""Pointwise layers whose operands are requested several steps ahead.  Input gradients: reductions that end inside a 32-channel chunk, several tiles a CTA and a last one partly filled, CTAs of
+four and of eight warps, one and several column blocks, with a residual's addend, with the sums of a BatchNorm in front, with and without an activation that the gradient was not stored behind (the
+layer is the last).  Residual sums of more than 4 M elements that the layer behind forms as it loads.  And layers just outside these rules.  Each test reads from a profile which form ran."""
 import pytest
 
 import stage_inputs as si
@@ -90,11 +90,27 @@ def test_input_gradients(name):
     assert mine["block"][0] == threads and -(-h * w * B // (threads // 2)) >= tiles * mine["grid"][0]
 
 
-# formed by the layer: 256 -> 64 and 264 -> 40 on 16 510 pixels; not: 256 -> 136 (more columns than a CTA takes), 128 -> 64 on 33 020
-@pytest.mark.parametrize("c, c_out, B", [(256, 64, 1), (264, 40, 1), (256, 136, 1), (128, 64, 2)])
+SUMS = {
+    # channels of the sum, columns of the layer behind, h, w, micro-batch: formed by that layer?
+    "tile_tail": (256, 64, 61, 935, 1, True),
+    "chunk_tail_column_tail": (264, 56, 57013, 1, 1, True),
+    "long": (512, 64, 40, 977, 1, True),
+    "four_chunks": (128, 64, 100, 119, 5, True),
+    "columns_of_three_CTAs": (256, 136, 130, 127, 1, False),
+    "blocks_of_48_columns": (264, 40, 130, 127, 1, False),
+    "fewer_tiles_than_CTAs": (128, 64, 130, 127, 2, False),
+    "short": (120, 64, 57013, 1, 1, False),
+}
+
+
+@pytest.mark.parametrize("name", list(SUMS))
 @pytest.mark.parametrize("relu", [False, True])
-def test_large_sums(c, c_out, B, relu):
+def test_large_sums(name, relu):
+    c, c_out, h, w, B, formed = SUMS[name]
     net = [L("conv", 16, c, 1, 1, 0, -1, -1), L("bn", c, c, 0, 1, 0, 0, -1), L("conv", 16, c, 1, 1, 0, -1, -1), L("bn", c, c, 0, 1, 0, 2, -1), L("add", c, c, 0, 1, 0, 3, 1)]
     net += [L("relu", c, c, 0, 1, 0, 4, -1)] if relu else []
     net += [L("conv", c, c_out, 1, 1, 0, len(net) - 1, -1), L("bn", c_out, c_out, 0, 1, 0, len(net), -1)]
-    _check(net, 130, 127, B, "sum_%d_%d_%s" % (c, c_out, relu), relu)
+    assert c * h * w * B > 1 << 22
+    with kernels() as found:
+        _check(net, h, w, B, "sum_%s_%s" % (name, relu), relu)
+    assert _ahead(found, False).count(True) == int(formed)

@@ -89,7 +89,8 @@ uint32_t w_pitch(int K) {
 // and the issue time of all warps on the multiprocessor, per 32-channel chunk and column tile, plus the epilogue, which an addend makes longer;
 // weights are staged once per CTA.  Split form: one tile per CTA, waves over the chip.  Offered are the tilings that won somewhere: with two
 // pixel tiles per warp one CTA of eight warps or two of four; eight column tiles per warp only with one pixel tile (the epilogue holds four
-// vectors per column tile).  Before the model (one rule as in the forward): 128 -> 512 at 25 088 pixels 57.6 -> 52.2 us, 64 -> 64 at 100 352
+// vectors per column tile).  The timings are of kernels that request one step ahead; gradients that request several (deep_layer) take the tiling that the model names and were not fitted
+// again.  Before the model (one rule as in the forward): 128 -> 512 at 25 088 pixels 57.6 -> 52.2 us, 64 -> 64 at 100 352
 // 27.5 -> 21.4, 160 -> 960 at 784 8.1 -> 6.0, 384 -> 64 at 3136 10.5 -> 6.7.
 bool bwd_choose(int P, int K, int N, MmaTiling* out) {
     const int KCH = (K + 31) / 32, sms = sm_count();

@@ -27,15 +27,14 @@ size_t deep_smem(bool bwd, int K, const MmaTiling& c, int xf) {
     const size_t Kp = (size_t)(K + 31) / 32 * 32;
     return mma_smem(bwd, K, c) - (bwd && xf != XF_ACT ? 8 * Kp : 0) + (xf == XF_SUM ? 4 * Kp : 0) + (size_t)(c.mi == 1 ? Slots<1>::BYTES : Slots<2>::BYTES) * 32 * c.wm;
 }
-// Two kinds of gradients gain only where their operands, 32 MB and more, come from beyond L2 in good part: rows that are no whole 32-byte sectors (the copies pass L1 by, where a load in
-// registers finds the sector it shares with the row before), and, on the small maps of one CTA of eight warps, those behind an activation that is not in them yet.  A unit's forward and backward,
-// one step ahead against several (reduction -> columns of the gradient): 136 -> 256 at 10 000 pixels 49.8 us against 50.2, with a ReLU 52.0 against 53.0, but 264 -> 512 at 57 000 410 against 377;
-// with a ReLU 384 -> 512 at 10 000 165 against 167, at 57 000 524 against 495.  On larger maps a ReLU's short reductions stay alone (128 -> 512 at 25 088 pixels 103.7 either way) but gain beside
-// weight gradients: without them the ResNet stage at batch 32 takes 19 686 us a round instead of 19 521.  All others gain from 5 000 pixels on (512 -> 512 104.2 against 101.8) or stay (128 -> 64
-// at 25 088 44.5 against 44.6).
+// Rows that are no whole 32-byte sectors gain only where the two operands, 32 MB and more, come from beyond L2 in good part: the copies pass L1 by, where a load in registers finds the sector it
+// shares with the row before.  A unit's forward and backward, one step ahead against several (reduction -> columns of the gradient): 136 -> 256 at 10 000 pixels 49.8 us against 50.2, with a ReLU
+// 52.0 against 53.0, but 264 -> 512 at 57 000 410 against 377.  All others gain from 5 000 pixels on (512 -> 512 104.2 against 101.8) or stay (128 -> 64 at 25 088 44.5 against 44.6).  Behind an
+// activation that is not in them yet, small maps lose up to 1 us of 50 to 170 alone, but gain beside weight gradients: rounds of the ResNet stage, four micro-batches, without them below 20 000
+// pixels 5 494 us instead of 5 489 (10 192 pixels), 7 015 instead of 6 989 (15 680); of 32 samples without them below 8 M elements 19 686 instead of 19 521 (eight micro-batches).
 bool deep_layer(bool bwd, int P, int K, const MmaTiling& c, int xf) {
     const size_t smem = deep_smem(bwd, K, c, xf);
-    return c.wk == 1 && deep_form(bwd, c.mi, c.nj, xf) && K >= 128 && (!bwd || (K % 16 == 0 && (xf == XF_AFFINE || P >= 20000)) || (size_t)P * K >= (size_t)8 << 20) && smem <= SMEM_MOST &&
+    return c.wk == 1 && deep_form(bwd, c.mi, c.nj, xf) && K >= 128 && (!bwd || K % 16 == 0 || (size_t)P * K >= (size_t)8 << 20) && smem <= SMEM_MOST &&
            (smem + 1024) * c.ctas <= 227 * 1024;
 }
 

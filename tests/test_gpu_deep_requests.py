@@ -70,8 +70,9 @@ GRADIENTS = {
     "activation": (256, 264, "relu", None, 171, 193, 1, True, 128, 4, 6),
     "activation_relu6": (320, 272, "relu6", "behind", 171, 193, 1, True, 128, 5, 8),
     "activation_short": (512, 128, "relu", None, 28, 28, 32, True, 128, 8, 10),
-    # one step ahead: an activation or split sectors on smaller maps, short reductions, one tile a CTA
-    "activation_small": (256, 136, "relu", None, 109, 92, 1, False, 256, 4, 2),
+    "activation_eight_warps": (256, 144, "relu", None, 209, 79, 1, True, 256, 4, 3),
+    # one step ahead: rows that split sectors on smaller maps, short reductions, one tile a CTA
+    "split_sectors_activation": (256, 136, "relu", None, 109, 92, 1, False, 256, 4, 2),
     "split_sectors_small": (256, 136, None, None, 25, 1000, 1, False, 128, 4, 5),
     "short": (64, 120, None, None, 57013, 1, 1, False, 128, 1, 3),
     "one_tile": (64, 128, None, None, 13, 1000, 1, False, 256, 1, 1),

@@ -15,11 +15,12 @@ typedef void (*KernelFn)(const Args);
 constexpr size_t SMEM_MOST = 200 * 1024;
 // Whether a persistent layer's operands are requested several steps ahead (pw_mma.cuh): input gradients of 128 channels and more in blocks of 64 columns and the large residual sums of
 // defers_add (stage.cu), where a CTA has more than one tile.  Both read two operands, and a step took 0.75 to 1 us, a trip to memory, whatever its work was: ResNet stage at batch 32
-// 20 566 -> 19 614 us a round.  A forward of one operand has its steps in time, and slots only add a store and a load of shared memory a vector: 128 -> 512 at 25 088 pixels 27.3 -> 29.9 us,
+// 20 592 -> 19 523 us a round.  A forward of one operand has its steps in time, and slots only add a store and a load of shared memory a vector: 128 -> 512 at 25 088 pixels 27.3 -> 29.9 us,
 // 256 -> 512 39.3 -> 43.7, 256 -> 64 at 57 000 19.0 -> 21.0 (that stage with such forwards 19 735 instead of 19 622).  Only operands beyond L2 gain there: 512 -> 64 from 94 000 pixels on,
 // 49 -> 43.  In narrower blocks one step ahead is as good or better too: slots in all persistent kernels took half of MobileNetV2 with the head 4140 -> 4210 us, EfficientNet 6941 -> 7029,
 // the ragged stage 613 -> 637; input gradients in narrower blocks EfficientNet 6955 -> 6994 from 128 channels on, 6936 -> 6955 from 256; single tiles the ragged ResNet share 1681 -> 1689.
-// The form is built for what is launched: gradients with a transform, whose blocks of 64 columns bwd_choose offers one pixel tile a warp, and large sums, for which fwd_choose takes two.
+// The form is built for what is launched: gradients with a transform (the others have one operand), whose blocks of 64 columns bwd_choose offers one pixel tile a warp, and large sums, for which
+// fwd_choose takes two.  Where the slots do not fit beside the weights and coefficients, one step ahead stays: gradients of 512 channels behind an unapplied activation, two CTAs.
 constexpr bool deep_form(bool bwd, int mi, int nj, int xf) { return nj == 8 && (bwd ? mi == 1 && xf != XF_NONE : mi == 2 && xf == XF_SUM); }
 // The slots lie behind the coefficients that the transform has, not the most it could have: the 8 KB of two CTAs decide whether gradients of 512 channels in blocks of 64 columns fit two to a
 // multiprocessor (ResNet stage at batch 32 19 830 -> 19 636 us a round).  Five steps ahead instead of three: 19 855.
@@ -30,7 +31,7 @@ size_t deep_smem(bool bwd, int K, const MmaTiling& c, int xf) {
 // Rows that are no whole 32-byte sectors gain only where the two operands, 32 MB and more, come from beyond L2 in good part: the copies pass L1 by, where a load in registers finds the sector it
 // shares with the row before.  A unit's forward and backward, one step ahead against several (reduction -> columns of the gradient): 136 -> 256 at 10 000 pixels 49.8 us against 50.2, with a ReLU
 // 52.0 against 53.0, but 264 -> 512 at 57 000 410 against 377.  All others gain from 5 000 pixels on (512 -> 512 104.2 against 101.8) or stay (128 -> 64 at 25 088 44.5 against 44.6).  Behind an
-// activation that is not in them yet, small maps lose up to 1 us of 50 to 170 alone, but gain beside weight gradients: rounds of the ResNet stage, four micro-batches, without them below 20 000
+// activation that is not in them yet, small maps lose up to 1.4 us of 50 to 170 alone, but gain beside weight gradients: rounds of the ResNet stage, four micro-batches, without them below 20 000
 // pixels 5 494 us instead of 5 489 (10 192 pixels), 7 015 instead of 6 989 (15 680); of 32 samples without them below 8 M elements 19 686 instead of 19 521 (eight micro-batches).
 bool deep_layer(bool bwd, int P, int K, const MmaTiling& c, int xf) {
     const size_t smem = deep_smem(bwd, K, c, xf);
@@ -183,7 +184,7 @@ bool fwd_choose(int P, int K, int N, MmaTiling* out) {
 // 256 channels a side.  There the arithmetic of mma.sync (and the shared-memory reads of its weights) is the bound and the tensor-memory
 // pipeline of pw_tc.cu is as fast or faster: 64 -> 256 at 100 352 pixels 26.3 us against 29.3, backward to 256 channels 71 against 77.  To at
 // most 64 channels it is not: 256 -> 64 30.6 against 24.0, backward 45 against 42.  (One layer with its BatchNorm sums in a captured chain.)  Requests several steps ahead do not move the
-// line: with 256 -> 128 forward here the ResNet stage at batch 32 takes 19 660 us a round, with its backward 19 671, without 19 611.
+// line: with them and 256 -> 128 forward here the ResNet stage at batch 32 takes 19 660 us a round, with its backward 19 671, without 19 611.
 // With 192 to 256 channels on both sides the pipeline does not fit and pw_stream.cu and the one-tile kernel take the layer: 256 -> 256 on 50 176
 // pixels forward 33 us with its pass for the sums (37 here), backward with a transform 49 (72), without 23 (49).
 bool mma_choose(bool bwd, int P, int K, int N, MmaTiling* out) {

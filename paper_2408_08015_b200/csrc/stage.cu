@@ -635,8 +635,9 @@ static bool f32_unit(const asteroid_stage* s, const Unit& u, bool bwd, F32Tiling
 // A residual sum of two tensors without activations of their own, read next by a pointwise layer on the register-operand or float32
 // kernels: that layer forms it as it loads, and writes it out for the others.  Up to 4 M elements, where the sum is mostly a launch in the chain (a
 // round of a sixth of MobileNetV2 at batch 4 1681 -> 1647 us, of small images 1469 -> 1440); beyond, where every CTA of that layer takes all of its columns and has a reduction
-// long enough to request several steps ahead (pw_mma.cu): each operand is then read once, and the sum not again.  ResNet stage at batch 32, with such requests in all persistent layers: no large
-// sum left to the layer behind 19 871 us a round, all of them 19 651, those of 12.8 M elements in front of 512 -> 128 alone, whose columns take three CTAs, 20 055.
+// long enough to request several steps ahead (pw_mma.cu): each operand is then read once, and the sum not again.  In front of 256 -> 64, pass and layer 40.9 -> 28.5 us at 57 000 pixels,
+// 61.6 -> 39.3 at 100 352.  ResNet stage at batch 32, with such requests in all persistent layers: no large sum left to the layer behind 19 871 us a round, all of them 19 651, those of
+// 12.8 M elements in front of 512 -> 128 alone, whose columns take three CTAs, 20 055.
 // The value is the elementwise pass's: beyond 4 M elements to the bit, up to there but for the shifts, which are added first.
 static bool small_sum(const Val& sum) { return sum.elems <= (size_t)4 << 20; }
 static bool defers_add(const asteroid_stage* s, size_t ui) {
